@@ -334,20 +334,29 @@ __global__ void pair_correct_kernel(double *__restrict__ out, const double *__re
 }
 
 // ---------------------------------------------------------------------------
-// FP32 CUDA-core Gram over upper-triangle tiles of 128 x 128 items.
+// FP32 CUDA-core Gram over units (tile of 128 x 128 items of the upper
+// triangle, range of columns): unit u is range u / n_tiles of tile
+// u % n_tiles, so the units in flight read the same columns.
 // 256 threads, 8 x 8 outputs per thread (FP32x2 FMAs), K staged 16 at a
-// time through registers into transposed, double-buffered shared memory.
+// time through registers into transposed, double-buffered shared memory; two
+// CTAs per SM.  Bound by the FMA pipe, 0.80 of its measured rate inside a
+// full wave.  (Even and odd columns of one output in the two halves of an
+// FMA, operands staged untransposed by cp.async, ran 0.71 with 8 x 8 outputs
+// per thread and 0.62 with 8 x 4: an FMA2 with three distinct register pairs
+// issues slower than one that reuses a splatted operand.)
 // ---------------------------------------------------------------------------
 constexpr int kF32Tile = 128;
 constexpr int kF32K = 16;
 constexpr int kF32Pad = 4;
 
-template <int COVER>
+// PARTIAL = 1: the unit's partial Gram is added into FP64 `out` (zeroed by
+// the caller, scaled by the pass that follows); 0: whole tiles, scaled here.
+template <int COVER, int PARTIAL>
 __global__ void __launch_bounds__(256, 2)
 gram_f32_kernel(const float *__restrict__ C, int64_t n, int64_t Dp,
                 const double *__restrict__ rs, const int32_t *__restrict__ tiles,
-                int64_t n_tiles, int32_t *queue, void *out, const double *__restrict__ delta,
-                double dcorr) {
+                int32_t n_tiles, int32_t k_split, int32_t *queue, void *out,
+                const double *__restrict__ delta, double dcorr) {
   __shared__ __align__(16) float As[2][kF32K][kF32Tile + kF32Pad];
   __shared__ __align__(16) float Bs[2][kF32K][kF32Tile + kF32Pad];
   __shared__ int s_tile;
@@ -358,9 +367,12 @@ gram_f32_kernel(const float *__restrict__ C, int64_t n, int64_t Dp,
   for (;;) {
     if (tid == 0) s_tile = atomicAdd(queue, 1);
     __syncthreads();
-    const int64_t t = s_tile;
+    const int u = s_tile;
     __syncthreads();
-    if (t >= n_tiles) break;
+    if (u >= n_tiles * k_split) break;
+    const int range = u / n_tiles, t = u - range * n_tiles;
+    const int kb0 = (int)((int64_t)range * nk / k_split);
+    const int kb1 = (int)((int64_t)(range + 1) * nk / k_split);
     const int64_t i0 = (int64_t)tiles[2 * t] * kF32Tile;
     const int64_t j0 = (int64_t)tiles[2 * t + 1] * kF32Tile;
     // blocked copy: block (row block, k block) = 128 rows x 16 columns, contiguous
@@ -395,12 +407,12 @@ gram_f32_kernel(const float *__restrict__ C, int64_t n, int64_t Dp,
       }
     };
 
-    gload(0);
-    sstore(0);
+    gload(kb0);
+    sstore(kb0 & 1);
     __syncthreads();
-    for (int kb = 0; kb < nk; ++kb) {
+    for (int kb = kb0; kb < kb1; ++kb) {
       const int buf = kb & 1;
-      if (kb + 1 < nk) gload(kb + 1);
+      if (kb + 1 < kb1) gload(kb + 1);
 #pragma unroll
       for (int k = 0; k < kF32K; ++k) {
         float4 a0 = *reinterpret_cast<const float4 *>(&As[buf][k][ty * 4]);
@@ -417,30 +429,55 @@ gram_f32_kernel(const float *__restrict__ C, int64_t n, int64_t Dp,
           for (int b = 0; b < 4; ++b) acc[a][b] = __ffma2_rn(aa, bv[b], acc[a][b]);
         }
       }
-      if (kb + 1 < nk) sstore(buf ^ 1);
+      if (kb + 1 < kb1) sstore(buf ^ 1);
       __syncthreads();
     }
 
-    // epilogue: r = G * rs_i * rs_j in FP64, strict upper triangle only
+    // epilogue, strict upper triangle only: r = (G - D delta_i delta_j) rs_i
+    // rs_j in FP64, or the partial sums as they are
+    const int ni = (int)(n - i0 < kF32Tile ? n - i0 : kF32Tile);
+    const int nj = (int)(n - j0 < kF32Tile ? n - j0 : kF32Tile);
 #pragma unroll
     for (int a = 0; a < 8; ++a) {
-      const int64_t i = i0 + (a < 4 ? ty * 4 + a : 64 + ty * 4 + (a - 4));
-      if (i >= n) continue;
-      const double ri = COVER ? 0.0 : rs[i];
-      const double di = (COVER || !delta) ? 0.0 : dcorr * delta[i];
+      const int il = (a < 4 ? a : 60 + a) + ty * 4;
+      if (il < ni) {
+        const int64_t i = i0 + il;
+        const int first = (int)(i - j0) + 1;        // pairs need j0 + jl > i
+        const int64_t p0 = pair_index(i, j0, n);
+        const double ri = (COVER || PARTIAL) ? 0.0 : rs[i];
+        const double di = (COVER || PARTIAL || !delta) ? 0.0 : dcorr * delta[i];
 #pragma unroll
-      for (int b = 0; b < 8; ++b) {
-        const int64_t j = j0 + (b < 4 ? tx * 4 + b : 64 + tx * 4 + (b - 4));
-        if (j >= n || j <= i) continue;
-        const int64_t p = pair_index(i, j, n);
-        if (COVER) atomicAdd(reinterpret_cast<int32_t *>(out) + p, 1);
-        else
-          reinterpret_cast<double *>(out)[p] =
-              ((double)((b & 1) ? acc[a][b >> 1].y : acc[a][b >> 1].x) -
-               (delta ? di * delta[j] : 0.0)) * ri * rs[j];
+        for (int b = 0; b < 8; ++b) {
+          const int jl = (b < 4 ? b : 60 + b) + tx * 4;
+          if (jl >= nj || jl < first) continue;
+          const float g = (b & 1) ? acc[a][b >> 1].y : acc[a][b >> 1].x;
+          if (COVER) atomicAdd(reinterpret_cast<int32_t *>(out) + p0 + jl, 1);
+          else if (PARTIAL) atomicAdd(reinterpret_cast<double *>(out) + p0 + jl, (double)g);
+          else
+            reinterpret_cast<double *>(out)[p0 + jl] =
+                ((double)g - (delta ? di * delta[j0 + jl] : 0.0)) * ri * rs[j0 + jl];
+        }
       }
     }
   }
+}
+
+// Column ranges per tile of the FP32 Gram on `slots` co-resident CTAs.  The
+// units are equal, so a run costs ceil(units / slots) of them; a unit costs
+// its 16-column blocks and about kF32UnitBlocks more (first loads, epilogue),
+// twice that where it adds FP64 partials.  The smallest product wins; 1 keeps
+// whole tiles, written once.  (1024 x 65,536: 36 tiles on 304 slots took 5.64
+// ms, 288 units 1.37 ms; 4096 x 2^17: 528 tiles in two waves, the second three
+// quarters full, 40.6 ms, 35.1 ms in ranges.)
+int32_t f32_k_split(int64_t n_tiles, int64_t nk, int64_t slots) {
+  constexpr int64_t kF32UnitBlocks = 12, kMost = 64;
+  int64_t best = 1, cost = INT64_MAX;
+  for (int64_t k = 1; k <= std::min(nk, kMost); ++k) {
+    const int64_t c = ((n_tiles * k + slots - 1) / slots) *
+                      ((nk + k - 1) / k + (k > 1 ? 2 : 1) * kF32UnitBlocks);
+    if (c < cost) { cost = c; best = k; }
+  }
+  return (int32_t)best;
 }
 
 }  // namespace
@@ -579,20 +616,33 @@ cudaError_t launch_gram_f32(const float *C, int64_t n, int64_t Dp, const double 
   // issuing where 8 left it idle a third of the time)
   int per_sm = 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-          &per_sm, coverage ? gram_f32_kernel<1> : gram_f32_kernel<0>, 256, 0) != cudaSuccess ||
+          &per_sm, coverage ? gram_f32_kernel<1, 0> : gram_f32_kernel<0, 1>, 256, 0) !=
+          cudaSuccess ||
       per_sm < 1) {
     cudaGetLastError();
     per_sm = 1;
   }
-  int64_t grid = (int64_t)num_sms() * per_sm;
-  if (grid > n_tiles) grid = n_tiles;
+  const int64_t slots = (int64_t)num_sms() * per_sm;
+  const int32_t k_split = coverage ? 1 : f32_k_split(n_tiles, Dp / kF32K, slots);
+  if (n_tiles * k_split > INT32_MAX / 2) return cudaErrorInvalidValue;
+  if (k_split > 1) {
+    e = cudaMemsetAsync(out, 0, (size_t)(n * (n - 1) / 2) * sizeof(double), s);
+    if (e != cudaSuccess) return e;
+  }
+  const int grid = (int)std::min<int64_t>(slots, n_tiles * k_split);
+  const int32_t nt = (int32_t)n_tiles;
   if (coverage)
-    gram_f32_kernel<1><<<(int)grid, 256, 0, s>>>(C, n, Dp, rs, tiles, n_tiles, queue, out, delta,
-                                                 (double)D);
+    gram_f32_kernel<1, 0><<<grid, 256, 0, s>>>(C, n, Dp, rs, tiles, nt, 1, queue, out, delta,
+                                               (double)D);
+  else if (k_split == 1)
+    gram_f32_kernel<0, 0><<<grid, 256, 0, s>>>(C, n, Dp, rs, tiles, nt, 1, queue, out, delta,
+                                               (double)D);
   else
-    gram_f32_kernel<0><<<(int)grid, 256, 0, s>>>(C, n, Dp, rs, tiles, n_tiles, queue, out, delta,
-                                                 (double)D);
-  return cudaGetLastError();
+    gram_f32_kernel<0, 1><<<grid, 256, 0, s>>>(C, n, Dp, rs, tiles, nt, k_split, queue, out, delta,
+                                               (double)D);
+  e = cudaGetLastError();
+  if (e != cudaSuccess || k_split == 1) return e;
+  return launch_pair_finalize(reinterpret_cast<double *>(out), rs, delta, n, D, s);
 }
 
 }  // namespace ap

@@ -43,6 +43,20 @@ def test_pearson_all_pairs_match_oracle(ap, oracle_lib, n, D):
             assert np.abs(got - ref).max() <= PEARSON_ATOL
 
 
+@pytest.mark.parametrize("n,D", [(130, 1000),     # a ragged second tile, 2 ranges of blocks
+                                 (385, 4100),     # ranges that do not divide the row
+                                 (128, 70000),    # one tile, the most ranges
+                                 (900, 17)])      # whole tiles: rows of a single range
+def test_pearson_fp32_column_ranges(ap, oracle_lib, n, D):
+    """The FP32 Gram's split of a tile's columns into ranges, whose partial
+    sums meet in FP64, and the whole tiles of short rows."""
+    X = synth.vectors_grouped(n, D, seed=n)
+    pi, pj = oracle_lib.all_pairs(n)
+    ref = oracle_lib.pearson(X.numpy(), pi, pj)
+    got = _run(ap, X, ap.AP_PREC_FP32, precisions=(ap.AP_PREC_FP32,))
+    assert np.all(np.abs(got - ref) <= pearson_tolerance(X.numpy(), pi, pj, ap.AP_PREC_FP32))
+
+
 @pytest.mark.parametrize("D", [4096, 1 << 16])
 def test_pearson_strongly_correlated(ap, oracle_lib, D):
     # long correlated chains: the accumulation must not drift (a single FP32

@@ -41,11 +41,72 @@ __host__ __device__ __forceinline__ int64_t pair_index(int64_t i, int64_t j, int
 
 // ---------------------------------------------------------------------------
 // point-cloud storage: items sorted by the planner, padded to a multiple of
-// 4 points; 2-D points packed as float4 {x, y, s2k, lw}, 3-D as
-// float4 {x, y, z, s2k} plus float lw[], where s2k = sigma^2 / (log2(e)/2)
-// and lw = log2(weight) (-inf for padding), so that
-//   w_b * exp(-d^2 / (2 (sa^2 + sb^2))) = 2^(lw_b - d^2 / (s2k_a + s2k_b)).
+// 4 points, held in pairs of points so that one packed FP32x2 operation takes
+// two of them as they lie: pair q (points 2q, 2q + 1) is
+//   2-D  {x0, x1, y0, y1} {s0, s1, l0, l1}
+//   3-D  {x0, x1, y0, y1} {z0, z1, s0, s1}, and {l0, l1} in lw[]
+// with s = s2k = -sigma^2 / (log2(e)/2) (negated) and l = log2(weight) (-inf
+// for padding), so that
+//   w_b * exp(-d^2 / (2 (sa^2 + sb^2))) = 2^(l_b + d^2 / (s_a + s_b)).
 // ---------------------------------------------------------------------------
+//
+// The a-side of the pair sums.  Four consecutive storage points (a group)
+// belong to one item; a warp job holds R points per lane.  An item's groups
+// split into fragments by its own size alone: runs of 8 R groups, each filling
+// a warp, then pieces of up to 8 groups.  Pieces of a block's items share
+// warps (four pieces of 8 groups at R = 4), so the lanes stay filled at any
+// item size; one partial sum per fragment and partner (a row).
+__host__ __device__ __forceinline__ int32_t cloud_rows(int64_t cnt, int32_t R) {
+  const int64_t g = (cnt + 3) / 4, full = 8 * R;
+  return (int32_t)(g / full + (g % full + 7) / 8);
+}
+// Lane descriptor: x = group of four storage points (-1: idle), y = row (10
+// bits), lane's place in its fragment (5), lanes of the fragment - 1 (5), item
+// of the block (5), points per lane 1 << re (2), first point of the group in
+// units of them (2).
+__host__ __device__ __forceinline__ int32_t pack_lane(int32_t row, int32_t t, int32_t len,
+                                                      int32_t il, int32_t re, int32_t sub) {
+  return row | t << 10 | (len - 1) << 15 | il << 20 | re << 25 | sub << 27;
+}
+// points per lane (as a power of two) of a job with `pieces` pieces of 8 groups
+__host__ __device__ __forceinline__ int32_t job_re(int32_t pieces) {
+  return pieces <= 1 ? 0 : pieces == 2 ? 1 : 2;
+}
+// lane `lane` of job k of a single item of G groups starting at group grp0
+__host__ __device__ __forceinline__ int2 cloud_lane_desc(int32_t k, int32_t lane, int32_t grp0,
+                                                         int32_t G, int32_t R, int32_t row0,
+                                                         int32_t il) {
+  const int32_t full = 8 * R, nfull = G / full;
+  int2 d;
+  if (k < nfull) {
+    const int32_t lpg = 4 / R;
+    d.x = grp0 + k * full + lane / lpg;
+    d.y = pack_lane(row0 + k, lane, 32, il, R == 4 ? 2 : 1, lane % lpg);
+    return d;
+  }
+  const int32_t rem = G - nfull * full, re = job_re((rem + 7) / 8), lpg = 4 >> re;
+  const int32_t gl = lane / lpg, in = gl < rem, left = rem - (gl & ~7);
+  d.x = in ? grp0 + nfull * full + gl : -1;
+  d.y = pack_lane(in ? row0 + nfull + (gl >> 3) : 0, in ? (gl & 7) * lpg + lane % lpg : 0,
+                  in ? (left < 8 ? left : 8) * lpg : 1, il, re, lane % lpg);
+  return d;
+}
+
+// a tile plan of a cloud set (plan.cpp): blocks, their warp jobs, the tiles
+struct CloudPlanHost {
+  std::vector<int32_t> bstart;      // block b = storage items [bstart[b], bstart[b+1])
+  std::vector<int32_t> bmeta;       // [blocks][8]: item begin, end, first group, groups,
+                                    // first job (-1: one item, see cloud_lane_desc), jobs,
+                                    // rows, 0; then the single items that tiles split at the
+                                    // end of the list take as their J side
+  std::vector<int32_t> desc;        // [jobs][32][2] lane descriptors
+  std::vector<int32_t> items;       // per stored item {first group, points, original id,
+                                    // first row in its block}
+  std::vector<int32_t> tiles;       // block pairs (I <= J), indices into bmeta
+  int32_t max_rows = 1, max_items = 1, max_pts = 4;
+  bool largest_first = false;
+};
+
 struct CloudStore {
   int dim = 2;
   int64_t n = 0;
@@ -55,26 +116,26 @@ struct CloudStore {
   std::vector<int64_t> h_poff;      // padded offsets in storage order [n+1]
   int64_t total_pts = 0;            // padded
   float4 *d_pts = nullptr;          // [total_pts]
-  float *d_lw = nullptr;            // [total_pts] (3-D with weights only)
+  float *d_lw = nullptr;            // [total_pts] (3-D only)
   int64_t *d_poff = nullptr;        // [n+1]
   int32_t *d_cnt = nullptr;         // [n] real points per stored item
-  int32_t *d_perm = nullptr;        // [n]
+  int32_t *d_perm = nullptr;        // [n] storage position -> original item id
   // tile plan (rebuilt when the tuned parameters change)
   int32_t block_items = 0, block_pts = 0, reg_r = 0;
-  int32_t max_rj = 0;               // most row jobs (chunks of 32 reg_r points) of a block
+  int32_t max_rows = 0, max_items = 0, max_pts = 0;   // of any block
   bool sorted = false;
   // pair lists: tiles are listed pairs of one-item blocks, outputs by list
   // position (set only on the temporary copy a list run launches with)
   bool list_mode = false;
   std::vector<int32_t> h_iperm;     // original item id -> storage position
-  int32_t *d_bstart_single = nullptr;   // [n + 1]: block b = item b
+  int32_t *d_bmeta_single = nullptr;    // [n][8]: block b = item b
   int32_t *d_list_tiles = nullptr;  // [list_cap][2] storage positions
   int64_t list_cap = 0;
-  std::vector<int32_t> h_bstart;    // block b = storage items [bstart[b], bstart[b+1])
-  int32_t *d_bstart = nullptr;
+  int32_t *d_bmeta = nullptr;       // as in CloudPlanHost
+  int32_t *d_desc = nullptr;
+  int32_t *d_items = nullptr;
   int32_t *d_tiles = nullptr;       // [n_tiles][2] block pairs (I <= J)
   int64_t n_tiles = 0;
-  int64_t tiles_cap = 0;
   // particle scores: re-scaled storage per score (index score - 1), built on
   // first use, and the GMM L2 self terms per original item
   float4 *d_pts_score[2] = {nullptr, nullptr};
@@ -295,10 +356,15 @@ namespace ap {
 void dc_block_pairs(int64_t nb, std::vector<int32_t> &out);
 // Group storage-ordered items into blocks of at most max_items items and
 // max_pts padded points (an item larger than max_pts forms its own block).
-// Blocks also respect max_chunks = sum over items of ceil(cnt / chunk).
+// Blocks of several items also respect max_rows partial rows (cloud_rows).
 void make_blocks(const std::vector<int64_t> &poff, const std::vector<int64_t> &cnt,
-                 int32_t max_items, int64_t max_pts, int64_t chunk, int64_t max_chunks,
+                 int32_t max_items, int64_t max_pts, int32_t reg_r, int64_t max_rows,
                  std::vector<int32_t> &bstart);
+// the whole tile plan: blocks, the packing of their items' pieces into warp
+// jobs, and the tiles in the order they are popped, the last split_tail of
+// them split into one tile per item of J
+void make_cloud_plan(const std::vector<int64_t> &poff, const std::vector<int64_t> &cnt,
+                     const std::vector<int32_t> &perm, int64_t split_tail, int32_t block_items, int32_t block_pts, int32_t reg_r, CloudPlanHost &out);
 
 // ---------------------------------------------------------------------------
 // kernel launchers
@@ -410,9 +476,6 @@ void tc_tiles(int64_t n, std::vector<int32_t> &tiles);   // (I-block of 128, J-b
 // first (point pairs per tile); returns whether it reordered
 bool order_cloud_tiles(const std::vector<int32_t> &bstart, const std::vector<int64_t> &cnt,
                        int64_t total_pts, std::vector<int32_t> &tiles);
-// the most row jobs (chunks of `chunk` points) any block of a cloud plan has
-int32_t max_row_jobs(const std::vector<int32_t> &bstart, const std::vector<int64_t> &cnt,
-                     int64_t chunk);
 // split-K units of the tiles: waves of `group` tiles, column range-major
 // inside each wave (k_split ranges of the nchunks 64-column chunks)
 void panel_units(const std::vector<int32_t> &tiles, int64_t nchunks, int64_t group,
@@ -456,12 +519,22 @@ ap_status create_sparse(const ap_items_desc *d, ap_items *it, cudaStream_t s);
 void free_sparse(SparseStore &sp);
 cudaError_t launch_sparse_cosine(const SparseStore &sp, double *out, int coverage,
                                  int32_t *queue, cudaStream_t s);
-constexpr int kOverlapMaxRowJobs = 128;   // chunks of one I block
+// words of a handle's d_queue block: [0] tile-queue head, [1] status word,
+// [2] scratch, and for clouds their own queue head (zero between launches:
+// the CTA that takes the last pop resets it) and traits of the set: some s2k
+// or coordinate is outside the range in which two terms may share a
+// reciprocal; some weight is not 1
+constexpr int kQueueClouds = 3, kQueueTraits = 4;
+constexpr int32_t kCloudWide = 1, kCloudWeighted = 2;
+// tiles at the end of a cloud plan's list that are split: one per CTA slot
+// (four CTAs of four warps per SM)
+constexpr int64_t kSplitTailPerSm = 4;
+constexpr int kOverlapMaxRows = 128;      // partial rows of a block of several items
 constexpr int kOverlapMaxBlockItems = 32;
 cudaError_t launch_cloud_pack(const float *x, const float *y, const float *z,
                               const float *sigma, const float *w, const int64_t *src_off,
                               const int32_t *perm, const int64_t *poff, int64_t n, int dim,
-                              float4 *pts, float *lw, cudaStream_t s);
+                              float4 *pts, float *lw, int32_t *traits, cudaStream_t s);
 
 int num_sms();
 
@@ -496,6 +569,11 @@ void dfree(T *&p) {
 struct CloudPlanChoice { int32_t block_items, block_pts, reg_r; bool sorted; };
 CloudPlanChoice choose_cloud_plan(const CloudStore &c);
 ap_status build_cloud_plan(ap_items *it, const CloudPlanChoice &ch, cudaStream_t s = nullptr);
+// copy a plan to the device into c (its plan buffers hold nothing before)
+ap_status upload_cloud_plan(CloudStore &c, const CloudPlanHost &h, cudaStream_t s);
+void free_cloud_plan(CloudStore &c);
+// per item of the set: {its block of one, 8 ints} as in CloudPlanHost::bmeta
+void single_item_blocks(const CloudStore &c, int32_t reg_r, std::vector<int32_t> &bmeta);
 // smallest a-points-per-lane that keeps the largest item within the row jobs
 int32_t min_reg_r(const CloudStore &c);
 

@@ -56,7 +56,7 @@ void free_items(ap_items *it) {
   cudaDeviceSynchronize();          // queued host functions may still use the host cache
   CloudStore &c = it->cl;
   dfree(c.d_pts); dfree(c.d_lw); dfree(c.d_poff); dfree(c.d_cnt); dfree(c.d_perm);
-  dfree(c.d_bstart); dfree(c.d_tiles); dfree(c.d_bstart_single); dfree(c.d_list_tiles);
+  free_cloud_plan(c); dfree(c.d_bmeta_single); dfree(c.d_list_tiles);
   for (int k = 0; k < 2; ++k) { dfree(c.d_pts_score[k]); dfree(c.d_lw_score[k]); }
   dfree(c.d_self);
   VecStore &v = it->vec;
@@ -93,48 +93,62 @@ CloudPlanChoice choose_cloud_plan(const CloudStore &c) {
   // uneven 3-D sets are sorted by size (transforms are 2-D only and need the
   // original order to know which item of a pair is moved)
   ch.sorted = (c.dim == 3) && mx > 4 * std::max<int64_t>(mn, 1);
-  // a-points per lane: enough chunk width for the largest item
-  ch.reg_r = std::max<int32_t>(2, min_reg_r(c));
-  ch.block_pts = 4096;
-  // block size: enough tiles to keep every SM busy several times over
-  const int64_t want_tiles = (int64_t)num_sms() * 16;
-  ch.block_items = kOverlapMaxBlockItems;
-  while (ch.block_items > 2) {
-    int64_t nb = (c.n + ch.block_items - 1) / ch.block_items;
-    if (nb * (nb + 1) / 2 >= want_tiles) break;
-    ch.block_items /= 2;
-  }
+  ch.reg_r = 4;
+  // blocks of about 1/60 of the points: 1800 tiles, 12 per SM before the last
+  // ones are split; at most kCloudBlockPts points, which one staging window
+  // holds.  Eight items at most: more would take shared memory for their
+  // partial sums from the CTAs.
+  constexpr int64_t kCloudBlockPts = 2048;
+  const int64_t want = (c.total_pts / 60 + 3) / 4 * 4;
+  ch.block_pts = (int32_t)std::min(std::max<int64_t>(want, 64), kCloudBlockPts);
+  ch.block_items = 8;
   return ch;
+}
+
+void free_cloud_plan(CloudStore &c) {
+  dfree(c.d_bmeta);
+  dfree(c.d_desc);
+  dfree(c.d_items);
+  dfree(c.d_tiles);
+}
+
+ap_status upload_cloud_plan(CloudStore &c, const CloudPlanHost &h, cudaStream_t s) {
+  // pageable sources: the copies are staged before the calls return
+  auto up = [&](int32_t **d, const std::vector<int32_t> &v) -> cudaError_t {
+    cudaError_t e = dmalloc(d, std::max<size_t>(v.size(), 8));
+    if (e == cudaSuccess && !v.empty())
+      e = cudaMemcpyAsync(*d, v.data(), v.size() * 4, cudaMemcpyHostToDevice, s);
+    return e;
+  };
+  AP_TRY(up(&c.d_bmeta, h.bmeta));
+  AP_TRY(up(&c.d_desc, h.desc));
+  AP_TRY(up(&c.d_items, h.items));
+  AP_TRY(up(&c.d_tiles, h.tiles));
+  c.n_tiles = (int64_t)h.tiles.size() / 2;
+  c.max_rows = h.max_rows;
+  c.max_items = h.max_items;
+  c.max_pts = h.max_pts;
+  return AP_OK;
 }
 
 ap_status build_cloud_plan(ap_items *it, const CloudPlanChoice &ch, cudaStream_t s) {
   CloudStore &c = it->cl;
   std::vector<int64_t> cnt(c.n);
   for (int64_t s = 0; s < c.n; ++s) cnt[s] = c.h_size[c.h_perm[s]];
-  std::vector<int32_t> bstart;
-  make_blocks(c.h_poff, cnt, ch.block_items, ch.block_pts, 32LL * ch.reg_r, kOverlapMaxRowJobs,
-              bstart);
-  std::vector<int32_t> tiles;
-  dc_block_pairs((int64_t)bstart.size() - 1, tiles);
-  const bool largest_first = order_cloud_tiles(bstart, cnt, c.total_pts, tiles);
-  dfree(c.d_bstart);
-  dfree(c.d_tiles);
-  AP_TRY(dmalloc(&c.d_bstart, bstart.size()));
-  AP_TRY(dmalloc(&c.d_tiles, std::max<size_t>(tiles.size(), 2)));
-  // pageable sources: the copies are staged before the calls return
-  AP_TRY(cudaMemcpyAsync(c.d_bstart, bstart.data(), bstart.size() * 4, cudaMemcpyHostToDevice, s));
-  if (!tiles.empty())
-    AP_TRY(cudaMemcpyAsync(c.d_tiles, tiles.data(), tiles.size() * 4, cudaMemcpyHostToDevice, s));
-  c.h_bstart = bstart;
-  c.max_rj = max_row_jobs(bstart, cnt, 32LL * ch.reg_r);
-  c.n_tiles = (int64_t)tiles.size() / 2;
+  CloudPlanHost h;
+  make_cloud_plan(c.h_poff, cnt, c.h_perm, kSplitTailPerSm * num_sms(), ch.block_items, ch.block_pts,
+                  ch.reg_r, h);
+  free_cloud_plan(c);
+  AP_TRY_ST(upload_cloud_plan(c, h, s));
   c.block_items = ch.block_items;
   c.block_pts = ch.block_pts;
+  // one-item blocks (pair lists) depend on the points per lane
+  if (c.reg_r != ch.reg_r) dfree(c.d_bmeta_single);
   c.reg_r = ch.reg_r;
   it->stats.tiles = c.n_tiles;
   it->stats.tile_m = ch.block_items;
   it->stats.tile_n = ch.block_items;
-  it->stats.order = largest_first ? 2 : 0;
+  it->stats.order = h.largest_first ? 2 : 0;
   ++it->plan_version;
   return AP_OK;
 }
@@ -158,9 +172,10 @@ ap_status create_clouds(const ap_items_desc *d, ap_items *it, cudaStream_t s) {
     return AP_ERR_INVALID_ARG;
   int64_t mx = 0;
   for (int64_t v : c.h_size) mx = std::max(mx, v);
-  if (mx > (int64_t)4 * 32 * kOverlapMaxRowJobs) return AP_ERR_UNSUPPORTED;   // > 16384 points
+  if (mx > (int64_t)4 * 32 * kOverlapMaxRows) return AP_ERR_UNSUPPORTED;   // > 16384 points
   c.unit_weights = (d->weight == nullptr);
 
+  for (int64_t v : c.h_size) c.total_pts += round_up(v, 4);
   CloudPlanChoice ch = choose_cloud_plan(c);
   c.sorted = ch.sorted;
   c.h_perm.resize(c.n);
@@ -176,7 +191,7 @@ ap_status create_clouds(const ap_items_desc *d, ap_items *it, cudaStream_t s) {
   std::vector<int32_t> cnt32(c.n);
   for (int64_t sidx = 0; sidx < c.n; ++sidx) cnt32[sidx] = (int32_t)c.h_size[c.h_perm[sidx]];
   AP_TRY(dmalloc(&c.d_pts, std::max<int64_t>(c.total_pts, 4)));
-  if (c.dim == 3 && !c.unit_weights) AP_TRY(dmalloc(&c.d_lw, std::max<int64_t>(c.total_pts, 4)));
+  if (c.dim == 3) AP_TRY(dmalloc(&c.d_lw, std::max<int64_t>(c.total_pts, 4)));
   AP_TRY(dmalloc(&c.d_poff, c.n + 1));
   AP_TRY(dmalloc(&c.d_cnt, std::max<int64_t>(c.n, 1)));
   AP_TRY(dmalloc(&c.d_perm, std::max<int64_t>(c.n, 1)));
@@ -195,7 +210,9 @@ ap_status create_clouds(const ap_items_desc *d, ap_items *it, cudaStream_t s) {
     const float *src[5] = {d->x, d->y, c.dim == 3 ? d->z : nullptr, d->sigma, d->weight};
     float *tmp[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};
     int64_t *d_src_off = nullptr;
-    cudaError_t e = cudaMallocAsync(reinterpret_cast<void **>(&d_src_off), (c.n + 1) * 8, s);
+    cudaError_t e = cudaMemsetAsync(it->d_queue + kQueueTraits, 0, sizeof(int32_t), s);
+    if (e == cudaSuccess)
+      e = cudaMallocAsync(reinterpret_cast<void **>(&d_src_off), (c.n + 1) * 8, s);
     if (e == cudaSuccess)
       e = cudaMemcpyAsync(d_src_off, off, (c.n + 1) * 8, cudaMemcpyHostToDevice, s);
     for (int k = 0; k < 5 && e == cudaSuccess; ++k) {
@@ -207,7 +224,7 @@ ap_status create_clouds(const ap_items_desc *d, ap_items *it, cudaStream_t s) {
     if (e == cudaSuccess) {
       auto pick = [&](int k) -> const float * { return d->data_on_host ? tmp[k] : src[k]; };
       e = launch_cloud_pack(pick(0), pick(1), pick(2), pick(3), pick(4), d_src_off, c.d_perm,
-                            c.d_poff, c.n, c.dim, c.d_pts, c.d_lw, s);
+                            c.d_poff, c.n, c.dim, c.d_pts, c.d_lw, it->d_queue + kQueueTraits, s);
     }
     for (int k = 0; k < 5; ++k)
       if (tmp[k]) cudaFreeAsync(tmp[k], s);
@@ -346,7 +363,7 @@ ap_status ensure_score_storage(ap_items *it, int score, cudaStream_t s) {
   CloudStore &c = it->cl;
   if (c.d_pts_score[score - 1]) return AP_OK;
   // the re-scaled storage (and the L2 self terms) on first use
-  const bool lw = score == 2 ? c.dim == 3 : c.d_lw != nullptr;
+  const bool lw = c.dim == 3;
   AP_TRY(dmalloc(&c.d_pts_score[score - 1], (size_t)std::max<int64_t>(c.total_pts, 1)));
   if (lw) AP_TRY(dmalloc(&c.d_lw_score[score - 1], (size_t)std::max<int64_t>(c.total_pts, 1)));
   AP_TRY(launch_cloud_rescore(c, score, c.d_pts_score[score - 1], c.d_lw_score[score - 1], s));
@@ -413,7 +430,7 @@ ap_status ap_create_items(const ap_items_desc *desc, void *stream, ap_items **ou
   cudaGetDevice(&it->device);
   ap_status st = AP_OK;
   cudaError_t e = dmalloc(&it->d_queue, 64);
-  if (e == cudaSuccess) e = cudaMemset(it->d_queue, 0, 64 * sizeof(int32_t));
+  if (e == cudaSuccess) e = cudaMemsetAsync(it->d_queue, 0, 64 * sizeof(int32_t), s);
   if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&it->copy_stream, cudaStreamNonBlocking);
   if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&it->graph_stream, cudaStreamNonBlocking);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&it->ev_a, cudaEventDisableTiming);
@@ -630,7 +647,11 @@ int32_t ap_last_device_error(ap_items *it) {
   if (!it || !it->d_status) return 0;
   int32_t v = 0;
   if (cudaMemcpy(&v, it->d_status, sizeof v, cudaMemcpyDeviceToHost) != cudaSuccess) return -1;
-  if (v != 0) cudaMemset(it->d_status, 0, sizeof v);
+  if (v != 0) {
+    cudaMemset(it->d_status, 0, sizeof v);
+    // an aborted launch leaves its clouds' queue part-way
+    cudaMemset(it->d_queue + kQueueClouds, 0, sizeof v);
+  }
   return v;
 }
 

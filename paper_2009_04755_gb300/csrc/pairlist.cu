@@ -302,11 +302,11 @@ ap_status cloud_list_plan(ap_items *it, const int32_t *pi, const int32_t *pj, in
     c.h_iperm.assign((size_t)c.n, 0);
     for (int64_t p = 0; p < c.n; ++p) c.h_iperm[c.h_perm[p]] = (int32_t)p;
   }
-  std::vector<int32_t> single((size_t)c.n + 1);
-  for (int64_t b = 0; b <= c.n; ++b) single[b] = (int32_t)b;
-  if (!c.d_bstart_single) {
-    AP_TRY(dmalloc(&c.d_bstart_single, single.size()));
-    AP_TRY(cudaMemcpy(c.d_bstart_single, single.data(), single.size() * 4,
+  if (!c.d_bmeta_single) {
+    std::vector<int32_t> single;
+    single_item_blocks(c, c.reg_r, single);
+    AP_TRY(dmalloc(&c.d_bmeta_single, std::max<size_t>(single.size(), 8)));
+    AP_TRY(cudaMemcpy(c.d_bmeta_single, single.data(), single.size() * 4,
                       cudaMemcpyHostToDevice));
   }
   if (c.list_cap < n_pairs) {
@@ -324,19 +324,17 @@ ap_status cloud_list_plan(ap_items *it, const int32_t *pi, const int32_t *pj, in
     tiles[2 * k + 1] = c.h_iperm[pj[k]];
   }
   AP_TRY(cudaMemcpy(c.d_list_tiles, tiles.data(), tiles.size() * 4, cudaMemcpyHostToDevice));
-  std::vector<int64_t> cnt((size_t)c.n);
-  for (int64_t p = 0; p < c.n; ++p) cnt[p] = c.h_size[c.h_perm[p]];
   lc = c;
   lc.list_mode = true;
-  lc.d_bstart = c.d_bstart_single;
+  lc.d_bmeta = c.d_bmeta_single;
   lc.d_tiles = c.d_list_tiles;
   lc.n_tiles = n_pairs;
-  lc.block_items = 1;
-  lc.max_rj = max_row_jobs(single, cnt, 32LL * c.reg_r);
-  // a J block is one item: stage as many points as the largest item has
-  int64_t most = 4;
-  for (int64_t p = 0; p < c.n; ++p) most = std::max(most, c.h_poff[p + 1] - c.h_poff[p]);
-  lc.block_pts = (int32_t)std::min<int64_t>(most, c.block_pts);
+  lc.max_items = lc.max_rows = 1;
+  lc.max_pts = 4;
+  for (int64_t p = 0; p < c.n; ++p) {
+    lc.max_rows = std::max(lc.max_rows, cloud_rows(c.h_size[c.h_perm[p]], c.reg_r));
+    lc.max_pts = std::max(lc.max_pts, (int32_t)(c.h_poff[p + 1] - c.h_poff[p]));
+  }
   return AP_OK;
 }
 

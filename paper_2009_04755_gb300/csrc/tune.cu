@@ -21,7 +21,7 @@ int32_t min_reg_r(const CloudStore &c) {
   int64_t mx = 0;
   for (int64_t s : c.h_size) mx = std::max(mx, s);
   int32_t r = 2;                        // a-points go in pairs (FP32x2)
-  while ((int64_t)r * 32 * kOverlapMaxRowJobs < mx && r < 4) r *= 2;
+  while ((int64_t)r * 32 * kOverlapMaxRows < mx && r < 4) r *= 2;
   return r;
 }
 
@@ -78,17 +78,33 @@ constexpr int64_t kLargestFirstBytes = 16ll << 20;
 bool order_cloud_tiles(const std::vector<int32_t> &bstart, const std::vector<int64_t> &cnt,
                        int64_t total_pts, std::vector<int32_t> &tiles) {
   if (total_pts * (int64_t)(sizeof(float4) + sizeof(float)) > kLargestFirstBytes) return false;
-  const size_t nt = tiles.size() / 2;
-  std::vector<std::pair<double, int64_t>> key(nt);
-  for (size_t t = 0; t < nt; ++t) key[t] = {-tile_cost(bstart, cnt, tiles[2 * t], tiles[2 * t + 1]), (int64_t)t};
-  std::stable_sort(key.begin(), key.end(),
-                   [](const std::pair<double, int64_t> &a, const std::pair<double, int64_t> &b) {
-                     return a.first < b.first;
-                   });
+  // counting sort on the cost in steps of a thousandth of the largest
+  constexpr int kSteps = 1000;
+  const size_t nt = tiles.size() / 2, nb = bstart.size() - 1;
+  std::vector<double> sum(nb, 0.0), sq(nb, 0.0);
+  for (size_t b = 0; b < nb; ++b)
+    for (int32_t k = bstart[b]; k < bstart[b + 1]; ++k) {
+      sum[b] += (double)cnt[k];
+      sq[b] += (double)cnt[k] * (double)cnt[k];
+    }
+  std::vector<double> cost(nt);
+  double most = 0.0;
+  for (size_t t = 0; t < nt; ++t) {
+    const int32_t I = tiles[2 * t], J = tiles[2 * t + 1];
+    cost[t] = I == J ? (sum[I] * sum[I] - sq[I]) / 2 : sum[I] * sum[J];
+    most = std::max(most, cost[t]);
+  }
+  std::vector<size_t> first(kSteps + 2, 0);
+  auto step = [&](size_t t) {
+    return most > 0.0 ? (size_t)((1.0 - cost[t] / most) * kSteps) : (size_t)0;
+  };
+  for (size_t t = 0; t < nt; ++t) ++first[step(t) + 1];
+  for (size_t k = 1; k < first.size(); ++k) first[k] += first[k - 1];
   std::vector<int32_t> out(tiles.size());
   for (size_t t = 0; t < nt; ++t) {
-    out[2 * t] = tiles[2 * key[t].second];
-    out[2 * t + 1] = tiles[2 * key[t].second + 1];
+    const size_t at = first[step(t)]++;
+    out[2 * at] = tiles[2 * t];
+    out[2 * at + 1] = tiles[2 * t + 1];
   }
   tiles.swap(out);
   return true;
@@ -219,7 +235,7 @@ extern "C" ap_status ap_tune(ap_items *it, int32_t mode, void *stream, ap_plan *
   const double budget = 2e10;
 
   float *d_out = nullptr, *d_g = nullptr;
-  int32_t *d_bstart = nullptr, *d_tiles = nullptr;
+  CloudStore cand;                       // no plan buffers yet
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   ap_status st = AP_OK;
   cudaError_t e = dmalloc(&d_out, (size_t)P);
@@ -231,14 +247,13 @@ extern "C" ap_status ap_tune(ap_items *it, int32_t mode, void *stream, ap_plan *
   double best_rate = -1.0;
   const int32_t rmin = min_reg_r(c);
   for (int32_t rr : {2, 4}) {
-    if (rr < rmin || e != cudaSuccess) continue;
+    if (rr < rmin) continue;
     for (int32_t bp : {2048, 4096, 8192}) {
       for (int32_t bi : {2, 4, 8, 16, 32}) {
-        if (e != cudaSuccess) break;
-        std::vector<int32_t> bstart, tiles;
-        make_blocks(c.h_poff, cnt, bi, bp, 32LL * rr, kOverlapMaxRowJobs, bstart);
-        dc_block_pairs((int64_t)bstart.size() - 1, tiles);
-        order_cloud_tiles(bstart, cnt, c.total_pts, tiles);
+        if (e != cudaSuccess || st != AP_OK) break;
+        CloudPlanHost plan;
+        make_cloud_plan(c.h_poff, cnt, c.h_perm, 0, bi, bp, rr, plan);
+        const std::vector<int32_t> &bstart = plan.bstart, &tiles = plan.tiles;
         const int64_t nt = (int64_t)tiles.size() / 2;
         std::vector<double> cost(nt);
         double total = 0;
@@ -258,23 +273,16 @@ extern "C" ap_status ap_tune(ap_items *it, int32_t mode, void *stream, ap_plan *
           sample.push_back(tiles[2 * t + 1]);
           scost += cost[t];
         }
-        dfree(d_bstart);
-        dfree(d_tiles);
-        e = dmalloc(&d_bstart, bstart.size());
-        if (e == cudaSuccess) e = dmalloc(&d_tiles, std::max<size_t>(sample.size(), 2));
-        if (e == cudaSuccess)
-          e = cudaMemcpy(d_bstart, bstart.data(), bstart.size() * 4, cudaMemcpyHostToDevice);
-        if (e == cudaSuccess && !sample.empty())
-          e = cudaMemcpy(d_tiles, sample.data(), sample.size() * 4, cudaMemcpyHostToDevice);
-        if (e != cudaSuccess) break;
-        CloudStore cand = c;                 // shallow copy pointing at the sample plan
-        cand.d_bstart = d_bstart;
-        cand.d_tiles = d_tiles;
-        cand.n_tiles = (int64_t)sample.size() / 2;
+        plan.tiles.swap(sample);
+        // a shallow copy of the set with the sample's plan
+        free_cloud_plan(cand);
+        cand = c;
+        cand.d_bmeta = cand.d_desc = cand.d_items = cand.d_tiles = nullptr;
         cand.block_items = bi;
         cand.block_pts = bp;
         cand.reg_r = rr;
-        cand.max_rj = max_row_jobs(bstart, cnt, 32LL * rr);
+        st = upload_cloud_plan(cand, plan, s);
+        if (st != AP_OK) break;
         auto launch = [&]() {
           return mode == 0 ? launch_overlap(cand, nullptr, d_out, 0, it->d_queue, s)
                            : launch_overlap_grad_q(cand, it->d_queue, nullptr, nullptr, d_g, d_out,
@@ -301,10 +309,10 @@ extern "C" ap_status ap_tune(ap_items *it, int32_t mode, void *stream, ap_plan *
     }
   }
   if (e != cudaSuccess) st = from_cuda(e);
+  cudaStreamSynchronize(s);                      // the last candidate's plan is still in use
   dfree(d_out);
   dfree(d_g);
-  dfree(d_bstart);
-  dfree(d_tiles);
+  free_cloud_plan(cand);
   if (e0) cudaEventDestroy(e0);
   if (e1) cudaEventDestroy(e1);
   if (st != AP_OK) return st;

@@ -127,3 +127,48 @@ def test_clouds_created_on_a_side_stream_from_pinned_host(ap, oracle_lib):
     s.synchronize()
     check_overlap(out.cpu().numpy(), ref, kappa, bound, "side stream")
     it.close()
+
+
+def _edge_clouds(dim, scale=1.0, weights=False, sizes=None):
+    """Sizes at the edges of a group of 4 points, a piece of 8 groups, a full
+    warp of 4 points per lane and (the last) of the staging windows."""
+    sizes = np.array(sizes or [1, 31, 32, 33, 36, 64, 65, 96, 127, 128, 129, 160, 161, 255, 257,
+                               2047, 2049, 4101])
+    off = np.concatenate([[0], np.cumsum(sizes)]).astype(np.int64)
+    rng = np.random.default_rng(int(off[-1]) + dim)
+    pts = rng.uniform(-0.3, 0.3, (int(off[-1]), 3)) * scale
+    sig = rng.uniform(0.03, 0.08, int(off[-1])) * scale
+    w = rng.uniform(0.5, 1.5, int(off[-1])) if weights else None
+    f32 = np.float32
+    return {"dim": dim, "offsets": off, "x": pts[:, 0].astype(f32), "y": pts[:, 1].astype(f32),
+            "z": pts[:, 2].astype(f32) if dim == 3 else None, "sigma": sig.astype(f32),
+            "weight": None if w is None else w.astype(f32)}
+
+
+@pytest.mark.parametrize("dim", [2, 3])
+@pytest.mark.parametrize("plan", [None, (4, 256, 2), (32, 8192, 4)])
+@pytest.mark.parametrize("kind", ["unit", "weighted", "tiny", "huge"])
+def test_overlap_fragment_and_window_edges(ap, oracle_lib, dim, plan, kind):
+    """Unit weights and weights take their own loops; lengths of 1e-12 (whose
+    s2k products leave the FP32 range) and coordinates of 1e16 the general
+    one.  The cost does not depend on the unit of length, so the oracle sees
+    the same set."""
+    scale = {"tiny": 1e-12, "huge": 1e16}.get(kind, 1.0)
+    c = _edge_clouds(dim, scale, kind == "weighted")
+    n = len(c["offsets"]) - 1
+    pi, pj = oracle_lib.all_pairs(n)
+    ref, kappa, bound = oracle_lib.overlap(c, pi, pj, with_cond=True)
+    with ap.Items.from_clouds(c) as it:
+        if plan:
+            it.set_plan(*plan)
+        f = it.run_pairs().cpu().numpy()
+        one = it.run_pairs_list(pi, pj).cpu().numpy()
+        cnt = it.run_pairs(ap.AP_FN_COVERAGE).cpu().numpy()
+        assert it.last_device_error() == 0
+    check_overlap(f, ref, kappa, bound, f"{kind} {dim}d {plan}")
+    assert np.all(cnt == 1)
+    if dim == 2:
+        # stored in item order: a listed pair sums the same fragments in the same order
+        np.testing.assert_array_equal(one, f)
+    else:
+        check_overlap(one, ref, kappa, bound, f"listed {kind} {dim}d {plan}")

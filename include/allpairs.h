@@ -208,7 +208,8 @@ typedef struct ap_plan {
  *   row whose shift missed its mean by D delta^2 > ss / 64 is written again
  *   centred on its mean.
  *   Sparse vectors: the CSR arrays copied, FP64 squared norms per row, and
- *   per column chunk of 2048 codes the first entry of every row in it.
+ *   per column chunk of 4096 codes the first entry of every row in it and
+ *   what its codes share (which decides how its pairs are summed).
  * Host-side planning (block and tile lists, sorting) happens before the call
  * returns; every copy and kernel of the call is ordered on `stream`, for all
  * kinds (host sources: pageable memory is staged by the copy calls, pinned

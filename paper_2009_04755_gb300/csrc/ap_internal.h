@@ -306,8 +306,7 @@ namespace ap {
 // code >= c * kSparseChunk, relative to the row's start (chunk-major, so the
 // bounds of 32 consecutive rows in one chunk are one coalesced load)
 constexpr int kSparseChunk = 4096;
-constexpr int kSparseBlock = 32;     // items i of a tile
-constexpr int kSparseBlockJ = 64;    // items j of a tile
+constexpr int kSparseBlock = 128;    // items of a tile side
 struct SparseStore {
   int64_t n = 0, dim = 0, nnz = 0, n_chunks = 0;
   int64_t *d_off = nullptr;
@@ -315,11 +314,11 @@ struct SparseStore {
   float *d_val = nullptr;
   int32_t *d_cptr = nullptr;        // [n_chunks + 1][n]
   double *d_rs = nullptr;           // 1 / sqrt(sum of squares), NaN for none
-  int32_t *d_tiles = nullptr;       // block pairs (I <= J) of 32 items
+  int32_t *d_tiles = nullptr;       // block pairs (I <= J) of 128 items
   int64_t n_tiles = 0;
-  // per block of 32 items: the item (0..31) each row slot j of a tile takes;
-  // slots w and w + 16 (one warp) pair a heavy row with a light one
-  int32_t *d_jperm = nullptr;
+  int32_t *d_chunks = nullptr;      // [n_join + n_dense]: chunks with shared codes, by way
+  int64_t n_join = 0, n_dense = 0;
+  unsigned long long *d_heads = nullptr;   // unit queues of the two kernels
 };
 }  // namespace ap
 
@@ -517,8 +516,7 @@ cudaError_t launch_cloud_self(const CloudStore &cs, const float4 *pts, const flo
 // sparse vectors (sparse.cu)
 ap_status create_sparse(const ap_items_desc *d, ap_items *it, cudaStream_t s);
 void free_sparse(SparseStore &sp);
-cudaError_t launch_sparse_cosine(const SparseStore &sp, double *out, int coverage,
-                                 int32_t *queue, cudaStream_t s);
+cudaError_t launch_sparse_cosine(const SparseStore &sp, void *out, int coverage, cudaStream_t s);
 // words of a handle's d_queue block: [0] tile-queue head, [1] status word,
 // [2] scratch, and for clouds their own queue head (zero between launches:
 // the CTA that takes the last pop resets it) and traits of the set: some s2k

@@ -6,30 +6,28 @@
 //
 // Rows are CSR (strictly increasing int32 codes, FP32 values) over an index
 // space of `dim` codes (20^k k-mers), cut into chunks of kSparseChunk codes.
-// Schedule: persistent CTAs pop tiles (a block of 32 items I x a block of 64
-// items J, every block pair holding a pair i < j, Sec. IV-B) from an atomic
-// queue.  The 16 warps walk the chunks together, for 8 rows of I at a time:
-// per chunk warps 0-7 each scatter one row i into the dense form of the
-// chunk in shared memory, and after a barrier every lane reads its share of
-// the chunk's entries of the warp's four rows j (once, into registers) and
-// multiplies each against the 8 rows i.  The dense form is code-major, the 8
-// rows' values of one code side by side (32 bytes), so one 16-byte load
-// gathers four rows; the two 16-byte groups of a code are XOR-swizzled by
-// code bit 1, which spreads the loads of random codes over the bank groups.
-// The barriers pace every chunk step by its busiest warp, so the rows j of a
-// block are dealt to the warps by entry count in a snake (heavy and light
-// rows alternate).  Each warp copies the next chunk's entries of its rows (up
-// to 64 per row) into a two-stage shared-memory ring with cp.async while it
-// works on the current one, so the chunk loop does not wait on DRAM.  Per
-// lane the FP32 products are summed over up to 64 chunks, then folded into
-// FP64 pair sums in shared memory.  (Tiles of 32 x 32 items with 16 rows i
-// per pass over chunks of 2048 codes ran 2.99 s on the 2500-item set, these
-// 2.89 s: the lookups, not the chunk steps, set the pace.)
+// A pair's sum needs only the codes that both rows hold, which for a code in
+// p of the n rows is p (p - 1) / 2 products.  Each chunk takes the cheaper of
+// two ways, decided at creation from its codes' counts:
+//
+//   join    few rows per code: one CTA sorts the chunk's entries by code in
+//           shared memory (count, scan, scatter) and adds every pair of
+//           entries of a code into the FP64 output, one product each;
+//   dense   many rows per code: the FP32 Gram of the chunk's dense form, tiles
+//           of 128 x 128 rows, 32 codes at a time scattered straight from the
+//           CSR rows into shared memory (nothing dense in global memory), FP32
+//           sums over one chunk added into the FP64 output.
+//
+// A last pass scales by the norms.  (Before, every chunk was made dense for 8
+// rows at a time in tiles of 32 x 64 rows, one product per entry of row j and
+// row i whether row i held the code or not: 256 rows of 20^6 codes, 1e5 to
+// 1.8e6 entries each, took 255 ms, 20 CTAs' work; now 10.4.)
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
 
 #include <algorithm>
+#include <type_traits>
 #include <vector>
 
 #include "ap_internal.h"
@@ -38,221 +36,393 @@ namespace ap {
 
 namespace {
 
-constexpr int kWarps = 16;                   // warps per CTA
-constexpr int kThreads = 32 * kWarps;
-constexpr int kRows = 8;                     // rows i per pass: the dense form's rows
-constexpr int kGroups = kRows / 4;           // 16-byte groups of a code in the dense form
-constexpr int BI = kSparseBlock;             // items i of a tile
-constexpr int BJ = kSparseBlockJ;            // items j of a tile
-constexpr int kJ = BJ / kWarps;              // rows j per warp
-constexpr int kStage = 64;                   // staged entries per row and chunk
 constexpr int W = kSparseChunk;
-constexpr int kFoldChunks = 64;
 
-// word of row q (0..kRows-1) at chunk code k in the swizzled dense form
-__device__ __forceinline__ int dense_at(int k, int q) {
-  return k * kRows + ((((q >> 2) ^ (k >> 1)) & (kGroups - 1)) << 2) + (q & 3);
+// ---------------------------------------------------------------------------
+// join
+// ---------------------------------------------------------------------------
+// Bound by the FP64 additions at L2 (one per product, 1.8e11 a second) where
+// many rows share codes, by the latency of the two passes over the entries
+// where few do (15 ps an entry over the GPU: 122 million entries and as many
+// products in 2.3 ms, 256 rows of 20^6 codes).  Two CTAs per SM.
+constexpr int kJoinThreads = 512;
+constexpr int kJoinCap = 9216;             // entries sorted at a time
+constexpr size_t kJoinSmem = (size_t)(W + 1) * 4 + 12 + (size_t)kJoinCap * 10;
+
+// f(row, entry index in the CSR arrays) for the entries of chunk c: eight
+// lanes on consecutive entries of a row (a chunk of a composition vector
+// holds a few dozen), a whole warp where there are fewer rows than octets
+template <class F>
+__device__ __forceinline__ void for_entries(const int64_t *__restrict__ off,
+                                            const int32_t *__restrict__ cptr, int64_t n, int64_t c,
+                                            F f) {
+  const int lpr = n * 8 >= blockDim.x ? 8 : 32;
+  const int sub = threadIdx.x & (lpr - 1);
+  for (int64_t r = threadIdx.x / lpr; r < n; r += blockDim.x / lpr) {
+    const int e1 = cptr[(c + 1) * n + r];
+    const int64_t b = off[r];
+#pragma unroll 4
+    for (int e = cptr[c * n + r] + sub; e < e1; e += lpr) f((int32_t)r, b + e);
+  }
 }
 
-// asynchronous 4-byte copy global -> shared; src_bytes 0 writes zeros and
-// reads nothing
-__device__ __forceinline__ void cp_async4(void *dst, const void *src, uint32_t src_bytes) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(
-                   (uint32_t)__cvta_generic_to_shared(dst)),
-               "l"(src), "r"(src_bytes)
-               : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() {
-  asm volatile("cp.async.commit_group;" ::: "memory");
-}
-__device__ __forceinline__ void cp_async_wait_prev() {
-  asm volatile("cp.async.wait_group 1;" ::: "memory");
+// exclusive scan of s[0, W) in place, s[W] = total (kJoinThreads threads)
+__device__ __forceinline__ void scan_counts(int32_t *s, int32_t *wsum) {
+  constexpr int PER = W / kJoinThreads;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  int32_t v[PER], sum = 0;
+#pragma unroll
+  for (int q = 0; q < PER; ++q) {
+    v[q] = s[threadIdx.x * PER + q];
+    sum += v[q];
+  }
+  int32_t inc = sum;
+  for (int o = 1; o < 32; o <<= 1) {
+    const int32_t x = __shfl_up_sync(0xffffffffu, inc, o);
+    if (lane >= o) inc += x;
+  }
+  if (lane == 31) wsum[warp] = inc;
+  __syncthreads();
+  int32_t before = 0;
+  for (int w = 0; w < warp; ++w) before += wsum[w];
+  int32_t at = before + inc - sum;
+#pragma unroll
+  for (int q = 0; q < PER; ++q) {
+    s[threadIdx.x * PER + q] = at;
+    at += v[q];
+  }
+  if (threadIdx.x == kJoinThreads - 1) s[W] = at;
+  __syncthreads();
 }
 
-// One warp's staging of a chunk: up to kStage entries (2 per lane) of its row
-// i (dense-row owners) and of its kJ rows j, filled by cp.async one chunk
-// ahead.
-struct WarpStage {
-  int32_t code[1 + kJ][kStage];
-  float val[1 + kJ][kStage];
-};
-
-template <int COVER>
-__global__ void __launch_bounds__(kThreads, 1)
-sparse_cos_kernel(const int64_t *__restrict__ off, const int32_t *__restrict__ idx,
-                  const float *__restrict__ val, const int32_t *__restrict__ cptr,
-                  const double *__restrict__ rs, int64_t n, int64_t n_chunks,
-                  const int32_t *__restrict__ tiles, int64_t n_tiles,
-                  const int32_t *__restrict__ jperm, int32_t *queue, void *out) {
+__global__ void __launch_bounds__(kJoinThreads, 2)
+sparse_join_kernel(const int64_t *__restrict__ off, const int32_t *__restrict__ idx,
+                   const float *__restrict__ val, const int32_t *__restrict__ cptr, int64_t n,
+                   const int32_t *__restrict__ chunks, int32_t n_chunks,
+                   unsigned long long *queue, double *__restrict__ out) {
   extern __shared__ __align__(16) uint8_t smem[];
-  float *dense = reinterpret_cast<float *>(smem);                     // [W][kRows], swizzled
-  double *s_g = reinterpret_cast<double *>(dense + kRows * W);        // [BI][BJ]
-  WarpStage *stage = reinterpret_cast<WarpStage *>(s_g + BI * BJ);    // [kWarps][2]
-  __shared__ int s_tile;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  // warps 0..kRows-1 each own one dense row (scatter and clear it, so the
-  // clearing of a chunk and the next chunk's scatter stay in program order)
-  const int wr = warp % kRows;
-  const bool owner = warp < kRows;
-  for (int k = threadIdx.x; k < kRows * W; k += kThreads) dense[k] = 0.f;
-  WarpStage *my_stage = stage + warp * 2;
-
+  int32_t *s_at = reinterpret_cast<int32_t *>(smem);              // [W + 1] code starts
+  int32_t *s_row = s_at + W + 4;                                  // [kJoinCap]
+  float *s_val = reinterpret_cast<float *>(s_row + kJoinCap);     // [kJoinCap]
+  uint16_t *s_code = reinterpret_cast<uint16_t *>(s_val + kJoinCap);
+  __shared__ int32_t s_wsum[kJoinThreads / 32];
+  __shared__ unsigned long long s_unit;
   for (;;) {
-    if (threadIdx.x == 0) s_tile = atomicAdd(queue, 1);
+    if (threadIdx.x == 0) s_unit = atomicAdd(queue, 1ull);
+    for (int k = threadIdx.x; k < W; k += kJoinThreads) s_at[k] = 0;
     __syncthreads();
-    const int64_t t = s_tile;
-    if (t >= n_tiles) break;
-    const int64_t i0 = (int64_t)tiles[2 * t] * BI, j0 = (int64_t)tiles[2 * t + 1] * BJ;
-    const int32_t *jslot = jperm + (int64_t)tiles[2 * t + 1] * BJ;   // item of each row slot of J
-    for (int q = threadIdx.x; q < BI * BJ; q += kThreads) s_g[q] = 0.0;
+    const int64_t u = (int64_t)s_unit;
+    if (u >= n_chunks) break;
+    const int64_t c = chunks[u];
+    const int32_t code0 = (int32_t)(c * W);
+    for_entries(off, cptr, n, c, [&](int32_t, int64_t e) { atomicAdd(&s_at[idx[e] - code0], 1); });
     __syncthreads();
-
-    if (!COVER) {
-      for (int pass = 0; pass < BI / kRows; ++pass) {
-        // the warp's rows: r = 0 its row i (owners only: dense row wr),
-        // r = 1.. its rows j (slots warp + (r - 1) * kWarps)
-        int64_t row[1 + kJ], base[1 + kJ];
-        bool valid[1 + kJ];
-        row[0] = i0 + pass * kRows + wr;
-#pragma unroll
-        for (int h = 0; h < kJ; ++h) row[1 + h] = j0 + jslot[warp + h * kWarps];
-        // pairs need j > i: a row j at or before every row i of the pass has none
-        const int64_t i_first = i0 + pass * kRows;
-#pragma unroll
-        for (int r = 0; r <= kJ; ++r) {
-          valid[r] = row[r] < n && (r == 0 ? owner : row[r] > i_first);
-          base[r] = valid[r] ? off[row[r]] : 0;
+    scan_counts(s_at, s_wsum);
+    const int32_t total = s_at[W];
+    // codes [a, b) hold at most kJoinCap entries: usually the whole chunk (no
+    // code alone holds more, or the chunk would be a dense one)
+    for (int a = 0; a < W;) {
+      const int32_t first = s_at[a];
+      if (first == total) break;
+      int b = W, lo = a + 1;
+      if (total - first > kJoinCap) {
+        for (int hi = W; lo < hi;) {                // last b with s_at[b] - first <= kJoinCap
+          const int mid = (lo + hi + 1) >> 1;
+          if (s_at[mid] - first <= kJoinCap) lo = mid;
+          else hi = mid - 1;
         }
-        float acc[kJ][kRows];
-#pragma unroll
-        for (int h = 0; h < kJ; ++h)
-#pragma unroll
-          for (int q = 0; q < kRows; ++q) acc[h][q] = 0.f;
-        // one entry (code k of the chunk, value v) of a row j against the
-        // kRows rows i: kGroups 16-byte loads of the dense form
-        auto product = [&](int32_t k, float v, float (&a)[kRows]) {
-          const float4 *dk = reinterpret_cast<const float4 *>(dense + k * kRows);
-#pragma unroll
-          for (int g = 0; g < kGroups; ++g) {
-            const float4 d = dk[(g ^ (k >> 1)) & (kGroups - 1)];
-            a[4 * g + 0] = fmaf(d.x, v, a[4 * g + 0]);
-            a[4 * g + 1] = fmaf(d.y, v, a[4 * g + 1]);
-            a[4 * g + 2] = fmaf(d.z, v, a[4 * g + 2]);
-            a[4 * g + 3] = fmaf(d.w, v, a[4 * g + 3]);
-          }
-        };
-        int since = 0;
-        // chunk starts b0..b3 = cptr of chunks c .. c + 3 (relative to the row)
-        int32_t b0[1 + kJ], b1[1 + kJ], b2[1 + kJ], b3[1 + kJ];
-        auto bound = [&](int r, int64_t cn, bool in_range) -> int32_t {
-          return (valid[r] && in_range) ? cptr[cn + row[r]] : 0;   // cn = c * n
-        };
-        // copies of chunk c's first kStage entries of every row into stage s;
-        // slots past a row's entries are not copied (nothing reads them)
-        auto stage_copy = [&](int64_t c, const int32_t *lo, const int32_t *hi, int s) {
-#pragma unroll
-          for (int r = 0; r <= kJ; ++r) {
-#pragma unroll
-            for (int u = 0; u < kStage / 32; ++u) {
-              const int32_t e = lo[r] + u * 32 + lane;
-              if (c < n_chunks && e < hi[r]) {
-                const int64_t g = base[r] + e;
-                cp_async4(&my_stage[s].code[r][u * 32 + lane], idx + g, 4u);
-                cp_async4(&my_stage[s].val[r][u * 32 + lane], val + g, 4u);
-              }
-            }
-          }
-          cp_async_commit();
-        };
-#pragma unroll
-        for (int r = 0; r <= kJ; ++r) {
-          b0[r] = bound(r, 0, true);
-          b1[r] = bound(r, n, 1 <= n_chunks);
-          b2[r] = bound(r, 2 * n, 2 <= n_chunks);
-        }
-        stage_copy(0, b0, b1, 0);
-        for (int64_t c = 0; c < n_chunks; ++c) {
-          const int32_t code0 = (int32_t)(c * W);
-          const int s = (int)(c & 1);
-          const int64_t cn3 = (c + 3) * n;
-#pragma unroll
-          for (int r = 0; r <= kJ; ++r) b3[r] = bound(r, cn3, c + 3 <= n_chunks);
-          stage_copy(c + 1, b1, b2, s ^ 1);            // the next chunk, in flight
-          cp_async_wait_prev();                        // this chunk's copies landed
-          const WarpStage &st = my_stage[s];
-          // scatter row i (staged entries, then any beyond the stage)
-          const int32_t ni = b1[0] - b0[0];
-#pragma unroll
-          for (int u = 0; u < kStage / 32; ++u)
-            if (u * 32 + lane < ni)
-              dense[dense_at(st.code[0][u * 32 + lane] - code0, wr)] = st.val[0][u * 32 + lane];
-          for (int32_t e = kStage + lane; e < ni; e += 32) {
-            const int64_t g = base[0] + b0[0] + e;
-            dense[dense_at(__ldg(idx + g) - code0, wr)] = __ldg(val + g);
-          }
-          __syncthreads();
-          // every entry of the warp's rows j in this chunk against the
-          // kRows rows i held in the dense arrays
-#pragma unroll
-          for (int h = 0; h < kJ; ++h) {
-            if (!valid[1 + h]) continue;
-            const int32_t nj = b1[1 + h] - b0[1 + h];
-#pragma unroll
-            for (int u = 0; u < kStage / 32; ++u) {
-              if (u * 32 + lane < nj)
-                product(st.code[1 + h][u * 32 + lane] - code0, st.val[1 + h][u * 32 + lane],
-                        acc[h]);
-            }
-            for (int32_t e = kStage + lane; e < nj; e += 32) {
-              const int64_t g = base[1 + h] + b0[1 + h] + e;
-              product(__ldg(idx + g) - code0, __ldg(val + g), acc[h]);
-            }
-          }
-          __syncthreads();
-#pragma unroll
-          for (int u = 0; u < kStage / 32; ++u)
-            if (u * 32 + lane < ni) dense[dense_at(st.code[0][u * 32 + lane] - code0, wr)] = 0.f;
-          for (int32_t e = kStage + lane; e < ni; e += 32)
-            dense[dense_at(__ldg(idx + base[0] + b0[0] + e) - code0, wr)] = 0.f;
-#pragma unroll
-          for (int r = 0; r <= kJ; ++r) { b0[r] = b1[r]; b1[r] = b2[r]; b2[r] = b3[r]; }
-          if (++since == kFoldChunks || c + 1 == n_chunks) {
-            since = 0;
-            // fold the lanes' FP32 sums into the FP64 pair sums
-#pragma unroll
-            for (int h = 0; h < kJ; ++h)
-#pragma unroll
-              for (int q = 0; q < kRows; ++q) {
-                double v = (double)acc[h][q];
-                for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-                if (lane == 0) s_g[(pass * kRows + q) * BJ + warp + h * kWarps] += v;
-                acc[h][q] = 0.f;
-              }
-          }
-        }
-        asm volatile("cp.async.wait_all;" ::: "memory");   // the last (empty) group
+        b = lo;
       }
-    }
-    __syncthreads();
-    for (int q = threadIdx.x; q < BI * BJ; q += kThreads) {
-      const int il = q / BJ, slot = q - il * BJ;
-      const int64_t i = i0 + il, j = j0 + jslot[slot];
-      if (i >= n || j >= n || j <= i) continue;
-      const int64_t p = pair_index(i, j, n);
-      if (COVER) atomicAdd(reinterpret_cast<int32_t *>(out) + p, 1);
-      else reinterpret_cast<double *>(out)[p] = s_g[q] * rs[i] * rs[j];
+      const int32_t count = s_at[b] - first;
+      __syncthreads();                              // every thread has read the starts
+      for_entries(off, cptr, n, c, [&](int32_t row, int64_t e) {
+        const int k = idx[e] - code0;
+        if (k < a || k >= b) return;
+        const int32_t at = atomicAdd(&s_at[k], 1) - first;   // s_at[k] becomes the code's end
+        s_row[at] = row;
+        s_val[at] = val[e];
+        s_code[at] = (uint16_t)k;
+      });
+      __syncthreads();
+      for (int e = threadIdx.x; e < count; e += kJoinThreads) {
+        const int end = s_at[s_code[e]] - first;
+        const int64_t r = s_row[e];
+        const float v = s_val[e];
+        for (int f = e + 1; f < end; ++f) {
+          const int64_t q = s_row[f];
+          const int64_t i = r < q ? r : q, j = r < q ? q : r;
+          atomicAdd(out + pair_index(i, j, n), (double)__fmul_rn(v, s_val[f]));
+        }
+      }
+      __syncthreads();                              // before the entries are replaced
+      a = b;
     }
     __syncthreads();
   }
 }
 
+// per chunk: {most entries of one code, entries, products}, at creation
+struct ChunkCount { int32_t most, pad; int64_t entries, products; };
+__global__ void __launch_bounds__(kJoinThreads)
+sparse_count_kernel(const int64_t *__restrict__ off, const int32_t *__restrict__ idx,
+                    const int32_t *__restrict__ cptr, int64_t n, int64_t n_chunks,
+                    ChunkCount *__restrict__ out) {
+  __shared__ int32_t s_cnt[W];
+  __shared__ int32_t s_most;
+  __shared__ unsigned long long s_sum[2];
+  for (int64_t c = blockIdx.x; c < n_chunks; c += gridDim.x) {
+    for (int k = threadIdx.x; k < W; k += kJoinThreads) s_cnt[k] = 0;
+    if (threadIdx.x == 0) { s_most = 0; s_sum[0] = s_sum[1] = 0; }
+    __syncthreads();
+    const int32_t code0 = (int32_t)(c * W);
+    for_entries(off, cptr, n, c, [&](int32_t, int64_t e) {
+      const uint32_t k = (uint32_t)(idx[e] - code0);
+      if (k < (uint32_t)W) atomicAdd(&s_cnt[k], 1);        // (rows not yet known to be in order)
+    });
+    __syncthreads();
+    int32_t most = 0;
+    unsigned long long ent = 0, prod = 0;
+    for (int k = threadIdx.x; k < W; k += kJoinThreads) {
+      const int64_t p = s_cnt[k];
+      most = max(most, s_cnt[k]);
+      ent += (unsigned long long)p;
+      prod += (unsigned long long)(p * (p - 1) / 2);
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+      most = max(most, __shfl_xor_sync(0xffffffffu, most, o));
+      ent += __shfl_xor_sync(0xffffffffu, ent, o);
+      prod += __shfl_xor_sync(0xffffffffu, prod, o);
+    }
+    if ((threadIdx.x & 31) == 0) {
+      atomicMax(&s_most, most);
+      atomicAdd(&s_sum[0], ent);
+      atomicAdd(&s_sum[1], prod);
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) out[c] = {s_most, 0, (int64_t)s_sum[0], (int64_t)s_sum[1]};
+    __syncthreads();
+  }
+}
+
+// ---------------------------------------------------------------------------
+// dense
+// ---------------------------------------------------------------------------
+// Units (tile of 128 x 128 rows, dense chunk or a part of one), a part's tiles
+// in a row so that they read its entries from L2.  256 threads, 8 x 8 outputs each as in
+// the FP32 Gram of dense vectors, two CTAs per SM; the FMA pipe is busy 0.53
+// of the time, the rest goes into bringing a stage in between two barriers (976
+// chunks of 256 rows of which a code is in 31: 8.3 ms; joining them takes 11).
+// Each warp brings in 32 of the 256 rows: eight lanes read the next eight
+// entries of a row (one or two sectors), so a warp load covers four rows.
+constexpr int kDenseTile = 128;
+constexpr int kDenseStage = 32;                       // codes per stage
+constexpr int kDenseLd = kDenseTile + 4;
+constexpr int kDenseBuf = kDenseStage * kDenseLd;     // floats of one operand's stage
+constexpr int kDenseAhead = 8;                        // entries of a row staged at a time
+constexpr size_t kDenseSmem = (size_t)4 * kDenseBuf * 4 + 256 * (4 + 4 + 8) +
+                              (size_t)256 * kDenseAhead * 8;
+
+// asynchronous 4-byte copy global -> shared
+__device__ __forceinline__ void cp_async4(void *dst, const void *src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(
+                   (uint32_t)__cvta_generic_to_shared(dst)),
+               "l"(src)
+               : "memory");
+}
+
+template <int COVER>
+__global__ void __launch_bounds__(256, 2)
+sparse_dense_kernel(const int64_t *__restrict__ off, const int32_t *__restrict__ idx,
+                    const float *__restrict__ val, const int32_t *__restrict__ cptr, int64_t n,
+                    const int32_t *__restrict__ chunks, int32_t n_chunks,
+                    int32_t split, const int32_t *__restrict__ tiles, int64_t n_tiles,
+                    unsigned long long *queue, void *out) {
+  extern __shared__ __align__(16) float dsm[];
+  float *s_buf = dsm;                                              // [2][A, B][stage][ld]
+  int64_t *s_base = reinterpret_cast<int64_t *>(dsm + 4 * kDenseBuf);   // [256] rows A, rows B
+  int32_t *s_ptr = reinterpret_cast<int32_t *>(s_base + 256);      // next entry
+  int32_t *s_end = s_ptr + 256;
+  int32_t *s_code = s_end + 256;                                   // [256][kDenseAhead]
+  float *s_val = reinterpret_cast<float *>(s_code + 256 * kDenseAhead);
+  __shared__ unsigned long long s_unit;
+  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+  const int warp = tid >> 5, lane = tid & 31, sub = lane & 7;
+
+  for (;;) {
+    if (tid == 0) s_unit = atomicAdd(queue, 1ull);
+    __syncthreads();
+    const int64_t u = (int64_t)s_unit;
+    __syncthreads();
+    if (u >= n_tiles * split * n_chunks) break;
+    const int64_t part = u / n_tiles, t = u - part * n_tiles;   // part of a chunk, tile
+    const int64_t i0 = (int64_t)tiles[2 * t] * kDenseTile;
+    const int64_t j0 = (int64_t)tiles[2 * t + 1] * kDenseTile;
+    const bool diag = i0 == j0;
+    float2 acc[8][4];
+#pragma unroll
+    for (int a = 0; a < 8; ++a)
+#pragma unroll
+      for (int b = 0; b < 4; ++b) acc[a][b] = make_float2(0.f, 0.f);
+
+    if (!COVER) {
+      const int64_t c = chunks[part / split];
+      const int stages = W / kDenseStage / split;
+      const int32_t code0 = (int32_t)(c * W + (part % split) * (W / split));
+      {
+        const int64_t row = tid < kDenseTile ? i0 + tid : j0 + tid - kDenseTile;
+        const bool in = row < n;
+        s_base[tid] = in ? off[row] : 0;
+        int32_t lo = in ? cptr[c * n + row] : 0, hi = in ? cptr[(c + 1) * n + row] : 0;
+        s_end[tid] = hi;
+        if (split > 1)                              // first entry of this part
+          while (lo < hi) {
+            const int32_t mid = lo + ((hi - lo) >> 1);
+            if (idx[s_base[tid] + mid] < code0) lo = mid + 1;
+            else hi = mid;
+          }
+        s_ptr[tid] = lo;
+      }
+      __syncthreads();
+      // the warps share the rows, four to a load (rr0 + 4 q, q < nq); a
+      // diagonal tile's rows B are its rows A, and one operand serves both
+      const int nq = diag ? 4 : 8, rr0 = warp * 4 * nq + (lane >> 3);
+      // the next eight entries of a row of this lane's into the staging area
+      auto load = [&](int q) {
+        const int rr = rr0 + 4 * q, p = s_ptr[rr] + sub;
+        if (p < s_end[rr]) {
+          const int64_t e = s_base[rr] + p;
+          cp_async4(&s_code[rr * kDenseAhead + sub], idx + e);
+          cp_async4(&s_val[rr * kDenseAhead + sub], val + e);
+        } else {
+          s_code[rr * kDenseAhead + sub] = -1;
+        }
+      };
+      // those of the stage's codes into its buffer; more while a row has them
+      // (each lane reads what it staged itself)
+      auto scatter = [&](int buf, int32_t k0) {
+        float *dst = s_buf + (2 * buf + (rr0 >> 7)) * kDenseBuf;
+        asm volatile("cp.async.wait_all;" ::: "memory");
+        auto place = [&](int q) -> bool {          // whether some row may have more
+          const int rr = rr0 + 4 * q, at = rr * kDenseAhead + sub;
+          const int32_t code = s_code[at];
+          const bool in = (uint32_t)(code - k0) < (uint32_t)kDenseStage;   // codes come in order
+          if (in) dst[(code - k0) * kDenseLd + (rr & 127)] = s_val[at];
+          const uint32_t m = __ballot_sync(0xffffffffu, in);
+          const int taken = __popc((m >> (lane & 24)) & 0xffu);
+          if (sub == 0 && taken) s_ptr[rr] += taken;
+          return __any_sync(0xffffffffu, taken == 8);
+        };
+        uint32_t more = 0;
+#pragma unroll 4
+        for (int q = 0; q < nq; ++q) more |= place(q) ? 1u << q : 0u;
+        for (; more; more &= more - 1) {
+          const int q = __ffs(more) - 1;
+          do {
+            __syncwarp();
+            load(q);
+            asm volatile("cp.async.wait_all;" ::: "memory");
+          } while (place(q));
+        }
+      };
+      auto zero = [&](int buf) {
+        float4 *z = reinterpret_cast<float4 *>(s_buf + 2 * buf * kDenseBuf);
+        for (int k = tid; k < 2 * kDenseBuf / 4; k += 256) z[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+      };
+      auto load_all = [&]() {
+#pragma unroll 4
+        for (int q = 0; q < nq; ++q) load(q);
+      };
+      // outputs (a, b) of one code; SKIP: a diagonal tile has no pair among
+      // the rows 64.. and columns ..63
+      auto product = [&](const float *As, const float *Bs, auto skip) {
+        constexpr bool SKIP = decltype(skip)::value;
+#pragma unroll 8
+        for (int k = 0; k < kDenseStage; ++k) {
+          const float4 a0 = *reinterpret_cast<const float4 *>(As + k * kDenseLd + ty * 4);
+          const float4 a1 = *reinterpret_cast<const float4 *>(As + k * kDenseLd + 64 + ty * 4);
+          const float4 b0 = *reinterpret_cast<const float4 *>(Bs + k * kDenseLd + tx * 4);
+          const float4 b1 = *reinterpret_cast<const float4 *>(Bs + k * kDenseLd + 64 + tx * 4);
+          const float av[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
+          const float2 bv[4] = {make_float2(b0.x, b0.y), make_float2(b0.z, b0.w),
+                                make_float2(b1.x, b1.y), make_float2(b1.z, b1.w)};
+#pragma unroll
+          for (int a = 0; a < 8; ++a) {
+            const float2 aa = make_float2(av[a], av[a]);
+#pragma unroll
+            for (int b = SKIP && a >= 4 ? 2 : 0; b < 4; ++b)
+              acc[a][b] = __ffma2_rn(aa, bv[b], acc[a][b]);
+          }
+        }
+      };
+      load_all();
+      zero(0);
+      __syncthreads();
+      scatter(0, code0);
+      __syncthreads();
+      for (int st = 0; st < stages; ++st) {
+        const int buf = st & 1;
+        const bool more = st + 1 < stages;
+        if (more) {
+          load_all();
+          zero(buf ^ 1);
+        }
+        const float *As = s_buf + 2 * buf * kDenseBuf;
+        if (diag) product(As, As, std::true_type());
+        else product(As, As + kDenseBuf, std::false_type());
+        __syncthreads();                            // the other buffer is clear
+        if (more) scatter(buf ^ 1, code0 + (st + 1) * kDenseStage);
+        __syncthreads();
+      }
+    }
+
+    const int ni = (int)(n - i0 < kDenseTile ? n - i0 : kDenseTile);
+    const int nj = (int)(n - j0 < kDenseTile ? n - j0 : kDenseTile);
+#pragma unroll
+    for (int a = 0; a < 8; ++a) {
+      const int il = (a < 4 ? a : 60 + a) + ty * 4;
+      if (il < ni) {
+        const int64_t i = i0 + il;
+        const int first = (int)(i - j0) + 1;        // pairs need j0 + jl > i
+        const int64_t p0 = pair_index(i, j0, n);
+#pragma unroll
+        for (int b = 0; b < 8; ++b) {
+          const int jl = (b < 4 ? b : 60 + b) + tx * 4;
+          if (jl >= nj || jl < first) continue;
+          if (COVER) atomicAdd(reinterpret_cast<int32_t *>(out) + p0 + jl, 1);
+          else
+            atomicAdd(reinterpret_cast<double *>(out) + p0 + jl,
+                      (double)((b & 1) ? acc[a][b >> 1].y : acc[a][b >> 1].x));
+        }
+      }
+    }
+  }
+}
+
+// out[p] *= rs_i rs_j over the packed triangle
+__global__ void sparse_scale_kernel(double *__restrict__ out, const double *__restrict__ rs,
+                                    int64_t n) {
+  for (int64_t i = blockIdx.x; i < n - 1; i += gridDim.x) {
+    const double ri = rs[i];
+    const int64_t p0 = pair_index(i, i + 1, n);
+    for (int64_t j = i + 1 + threadIdx.x; j < n; j += blockDim.x)
+      out[p0 + (j - i - 1)] *= ri * rs[j];
+  }
+}
+
+// measured on a GB300: see sparse_join_kernel and sparse_dense_kernel
+constexpr double kJoinProductPs = 5.6, kJoinEntryPs = 15.0;
+constexpr double kDenseTilePs = 2.6e6;
+
 // row checks (strictly increasing codes in [0, dim)), FP64 squared norms
-__global__ void sparse_rows_kernel(const int64_t *__restrict__ off, const int32_t *__restrict__ idx,
-                                   const float *__restrict__ val, int64_t n, int64_t dim,
-                                   double *__restrict__ rs, int32_t *bad) {
-  __shared__ double red[8];
+constexpr int kRowThreads = 512;
+__global__ void __launch_bounds__(kRowThreads)
+sparse_rows_kernel(const int64_t *__restrict__ off, const int32_t *__restrict__ idx,
+                   const float *__restrict__ val, int64_t n, int64_t dim, double *__restrict__ rs,
+                   int32_t *bad) {
+  __shared__ double red[kRowThreads / 32];
   for (int64_t i = blockIdx.x; i < n; i += gridDim.x) {
     double s = 0.0;
+#pragma unroll 4
     for (int64_t e = off[i] + threadIdx.x; e < off[i + 1]; e += blockDim.x) {
       const int32_t k = idx[e];
       if (k < 0 || k >= dim || (e > off[i] && idx[e - 1] >= k)) atomicExch(bad, 1);
@@ -298,7 +468,8 @@ void free_sparse(SparseStore &sp) {
   dfree(sp.d_cptr);
   dfree(sp.d_rs);
   dfree(sp.d_tiles);
-  dfree(sp.d_jperm);
+  dfree(sp.d_chunks);
+  dfree(sp.d_heads);
 }
 
 ap_status create_sparse(const ap_items_desc *d, ap_items *it, cudaStream_t s) {
@@ -329,7 +500,7 @@ ap_status create_sparse(const ap_items_desc *d, ap_items *it, cudaStream_t s) {
   AP_TRY(cudaMemsetAsync(d_bad, 0, 4, s));
   if (sp.n > 0) {
     const int g = (int)std::min<int64_t>(sp.n, 65535);
-    sparse_rows_kernel<<<g, 256, 0, s>>>(sp.d_off, sp.d_idx, sp.d_val, sp.n, sp.dim, sp.d_rs,
+    sparse_rows_kernel<<<g, kRowThreads, 0, s>>>(sp.d_off, sp.d_idx, sp.d_val, sp.n, sp.dim, sp.d_rs,
                                          d_bad);
     AP_TRY(cudaGetLastError());
     const int64_t total = (sp.n_chunks + 1) * sp.n;
@@ -337,64 +508,98 @@ ap_status create_sparse(const ap_items_desc *d, ap_items *it, cudaStream_t s) {
     sparse_cptr_kernel<<<g2, 256, 0, s>>>(sp.d_off, sp.d_idx, sp.n, sp.n_chunks, sp.d_cptr);
     AP_TRY(cudaGetLastError());
   }
-  // row slots of each J block of BJ items, dealt to the warps by entry
-  // count in a snake (warp w takes slots w, w + kWarps, ...: the w-th
-  // heaviest row, the w-th lightest of the next kWarps, ...), so every
-  // warp's rows j weigh about the same (rows past n count as empty)
-  const int64_t nbi = (sp.n + BI - 1) / BI, nbj = (sp.n + BJ - 1) / BJ;
-  std::vector<int32_t> jperm((size_t)std::max<int64_t>(nbj, 1) * BJ);
-  for (int64_t b = 0; b < nbj; ++b) {
-    int32_t order[BJ];
-    auto cnt = [&](int32_t l) {
-      const int64_t i = b * BJ + l;
-      return i < sp.n ? off[i + 1] - off[i] : (int64_t)-1;
-    };
-    for (int32_t l = 0; l < BJ; ++l) order[l] = l;
-    std::stable_sort(order, order + BJ, [&](int32_t a, int32_t c) { return cnt(a) > cnt(c); });
-    for (int h = 0; h < kJ; ++h)
-      for (int w = 0; w < kWarps; ++w)
-        jperm[(size_t)b * BJ + w + h * kWarps] = order[h * kWarps + ((h & 1) ? kWarps - 1 - w : w)];
+  // what each chunk holds, read back with the verdict on the rows
+  std::vector<ChunkCount> count((size_t)(sp.n > 0 ? sp.n_chunks : 0));
+  ChunkCount *d_count = nullptr;
+  if (!count.empty()) {
+    AP_TRY(dmalloc(&d_count, count.size()));
+    const int g = (int)std::min<int64_t>(sp.n_chunks, (int64_t)num_sms() * 4);
+    sparse_count_kernel<<<g, kJoinThreads, 0, s>>>(sp.d_off, sp.d_idx, sp.d_cptr, sp.n,
+                                                   sp.n_chunks, d_count);
   }
-  AP_TRY(dmalloc(&sp.d_jperm, jperm.size()));
-  AP_TRY(cudaMemcpyAsync(sp.d_jperm, jperm.data(), jperm.size() * 4, cudaMemcpyHostToDevice, s));
-  // tiles (I block of BI items, J block of BJ items) holding a pair i < j,
-  // the J blocks in order and within each its I blocks
+  int32_t bad = 0;
+  cudaError_t e = cudaGetLastError();
+  if (e == cudaSuccess) e = cudaMemcpyAsync(&bad, d_bad, 4, cudaMemcpyDeviceToHost, s);
+  if (e == cudaSuccess && !count.empty())
+    e = cudaMemcpyAsync(count.data(), d_count, count.size() * sizeof(ChunkCount),
+                        cudaMemcpyDeviceToHost, s);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+  dfree(d_count);
+  if (e != cudaSuccess) return from_cuda(e);
+  if (bad) return AP_ERR_INVALID_ARG;
+
   std::vector<int32_t> tiles;
-  for (int64_t bj = 0; bj < nbj; ++bj)
-    for (int64_t bi = 0; bi < nbi && bi * BI < (bj + 1) * BJ - 1; ++bi) {
-      tiles.push_back((int32_t)bi);
-      tiles.push_back((int32_t)bj);
-    }
+  dc_block_pairs((sp.n + kDenseTile - 1) / kDenseTile, tiles);
   sp.n_tiles = (int64_t)tiles.size() / 2;
+  // Each chunk by the cheaper way (picoseconds of the whole GPU): a join adds
+  // kJoinProductPs per product and kJoinEntryPs per entry, a dense chunk costs
+  // kDenseTilePs per tile whatever it holds.  A code in more rows than a join
+  // sorts at a time makes its chunk a dense one.  join chunks first in the list
+  std::vector<int32_t> join, dense;
+  for (int64_t c = 0; c < (int64_t)count.size(); ++c) {
+    const ChunkCount &k = count[c];
+    if (k.products == 0) continue;               // no code in two rows
+    const double way_join = kJoinProductPs * (double)k.products + kJoinEntryPs * (double)k.entries;
+    const bool d = k.most > kJoinCap || way_join > kDenseTilePs * (double)sp.n_tiles;
+    (d ? dense : join).push_back((int32_t)c);
+  }
+  // heaviest joins first: their times differ, and the queue ends with a tail
+  std::stable_sort(join.begin(), join.end(), [&](int32_t a, int32_t b) {
+    return count[a].products + count[a].entries > count[b].products + count[b].entries;
+  });
+  sp.n_join = (int64_t)join.size();
+  sp.n_dense = (int64_t)dense.size();
+  join.insert(join.end(), dense.begin(), dense.end());
+  AP_TRY(dmalloc(&sp.d_chunks, std::max<size_t>(join.size(), 1)));
   AP_TRY(dmalloc(&sp.d_tiles, std::max<size_t>(tiles.size(), 2)));
+  AP_TRY(dmalloc(&sp.d_heads, 2));
+  if (!join.empty())
+    AP_TRY(cudaMemcpyAsync(sp.d_chunks, join.data(), join.size() * 4, cudaMemcpyHostToDevice, s));
   if (!tiles.empty())
     AP_TRY(cudaMemcpyAsync(sp.d_tiles, tiles.data(), tiles.size() * 4, cudaMemcpyHostToDevice, s));
-  int32_t bad = 0;
-  AP_TRY(cudaMemcpyAsync(&bad, d_bad, 4, cudaMemcpyDeviceToHost, s));
-  AP_TRY(cudaStreamSynchronize(s));
-  if (bad) return AP_ERR_INVALID_ARG;
   it->stats.tiles = sp.n_tiles;
-  it->stats.tile_m = BI;
-  it->stats.tile_n = BJ;
+  it->stats.tile_m = it->stats.tile_n = kSparseBlock;
   return AP_OK;
 }
 
-cudaError_t launch_sparse_cosine(const SparseStore &sp, double *out, int coverage,
-                                 int32_t *queue, cudaStream_t s) {
+cudaError_t launch_sparse_cosine(const SparseStore &sp, void *out, int coverage, cudaStream_t s) {
   if (sp.n_tiles <= 0) return cudaSuccess;
-  const size_t smem = (size_t)kRows * W * 4 + (size_t)BI * BJ * 8 +
-                      (size_t)kWarps * 2 * sizeof(WarpStage);
-  void (*kern)(const int64_t *, const int32_t *, const float *, const int32_t *, const double *,
-               int64_t, int64_t, const int32_t *, int64_t, const int32_t *, int32_t *, void *) =
-      coverage ? sparse_cos_kernel<1> : sparse_cos_kernel<0>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = cudaMemsetAsync(sp.d_heads, 0, 2 * sizeof(*sp.d_heads), s);
   if (e != cudaSuccess) return e;
-  e = cudaMemsetAsync(queue, 0, sizeof(int32_t), s);
+  const int64_t slots = 2 * (int64_t)num_sms();      // two CTAs per SM, both kernels
+  if (coverage) {
+    sparse_dense_kernel<1><<<(int)std::min(slots, sp.n_tiles), 256, 0, s>>>(
+        sp.d_off, sp.d_idx, sp.d_val, sp.d_cptr, sp.n, sp.d_chunks, 1, 1, sp.d_tiles, sp.n_tiles,
+        sp.d_heads, out);
+    return cudaGetLastError();
+  }
+  double *o = reinterpret_cast<double *>(out);
+  e = cudaMemsetAsync(o, 0, (size_t)(sp.n * (sp.n - 1) / 2) * sizeof(double), s);
   if (e != cudaSuccess) return e;
-  const int64_t grid = std::min<int64_t>((int64_t)num_sms(), sp.n_tiles);
-  kern<<<(int)grid, kThreads, smem, s>>>(sp.d_off, sp.d_idx, sp.d_val, sp.d_cptr, sp.d_rs, sp.n,
-                                         sp.n_chunks, sp.d_tiles, sp.n_tiles, sp.d_jperm, queue,
-                                         out);
+  if (sp.n_dense > 0) {
+    e = cudaFuncSetAttribute(sparse_dense_kernel<0>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)kDenseSmem);
+    if (e != cudaSuccess) return e;
+    // parts of a chunk where whole ones leave SMs idle (at least 4 stages each)
+    int32_t split = 1;
+    while (split < 32 && sp.n_dense * sp.n_tiles * split < slots) split *= 2;
+    const int64_t units = sp.n_dense * sp.n_tiles * split;
+    sparse_dense_kernel<0><<<(int)std::min(slots, units), 256, kDenseSmem, s>>>(
+        sp.d_off, sp.d_idx, sp.d_val, sp.d_cptr, sp.n, sp.d_chunks + sp.n_join,
+        (int32_t)sp.n_dense, split, sp.d_tiles, sp.n_tiles, sp.d_heads, out);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  }
+  if (sp.n_join > 0) {
+    e = cudaFuncSetAttribute(sparse_join_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)kJoinSmem);
+    if (e != cudaSuccess) return e;
+    sparse_join_kernel<<<(int)std::min(slots, sp.n_join), kJoinThreads, kJoinSmem, s>>>(
+        sp.d_off, sp.d_idx, sp.d_val, sp.d_cptr, sp.n, sp.d_chunks, (int32_t)sp.n_join,
+        sp.d_heads + 1, o);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  }
+  const int grid = (int)std::min<int64_t>(sp.n - 1, 65535);
+  sparse_scale_kernel<<<grid, 256, 0, s>>>(o, sp.d_rs, sp.n);
   return cudaGetLastError();
 }
 

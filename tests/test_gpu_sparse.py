@@ -82,3 +82,32 @@ def test_cosine_rejects_bad_rows(ap):
     with pytest.raises(ap.APError):                            # duplicate code
         ap.Items.from_sparse(off, np.array([1, 5, 5, 0, 2], np.int32),
                              np.ones(5, np.float32), 100)
+
+
+@pytest.mark.parametrize("n,dim,lo,hi", [
+    (130, 4097, 1500, 4097),      # dense chunks, two row blocks, a chunk of one code
+    (129, 20000, 5, 60),          # join chunks, a ragged row block
+    (40, 12288, 8, 4000),         # rows a hundred times as heavy as others
+    (700, 8192, 20, 300)])        # join chunks sorted in several rounds
+def test_cosine_join_and_dense_chunks(ap, oracle_lib, n, dim, lo, hi):
+    rng = np.random.default_rng(n)
+    sizes = np.exp(rng.uniform(np.log(lo), np.log(hi), n)).astype(np.int64).clip(lo, hi)
+    rows = [np.sort(rng.choice(dim, s, replace=False)) for s in sizes]
+    off = np.concatenate([[0], np.cumsum(sizes)]).astype(np.int64)
+    idx = np.concatenate(rows).astype(np.int32)
+    val = (0.6 * rng.standard_normal(dim)[idx] + rng.standard_normal(len(idx))).astype(np.float32)
+    _check(ap, oracle_lib, off, idx, val, dim)
+
+
+def test_cosine_chunks_mixed(ap, oracle_lib):
+    """Frequent codes in a few chunks (dense), rare ones in the rest (join),
+    and one code that every row holds."""
+    rng = np.random.default_rng(5)
+    n, dim = 150, 40960
+    rows = [np.unique(np.concatenate([[0], rng.choice(8192, 2500, replace=False),
+                                      8192 + rng.choice(dim - 8192, 120, replace=False)]))
+            for _ in range(n)]
+    off = np.concatenate([[0], np.cumsum([len(r) for r in rows])]).astype(np.int64)
+    idx = np.concatenate(rows).astype(np.int32)
+    val = (rng.standard_normal(dim)[idx] + rng.standard_normal(len(idx))).astype(np.float32)
+    _check(ap, oracle_lib, off, idx, val, dim, device_input=True)

@@ -181,9 +181,9 @@ typedef struct ap_plan {
    * range by range inside waves of one tile per SM, so the tiles in flight
    * read the same columns and share them in L2; the partial Grams meet in
    * FP64 in the output, which a last pass scales by rs_i rs_j.  The default
-   * (set at creation, and by ap_set_plan with k_split = -1): ranges of about
-   * 16384 columns and at least two units per SM, at most one range per 64
-   * columns; 0 where that gives one range */
+   * (set at creation, and by ap_set_plan with k_split = -1): ranges of at most
+   * 16384 and at least 64 columns, as many as fill whole rounds of the units
+   * that run at once; 0 where that gives one range */
   int32_t k_split;
   /* vector sets only: CTAs per tensor-core MMA.  2 (the default; 0 in
    * ap_set_plan asks for it): the units are 256 x 256 block pairs, each

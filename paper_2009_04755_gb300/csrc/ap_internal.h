@@ -39,6 +39,17 @@ __host__ __device__ __forceinline__ int64_t pair_index(int64_t i, int64_t j, int
   return i * n - (i * (i + 1)) / 2 + (j - i - 1);
 }
 
+// float -> double on the integer pipe: GB300 converts on its FP64 pipe, two
+// values per clock and SM, which an epilogue of 32,768 sums a CTA feels
+#ifdef __CUDACC__
+__device__ __forceinline__ double widen(float x) {
+  const uint32_t u = __float_as_uint(x), m = u & 0x7fffffffu;
+  if (m - 0x00800000u >= 0x7f000000u && m != 0) return (double)x;   // subnormal, infinite, NaN
+  const uint32_t hi = (u & 0x80000000u) | (m ? (m >> 3) + 0x38000000u : 0u);
+  return __hiloint2double((int)hi, (int)(u << 29));
+}
+#endif
+
 // ---------------------------------------------------------------------------
 // point-cloud storage: items sorted by the planner, padded to a multiple of
 // 4 points, held in pairs of points so that one packed FP32x2 operation takes
@@ -195,7 +206,6 @@ struct VecStore {
   double *d_mu = nullptr, *d_ss = nullptr, *d_rs = nullptr;   // FP64 per item (d_mu: the shift)
   double *d_delta_all = nullptr;    // mean - shift per item
   double *d_partc = nullptr;        // [n][kSplitParts] partial sums of c
-  int32_t *d_recentre = nullptr;    // [n + 1]: count, rows centred again
   double *d_part = nullptr;         // [n][kSplitParts] partial sums of c^2
   int64_t n_rows_alloc = 0;         // rows rounded up to the row block
   __nv_bfloat16 *d_hi = nullptr, *d_lo = nullptr;              // [n][Dp]
@@ -244,6 +254,8 @@ struct VecStore {
   // columns: k_split = 0 and coverage)
   int32_t mma_ctas = 2;
   int32_t *d_pair_units = nullptr; int64_t n_pair_units = 0;
+  float *d_planes = nullptr;        // [n_planes][n (n - 1) / 2] partial Grams of d_pair_units;
+  int64_t n_planes = 0;             // without them the units add into the output
   int32_t *d_pair_whole = nullptr; int64_t n_pair_whole = 0;
   std::vector<int32_t> h_tiles_tc;
   int32_t *d_tiles_f32 = nullptr; int64_t n_tiles_f32 = 0;
@@ -383,21 +395,23 @@ __host__ __device__ __forceinline__ size_t blocked_offset(int64_t row, int64_t k
 }
 cudaError_t launch_vec_mean(const float *X, int64_t n, int64_t D, int64_t ld, double *mu,
                             cudaStream_t s);
-// the single-pass load pipeline of vectors: per row a shift (the mean of
+// the load pipeline of vectors in one launch: per row a shift (the mean of
 // evenly spread samples), then the centred split / FP32 copies and the FP64
 // sums of c and c^2 in one pass, then delta = mean - shift, ss and rs; rows
 // whose shift missed the mean by D delta^2 > ss / 64 are redone from the
-// exact mean.  recentre: device int32 [n + 1] scratch (count, rows).
+// exact mean.
 cudaError_t launch_vec_prep(const float *X, int64_t row0, int64_t out_row0, int64_t n, int64_t D,
                             int64_t ld, int64_t Dp, __nv_bfloat16 *hi, __nv_bfloat16 *lo,
-                            float *c32, double *shift, double *part, double *part_c,
-                            double *delta, double *ss, double *rs, int32_t *recentre,
+                            float *c32, double *shift, double *delta, double *ss, double *rs,
                             cudaStream_t s);
 // out[p] -= (D delta_i rs_i)(delta_j rs_j) over the packed triangle: the
 // mean correction of pairs the Gram kernel already scaled by rs_i rs_j
 cudaError_t launch_pair_correct(double *out, const double *rs, const double *delta, int64_t n,
                                 int64_t D, cudaStream_t s);
 // out[p] = (out[p] - D delta_i delta_j) rs_i rs_j over the packed triangle
+// out[p] = (sum over r of planes[r][p] - D delta_i delta_j) rs_i rs_j
+cudaError_t launch_pair_planes(double *out, const float *planes, int64_t k, const double *rs,
+                               const double *delta, int64_t n, int64_t D, cudaStream_t s);
 cudaError_t launch_pair_finalize(double *out, const double *rs, const double *delta, int64_t n,
                                  int64_t D, cudaStream_t s);
 // columns [col0, col0 + width) of rows row0.. (cols of them real, staged
@@ -448,6 +462,13 @@ cudaError_t launch_gram_tc2(const void *tmap_hi, const void *tmap_lo, int64_t n,
                             const int32_t *units, int64_t n_units, int32_t *queue,
                             int32_t *status, double *g64, void *out, int coverage, int atomic,
                             uint64_t budget, int32_t debug, cudaStream_t s);
+// split-K units of the resident set, listed by pair_units with k_split ranges
+// of at most kKSplitCols columns: range r's partial Grams stored as FP32 in
+// planes[r][n (n - 1) / 2]
+cudaError_t launch_gram_tc2_store(const void *tmap_hi, const void *tmap_lo, int64_t n,
+                                  const int32_t *units, int64_t n_units, int64_t k_split,
+                                  int32_t *queue, int32_t *status, float *planes, uint64_t budget,
+                                  int32_t debug, cudaStream_t s);
 // CTA pairs of one launch (clusters of two that fit on the device at once)
 int64_t tc2_pairs();
 // units of the CTA-pair Gram over the resident set: macro pairs (I <= J, 256
@@ -481,7 +502,8 @@ void panel_units(const std::vector<int32_t> &tiles, int64_t nchunks, int64_t gro
                  int64_t k_split, std::vector<int32_t> &units);
 // the split-K schedule of a vector set's split-BF16 Gram: k_split column
 // ranges per tile (0 whole tiles, -1 the default rule of default_k_split)
-int32_t default_k_split(int64_t n_tiles, int64_t Dp);
+int32_t default_k_split(int64_t n_tiles, int64_t slots, int64_t Dp, int64_t pairs);
+constexpr int64_t kPlaneBytes = 256ll << 20;    // most the planes of a set may take
 ap_status set_vector_plan(ap_items *it, int32_t k_split, int32_t mma_ctas = 0);
 
 // the particle scores' re-scaled cloud storage and L2 self terms, built on
@@ -523,6 +545,7 @@ cudaError_t launch_sparse_cosine(const SparseStore &sp, void *out, int coverage,
 // or coordinate is outside the range in which two terms may share a
 // reciprocal; some weight is not 1
 constexpr int kQueueClouds = 3, kQueueTraits = 4;
+constexpr int kQueuePairs = 5;          // head of the CTA-pair Gram's queue, reset the same way
 constexpr int32_t kCloudWide = 1, kCloudWeighted = 2;
 // tiles at the end of a cloud plan's list that are split: one per CTA slot
 // (four CTAs of four warps per SM)

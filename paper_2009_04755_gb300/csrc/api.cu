@@ -62,9 +62,9 @@ void free_items(ap_items *it) {
   VecStore &v = it->vec;
   dfree(v.d_mu); dfree(v.d_ss); dfree(v.d_rs); dfree(v.d_part); dfree(v.d_hi); dfree(v.d_lo); dfree(v.d_c32);
   dfree(v.d_rows);
-  dfree(v.d_partc); dfree(v.d_delta_all); dfree(v.d_recentre);
+  dfree(v.d_partc); dfree(v.d_delta_all);
   dfree(v.d_stage); dfree(v.d_tiles_tc); dfree(v.d_tiles_f32); dfree(v.d_g64);
-  dfree(v.d_panel_units); dfree(v.d_pair_units); dfree(v.d_pair_whole);
+  dfree(v.d_panel_units); dfree(v.d_pair_units); dfree(v.d_pair_whole); dfree(v.d_planes);
   free_out_of_core(v);
   free_sparse(it->sp);
   free_tc_tensor_maps(v.tmap_hi, v.tmap_lo);
@@ -244,8 +244,8 @@ ap_status vec_load(ap_items *it, const float *data, int on_host, cudaStream_t s)
   const bool f32 = (v.precisions & (1u << AP_PREC_FP32)) != 0;
   if (!on_host) {
     AP_TRY(launch_vec_prep(data, 0, 0, v.n, v.D, v.ld, v.Dp, split ? v.d_hi : nullptr,
-                           split ? v.d_lo : nullptr, f32 ? v.d_c32 : nullptr, v.d_mu, v.d_part,
-                           v.d_partc, v.d_delta_all, v.d_ss, v.d_rs, v.d_recentre, s));
+                           split ? v.d_lo : nullptr, f32 ? v.d_c32 : nullptr, v.d_mu,
+                           v.d_delta_all, v.d_ss, v.d_rs, s));
     return AP_OK;
   }
   // host source: two staging buffers, copies on the copy stream overlap the
@@ -273,8 +273,8 @@ ap_status vec_load(ap_items *it, const float *data, int on_host, cudaStream_t s)
     if (e == cudaSuccess) e = cudaStreamWaitEvent(s, copied[b], 0);
     if (e == cudaSuccess)
       e = launch_vec_prep(stage, r0, r0, nr, v.D, v.ld, v.Dp, split ? v.d_hi : nullptr,
-                          split ? v.d_lo : nullptr, f32 ? v.d_c32 : nullptr, v.d_mu, v.d_part,
-                          v.d_partc, v.d_delta_all, v.d_ss, v.d_rs, v.d_recentre, s);
+                          split ? v.d_lo : nullptr, f32 ? v.d_c32 : nullptr, v.d_mu,
+                           v.d_delta_all, v.d_ss, v.d_rs, s);
     if (e == cudaSuccess) e = cudaEventRecord(done[b], s);
   }
   if (e != cudaSuccess) st = from_cuda(e);
@@ -311,7 +311,6 @@ ap_status create_vectors(const ap_items_desc *d, ap_items *it, cudaStream_t s) {
   AP_TRY(dmalloc(&v.d_part, (size_t)nn * kSplitParts));
   AP_TRY(dmalloc(&v.d_partc, (size_t)nn * kSplitParts));
   AP_TRY(dmalloc(&v.d_delta_all, nn));
-  AP_TRY(dmalloc(&v.d_recentre, nn + 1));
   // out-of-core: items stay in host memory and stream through the slot cache
   if (d->slot_cache_bytes) return create_out_of_core(d, it);
   // blocked copies cover whole row blocks; the padding rows stay zero
@@ -507,18 +506,26 @@ ap_status ap_run_pairs(ap_items *it, int32_t fn, int32_t precision, const float 
     if (!use_split && !have_f32) return AP_ERR_STATE;
     const bool pairs = v.mma_ctas == 2;
     if (use_split && !cover && v.k_split > 0) {
-      // split-K units in waves: partial Grams meet in FP64 in `out`
-      AP_TRY(cudaMemsetAsync(out, 0, (size_t)(n * (n - 1) / 2) * sizeof(double), s));
-      if (pairs)
-        AP_TRY(launch_gram_tc2(v.tmap_hi, v.tmap_lo, v.n, v.d_rs, v.d_pair_units, v.n_pair_units,
-                               it->d_queue, it->d_status, v.d_g64, out, 0, 1,
-                               it->wait_budget_ns, it->debug, s));
-      else
-        AP_TRY(launch_gram_tc(v.tmap_hi, v.tmap_lo, v.n, v.Dp, v.d_rs, v.d_panel_units,
-                              v.n_panel_units, it->d_queue, it->d_status, v.d_g64, out, 0, 1,
-                              it->wait_budget_ns, it->debug, s));
-      AP_TRY(launch_pair_finalize(reinterpret_cast<double *>(out), v.d_rs, v.d_delta_all, v.n,
-                                  v.D, s));
+      // split-K units in waves: partial Grams in planes that the scaling pass
+      // sums, or added in FP64 into `out`
+      double *o = reinterpret_cast<double *>(out);
+      if (pairs && v.d_planes) {
+        AP_TRY(launch_gram_tc2_store(v.tmap_hi, v.tmap_lo, v.n, v.d_pair_units, v.n_pair_units,
+                                     v.n_planes, it->d_queue, it->d_status, v.d_planes,
+                                     it->wait_budget_ns, it->debug, s));
+        AP_TRY(launch_pair_planes(o, v.d_planes, v.n_planes, v.d_rs, v.d_delta_all, v.n, v.D, s));
+      } else {
+        AP_TRY(cudaMemsetAsync(out, 0, (size_t)(n * (n - 1) / 2) * sizeof(double), s));
+        if (pairs)
+          AP_TRY(launch_gram_tc2(v.tmap_hi, v.tmap_lo, v.n, v.d_rs, v.d_pair_units,
+                                 v.n_pair_units, it->d_queue, it->d_status, v.d_g64, out, 0, 1,
+                                 it->wait_budget_ns, it->debug, s));
+        else
+          AP_TRY(launch_gram_tc(v.tmap_hi, v.tmap_lo, v.n, v.Dp, v.d_rs, v.d_panel_units,
+                                v.n_panel_units, it->d_queue, it->d_status, v.d_g64, out, 0, 1,
+                                it->wait_budget_ns, it->debug, s));
+        AP_TRY(launch_pair_finalize(o, v.d_rs, v.d_delta_all, v.n, v.D, s));
+      }
       it->stats.tiles = pairs ? v.n_pair_units : v.n_panel_units;
       it->stats.tile_m = pairs ? 2 * kTcTileM : kTcTileM;
       it->stats.tile_n = kTcTileN;
@@ -648,8 +655,9 @@ int32_t ap_last_device_error(ap_items *it) {
   if (cudaMemcpy(&v, it->d_status, sizeof v, cudaMemcpyDeviceToHost) != cudaSuccess) return -1;
   if (v != 0) {
     cudaMemset(it->d_status, 0, sizeof v);
-    // an aborted launch leaves its clouds' queue part-way
+    // an aborted launch leaves its queue part-way
     cudaMemset(it->d_queue + kQueueClouds, 0, sizeof v);
+    cudaMemset(it->d_queue + kQueuePairs, 0, sizeof v);
   }
   return v;
 }

@@ -65,6 +65,9 @@ constexpr int kRing = 4;                     // units handed out ahead
 // epilogue warps of both CTAs
 constexpr int kUnitConsumers = 2 + 2 * kEpiWarps;
 constexpr int kChainStages = 8;              // one accumulation chain = 256 columns of D
+// units of up to 2048 columns take chains of 128: the longer chain's truncation
+// (4.9e-6 of the 2-norm against 4.4e-6 at 2360 x 517) buys nothing there
+constexpr int kShortUnit = 2048 / BK, kShortChain = 4;
 constexpr int kHeadStages = 2;               // the first two chains of a unit: 64 columns
 constexpr float kSeedBeta = 0.9f;
 constexpr int kFlushCols = 16384;
@@ -112,30 +115,45 @@ __device__ __forceinline__ void mbar_complete_tx(uint32_t bar, uint32_t bytes) {
   asm volatile("mbarrier.complete_tx.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
 }
 
-__device__ __forceinline__ int64_t chain_first(int64_t c) {
-  return c < 2 ? c * kHeadStages : 2 * kHeadStages + (c - 2) * kChainStages;
+__device__ __forceinline__ int64_t chain_length(int64_t nkb) {
+  return nkb <= kShortUnit ? kShortChain : kChainStages;
+}
+__device__ __forceinline__ int64_t chain_first(int64_t c, int64_t nkb) {
+  return c < 2 ? c * kHeadStages : 2 * kHeadStages + (c - 2) * chain_length(nkb);
 }
 __device__ __forceinline__ int64_t chain_stages(int64_t c, int64_t nkb) {
-  const int64_t len = c < 2 ? kHeadStages : kChainStages, left = nkb - chain_first(c);
+  const int64_t len = c < 2 ? kHeadStages : chain_length(nkb), left = nkb - chain_first(c, nkb);
   return left < len ? left : len;
 }
 __device__ __forceinline__ int64_t chain_count(int64_t nkb) {
+  const int64_t len = chain_length(nkb);
   return nkb <= 2 * kHeadStages ? (nkb + kHeadStages - 1) / kHeadStages
-                                : 2 + (nkb - 2 * kHeadStages + kChainStages - 1) / kChainStages;
+                                : 2 + (nkb - 2 * kHeadStages + len - 1) / len;
 }
 
-// ATOMIC = 1: the unit's partial Gram is added into FP64 `out` (split-K: several
-// column ranges of one block pair); ATOMIC = 0: whole block pairs, out = G rs_i rs_j.
-// COVER = 1: no arithmetic, each pair of the unit adds 1 to int32 `out`.
+// OUT: what becomes of a unit's partial Gram.  kWhole: the unit is a whole
+// block pair, out = G rs_i rs_j; kAdd: added into FP64 `out`; kStore: stored as
+// FP32 sums in plane `range` of `out` (n (n - 1) / 2 floats each), range = the
+// unit's place in the split of its block pair (SplitOrder); kCover: no
+// arithmetic, each pair of the unit adds 1 to int32 `out`.
+// kStore needs no cleared output and leaves the sums' order fixed: a run is two
+// launches (100 x 1000: 21 us against 35 with the output cleared, added into and
+// scaled); large sets, whose planes would be too many bytes, add.
 // Registers: each of the SM's four sub-partitions holds 16384 of them and
 // ten warps put three warps on two sub-partitions, so 3 x 32 x 168 = 16128
 // is the most a thread may take and the CTA still launch.
-template <int COVER, int ATOMIC>
+enum Out { kWhole = 0, kAdd = 1, kStore = 2, kCover = 3 };
+// the order pair_units lists units in: waves of `group` block pairs, in each
+// the first range of every block pair, then the second, ...
+struct SplitOrder { int32_t tiles, group, k_split; };
+
+template <int OUT>
 __global__ void __maxnreg__(168)
 gram_tc2_kernel(const __grid_constant__ CUtensorMap tm_hi, const __grid_constant__ CUtensorMap tm_lo,
                 int64_t n, const double *__restrict__ rs, const int32_t *__restrict__ units,
                 int32_t n_units, int32_t *queue, int32_t *status, double *__restrict__ g64,
-                void *out, uint64_t budget, int32_t debug) {
+                void *out, SplitOrder order, uint64_t budget, int32_t debug) {
+  constexpr bool COVER = OUT == kCover;
   extern __shared__ uint8_t smem_raw[];
   uint8_t *smem = reinterpret_cast<uint8_t *>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
@@ -235,7 +253,12 @@ gram_tc2_kernel(const __grid_constant__ CUtensorMap tm_hi, const __grid_constant
           abort_pair(DEV_TIMEOUT_UNIT);
           break;
         }
+        // each pair of CTAs pops once past the last unit; the last of these
+        // pops leaves the queue as it was found (an aborted run does not, and
+        // nothing runs until the host has cleared the status and the queue)
         t = atomicAdd(queue, 1);
+        if (t == n_units + (int32_t)(gridDim.x >> 1) - 1)
+          *reinterpret_cast<volatile int32_t *>(queue) = 0;
         if (*s_abort || *reinterpret_cast<volatile int32_t *>(status) != 0) t = n_units;
         if (t > n_units) t = n_units;
         ring[us] = t;
@@ -424,7 +447,7 @@ gram_tc2_kernel(const __grid_constant__ CUtensorMap tm_hi, const __grid_constant
         tc_fence_before();
         __syncwarp();
         if (lane == 0) arrive_leader(bar(B_TEMPTY + a));
-        if (kb_since >= kFlushKb && c + 1 < nchains) {
+        if (OUT != kStore && kb_since >= kFlushKb && c + 1 < nchains) {
           kb_since = 0;
           // fold the FP32 partial sums into FP64 scratch ([col][row] layout)
 #pragma unroll
@@ -438,6 +461,12 @@ gram_tc2_kernel(const __grid_constant__ CUtensorMap tm_hi, const __grid_constant
         }
       }
       if (!ok) break;
+      int32_t range = 0;
+      if (OUT == kStore) {
+        const int32_t wave = t / (order.group * order.k_split);
+        const int32_t left = order.tiles - wave * order.group;
+        range = (t - wave * order.group * order.k_split) / (left < order.group ? left : order.group);
+      }
       // output: 32 columns at a time through the warp's transpose buffer, so
       // that one warp instruction covers 32 consecutive pairs (i, j..j+31)
       // of one row
@@ -450,20 +479,28 @@ gram_tc2_kernel(const __grid_constant__ CUtensorMap tm_hi, const __grid_constant
         }
         __syncwarp();
         const int64_t jc = j + cb * 32;
-#pragma unroll 1
+        // rows r < r_end exist and lie above the diagonal; row i + 1's pair
+        // with jc comes n - i - 2 places after row i's
+        const int64_t ir = i0 + q * 32;
+        const int64_t lim = jc < n ? jc - ir : 0;      // i < jc implies i < n
+        const int r_end = lim < 32 ? (int)(lim > 0 ? lim : 0) : 32;
+        int64_t p = pair_index(ir, jc, n);
+        if (OUT == kStore) p += (int64_t)range * (n * (n - 1) / 2);
+#pragma unroll 4
         for (int r = 0; r < 32; ++r) {
-          const int64_t i = i0 + q * 32 + r;
-          if (i < n && jc > i && jc < n) {
-            const int64_t p = pair_index(i, jc, n);
+          if (r < r_end) {
             if (COVER) {
               atomicAdd(reinterpret_cast<int32_t *>(out) + p, 1);
+            } else if (OUT == kStore) {
+              reinterpret_cast<float *>(out)[p] = tb[r * kTrStride + lane];
             } else {
-              double g = (double)tb[r * kTrStride + lane];
+              double g = widen(tb[r * kTrStride + lane]);
               if (flushed) g += my_g64[(size_t)(h * (BN / 2) + cb * 32 + lane) * BM + q * 32 + r];
-              if (ATOMIC) atomicAdd(reinterpret_cast<double *>(out) + p, g);
-              else reinterpret_cast<double *>(out)[p] = g * rs[i] * rs[jc];
+              if (OUT == kAdd) atomicAdd(reinterpret_cast<double *>(out) + p, g);
+              else reinterpret_cast<double *>(out)[p] = g * rs[ir + r] * rs[jc];
             }
           }
+          p += n - ir - r - 2;
         }
         __syncwarp();
       }
@@ -503,11 +540,15 @@ gram_tc2_kernel(const __grid_constant__ CUtensorMap tm_hi, const __grid_constant
 }
 
 using Kern2 = void (*)(CUtensorMap, CUtensorMap, int64_t, const double *, const int32_t *, int32_t,
-                       int32_t *, int32_t *, double *, void *, uint64_t, int32_t);
+                       int32_t *, int32_t *, double *, void *, SplitOrder, uint64_t, int32_t);
 
-Kern2 pick(int coverage, int atomic) {
-  return coverage ? gram_tc2_kernel<1, 0>
-                  : (atomic ? gram_tc2_kernel<0, 1> : gram_tc2_kernel<0, 0>);
+Kern2 pick(int out) {
+  switch (out) {
+    case kCover: return gram_tc2_kernel<kCover>;
+    case kStore: return gram_tc2_kernel<kStore>;
+    case kAdd: return gram_tc2_kernel<kAdd>;
+  }
+  return gram_tc2_kernel<kWhole>;
 }
 
 cudaLaunchConfig_t launch_cfg(int pairs, cudaStream_t s, cudaLaunchAttribute *attr) {
@@ -526,15 +567,14 @@ cudaLaunchConfig_t launch_cfg(int pairs, cudaStream_t s, cudaLaunchAttribute *at
 }
 
 std::mutex g_tc2_mutex;
-bool g_tc2_attr[3] = {false, false, false};
+bool g_tc2_attr[4] = {false, false, false, false};
 
-cudaError_t ensure_attr(int coverage, int atomic) {
-  const int v = coverage ? 2 : atomic;
+cudaError_t ensure_attr(int out) {
   std::lock_guard<std::mutex> lock(g_tc2_mutex);
-  if (g_tc2_attr[v]) return cudaSuccess;
-  cudaError_t e = cudaFuncSetAttribute(pick(coverage, atomic),
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
-  if (e == cudaSuccess) g_tc2_attr[v] = true;
+  if (g_tc2_attr[out]) return cudaSuccess;
+  cudaError_t e = cudaFuncSetAttribute(pick(out), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       SMEM_BYTES);
+  if (e == cudaSuccess) g_tc2_attr[out] = true;
   return e;
 }
 
@@ -551,9 +591,9 @@ int64_t tc2_pairs() {
   int v = 0;
   cudaLaunchAttribute attr[1];
   cudaLaunchConfig_t cfg = launch_cfg(1, nullptr, attr);
-  if (cudaFuncSetAttribute(gram_tc2_kernel<0, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  if (cudaFuncSetAttribute(gram_tc2_kernel<kAdd>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            SMEM_BYTES) != cudaSuccess ||
-      cudaOccupancyMaxActiveClusters(&v, gram_tc2_kernel<0, 1>, &cfg) != cudaSuccess || v <= 0) {
+      cudaOccupancyMaxActiveClusters(&v, gram_tc2_kernel<kAdd>, &cfg) != cudaSuccess || v <= 0) {
     cudaGetLastError();
     v = num_sms() / 2;
   }
@@ -561,25 +601,41 @@ int64_t tc2_pairs() {
   return v;
 }
 
-cudaError_t launch_gram_tc2(const void *tmap_hi, const void *tmap_lo, int64_t n, const double *rs,
-                            const int32_t *units, int64_t n_units, int32_t *queue,
-                            int32_t *status, double *g64, void *out, int coverage, int atomic,
-                            uint64_t budget, int32_t debug, cudaStream_t s) {
+namespace {
+cudaError_t launch(const void *tmap_hi, const void *tmap_lo, int64_t n, const double *rs,
+                   const int32_t *units, int64_t n_units, int32_t *queue, int32_t *status,
+                   double *g64, void *out, int what, SplitOrder order, uint64_t budget,
+                   int32_t debug, cudaStream_t s) {
   if (n_units <= 0) return cudaSuccess;
   if (n_units > INT32_MAX / 2) return cudaErrorInvalidValue;
-  cudaError_t e = ensure_attr(coverage, atomic);
-  if (e != cudaSuccess) return e;
-  e = cudaMemsetAsync(queue, 0, sizeof(int32_t), s);
+  cudaError_t e = ensure_attr(what);
   if (e != cudaSuccess) return e;
   int64_t pairs = tc2_pairs();
   if (pairs > n_units) pairs = n_units;
   cudaLaunchAttribute attr[1];
   cudaLaunchConfig_t cfg = launch_cfg((int)pairs, s, attr);
-  return cudaLaunchKernelEx(&cfg, pick(coverage, atomic),
-                            *reinterpret_cast<const CUtensorMap *>(tmap_hi),
+  return cudaLaunchKernelEx(&cfg, pick(what), *reinterpret_cast<const CUtensorMap *>(tmap_hi),
                             *reinterpret_cast<const CUtensorMap *>(tmap_lo), n, rs, units,
-                            (int32_t)n_units, queue, status, g64, out,
+                            (int32_t)n_units, queue + kQueuePairs, status, g64, out, order,
                             (uint64_t)(budget ? budget : kWaitBudgetNs), debug);
+}
+}  // namespace
+
+cudaError_t launch_gram_tc2(const void *tmap_hi, const void *tmap_lo, int64_t n, const double *rs,
+                            const int32_t *units, int64_t n_units, int32_t *queue,
+                            int32_t *status, double *g64, void *out, int coverage, int atomic,
+                            uint64_t budget, int32_t debug, cudaStream_t s) {
+  return launch(tmap_hi, tmap_lo, n, rs, units, n_units, queue, status, g64, out,
+                coverage ? kCover : atomic ? kAdd : kWhole, SplitOrder{}, budget, debug, s);
+}
+
+cudaError_t launch_gram_tc2_store(const void *tmap_hi, const void *tmap_lo, int64_t n,
+                                  const int32_t *units, int64_t n_units, int64_t k_split,
+                                  int32_t *queue, int32_t *status, float *planes, uint64_t budget,
+                                  int32_t debug, cudaStream_t s) {
+  const SplitOrder order{(int32_t)(n_units / k_split), (int32_t)tc2_pairs(), (int32_t)k_split};
+  return launch(tmap_hi, tmap_lo, n, nullptr, units, n_units, queue, status, nullptr, planes,
+                kStore, order, budget, debug, s);
 }
 
 }  // namespace ap

@@ -347,12 +347,11 @@ static ap_status alloc_slices(VecStore &v) {
   AP_TRY_ST(alloc_raw_ring(v, ring, (size_t)kMacro * v.slice_cols));
   // every block pair of the triangle on CTA pairs, split-K units in waves
   // over one chunk
-  std::vector<int32_t> tiles, units;
-  tc_tiles(v.n, tiles);
-  const int64_t nt = (int64_t)tiles.size() / 2;
+  std::vector<int32_t> units;
+  const int64_t nb = (v.n + kTcTileN - 1) / kTcTileN, nt = nb * (nb + 1) / 2;
   const int64_t nch = v.slice_cols / kOocChunkCols;
-  pair_units(v.n, nch, tc2_pairs(), std::max<int32_t>(1, default_k_split(nt, v.slice_cols)),
-             units);
+  pair_units(v.n, nch, tc2_pairs(),
+             std::max<int32_t>(1, default_k_split(nt, tc2_pairs(), v.slice_cols, 0)), units);
   v.n_slice_units = (int64_t)units.size() / kOocTileInts;
   AP_TRY(dmalloc(&v.d_slice_units, std::max<size_t>(units.size(), kOocTileInts)));
   if (!units.empty())
@@ -535,8 +534,8 @@ ap_status run_out_of_core(ap_items *it, void *out, int coverage, cudaStream_t s)
         AP_TRY(cudaStreamWaitEvent(s, v.ev_raw_ready[b], 0));
         const size_t slot_off = (size_t)slot * kMacro * v.Dp;
         AP_TRY(launch_vec_prep(raw, r0, 0, rows, v.D, v.ld, v.Dp, v.d_pool_hi + slot_off,
-                               v.d_pool_lo + slot_off, nullptr, v.d_mu, v.d_part, v.d_partc,
-                               v.d_delta_all, v.d_ss, v.d_rs, v.d_recentre, s));
+                               v.d_pool_lo + slot_off, nullptr, v.d_mu, v.d_delta_all, v.d_ss,
+                               v.d_rs, s));
         AP_TRY(cudaEventRecord(v.ev_raw_free[b], s));
         v.ring_used[b] = 1;
         h2d += (uint64_t)rows * v.ld * 4;
@@ -680,8 +679,7 @@ static ap_status build_stream_units(VecStore &v, int64_t C) {
         macro.push_back((int32_t)a);
         macro.push_back((int32_t)m);
       }
-      // split-K: the rule of the single-CTA tiles (two 128-row tiles per pair)
-      const int64_t ks = std::max<int32_t>(1, default_k_split(2 * (m + 1), w));
+      const int64_t ks = std::max<int32_t>(1, default_k_split(m + 1, tc2_pairs(), w, 0));
       pair_units_of(macro, nch, tc2_pairs(), ks, col_units);
       for (size_t u = 0; u < col_units.size(); u += kOocTileInts) {
         col_units[u + 6] += (int32_t)off;
@@ -824,9 +822,8 @@ ap_status stream_load_and_run(ap_items *it, const float *h, double *out, cudaStr
     AP_TRY(cudaStreamWaitEvent(it->prep_stream, v.ev_raw_ready[b], 0));
     const int t_prep = tr.begin(2, AP_STAGE_PREPROCESS, (int64_t)m, 0, it->prep_stream);
     AP_TRY(launch_vec_prep(raw, r0, r0, rows, v.D, v.ld, v.Dp, split ? v.d_hi : nullptr,
-                           split ? v.d_lo : nullptr, f32 ? v.d_c32 : nullptr, v.d_mu, v.d_part,
-                           v.d_partc, v.d_delta_all, v.d_ss, v.d_rs, v.d_recentre,
-                           it->prep_stream));
+                           split ? v.d_lo : nullptr, f32 ? v.d_c32 : nullptr, v.d_mu,
+                           v.d_delta_all, v.d_ss, v.d_rs, it->prep_stream));
     tr.end(t_prep, it->prep_stream);
     AP_TRY(cudaEventRecord(v.ev_raw_free[b], it->prep_stream));
     AP_TRY(cudaEventRecord(v.ev_prepped[b], it->prep_stream));

@@ -151,7 +151,7 @@ sparse_join_kernel(const int64_t *__restrict__ off, const int32_t *__restrict__ 
         for (int f = e + 1; f < end; ++f) {
           const int64_t q = s_row[f];
           const int64_t i = r < q ? r : q, j = r < q ? q : r;
-          atomicAdd(out + pair_index(i, j, n), (double)__fmul_rn(v, s_val[f]));
+          atomicAdd(out + pair_index(i, j, n), widen(__fmul_rn(v, s_val[f])));
         }
       }
       __syncthreads();                              // before the entries are replaced
@@ -391,7 +391,7 @@ sparse_dense_kernel(const int64_t *__restrict__ off, const int32_t *__restrict__
           if (COVER) atomicAdd(reinterpret_cast<int32_t *>(out) + p0 + jl, 1);
           else
             atomicAdd(reinterpret_cast<double *>(out) + p0 + jl,
-                      (double)((b & 1) ? acc[a][b >> 1].y : acc[a][b >> 1].x));
+                      widen((b & 1) ? acc[a][b >> 1].y : acc[a][b >> 1].x));
         }
       }
     }

@@ -142,13 +142,40 @@ extern "C" ap_status ap_get_plan(const ap_items *it, ap_plan *out) {
   return AP_OK;
 }
 
-int32_t ap::default_k_split(int64_t n_tiles, int64_t Dp) {
-  // column ranges of about kKSplitCols columns, and at least two units per SM
+namespace {
+// whether the ranges of k_split keep to FP32 sums and their planes to the limit
+bool planes_fit(int64_t k_split, int64_t Dp, int64_t pairs) {
   const int64_t nch = Dp / kOocChunkCols;
-  int64_t k = (Dp + kKSplitCols - 1) / kKSplitCols;
-  if (n_tiles > 0) k = std::max<int64_t>(k, (2LL * num_sms() + n_tiles - 1) / n_tiles);
-  k = std::min<int64_t>(k, std::min<int64_t>(nch, kMaxKSplit));
-  return k <= 1 ? 0 : (int32_t)k;
+  return k_split > 0 && (nch + k_split - 1) / k_split * kOocChunkCols <= kKSplitCols &&
+         k_split * pairs * (int64_t)sizeof(float) <= kPlaneBytes;
+}
+}  // namespace
+
+// Column ranges per tile, in microseconds: a run costs ceil(units / slots)
+// rounds of units, a unit its 64-column chunks (one each) and about kUnitUs
+// more (the pipeline's start, and an epilogue that the next unit's MMAs cover
+// for two chunks), and where its partial Grams go into planes the scaling pass
+// one FP64 addition a pair and range.  Ranges of at most kKSplitCols columns,
+// which the units in flight share in L2.  The cheapest wins.  1000 x 50,000, 10
+// block pairs on 76 CTA pairs: 7 ranges fill one round and take 141 us with the
+// scaling, 15 two rounds 167, 16 (the two units per SM of an earlier rule) a
+// third round 206; 547 x 15,252, 6 block pairs: 12 ranges 50 us, 8 54, 16 68.
+int32_t ap::default_k_split(int64_t n_tiles, int64_t slots, int64_t Dp, int64_t pairs) {
+  constexpr double kUnitUs = 20.0, kPlaneAddsPerUs = 6e5;
+  const int64_t nch = Dp / kOocChunkCols;
+  const int64_t most = std::min<int64_t>(nch, kMaxKSplit);
+  const int64_t least = std::min<int64_t>((Dp + kKSplitCols - 1) / kKSplitCols, most);
+  int64_t best = least;
+  double cost = 1e300;
+  for (int64_t k = least; k <= most && n_tiles > 0; ++k) {
+    const double rounds = (double)((n_tiles * k + slots - 1) / slots);
+    const double unit = (double)((nch + k - 1) / k);
+    const double c = rounds * (unit + kUnitUs) +
+                     (pairs > 0 && planes_fit(k, Dp, pairs) ? (double)(k * pairs) / kPlaneAddsPerUs
+                                                            : 0.0);
+    if (c < cost) { cost = c; best = k; }
+  }
+  return best <= 1 ? 0 : (int32_t)best;
 }
 
 namespace {
@@ -171,12 +198,18 @@ ap_status ap::set_vector_plan(ap_items *it, int32_t k_split, int32_t mma_ctas) {
   if (!v.d_hi) return AP_ERR_STATE;
   if (mma_ctas == 0) mma_ctas = 2;
   if (mma_ctas != 1 && mma_ctas != 2) return AP_ERR_INVALID_ARG;
-  if (k_split < 0) k_split = default_k_split(v.n_tiles_tc, v.Dp);
+  if (k_split < 0) {
+    const int64_t nb = (v.n + kTcTileN - 1) / kTcTileN;
+    k_split = mma_ctas == 2
+                  ? default_k_split(nb * (nb + 1) / 2, tc2_pairs(), v.Dp, v.n * (v.n - 1) / 2)
+                  : default_k_split(v.n_tiles_tc, num_sms(), v.Dp, 0);
+  }
   cudaError_t e = cudaDeviceSynchronize();      // the old units may still be in use
   if (e != cudaSuccess) return from_cuda(e);
   dfree(v.d_panel_units);
   dfree(v.d_pair_units);
   dfree(v.d_pair_whole);
+  dfree(v.d_planes);
   v.n_panel_units = v.n_pair_units = v.n_pair_whole = 0;
   v.k_split = 0;
   v.mma_ctas = mma_ctas;
@@ -190,6 +223,13 @@ ap_status ap::set_vector_plan(ap_items *it, int32_t k_split, int32_t mma_ctas) {
   if (mma_ctas == 2) {
     pair_units(v.n, nch, tc2_pairs(), k_split, units);
     AP_TRY_ST(upload_units(units, &v.d_pair_units, &v.n_pair_units));
+    v.n_planes = std::min<int64_t>(k_split, nch);            // the ranges that were listed
+    const int64_t P = v.n * (v.n - 1) / 2;
+    if (P > 0 && planes_fit(v.n_planes, v.Dp, P) &&
+        dmalloc(&v.d_planes, (size_t)(v.n_planes * P)) != cudaSuccess) {
+      cudaGetLastError();                       // no room: the units add into the output
+      v.d_planes = nullptr;
+    }
   } else {
     panel_units(v.h_tiles_tc, nch, tc_grid(v.n_tiles_tc), k_split, units);
     AP_TRY_ST(upload_units(units, &v.d_panel_units, &v.n_panel_units));

@@ -15,6 +15,7 @@
 // thread) are folded into FP64 accumulators, and the centring subtracts the
 // FP64 shift as a two-float pair (x - s_hi) - s_lo, which keeps c accurate
 // to a few ulps of c itself even when |s| >> |c|.
+#include <cooperative_groups.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -26,6 +27,8 @@
 namespace ap {
 
 namespace {
+
+namespace cg = cooperative_groups;
 
 constexpr int kStatsThreads = 512;
 constexpr int kSplitThreads = 256;
@@ -94,8 +97,7 @@ vec_mean_kernel(const float *__restrict__ X, int64_t n, int64_t D, int64_t ld,
 // CTA's FP64 partials of sum_k c_k^2 and sum_k c_k into slot blockIdx.x of
 // the row (set when first_chunk, else added, so column chunks accumulate).
 // Grid: x = column ranges of a row (thread t of CTA b takes the float4
-// groups b * blockDim + t + m * stride), y = rows (strided), or only the rows
-// of list = [count, rows...].
+// groups b * blockDim + t + m * stride), y = rows (strided).
 //
 // Blocked offsets advance by constants: the group stride is a multiple of 8
 // float4 (one 32-column block), so a thread's column within a block is fixed
@@ -128,7 +130,7 @@ vec_split_kernel(const float *__restrict__ X, int64_t row0, int64_t out_row0, in
                  __nv_bfloat16 *__restrict__ hi, __nv_bfloat16 *__restrict__ lo,
                  float *__restrict__ c32, double *__restrict__ part,
                  double *__restrict__ part_c, int first_chunk,
-                 const int32_t *__restrict__ list, int64_t col0, int64_t Dl) {
+                 int64_t col0, int64_t Dl) {
   // Dp columns (D of them real) of each row go to columns col0.. (a multiple
   // of 32) of blocked copies Dl columns wide
   __shared__ double2 red[kSplitThreads];
@@ -140,9 +142,7 @@ vec_split_kernel(const float *__restrict__ X, int64_t row0, int64_t out_row0, in
   const int64_t qa = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   constexpr size_t kTileTc = (size_t)kRowBlock * kTcKBlock, kTile32 = (size_t)kRowBlock * kF32KBlock;
   const size_t d_tc = (size_t)(stq >> 3) * kTileTc, d_32 = (size_t)(stq >> 2) * kTile32;
-  const int64_t nrows = list ? (int64_t)list[0] : n;
-  for (int64_t t = blockIdx.y; t < nrows; t += gridDim.y) {
-    const int64_t lr = list ? (int64_t)list[1 + t] : t;
+  for (int64_t lr = blockIdx.y; lr < n; lr += gridDim.y) {
     const int64_t row = row0 + lr;             // global item index (statistics)
     const int64_t orow = out_row0 + lr;        // row of the blocked copies
     const float *x = X + lr * ld;
@@ -224,23 +224,196 @@ vec_split_kernel(const float *__restrict__ X, int64_t row0, int64_t out_row0, in
 }
 
 
-// The shift of each row: the FP64 mean of up to kShiftSamples values spread
-// evenly over the row; rows are centred on it in the single pass that
-// follows, and the exact mean enters at the end (delta_i = mu_i - s_i from
-// the same pass's sums).  One warp per row.
+// ---------------------------------------------------------------------------
+// The load pipeline of resident rows in one launch: per row the shift (the
+// FP64 mean of up to kShiftSamples values spread evenly over the row), the
+// pass that centres on it, writes the copies and sums c and c^2, the
+// statistics, and for a row whose shift missed its mean by D delta^2 >
+// kRecentreRatio ss a second pass centred on the mean.
+//
+// Bound by HBM (read 4 bytes, write 4 per value).  A row belongs to one CTA, or
+// to a cluster of up to eight that share its columns and meet in distributed
+// shared memory, where rows are too few to fill the SMs (prep_cluster); four
+// CTAs per SM are in different phases, so one row's sampling and sums run
+// beside the others' streams.  As separate launches (shift, split over 16 CTAs a
+// row, statistics, second split over the rows that need it, statistics) the
+// same work took 190 us for 1000 x 50,000, now 88, and six launches' worth of
+// latency for a few short rows (100 x 1000: 49 us, now 9).
+//
+// Rows may start at any float: a row off the 16-byte grid reads the two
+// aligned vectors that hold its four columns and selects.
+// ---------------------------------------------------------------------------
 constexpr int kShiftSamples = 1024;
-__global__ void vec_shift_kernel(const float *__restrict__ X, int64_t n, int64_t D, int64_t ld,
-                                 double *__restrict__ shift) {
-  const int lane = threadIdx.x & 31;
-  const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
+// A row whose shift misses its mean by D delta^2 > ss / 64 is centred again
+// on the exact mean: the shifted rows' common part D delta_i delta_j then
+// stays below 1/64 of sqrt(ss_i ss_j), so it adds nothing measurable to the
+// rounding of the Gram's FP32 chains.
+constexpr double kRecentreRatio = 1.0 / 64.0;
+
+template <bool CLUSTER, bool ALIGNED>
+__global__ void __launch_bounds__(kSplitThreads, 4)
+vec_prep_kernel(const float *__restrict__ X, int64_t row0, int64_t out_row0, int64_t n, int64_t D,
+                int64_t ld, int64_t Dp, __nv_bfloat16 *__restrict__ hi,
+                __nv_bfloat16 *__restrict__ lo, float *__restrict__ c32,
+                double *__restrict__ shift_out, double *__restrict__ delta,
+                double *__restrict__ ss, double *__restrict__ rs) {
+  __shared__ double2 red[kSplitThreads];
+  __shared__ double2 s_sum[3];                   // this CTA's sums: samples, first, second pass
+  __shared__ float2 s_shift;
+  __shared__ int s_again;
+  const cg::cluster_group cluster = cg::this_cluster();
+  const int C = CLUSTER ? (int)cluster.num_blocks() : 1;
+  const int rank = CLUSTER ? (int)cluster.block_rank() : 0;
+  const int tid = threadIdx.x;
+  const int64_t q4 = Dp >> 2, qf = D >> 2;       // float4 groups of a padded row, whole ones
+  const int64_t nkb_tc = Dp / kTcKBlock, nkb_32 = Dp / kF32KBlock;
+  const int64_t stq = (int64_t)C * kSplitThreads;
+  const int64_t qa = (int64_t)rank * kSplitThreads + tid;
+  constexpr size_t kTileTc = (size_t)kRowBlock * kTcKBlock, kTile32 = (size_t)kRowBlock * kF32KBlock;
+  const size_t d_tc = (size_t)(stq >> 3) * kTileTc, d_32 = (size_t)(stq >> 2) * kTile32;
   const int64_t count = D < kShiftSamples ? D : kShiftSamples, stride = D / count;
-  for (int64_t row = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); row < n;
-       row += warps) {
-    const float *x = X + row * ld;
+
+  // sums of the whole row, in thread 0 (FP64 runs at a small fraction of the
+  // FP32 rate, so one warp adds the CTA's and one thread the cluster's)
+  auto row_sums = [&](double a, double b, int which) -> double2 {
+    red[tid] = make_double2(a, b);
+    __syncthreads();
+    if (tid < 32) {
+      double x = 0.0, y = 0.0;
+      for (int k = tid; k < kSplitThreads; k += 32) {
+        x += red[k].x;
+        y += red[k].y;
+      }
+      for (int o = 16; o > 0; o >>= 1) {
+        x += __shfl_down_sync(0xffffffffu, x, o);
+        y += __shfl_down_sync(0xffffffffu, y, o);
+      }
+      if (tid == 0) s_sum[which] = make_double2(x, y);
+    }
+    if (CLUSTER) cluster.sync();
+    double2 t = make_double2(0.0, 0.0);
+    if (tid == 0) {
+      t = s_sum[which];
+      if (CLUSTER) {
+        t = make_double2(0.0, 0.0);
+        for (int c = 0; c < C; ++c) {            // rank order: the same sum in every CTA
+          const double2 v = *cluster.map_shared_rank(&s_sum[which], c);
+          t.x += v.x;
+          t.y += v.y;
+        }
+      }
+    }
+    return t;
+  };
+
+  for (int64_t lr = blockIdx.x / C; lr < n; lr += gridDim.x / C) {
+    const int64_t row = row0 + lr;               // global item index (statistics)
+    const int64_t orow = out_row0 + lr;          // row of the blocked copies
+    const float *x = X + lr * ld;
+    const int off = ALIGNED ? 0 : (int)((reinterpret_cast<uintptr_t>(x) >> 2) & 3);
+    const float4 *x4 = reinterpret_cast<const float4 *>(x - off);
     double acc = 0.0;
-    for (int64_t k = lane; k < count; k += 32) acc += (double)__ldg(x + k * stride);
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if (lane == 0) shift[row] = acc / (double)count;
+    for (int64_t k = qa; k < count; k += stq) acc += (double)__ldg(x + k * stride);
+    double sh = row_sums(acc, 0.0, 0).x / (double)count;      // (thread 0)
+    for (int pass = 0;; ++pass) {
+      if (tid == 0) {
+        const float mh = (float)sh;
+        s_shift = make_float2(mh, (float)(sh - (double)mh));
+      }
+      __syncthreads();
+      const float mh = s_shift.x, ml = s_shift.y;
+      const int64_t rb = orow / kRowBlock, ri = orow % kRowBlock;
+      size_t o_tc = ((size_t)rb * nkb_tc + (size_t)(qa >> 3)) * kTileTc + (size_t)ri * kTcKBlock +
+                    4 * (size_t)(qa & 7);
+      size_t o_32 = ((size_t)rb * nkb_32 + (size_t)(qa >> 2)) * kTile32 + (size_t)ri * kF32KBlock +
+                    4 * (size_t)(qa & 3);
+      double acc2 = 0.0, acc1 = 0.0;
+      float psum = 0.f, psum_c = 0.f;
+      auto put = [&](const float4 &v) {
+        const float c[4] = {(v.x - mh) - ml, (v.y - mh) - ml, (v.z - mh) - ml, (v.w - mh) - ml};
+        psum += (c[0] * c[0] + c[1] * c[1]) + (c[2] * c[2] + c[3] * c[3]);
+        psum_c += (c[0] + c[1]) + (c[2] + c[3]);
+        split_store(c, hi, lo, c32, o_tc, o_32);
+        o_tc += d_tc;
+        o_32 += d_32;
+      };
+      // columns 4 q .. 4 q + 3 out of the aligned vectors q and q + 1
+      auto pick = [&](const float4 &a, const float4 &b) -> float4 {
+        return off == 1 ? make_float4(a.y, a.z, a.w, b.x)
+                        : off == 2 ? make_float4(a.z, a.w, b.x, b.y) : make_float4(a.w, b.x, b.y, b.z);
+      };
+      int64_t q = qa;
+      // four groups per trip, all loads issued before any is used
+      for (int trips = 0; q + 3 * stq < qf; q += 4 * stq) {
+        float4 v[4];
+        if (ALIGNED || off == 0) {
+#pragma unroll
+          for (int u = 0; u < 4; ++u) v[u] = __ldg(x4 + q + u * stq);
+        } else {
+          float4 w[4];
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            v[u] = __ldg(x4 + q + u * stq);
+            w[u] = __ldg(x4 + q + u * stq + 1);
+          }
+#pragma unroll
+          for (int u = 0; u < 4; ++u) v[u] = pick(v[u], w[u]);
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) put(v[u]);
+        if (++trips == 4) {                      // 64 elements per FP32 partial
+          acc2 += (double)psum;
+          acc1 += (double)psum_c;
+          psum = psum_c = 0.f;
+          trips = 0;
+        }
+      }
+      // the rest: at most three whole groups, loaded together, then one group
+      // at a time bounds checked (ragged end, padding)
+      {
+        float4 v[3];
+        int m = 0;
+#pragma unroll
+        for (int u = 0; u < 3; ++u)
+          if (q + u * stq < qf) {
+            v[u] = __ldg(x4 + q + u * stq);
+            if (off) v[u] = pick(v[u], __ldg(x4 + q + u * stq + 1));
+            m = u + 1;
+          }
+#pragma unroll
+        for (int u = 0; u < 3; ++u)
+          if (u < m) put(v[u]);
+        q += m * stq;
+      }
+      for (; q < q4; q += stq) {
+        const int64_t k = q << 2;
+        float c[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) c[e] = (k + e < D) ? (__ldg(x + k + e) - mh) - ml : 0.f;
+        psum += (c[0] * c[0] + c[1] * c[1]) + (c[2] * c[2] + c[3] * c[3]);
+        psum_c += (c[0] + c[1]) + (c[2] + c[3]);
+        split_store(c, hi, lo, c32, o_tc, o_32);
+        o_tc += d_tc;
+        o_32 += d_32;
+      }
+      const double2 t = row_sums(acc2 + (double)psum, acc1 + (double)psum_c, 1 + pass);
+      if (tid == 0) {
+        const double d = t.y / (double)D, v = t.x - t.y * d;
+        s_again = pass == 0 && v > 0.0 && (double)D * d * d > kRecentreRatio * v;
+        if (s_again) {
+          sh += d;
+        } else if (rank == 0) {
+          shift_out[row] = sh;
+          delta[row] = d;
+          ss[row] = v;
+          rs[row] = v > 0.0 ? 1.0 / sqrt(v) : __longlong_as_double(0x7ff8000000000000ll);
+        }
+      }
+      __syncthreads();
+      if (!s_again) break;
+    }
+    if (CLUSTER) cluster.sync();                 // peers have read this CTA's sums
+    else __syncthreads();
   }
 }
 
@@ -275,22 +448,13 @@ __global__ void vec_shift_runs_kernel(const float *__restrict__ X, int64_t n, in
   }
 }
 
-// A row whose shift misses its mean by D delta^2 > ss / 64 is centred again
-// on the exact mean: the shifted rows' common part D delta_i delta_j then
-// stays below 1/64 of sqrt(ss_i ss_j), so it adds nothing measurable to the
-// rounding of the Gram's FP32 chains.
-constexpr double kRecentreRatio = 1.0 / 64.0;
-
 // Column-sliced rows centred on shifts s_i: with S1 = sum_k c_ik and
 // S2 = sum_k c_ik^2 over all D columns (c = x - s), delta_i = mu_i - s_i =
 // S1 / D and ss_i = S2 - S1 delta_i (the shifted-data form of the variance).
-// list (optional): rows beyond kRecentreRatio get shift += delta and are
-// appended to list = [count, rows...].
 __global__ void slice_stats_kernel(const double *__restrict__ part,
                                    const double *__restrict__ part_c, int64_t n, int nparts,
                                    int64_t D, double *__restrict__ delta,
-                                   double *__restrict__ ss, double *__restrict__ rs,
-                                   double *__restrict__ shift, int32_t *__restrict__ list) {
+                                   double *__restrict__ ss, double *__restrict__ rs) {
   for (int64_t row = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; row < n;
        row += (int64_t)gridDim.x * blockDim.x) {
     double s1 = 0.0, s2 = 0.0;
@@ -302,10 +466,6 @@ __global__ void slice_stats_kernel(const double *__restrict__ part,
     delta[row] = d;
     ss[row] = v;
     rs[row] = v > 0.0 ? 1.0 / sqrt(v) : __longlong_as_double(0x7ff8000000000000ll);
-    if (list && v > 0.0 && (double)D * d * d > kRecentreRatio * v) {
-      shift[row] += d;
-      list[1 + atomicAdd(list, 1)] = (int32_t)row;
-    }
   }
 }
 
@@ -318,6 +478,25 @@ __global__ void slice_finalize_kernel(double *__restrict__ out, const double *__
     const int64_t p0 = pair_index(i, i + 1, n);
     for (int64_t j = i + 1 + threadIdx.x; j < n; j += blockDim.x)
       out[p0 + (j - i - 1)] = (out[p0 + (j - i - 1)] - di * delta[j]) * (ri * rs[j]);
+  }
+}
+
+// the same over the planes of a split Gram: FP32 partial sums in order, FP64.
+// Bound by the FP64 additions (two per clock and SM), k of them a pair.
+__global__ void pair_planes_kernel(double *__restrict__ out, const float *__restrict__ planes,
+                                   int64_t k, const double *__restrict__ rs,
+                                   const double *__restrict__ delta, int64_t n, int64_t D) {
+  const int64_t P = n * (n - 1) / 2;
+  for (int64_t i = blockIdx.x; i < n - 1; i += gridDim.x) {
+    const double ri = rs[i], di = (double)D * delta[i];
+    const int64_t p0 = pair_index(i, i + 1, n);
+    for (int64_t j = i + 1 + threadIdx.x; j < n; j += blockDim.x) {
+      const float *src = planes + p0 + (j - i - 1);
+      double g = 0.0;
+#pragma unroll 8
+      for (int64_t r = 0; r < k; ++r) g += widen(__ldcs(src + r * P));
+      out[p0 + (j - i - 1)] = (g - di * delta[j]) * (ri * rs[j]);
+    }
   }
 }
 
@@ -452,7 +631,7 @@ gram_f32_kernel(const float *__restrict__ C, int64_t n, int64_t Dp,
           if (jl >= nj || jl < first) continue;
           const float g = (b & 1) ? acc[a][b >> 1].y : acc[a][b >> 1].x;
           if (COVER) atomicAdd(reinterpret_cast<int32_t *>(out) + p0 + jl, 1);
-          else if (PARTIAL) atomicAdd(reinterpret_cast<double *>(out) + p0 + jl, (double)g);
+          else if (PARTIAL) atomicAdd(reinterpret_cast<double *>(out) + p0 + jl, widen(g));
           else
             reinterpret_cast<double *>(out)[p0 + jl] =
                 ((double)g - (delta ? di * delta[j0 + jl] : 0.0)) * ri * rs[j0 + jl];
@@ -509,12 +688,12 @@ cudaError_t launch_vec_split_slice(const float *X, int64_t row0, int64_t n, int6
   const bool vec4 = (ld % 4 == 0) && ((reinterpret_cast<uintptr_t>(X) & 15) == 0);
   if (vec4)
     vec_split_kernel<true><<<grid, kSplitThreads, 0, s>>>(
-        X, row0, row0, n, cols, ld, cols_p, shift, hi, lo, nullptr, part, part_c, first_chunk,
-        nullptr, 0, cols_p);
+        X, row0, row0, n, cols, ld, cols_p, shift, hi, lo, nullptr, part, part_c, first_chunk, 0,
+        cols_p);
   else
     vec_split_kernel<false><<<grid, kSplitThreads, 0, s>>>(
-        X, row0, row0, n, cols, ld, cols_p, shift, hi, lo, nullptr, part, part_c, first_chunk,
-        nullptr, 0, cols_p);
+        X, row0, row0, n, cols, ld, cols_p, shift, hi, lo, nullptr, part, part_c, first_chunk, 0,
+        cols_p);
   return cudaGetLastError();
 }
 
@@ -528,51 +707,48 @@ cudaError_t launch_vec_split_cols(const float *X, int64_t row0, int64_t n, int64
   const bool vec4 = (ld % 4 == 0) && ((reinterpret_cast<uintptr_t>(X) & 15) == 0);
   if (vec4)
     vec_split_kernel<true><<<grid, kSplitThreads, 0, s>>>(
-        X, row0, row0, n, cols, ld, width, shift, hi, lo, c32, part, part_c, first_chunk, nullptr,
-        col0, Dl);
+        X, row0, row0, n, cols, ld, width, shift, hi, lo, c32, part, part_c, first_chunk, col0,
+        Dl);
   else
     vec_split_kernel<false><<<grid, kSplitThreads, 0, s>>>(
-        X, row0, row0, n, cols, ld, width, shift, hi, lo, c32, part, part_c, first_chunk, nullptr,
-        col0, Dl);
+        X, row0, row0, n, cols, ld, width, shift, hi, lo, c32, part, part_c, first_chunk, col0,
+        Dl);
   return cudaGetLastError();
+}
+
+// CTAs per row, a power of two, at most eight: as many as give every SM its
+// four, while each keeps 2048 columns; and eight of a row so long that each
+// still has 65,536 (4096 x 2^20: 5.47 ms with eight, 6.31 with one, whose writes
+// meet 608 rows at once; 1000 x 50,000: 88 us with one, 97 with two)
+int prep_cluster(int64_t n, int64_t Dp) {
+  int c = 1;
+  while (c < 8 && ((n * c < 4 * (int64_t)num_sms() && Dp / (2 * c) >= 2048) ||
+                   Dp / (2 * c) >= 65536))
+    c *= 2;
+  return c;
 }
 
 cudaError_t launch_vec_prep(const float *X, int64_t row0, int64_t out_row0, int64_t n, int64_t D,
                             int64_t ld, int64_t Dp, __nv_bfloat16 *hi, __nv_bfloat16 *lo,
-                            float *c32, double *shift, double *part, double *part_c,
-                            double *delta, double *ss, double *rs, int32_t *recentre,
+                            float *c32, double *shift, double *delta, double *ss, double *rs,
                             cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
-  const int sg = (int)std::min<int64_t>((n + 7) / 8, 65535);
-  vec_shift_kernel<<<sg, 256, 0, s>>>(X, n, D, ld, shift + row0);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  const bool vec4 = (ld % 4 == 0) && ((reinterpret_cast<uintptr_t>(X) & 15) == 0);
-  auto split = [&](dim3 grid, const int32_t *list) {
-    if (vec4)
-      vec_split_kernel<true><<<grid, kSplitThreads, 0, s>>>(
-          X, row0, out_row0, n, D, ld, Dp, shift, hi, lo, c32, part, part_c, 1, list, 0, Dp);
-    else
-      vec_split_kernel<false><<<grid, kSplitThreads, 0, s>>>(
-          X, row0, out_row0, n, D, ld, Dp, shift, hi, lo, c32, part, part_c, 1, list, 0, Dp);
-    return cudaGetLastError();
-  };
-  const int fg = (int)((n + 255) / 256 < 4096 ? (n + 255) / 256 : 4096);
-  auto stats = [&](int32_t *list) {
-    slice_stats_kernel<<<fg, 256, 0, s>>>(part + row0 * kSplitParts, part_c + row0 * kSplitParts,
-                                          n, kSplitParts, D, delta + row0, ss + row0, rs + row0,
-                                          shift + row0, list);
-    return cudaGetLastError();
-  };
-  if ((e = split(dim3(kSplitParts, (unsigned)(n < 65535 ? n : 65535)), nullptr)) != cudaSuccess)
-    return e;
-  if ((e = cudaMemsetAsync(recentre, 0, sizeof(int32_t), s)) != cudaSuccess) return e;
-  if ((e = stats(recentre)) != cudaSuccess) return e;
-  // the rows the sampled shift served badly, again from the exact mean (the
-  // list is normally empty and the CTAs return at once)
-  if ((e = split(dim3(kSplitParts, (unsigned)(n < 256 ? n : 256)), recentre)) != cudaSuccess)
-    return e;
-  return stats(nullptr);
+  const int c = prep_cluster(n, Dp);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(std::min<int64_t>(n, 1 << 24) * c), 1, 1);
+  cfg.blockDim = dim3(kSplitThreads, 1, 1);
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = c;
+  attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = c > 1 ? 1 : 0;
+  const bool al = (ld % 4 == 0) && ((reinterpret_cast<uintptr_t>(X) & 15) == 0);
+  auto kern = c > 1 ? (al ? vec_prep_kernel<true, true> : vec_prep_kernel<true, false>)
+                    : (al ? vec_prep_kernel<false, true> : vec_prep_kernel<false, false>);
+  return cudaLaunchKernelEx(&cfg, kern, X, row0, out_row0, n, D, ld, Dp, hi, lo, c32, shift, delta,
+                            ss, rs);
 }
 
 cudaError_t launch_pair_correct(double *out, const double *rs, const double *delta, int64_t n,
@@ -580,6 +756,14 @@ cudaError_t launch_pair_correct(double *out, const double *rs, const double *del
   if (n < 2) return cudaSuccess;
   const int grid = (int)(n - 1 < 65535 ? n - 1 : 65535);
   pair_correct_kernel<<<grid, 256, 0, s>>>(out, rs, delta, n, D);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_pair_planes(double *out, const float *planes, int64_t k, const double *rs,
+                               const double *delta, int64_t n, int64_t D, cudaStream_t s) {
+  if (n < 2) return cudaSuccess;
+  const int grid = (int)(n - 1 < 65535 ? n - 1 : 65535);
+  pair_planes_kernel<<<grid, 256, 0, s>>>(out, planes, k, rs, delta, n, D);
   return cudaGetLastError();
 }
 
@@ -596,8 +780,7 @@ cudaError_t launch_slice_finalize(const double *part, const double *part_c, int6
                                   cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
   const int fg = (int)((n + 255) / 256 < 4096 ? (n + 255) / 256 : 4096);
-  slice_stats_kernel<<<fg, 256, 0, s>>>(part, part_c, n, kSplitParts, D, delta, ss, rs, nullptr,
-                                        nullptr);
+  slice_stats_kernel<<<fg, 256, 0, s>>>(part, part_c, n, kSplitParts, D, delta, ss, rs);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess || n < 2) return e;
   const int grid = (int)(n - 1 < 65535 ? n - 1 : 65535);

@@ -334,3 +334,40 @@ def test_load_and_run_column_chunks(ap, oracle_lib, n, D):
     copies = [e for e in tr if e["stage"] == "copy"]
     assert len(copies) == chunks * ((n + 255) // 256)
     assert sum(e["bytes"] for e in copies) == n * D * 4
+
+
+@pytest.mark.parametrize("off", [0, 1, 2, 3])
+@pytest.mark.parametrize("n,D", [(3, 70001),      # a cluster of eight CTAs a row
+                                 (40, 9000),      # of four
+                                 (700, 1030),     # one CTA a row, ragged end
+                                 (5, 3)])
+def test_pearson_rows_off_the_vector_grid(ap, oracle_lib, n, D, off):
+    """Rows that start `off` floats past a 16-byte boundary (a window into
+    wider rows), some of whose sampled shift misses their mean, so that they
+    are centred a second time."""
+    rng = np.random.default_rng(100 * n + off)
+    wide = rng.standard_normal((n, D + 8 - D % 4)).astype(np.float32)
+    X = wide[:, off:off + D]
+    if D >= 2048:
+        X[::3, ::D // min(D, 1024)] += 30.0       # the sampled places alone
+    pi, pj = oracle_lib.all_pairs(n)
+    ref = oracle_lib.pearson(np.ascontiguousarray(X), pi, pj)
+    dev = torch.from_numpy(wide).cuda()[:, off:off + D]
+    both = (ap.AP_PREC_SPLIT_BF16, ap.AP_PREC_FP32)
+    with ap.Items.from_vectors(dev, precisions=both) as it:
+        for prec in both:
+            got = it.run_pairs(ap.AP_FN_PEARSON, prec).cpu().numpy()
+            tol = pearson_tolerance(np.ascontiguousarray(X), pi, pj, prec)
+            assert np.all(np.abs(got - ref) <= tol), float((np.abs(got - ref) / tol).max())
+
+
+def test_pearson_split_runs_repeat_bits(ap):
+    """Partial Grams kept in planes are summed in order: runs repeat their
+    bits, across updates and after a coverage run on the same handle."""
+    X = synth.vectors_grouped(600, 5000, seed=3).cuda()
+    with ap.Items.from_vectors(X) as it:
+        a = it.run_pairs()
+        assert it.plan()["k_split"] > 1
+        cnt = it.run_pairs(ap.AP_FN_COVERAGE)
+        it.update(X)
+        assert torch.equal(a, it.run_pairs()) and bool((cnt == 1).all())

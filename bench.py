@@ -281,10 +281,9 @@ def ours(args):
                        "parallelism": "replicas" if ws > 1 else "single",
                        "l2": "inputs (32 GiB raw + 32 GiB hi/lo) far larger than L2"},
             "roofline": roofline, "gram_ms": gram_avg,
-            # per step: vec_shift, vec_split, slice_stats, vec_split over the rows
-            # centred again (normally none), slice_stats, gram_tc, and the pass
-            # that scales (split-K) or corrects (whole tiles) the pairs
-            "gpu_launches": 7 * args.steps}
+            # per step: vec_prep, gram_tc2, and the pass that scales (split-K) or
+            # corrects (whole tiles) the pairs
+            "gpu_launches": 3 * args.steps}
     if clk:
         line["clocks"] = {k: clk[k] for k in ("sm_mhz", "sm_max_mhz", "reasons")}
 
@@ -402,7 +401,8 @@ def ours(args):
 # SFU (MUFU) throughput of a GB300 SM, measured with independent chains of
 # each instruction: ex2.approx 30.2 and rcp.approx 15.2 results per clock;
 # the overlap kernels' roofline is 152 SMs x the SM clock seen during the run
-# x the point-pair rate these allow (one rcp and one ex2 per point pair)
+# x the point-pair rate these allow (one ex2 per point pair, and one rcp per
+# point pair of the adjoint and per two of the costs)
 EX2_PER_CLK_PER_SM = 32
 RCP_PER_CLK_PER_SM = 16
 OOC_N, OOC_DIM, OOC_CACHE = 8192, 3 << 20, 48 << 30
@@ -618,8 +618,9 @@ def run_pearson_list_workload(args):
                        "l2": "each step reads 168 GB of rows, far larger than L2"},
             "roofline": {"bound": "hbm", "achieved": gbs, "peak": peak, "unit": "GB/s",
                          "frac": gbs / peak, "traffic": None,
-                         "kernel": "pearson_rows_kernel (with list_rows_kernel's row-major "
-                                   "copy and the host sort, over the whole call)",
+                         "kernel": "pearson_list_kernel (with the host grouping, over the whole "
+                                   "call; rows listed more than once meet in L2, so the rate "
+                                   "may exceed the peak)",
                          "peak_kind": f"{pk_kind} HBM copy",
                          "algorithmic_bytes_per_step": bytes_step},
             "gpu_launches": 2 * args.steps}
@@ -648,11 +649,6 @@ def run_pearson_list_workload(args):
 
 
 SPARSE_N, SPARSE_DIM = 2500, 20 ** 6
-# shared-memory / L1 data path of an SM: 128 bytes per clock; a probe of the
-# sparse cosine moves 12 (a 4-byte gather from the dense chunk + the 8-byte
-# entry it multiplies)
-L1_BYTES_PER_CLK_PER_SM = 128
-SPARSE_BYTES_PER_PROBE = 12
 
 
 def run_sparse_workload(args):
@@ -684,9 +680,10 @@ def run_sparse_workload(args):
     torch.cuda.synchronize()
     clk = clocks.stop()
     ms = e0.elapsed_time(e1) / args.steps
-    sm_mhz = clk["sm_mhz"] if clk else 2070.0
-    achieved = probes * SPARSE_BYTES_PER_PROBE / (ms / 1e3) / 1e9
-    peak = L1_BYTES_PER_CLK_PER_SM * 152 * sm_mhz * 1e6 / 1e9
+    pk, pk_kind = peaks()
+    peak = pk["hbm_gbs"]
+    bytes_step = 8.0 * float(nnz.sum()) + 8.0 * P
+    achieved = bytes_step / (ms / 1e3) / 1e9
     line = {"metric": METRIC, "value": P / (ms / 1e3), "unit": "pairs/s", "n_gpus": 1,
             "steps": args.steps, "warmup": max(args.warmup, 3), "ms_per_step": ms,
             "higher_is_better": True, "scaling": "weak", "vs_baseline": None,
@@ -694,11 +691,12 @@ def run_sparse_workload(args):
             "config": {"workload": f"cosine_sparse_n{n}", "n_items": n, "dim": SPARSE_DIM,
                        "nnz_total": int(nnz.sum()), "pairs": P, "probes": probes},
             "probes_per_s": probes / (ms / 1e3),
-            "roofline": {"bound": "l1", "achieved": achieved, "peak": peak, "unit": "GB/s",
-                         "frac": achieved / peak, "traffic": None, "kernel": "sparse_cos_kernel",
-                         "peak_kind": "128 B/clk/SM shared/L1 data path x 152 SMs x median SM "
-                                      "clock; 12 B per probe"},
-            "gpu_launches": args.steps}
+            "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
+                         "frac": achieved / peak, "traffic": None,
+                         "kernel": "sparse_dense_kernel + sparse_join_kernel",
+                         "peak_kind": f"{pk_kind} HBM copy; every entry read once, every pair "
+                                      "written once"},
+            "gpu_launches": 3 * args.steps}
     if clk:
         line["clocks"] = {k: clk[k] for k in ("sm_mhz", "sm_max_mhz", "reasons")}
     if not args.no_cpu:
@@ -853,20 +851,20 @@ def measure_pipes():
     return out
 
 
-def mufu_roof(pipes, sm_mhz, n_sm):
-    """The overlap kernels' bound: one rcp and one ex2 per point pair on the
-    SM's MUFU pipe.  Returns (peak MUFU results/s in units of 1e12, point
-    pairs per clock per SM, how the rates were obtained)."""
+def mufu_roof(pipes, sm_mhz, n_sm, rcps=1.0):
+    """The MUFU bound of the overlap kernels: one ex2 and `rcps` rcp per point
+    pair.  Returns (peak MUFU results/s in units of 1e12, point pairs per
+    clock per SM, how the rates were obtained)."""
     if pipes:
         rcp, ex2 = pipes["rcp"]["per_clk_per_sm"], pipes["ex2"]["per_clk_per_sm"]
         kind = "ap_pipe_rate measured in this run"
     else:
         rcp, ex2 = RCP_PER_CLK_PER_SM, EX2_PER_CLK_PER_SM
         kind = "rates of an earlier probe"
-    pp = 1.0 / (1.0 / rcp + 1.0 / ex2)
-    return 2.0 * pp * n_sm * sm_mhz * 1e6 / 1e12, pp, \
-        f"one rcp ({rcp:.1f}/clk/SM) + one ex2 ({ex2:.1f}/clk/SM) per point pair ({kind}): " \
-        f"{2 * pp:.1f} MUFU results/clk/SM x {n_sm} SMs x median SM clock"
+    pp = 1.0 / (rcps / rcp + 1.0 / ex2)
+    return (1.0 + rcps) * pp * n_sm * sm_mhz * 1e6 / 1e12, pp, \
+        f"{rcps:g} rcp ({rcp:.1f}/clk/SM) + one ex2 ({ex2:.1f}/clk/SM) per point pair ({kind}): " \
+        f"{(1 + rcps) * pp:.1f} MUFU results/clk/SM x {n_sm} SMs x median SM clock"
 
 
 def cloud_record(wl, fn_name="overlap", steps=5, warmup=3, ref_pairs=2000, plan="",
@@ -958,10 +956,12 @@ def cloud_record(wl, fn_name="overlap", steps=5, warmup=3, ref_pairs=2000, plan=
     ms = e0.elapsed_time(e1) / steps
     evals = n_asc + (wl == "register_particles2d_n256") if reg else 1   # pair evaluations per step
     units = P * (n_asc if wl in ("register2d_n1024", "register2d_n1024_list") else 1)
-    mufu = 2.0 * point_pairs * evals
+    # costs share a reciprocal between two terms, the adjoint does not
+    rcps = 1.0 if reg else 0.5
+    mufu = (1.0 + rcps) * point_pairs * evals
     sm_mhz = clk["sm_mhz"] if clk else 2070.0
     n_sm = torch.cuda.get_device_properties(local).multi_processor_count
-    peak, _, peak_kind = mufu_roof(pipes, sm_mhz, n_sm)
+    peak, _, peak_kind = mufu_roof(pipes, sm_mhz, n_sm, rcps)
     achieved = mufu / (ms / 1e3) / 1e12
     line = {"metric": METRIC, "value": units / (ms / 1e3),
             "unit": {"register2d_n1024": "pair-steps/s", "register2d_n1024_list": "pair-steps/s",

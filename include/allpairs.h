@@ -264,13 +264,11 @@ ap_status ap_run_pairs(ap_items *items, int32_t fn, int32_t precision,
  *        transform applied to item pj[k] (2-D only).  A pair listed as
  *        (a < b) gives the bits of ap_run_pairs at a's and b's packed index.
  *   fn = AP_FN_PEARSON: resident vector sets; out device double[n_pairs];
- *        precision selects the representation (built at creation); one warp
- *        per pair, the Gram's three products per column in FP32, FP64 sums.
- *        A list of at least 32 pairs per 128-item row block it touches first
- *        copies those blocks into row-major rows of one 4-byte word per
- *        column, in a buffer of n_items x dim words (padded to 64) that the
- *        first such call allocates and the handle keeps until ap_destroy;
- *        where that allocation fails, the call reads the blocked rows.
+ *        precision selects the representation (built at creation); the
+ *        Gram's three products per column in FP32, FP64 sums, in column
+ *        slices; pairs that share a row are computed together.  The handle
+ *        keeps a buffer of the list's indices and one FP64 sum per pair and
+ *        slice (at most 256 MB of them, or one per pair) until ap_destroy.
  *   fn = AP_FN_COSINE: sparse sets; out device double[n_pairs]; the two
  *        rows' codes merged (FP32 products, FP64 sums).
  * Errors: AP_ERR_INVALID_ARG (fn/kind mismatch, an index out of range or a

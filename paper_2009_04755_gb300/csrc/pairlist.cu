@@ -9,15 +9,12 @@
 // in packed order (a < b) therefore gets exactly the operations, and the
 // bits, of the all-pairs run.
 //
-// Vectors use one warp per listed pair over the resident centred rows (split
-// BF16 or FP32 copy), the same three products per column as the tensor-core
-// Gram, summed in FP32 over 64 column blocks per lane and in FP64 after:
+// Vectors run over the resident centred rows (split BF16 or FP32 copy), the
+// same three products per column as the tensor-core Gram, summed in FP32 over
+// 64 columns per lane and in FP64 after:
 //   r_k = (sum_c c_a c_b - D delta_a delta_b) rs_a rs_b.
-// The blocked layout puts a row's 32-column pieces 8 KB apart, so a row is
-// read as scattered 64-byte pieces; the list is therefore run sorted by the
-// row blocks of its two items (smaller item first: r is symmetric), so that
-// the warps in flight read pieces of the same 8 KB blocks, and each result
-// goes back to its list position.
+// The list runs in column slices that the rows it touches share in L2, and
+// pairs with a row in common are computed together by one warp.
 // Sparse rows merge their sorted codes (one CTA per pair).
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -34,205 +31,141 @@ namespace {
 
 constexpr int kListThreads = 256;
 
+// Vector pairs.  Work is (column slice, group): a group is a row a and up to
+// kListGroup partner rows, one warp's; the slices come one after another, so
+// that the warps in flight read one slice of the touched rows, which stays in
+// L2: a row's pieces (64 bytes, 8 KB apart) come from memory about once, not
+// once per pair.  Bound by the L2 reads of the groups' rows.  3000 random pairs of
+// 1024 x 2^18 (1 GiB of rows, 6.3 GB listed, 4.2 GB after grouping): 0.62 ms
+// against 1.33 through a row-major copy of the touched blocks; 441 pairs of 389
+// x 139,141, which read the pieces once per pair before: 65 us against 668.
+// Slices of 12 and 40 MB and groups of 6 took as long, 6 MB 14% and groups of 8
+// (spilled) 70% longer; asking for the next slice's blocks ahead 6% longer.
+constexpr int kListGroup = 4;
+constexpr int64_t kListSliceBytes = 24ll << 20;  // of the touched rows
+
+struct ListPlan {
+  const int4 *groups;        // {a, first pair, pairs, 0}
+  const int32_t *a, *b;      // rows of the pairs in group order
+  const int32_t *pos;        // their places in the caller's list
+  int64_t n_groups, n_pairs, slice_cols, n_slices;
+};
+
 template <bool SPLIT>
 __global__ void __launch_bounds__(kListThreads)
 pearson_list_kernel(const __nv_bfloat16 *__restrict__ hi, const __nv_bfloat16 *__restrict__ lo,
-                    const float *__restrict__ c32, int64_t Dp, const int32_t *__restrict__ pi,
-                    const int32_t *__restrict__ pj, const int32_t *__restrict__ pos,
-                    int64_t n_pairs, const double *__restrict__ rs,
-                    const double *__restrict__ delta, int64_t D, double *__restrict__ out) {
+                    const float *__restrict__ c32, int64_t Dp, ListPlan L,
+                    double *__restrict__ part) {
+  constexpr int kblk = SPLIT ? kTcKBlock : kF32KBlock;             // columns of an 8 KB block
+  constexpr int64_t kBlock = (int64_t)kRowBlock * kblk;            // its elements
+  constexpr int kCols = SPLIT ? 8 : 4;                             // columns of a 16-byte load
+  constexpr int kTrip = 32 * kCols;                                // of a warp's trip
   const int lane = threadIdx.x & 31;
-  const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
-  for (int64_t k = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); k < n_pairs;
-       k += warps) {
-    const int64_t a = pi[k], b = pj[k];
-    double acc = 0.0;
-    float part = 0.f;
-    if (SPLIT) {
-      // lane l takes column l of every 32-column block (64 contiguous bytes
-      // per row and block for the warp)
-      // four blocks per trip, all sixteen loads issued before any product
-      // (Dp is a multiple of 64, so the block count is even, not always a
-      // multiple of four: the last trip may hold two)
-      const int64_t nkb = Dp / kTcKBlock;
-      constexpr size_t kBlock = (size_t)kRowBlock * kTcKBlock;   // elements per block
-      const size_t ra = blocked_offset(a, lane, nkb, kTcKBlock);
-      const size_t rb = blocked_offset(b, lane, nkb, kTcKBlock);
-      for (int64_t kb = 0; kb < nkb; kb += 4) {
-        float ha[4], la[4], hb[4], lb[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const bool in = kb + u < nkb;
-          const size_t o = (size_t)(kb + u) * kBlock;
-          ha[u] = in ? __bfloat162float(hi[ra + o]) : 0.f;
-          la[u] = in ? __bfloat162float(lo[ra + o]) : 0.f;
-          hb[u] = in ? __bfloat162float(hi[rb + o]) : 0.f;
-          lb[u] = in ? __bfloat162float(lo[rb + o]) : 0.f;
-        }
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          part = fmaf(ha[u], hb[u], part);
-          part = fmaf(ha[u], lb[u], part);
-          part = fmaf(la[u], hb[u], part);
-        }
-        if ((kb & 63) == 60) {                     // 64 blocks per FP32 partial
-          acc += (double)part;
-          part = 0.f;
-        }
-      }
-    } else {
-      const int64_t nkb = Dp / kF32KBlock;
-      for (int64_t col = lane, m = 0; col < Dp; col += 32, ++m) {
-        const float ca = c32[blocked_offset(a, col, nkb, kF32KBlock)];
-        const float cb = c32[blocked_offset(b, col, nkb, kF32KBlock)];
-        part = fmaf(ca, cb, part);
-        if ((m & 63) == 63) {
-          acc += (double)part;
-          part = 0.f;
-        }
-      }
-    }
-    acc += (double)part;
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if (lane == 0) out[pos[k]] = (acc - (double)D * delta[a] * delta[b]) * rs[a] * rs[b];
-  }
-}
-
-// Long lists read a row-major copy instead.  Scattered 64-byte pieces reach
-// about a quarter of the HBM copy rate; when the list reads the rows it
-// touches several times over, the call first copies the touched row blocks
-// into a row-major buffer of one 4-byte word per column (a split column's hi
-// and lo bf16 packed, hi in the low half; or the FP32 value), streaming the
-// blocked arrays once, and each pair then reads two contiguous rows.
-constexpr int kRowsCols = 128;                  // columns per relayout item
-constexpr int kRowsSlot = kRowBlock * 64 + 64;  // one staged 8 KB block + 64 B,
-                                                // so slots start 16 banks apart
-constexpr int kRowsSmem = 8 * kRowsSlot;
-constexpr int kRowsThreads = 256;
-
-__device__ __forceinline__ void cp_async16(void *dst, const void *src) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
-                   (uint32_t)__cvta_generic_to_shared(dst)),
-               "l"(src)
-               : "memory");
-}
-
-// Item (row block rb, column group g): the 128 columns from g * 128 of every
-// row of the block.  SPLIT: slots 0-3 hold hi's 32-column blocks, 4-7 lo's;
-// FP32: slots 0-7 hold 16-column blocks.  Each warp then writes whole rows'
-// 512-byte pieces.
-template <bool SPLIT>
-__global__ void __launch_bounds__(kRowsThreads, 3)
-list_rows_kernel(const __nv_bfloat16 *__restrict__ hi, const __nv_bfloat16 *__restrict__ lo,
-                 const float *__restrict__ c32, int64_t n, int64_t Dp,
-                 const int32_t *__restrict__ blocks, int64_t n_blocks,
-                 uint32_t *__restrict__ rows) {
-  extern __shared__ __align__(16) uint8_t st[];
-  const int64_t groups = (Dp + kRowsCols - 1) / kRowsCols;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  constexpr int kblk = SPLIT ? kTcKBlock : kF32KBlock;
   const int64_t nkb = Dp / kblk;
-  for (int64_t w = blockIdx.x; w < n_blocks * groups; w += gridDim.x) {
-    const int64_t rb = blocks[w / groups], col0 = (w % groups) * kRowsCols;
-    const int cols = (int)(Dp - col0 < kRowsCols ? Dp - col0 : kRowsCols);   // 128 or 64
-    const int per_slot = cols / kblk;            // staged blocks per array
-    // 512 16-byte chunks per staged block
-    for (int c = threadIdx.x; c < 8 * 512; c += kRowsThreads) {
-      const int slot = c >> 9, off = (c & 511) * 16;
-      const int kbl = SPLIT ? (slot & 3) : slot;
-      if (kbl >= per_slot) continue;
-      const int64_t kb = col0 / kblk + kbl;
-      const uint8_t *src;
-      if (SPLIT) {
-        const __nv_bfloat16 *arr = slot < 4 ? hi : lo;
-        src = reinterpret_cast<const uint8_t *>(arr + (size_t)(rb * nkb + kb) * kRowBlock * kblk);
-      } else {
-        src = reinterpret_cast<const uint8_t *>(c32 + (size_t)(rb * nkb + kb) * kRowBlock * kblk);
-      }
-      cp_async16(st + slot * kRowsSlot + off, src + off);
-    }
-    asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory");
-    __syncthreads();
-    const int c4 = lane * 4;                     // this lane's four columns
-    if (c4 < cols) {
-      for (int r = warp; r < kRowBlock; r += kRowsThreads / 32) {
-        const int64_t row = rb * kRowBlock + r;
-        if (row >= n) break;
-        uint4 o;
-        if (SPLIT) {
-          const int kbl = c4 / kTcKBlock, c = c4 % kTcKBlock;
-          const uint2 h = *reinterpret_cast<const uint2 *>(st + kbl * kRowsSlot +
-                                                           (r * kTcKBlock + c) * 2);
-          const uint2 l = *reinterpret_cast<const uint2 *>(st + (4 + kbl) * kRowsSlot +
-                                                           (r * kTcKBlock + c) * 2);
-          o.x = __byte_perm(h.x, l.x, 0x5410);
-          o.y = __byte_perm(h.x, l.x, 0x7632);
-          o.z = __byte_perm(h.y, l.y, 0x5410);
-          o.w = __byte_perm(h.y, l.y, 0x7632);
-        } else {
-          const int kbl = c4 / kF32KBlock, c = c4 % kF32KBlock;
-          o = *reinterpret_cast<const uint4 *>(st + kbl * kRowsSlot + (r * kF32KBlock + c) * 4);
-        }
-        *reinterpret_cast<uint4 *>(rows + (size_t)row * Dp + col0 + c4) = o;
-      }
-    }
-    __syncthreads();                             // before the slots are refilled
-  }
-}
+  const int64_t per_slice = (L.n_groups + kListThreads / 32 - 1) / (kListThreads / 32);
+  for (int64_t unit = blockIdx.x; unit < per_slice * L.n_slices; unit += gridDim.x) {
+    const int64_t s = unit / per_slice, cta = unit - s * per_slice;
+    const int64_t c0 = s * L.slice_cols, c1 = c0 + L.slice_cols < Dp ? c0 + L.slice_cols : Dp;
 
-// One warp per listed pair over the row-major copy: lane l takes four
-// consecutive columns of every 128, four such loads per row in flight; FP32
-// partials over 64 columns per lane, then FP64, as the blocked kernel.
-template <bool SPLIT>
-__global__ void __launch_bounds__(kListThreads)
-pearson_rows_kernel(const uint32_t *__restrict__ rows, int64_t Dp, const int32_t *__restrict__ pi,
-                    const int32_t *__restrict__ pj, const int32_t *__restrict__ pos,
-                    int64_t n_pairs, const double *__restrict__ rs,
-                    const double *__restrict__ delta, int64_t D, double *__restrict__ out) {
-  const int lane = threadIdx.x & 31;
-  const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
-  const int64_t nq = Dp / 4;                     // 16-byte words per row
-  for (int64_t k = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); k < n_pairs;
-       k += warps) {
-    const int64_t a = pi[k], b = pj[k];
-    const uint4 *ra = reinterpret_cast<const uint4 *>(rows + (size_t)a * Dp);
-    const uint4 *rb = reinterpret_cast<const uint4 *>(rows + (size_t)b * Dp);
-    double acc = 0.0;
-    float part = 0.f;
-    for (int64_t q0 = 0, t = 0; q0 < nq; q0 += 128, ++t) {
-      uint4 va[4], vb[4];
+    const int64_t gi = cta * (kListThreads / 32) + (threadIdx.x >> 5);
+    if (gi >= L.n_groups) continue;
+    const int4 g = L.groups[gi];
+    // a lane's first columns: load q of a trip covers block (q, lane >> 2)
+    const int64_t k0 = c0 / kblk + (lane >> 2);
+    auto at = [&](int64_t row) {
+      return ((row / kRowBlock) * nkb + k0) * kBlock + (row % kRowBlock) * kblk + (lane & 3) * kCols;
+    };
+    int64_t oa = at(g.x), ob[kListGroup];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int64_t q = q0 + u * 32 + lane;
-        const bool in = q < nq;
-        va[u] = in ? __ldg(ra + q) : make_uint4(0u, 0u, 0u, 0u);
-        vb[u] = in ? __ldg(rb + q) : make_uint4(0u, 0u, 0u, 0u);
+    for (int j = 0; j < kListGroup; ++j) ob[j] = at(L.b[g.y + (j < g.z ? j : 0)]);
+    float sum[kListGroup];
+    double acc[kListGroup];
+#pragma unroll
+    for (int j = 0; j < kListGroup; ++j) {
+      sum[j] = 0.f;
+      acc[j] = 0.0;
+    }
+    const uint4 z = make_uint4(0u, 0u, 0u, 0u);
+    auto load = [](const void *p, bool in) {
+      return in ? __ldg(reinterpret_cast<const uint4 *>(p)) : make_uint4(0u, 0u, 0u, 0u);
+    };
+    int trips = 0;
+    for (int64_t c = c0; c < c1; c += kTrip) {
+      const bool in = c + (lane >> 2) * kblk < c1;
+      uint4 ah, al = z, bh[kListGroup], bl[kListGroup];
+      if (SPLIT) {
+        ah = load(hi + oa, in);
+        al = load(lo + oa, in);
+      } else {
+        ah = load(c32 + oa, in);
       }
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const uint32_t wa[4] = {va[u].x, va[u].y, va[u].z, va[u].w};
-        const uint32_t wb[4] = {vb[u].x, vb[u].y, vb[u].z, vb[u].w};
+      for (int j = 0; j < kListGroup; ++j) {
+        bl[j] = z;
+        bh[j] = z;
+        if (j >= g.z) continue;
+        if (SPLIT) {
+          bh[j] = load(hi + ob[j], in);
+          bl[j] = load(lo + ob[j], in);
+        } else {
+          bh[j] = load(c32 + ob[j], in);
+        }
+      }
+      const uint32_t ahw[4] = {ah.x, ah.y, ah.z, ah.w}, alw[4] = {al.x, al.y, al.z, al.w};
+#pragma unroll
+      for (int j = 0; j < kListGroup; ++j) {
+        if (j >= g.z) continue;
+        const uint32_t bhw[4] = {bh[j].x, bh[j].y, bh[j].z, bh[j].w};
+        const uint32_t blw[4] = {bl[j].x, bl[j].y, bl[j].z, bl[j].w};
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
           if (SPLIT) {
-            const float ha = __uint_as_float(wa[e] << 16), la = __uint_as_float(wa[e] & 0xffff0000u);
-            const float hb = __uint_as_float(wb[e] << 16), lb = __uint_as_float(wb[e] & 0xffff0000u);
-            part = fmaf(ha, hb, part);
-            part = fmaf(ha, lb, part);
-            part = fmaf(la, hb, part);
+#pragma unroll
+            for (int w = 0; w < 2; ++w) {            // the word's low and high bf16
+              auto f = [&](uint32_t x) { return __uint_as_float(w ? x & 0xffff0000u : x << 16); };
+              sum[j] = fmaf(f(ahw[e]), f(bhw[e]), sum[j]);
+              sum[j] = fmaf(f(ahw[e]), f(blw[e]), sum[j]);
+              sum[j] = fmaf(f(alw[e]), f(bhw[e]), sum[j]);
+            }
           } else {
-            part = fmaf(__uint_as_float(wa[e]), __uint_as_float(wb[e]), part);
+            sum[j] = fmaf(__uint_as_float(ahw[e]), __uint_as_float(bhw[e]), sum[j]);
           }
         }
       }
-      if ((t & 3) == 3) {                        // 64 columns per lane
-        acc += (double)part;
-        part = 0.f;
+      oa += (int64_t)(kTrip / kblk) * kBlock;
+#pragma unroll
+      for (int j = 0; j < kListGroup; ++j) ob[j] += (int64_t)(kTrip / kblk) * kBlock;
+      if (++trips == 64 / kCols) {                   // 64 columns per lane
+        trips = 0;
+#pragma unroll
+        for (int j = 0; j < kListGroup; ++j) {
+          acc[j] += widen(sum[j]);
+          sum[j] = 0.f;
+        }
       }
     }
-    acc += (double)part;
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if (lane == 0) out[pos[k]] = (acc - (double)D * delta[a] * delta[b]) * rs[a] * rs[b];
+#pragma unroll
+    for (int j = 0; j < kListGroup; ++j) {
+      if (j >= g.z) continue;
+      double v = acc[j] + widen(sum[j]);
+      for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+      if (lane == 0) part[s * L.n_pairs + g.y + j] = v;
+    }
+  }
+}
+
+// the slices' sums in order, the mean correction and the scaling
+__global__ void pearson_list_sum_kernel(const double *__restrict__ part, ListPlan L,
+                                        const double *__restrict__ rs,
+                                        const double *__restrict__ delta, int64_t D,
+                                        double *__restrict__ out) {
+  for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < L.n_pairs;
+       q += (int64_t)gridDim.x * blockDim.x) {
+    double g = 0.0;
+#pragma unroll 8
+    for (int64_t s = 0; s < L.n_slices; ++s) g += part[s * L.n_pairs + q];
+    const int64_t a = L.a[q], b = L.b[q];
+    out[L.pos[q]] = (g - (double)D * delta[a] * delta[b]) * rs[a] * rs[b];
   }
 }
 
@@ -347,88 +280,104 @@ ap_status device_pairs(const int32_t *pi, const int32_t *pj, int64_t n_pairs, cu
   return AP_OK;
 }
 
-// the listed vector pairs sorted by the row blocks of their items (smaller
-// item first), with their list positions, then the distinct row blocks the
-// list touches: [a...][b...][position...][block...] on the device (the host
-// copy goes through a pageable buffer, staged by the call)
-ap_status device_pairs_by_block(const int32_t *pi, const int32_t *pj, int64_t n_pairs,
-                                int64_t n, cudaStream_t s, int32_t **d_idx,
-                                int64_t *n_blocks) {
-  std::vector<uint64_t> key((size_t)n_pairs);
+// The listed vector pairs in groups that share a row: each pair goes to the
+// end listed more often (r is symmetric), the pairs of a row in groups of up
+// to kListGroup.  Host arrays for one copy: [groups x 4][a][b][position].
+struct ListHost {
+  std::vector<int32_t> ints;
+  int64_t n_groups = 0, n_rows = 0;
+};
+void group_pairs(const int32_t *pi, const int32_t *pj, int64_t n_pairs, int64_t n, ListHost &h) {
+  // the rows listed, numbered; their counts
+  std::vector<int32_t> count((size_t)n, 0), first((size_t)n + 1, 0);
   for (int64_t k = 0; k < n_pairs; ++k) {
-    const uint32_t a = (uint32_t)std::min(pi[k], pj[k]), b = (uint32_t)std::max(pi[k], pj[k]);
-    const uint64_t blocks = ((uint64_t)(a / kRowBlock) << 16) | (uint64_t)(b / kRowBlock);
-    key[k] = (blocks << 32) | (uint64_t)k;     // row blocks < 2^16 (n <= INT32_MAX / 2)
+    ++count[pi[k]];
+    ++count[pj[k]];
   }
-  std::sort(key.begin(), key.end());
-  std::vector<int32_t> h((size_t)n_pairs * 3);
-  std::vector<uint8_t> touched((size_t)((n + kRowBlock - 1) / kRowBlock), 0);
-  for (int64_t q = 0; q < n_pairs; ++q) {
-    const int64_t k = (int64_t)(key[q] & 0xffffffffu);
-    h[q] = std::min(pi[k], pj[k]);
-    h[n_pairs + q] = std::max(pi[k], pj[k]);
-    h[2 * n_pairs + q] = (int32_t)k;
-    touched[h[q] / kRowBlock] = touched[h[n_pairs + q] / kRowBlock] = 1;
+  auto hub = [&](int64_t k) {
+    return count[pj[k]] > count[pi[k]] || (count[pj[k]] == count[pi[k]] && pj[k] < pi[k]) ? pj[k]
+                                                                                            : pi[k];
+  };
+  for (int64_t k = 0; k < n_pairs; ++k) ++first[hub(k) + 1];
+  for (int64_t i = 0; i < n; ++i) {
+    h.n_groups += (first[i + 1] + kListGroup - 1) / kListGroup;
+    h.n_rows += count[i] > 0;
+    first[i + 1] += first[i];
   }
-  for (size_t r = 0; r < touched.size(); ++r)
-    if (touched[r]) h.push_back((int32_t)r);
-  *n_blocks = (int64_t)h.size() - n_pairs * 3;
-  AP_TRY(dmalloc(d_idx, h.size()));
-  AP_TRY(cudaMemcpyAsync(*d_idx, h.data(), h.size() * 4, cudaMemcpyHostToDevice, s));
-  return AP_OK;
+  h.ints.resize((size_t)(4 * h.n_groups + 3 * n_pairs));
+  int32_t *g = h.ints.data(), *a = g + 4 * h.n_groups, *b = a + n_pairs, *pos = b + n_pairs;
+  for (int64_t i = 0; i < n; ++i)
+    for (int32_t q = first[i]; q < first[i + 1]; q += kListGroup, g += 4) {
+      g[0] = (int32_t)i;
+      g[1] = q;
+      g[2] = std::min<int32_t>(kListGroup, first[i + 1] - q);
+      g[3] = 0;
+    }
+  for (int64_t k = 0; k < n_pairs; ++k) {
+    const int32_t hk = hub(k), q = first[hk]++;
+    a[q] = hk;
+    b[q] = pi[k] == hk ? pj[k] : pi[k];
+    pos[q] = (int32_t)k;
+  }
 }
 
 }  // namespace
 
 cudaError_t launch_pearson_list(VecStore &v, bool split, const int32_t *pi,
-                                const int32_t *pj, const int32_t *pos, int64_t n_pairs,
-                                const int32_t *blocks, int64_t n_blocks, double *out,
+                                const int32_t *pj, int64_t n_pairs, double *out,
                                 cudaStream_t s) {
-  if (n_pairs <= 0) return cudaSuccess;
-  const int64_t need = (n_pairs + (kListThreads / 32) - 1) / (kListThreads / 32);
-  const int grid = (int)std::min<int64_t>(need, (int64_t)num_sms() * 8);
-  // the copy streams 2 x 128 rows per touched block at about the HBM rate;
-  // it pays once the list reads those rows, in 64-byte pieces at about a
-  // quarter of that rate, more than kRowsPairsPerBlock pairs per block
-  constexpr int64_t kRowsPairsPerBlock = 32;
-  if (n_pairs >= kRowsPairsPerBlock * n_blocks) {
-    if (!v.d_rows && dmalloc(&v.d_rows, (size_t)v.n * v.Dp) != cudaSuccess) {
-      cudaGetLastError();                       // no room: the blocked kernel
-      v.d_rows = nullptr;
-    }
-  }
-  if (v.d_rows && n_pairs >= kRowsPairsPerBlock * n_blocks) {
-    const cudaError_t e =
-        split ? cudaFuncSetAttribute(list_rows_kernel<true>,
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize, kRowsSmem)
-              : cudaFuncSetAttribute(list_rows_kernel<false>,
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize, kRowsSmem);
+  ListHost h;
+  group_pairs(pi, pj, n_pairs, v.n, h);
+  ListPlan L{};
+  L.n_groups = h.n_groups;
+  L.n_pairs = n_pairs;
+  // slices that the touched rows share in L2, and enough of them to give every
+  // SM sixteen warps; whole trips of 256 columns; fewer where the slices' sums
+  // would take more than kListPartBytes
+  constexpr int64_t kListPartBytes = 256ll << 20;
+  const int64_t share = kListSliceBytes / (4 * h.n_rows);
+  const int64_t spread = v.Dp * h.n_groups / (16 * (int64_t)num_sms());
+  const int64_t most = std::max<int64_t>(kListPartBytes / (8 * n_pairs), 1);
+  const int64_t least = (v.Dp + most - 1) / most;
+  L.slice_cols = (std::max(std::max<int64_t>(std::min(share, spread), 1024), least) + 255) / 256 * 256;
+  L.n_slices = (v.Dp + L.slice_cols - 1) / L.slice_cols;
+  // the handle's list buffer (the call before has synchronised its stream):
+  // partial sums, then the index arrays
+  const size_t head = (size_t)(L.n_slices * n_pairs) * sizeof(double);
+  const size_t ints_at = (head + 15) / 16 * 16, bytes = ints_at + h.ints.size() * 4;
+  cudaError_t e = cudaSuccess;
+  if (v.list_bytes < bytes) {
+    dfree(v.d_list);
+    v.list_bytes = 0;
+    e = dmalloc(&v.d_list, bytes + bytes / 4);
     if (e != cudaSuccess) return e;
-    const int64_t items = n_blocks * ((v.Dp + kRowsCols - 1) / kRowsCols);
-    const int rgrid = (int)std::min<int64_t>(items, (int64_t)num_sms() * 3 * 16);
-    if (split) {
-      list_rows_kernel<true><<<rgrid, kRowsThreads, kRowsSmem, s>>>(
-          v.d_hi, v.d_lo, nullptr, v.n, v.Dp, blocks, n_blocks, v.d_rows);
-      pearson_rows_kernel<true><<<grid, kListThreads, 0, s>>>(v.d_rows, v.Dp, pi, pj, pos, n_pairs,
-                                                              v.d_rs, v.d_delta_all, v.D, out);
-    } else {
-      list_rows_kernel<false><<<rgrid, kRowsThreads, kRowsSmem, s>>>(
-          nullptr, nullptr, v.d_c32, v.n, v.Dp, blocks, n_blocks, v.d_rows);
-      pearson_rows_kernel<false><<<grid, kListThreads, 0, s>>>(v.d_rows, v.Dp, pi, pj, pos,
-                                                               n_pairs, v.d_rs, v.d_delta_all,
-                                                               v.D, out);
-    }
-    return cudaGetLastError();
+    v.list_bytes = bytes + bytes / 4;
   }
-  if (split)
-    pearson_list_kernel<true><<<grid, kListThreads, 0, s>>>(v.d_hi, v.d_lo, nullptr, v.Dp, pi, pj,
-                                                            pos, n_pairs, v.d_rs, v.d_delta_all,
-                                                            v.D, out);
-  else
-    pearson_list_kernel<false><<<grid, kListThreads, 0, s>>>(nullptr, nullptr, v.d_c32, v.Dp, pi,
-                                                             pj, pos, n_pairs, v.d_rs,
-                                                             v.d_delta_all, v.D, out);
-  return cudaGetLastError();
+  uint8_t *buf = v.d_list;
+  // (a pageable source: staged before the call returns)
+  e = cudaMemcpyAsync(buf + ints_at, h.ints.data(), h.ints.size() * 4, cudaMemcpyHostToDevice, s);
+  if (e == cudaSuccess) {
+    const int32_t *ints = reinterpret_cast<const int32_t *>(buf + ints_at);
+    L.groups = reinterpret_cast<const int4 *>(ints);
+    L.a = ints + 4 * h.n_groups;
+    L.b = L.a + n_pairs;
+    L.pos = L.b + n_pairs;
+    double *part = reinterpret_cast<double *>(buf);
+    const int64_t per_slice = (h.n_groups + kListThreads / 32 - 1) / (kListThreads / 32);
+    const unsigned grid = (unsigned)std::min<int64_t>(per_slice * L.n_slices, 1 << 30);
+    if (split)
+      pearson_list_kernel<true><<<grid, kListThreads, 0, s>>>(v.d_hi, v.d_lo, nullptr, v.Dp, L,
+                                                              part);
+    else
+      pearson_list_kernel<false><<<grid, kListThreads, 0, s>>>(nullptr, nullptr, v.d_c32, v.Dp, L,
+                                                               part);
+    e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    const unsigned g2 = (unsigned)std::min<int64_t>((n_pairs + 127) / 128, 65535);
+    pearson_list_sum_kernel<<<g2, 128, 0, s>>>(part, L, v.d_rs, v.d_delta_all, v.D, out);
+    e = cudaGetLastError();
+  }
+  return e;
 }
 
 }  // namespace ap
@@ -460,28 +409,23 @@ extern "C" ap_status ap_run_pairs_list(ap_items *it, int32_t fn, int32_t precisi
       if (v.out_of_core) return AP_ERR_UNSUPPORTED;   // rows are not resident
       if ((split && !v.d_hi) || (!split && !v.d_c32)) return AP_ERR_STATE;
     }
-    int32_t *d_idx = nullptr;
-    int64_t n_blocks = 0;
-    ap_status st = sparse ? device_pairs(pi, pj, n_pairs, s, &d_idx)
-                          : device_pairs_by_block(pi, pj, n_pairs, n, s, &d_idx, &n_blocks);
     cudaError_t e = cudaSuccess;
-    if (st == AP_OK) {
-      if (sparse) {
-        const SparseStore &sp = it->sp;
-        const int grid = (int)std::min<int64_t>(n_pairs, (int64_t)num_sms() * 8);
-        cosine_list_kernel<<<grid, kMergeThreads, 0, s>>>(sp.d_off, sp.d_idx, sp.d_val, sp.d_rs,
-                                                           d_idx, d_idx + n_pairs, n_pairs,
-                                                           reinterpret_cast<double *>(out));
-        e = cudaGetLastError();
-      } else {
-        e = launch_pearson_list(it->vec, split, d_idx, d_idx + n_pairs, d_idx + 2 * n_pairs,
-                                n_pairs, d_idx + 3 * n_pairs, n_blocks,
-                                reinterpret_cast<double *>(out), s);
-      }
+    if (sparse) {
+      int32_t *d_idx = nullptr;
+      AP_TRY_ST(device_pairs(pi, pj, n_pairs, s, &d_idx));
+      const SparseStore &sp = it->sp;
+      const int grid = (int)std::min<int64_t>(n_pairs, (int64_t)num_sms() * 8);
+      cosine_list_kernel<<<grid, kMergeThreads, 0, s>>>(sp.d_off, sp.d_idx, sp.d_val, sp.d_rs,
+                                                         d_idx, d_idx + n_pairs, n_pairs,
+                                                         reinterpret_cast<double *>(out));
+      e = cudaGetLastError();
       if (e == cudaSuccess) e = cudaStreamSynchronize(s);   // before the index buffer goes
-      st = e == cudaSuccess ? AP_OK : from_cuda(e);
+      dfree(d_idx);
+    } else {
+      e = launch_pearson_list(it->vec, split, pi, pj, n_pairs, reinterpret_cast<double *>(out), s);
+      if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     }
-    dfree(d_idx);
+    const ap_status st = e == cudaSuccess ? AP_OK : from_cuda(e);
     return st;
   }
   CloudStore lc;

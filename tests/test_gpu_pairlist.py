@@ -204,3 +204,25 @@ def test_list_rejects_bad_pairs(ap):
         assert e.value.status == 6
         with pytest.raises(ap.APError):
             it.ascent_list([0], [1], torch.zeros(1, 3, device="cuda"), 1, 1e-3)
+
+
+@pytest.mark.parametrize("prec", [1, 0])
+@pytest.mark.parametrize("D", [63, 1024, 1088, 5000])
+def test_pearson_list_groups_and_slices(ap, oracle_lib, prec, D):
+    """Groups of pairs that share a row (a row paired with every other, in
+    either order, pairs listed twice, a lone pair) over one slice and several,
+    on lists that grow and shrink on one handle."""
+    n = 140
+    X = synth.vectors_grouped(n, D, seed=D).contiguous()
+    rng = np.random.default_rng(D)
+    hub = np.array([[5, j] if j % 2 else [j, 5] for j in range(n) if j != 5])
+    for pairs in (np.array([[3, 139]]), hub[:4], hub[:5], np.concatenate([hub, hub[::-1], [[0, 1]]]),
+                  hub[rng.permutation(len(hub))[:17]]):
+        pi, pj = pairs[:, 0].astype(np.int32), pairs[:, 1].astype(np.int32)
+        ref = oracle_lib.pearson(X.numpy(), pi, pj)
+        tol = pearson_tolerance(X.numpy(), pi, pj, prec)
+        if len(pairs) == 1:
+            it = ap.Items.from_vectors(X.cuda(), precisions=(prec,))
+        got = it.run_pairs_list(pi, pj, ap.AP_FN_PEARSON, prec).cpu().numpy()
+        assert np.all(np.abs(got - ref) <= tol), float((np.abs(got - ref) / tol).max())
+    it.close()

@@ -9,6 +9,7 @@
 #include <stdint.h>
 
 #include <functional>
+#include <memory>
 #include <string>
 #include <vector>
 
@@ -147,6 +148,10 @@ struct CloudStore {
   int32_t *d_items = nullptr;
   int32_t *d_tiles = nullptr;       // [n_tiles][2] block pairs (I <= J)
   int64_t n_tiles = 0;
+  // launch shapes already looked up for this plan's buffers (shared with the
+  // temporary copies a list run or the tuner launches with)
+  struct Fit { const void *kern; size_t smem; int threads; int64_t slots; };
+  std::shared_ptr<std::vector<Fit>> fits = std::make_shared<std::vector<Fit>>();
   // particle scores: re-scaled storage per score (index score - 1), built on
   // first use, and the GMM L2 self terms per original item
   float4 *d_pts_score[2] = {nullptr, nullptr};
@@ -297,12 +302,11 @@ struct NvtxRange {
 namespace ap {
 // a captured launch sequence, replayed with cudaGraphLaunch
 struct GraphKey {
-  int32_t kind;                    // 1 overlap, 2 coverage, 3 ascent, 4 L2, 5 Bhattacharyya
   const void *a, *b, *c, *d;       // buffers the sequence reads / writes
   float eta, fmin;
   int32_t n;
   bool operator==(const GraphKey &o) const {
-    return kind == o.kind && a == o.a && b == o.b && c == o.c && d == o.d && eta == o.eta &&
+    return a == o.a && b == o.b && c == o.c && d == o.d && eta == o.eta &&
            fmin == o.fmin && n == o.n;
   }
 };

@@ -94,12 +94,14 @@ CloudPlanChoice choose_cloud_plan(const CloudStore &c) {
   ch.sorted = (c.dim == 3) && mx > 4 * std::max<int64_t>(mn, 1);
   ch.reg_r = 4;
   // blocks of about 1/60 of the points: 1800 tiles, 12 per SM before the last
-  // ones are split; at most kCloudBlockPts points, which one staging window
-  // holds.  Eight items at most: more would take shared memory for their
+  // ones are split (256 clouds of 64-128 points: 420 points a block 126 us, 256
+  // 140, 768 134); at least 384, below which a small set's launch is all tiles
+  // (48 clouds of 20-60 points: 8.2 us with 384, 10.2 with 64); at most
+  // kCloudBlockPts, which one staging window holds.  Eight items at most: more would take shared memory for their
   // partial sums from the CTAs.
   constexpr int64_t kCloudBlockPts = 2048;
   const int64_t want = (c.total_pts / 60 + 3) / 4 * 4;
-  ch.block_pts = (int32_t)std::min(std::max<int64_t>(want, 64), kCloudBlockPts);
+  ch.block_pts = (int32_t)std::min(std::max<int64_t>(want, 384), kCloudBlockPts);
   ch.block_items = 8;
   return ch;
 }
@@ -138,6 +140,7 @@ ap_status build_cloud_plan(ap_items *it, const CloudPlanChoice &ch, cudaStream_t
   make_cloud_plan(c.h_poff, cnt, c.h_perm, kSplitTailPerSm * num_sms(), ch.block_items, ch.block_pts,
                   ch.reg_r, h);
   free_cloud_plan(c);
+  c.fits->clear();
   AP_TRY_ST(upload_cloud_plan(c, h, s));
   c.block_items = ch.block_items;
   c.block_pts = ch.block_pts;
@@ -564,28 +567,16 @@ ap_status ap_run_pairs(ap_items *it, int32_t fn, int32_t precision, const float 
   if (fn == AP_FN_GMM_L2 || fn == AP_FN_BHATTACHARYYA) {
     const int score = fn == AP_FN_GMM_L2 ? 1 : 2;
     AP_TRY_ST(ensure_score_storage(it, score, s));
-    GraphKey key{3 + score, params, out, nullptr, nullptr, 0.f, 0.f, 1};
-    ap_items *h = it;
-    ap_status st = run_graphed(it, key, s, [h, params, out, score](cudaStream_t cs) {
-      const CloudStore &c = h->cl;
-      return launch_score(c, score, c.d_pts_score[score - 1], c.d_lw_score[score - 1], c.d_self,
-                          params, reinterpret_cast<float *>(out), h->d_queue, cs);
-    });
-    if (st != AP_OK) return st;
+    const CloudStore &c = it->cl;
+    AP_TRY(launch_score(c, score, c.d_pts_score[score - 1], c.d_lw_score[score - 1], c.d_self,
+                        params, reinterpret_cast<float *>(out), it->d_queue, s));
     it->stats.tiles = it->cl.n_tiles;
     it->stats.item_loads = it->cl.n;
     it->stats.reuse_R = 1.0;
     it->stats.slot_hit_rate = 1.0;
     return AP_OK;
   }
-  {
-    GraphKey key{1 + cover, params, out, nullptr, nullptr, 0.f, 0.f, 1};
-    ap_items *h = it;
-    ap_status st = run_graphed(it, key, s, [h, params, out, cover](cudaStream_t cs) {
-      return launch_overlap(h->cl, params, reinterpret_cast<float *>(out), cover, h->d_queue, cs);
-    });
-    if (st != AP_OK) return st;
-  }
+  AP_TRY(launch_overlap(it->cl, params, reinterpret_cast<float *>(out), cover, it->d_queue, s));
   it->stats.tiles = it->cl.n_tiles;
   it->stats.item_loads = it->cl.n;
   it->stats.reuse_R = 1.0;
@@ -613,7 +604,7 @@ ap_status ap_ascent(ap_items *it, float *params, int32_t n_steps, float eta, flo
   if (!params) return AP_ERR_INVALID_ARG;
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   // the n_steps fused steps are replayed as one CUDA graph
-  GraphKey key{3, params, f_out, flags, nullptr, eta, fmin, n_steps};
+  GraphKey key{params, f_out, flags, nullptr, eta, fmin, n_steps};
   ap_items *h = it;
   return run_graphed(it, key, s, [h, params, n_steps, eta, fmin, f_out, flags](cudaStream_t cs) {
     for (int32_t k = 0; k < n_steps; ++k) {

@@ -708,18 +708,34 @@ cudaError_t launch_r(const CloudStore &cs, Params &P, cudaStream_t s) {
                       kMaxBlockItems * sizeof(int2) + 8 + 2 * sizeof(TileCtx) + 16;
   void (*kern)(Params) =
       cs.reg_r == 2 ? overlap_kernel<DIM, MODE, 2, SCORE> : overlap_kernel<DIM, MODE, 4, SCORE>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
   // listed pairs are tiles of one item against one, a few jobs each: one
   // warp per CTA and many CTAs per SM keep the warps busy (20 ascent steps on
   // 131K listed pairs: 114 ms at 8 warps per CTA, 89 at 4, 81 at 2, 79 at 1)
   const int threads = cs.list_mode ? 32 : kThreads;
-  int per_sm = 0;
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem);
-  if (e != cudaSuccess) return e;
-  if (per_sm < 1) per_sm = 1;
-  int64_t grid = (int64_t)num_sms() * per_sm;
-  if (grid > P.n_tiles) grid = P.n_tiles;
+  // the attribute and the CTAs that fit are looked up once per plan: the two
+  // calls take as long as a launch
+  int64_t slots = 0;
+  for (const CloudStore::Fit &f : *cs.fits)
+    if (f.kern == reinterpret_cast<const void *>(kern) && f.smem == smem && f.threads == threads)
+      slots = f.slots;
+  cudaError_t e = cudaSuccess;
+  if (slots == 0) {
+    // (the attribute is the kernel's, not the handle's: always the most a CTA
+    // may have, so that no handle lowers it for another)
+    int optin = 0, dev = 0;
+    e = cudaGetDevice(&dev);
+    if (e == cudaSuccess)
+      e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, optin);
+    if (e != cudaSuccess) return e;
+    int per_sm = 0;
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem);
+    if (e != cudaSuccess) return e;
+    slots = (int64_t)num_sms() * std::max(per_sm, 1);
+    cs.fits->push_back({reinterpret_cast<const void *>(kern), smem, threads, slots});
+  }
+  const int64_t grid = std::min(slots, P.n_tiles);
   kern<<<(int)grid, threads, smem, s>>>(P);
   return cudaGetLastError();
 }

@@ -83,3 +83,15 @@ def test_graph_replay_respects_new_buffers(ap):
         it.set_plan(4, 2048, 4)                   # a new plan invalidates the graphs
         b = it.run_pairs()
         assert torch.allclose(a, b, rtol=1e-5, atol=0)
+
+
+def test_handles_of_one_kernel_keep_their_launch_shapes(ap):
+    """Two sets run by the same kernel with different amounts of shared
+    memory, in turn: neither run changes what the other may use."""
+    big = synth.clouds_uniform(n=12, dim=2, size=(900, 2000), seed=1)
+    small = synth.clouds_uniform(n=12, dim=2, size=(5, 9), seed=2)
+    with ap.Items.from_clouds(big) as a, ap.Items.from_clouds(small) as b:
+        fa, fb = a.run_pairs().clone(), b.run_pairs().clone()
+        for _ in range(2):
+            assert torch.equal(a.run_pairs(), fa) and torch.equal(b.run_pairs(), fb)
+            assert a.run_pairs_list([0, 3], [1, 5]).shape == (2,)

@@ -55,7 +55,7 @@ void free_items(ap_items *it) {
   if (!it) return;
   cudaDeviceSynchronize();          // queued host functions may still use the host cache
   CloudStore &c = it->cl;
-  dfree(c.d_pts); dfree(c.d_lw); dfree(c.d_poff); dfree(c.d_cnt); dfree(c.d_perm);
+  dfree(c.d_pts); dfree(c.d_lw); dfree(c.d_boxes); dfree(c.d_poff); dfree(c.d_cnt); dfree(c.d_perm);
   free_cloud_plan(c); dfree(c.d_bmeta_single); dfree(c.d_list_tiles);
   for (int k = 0; k < 2; ++k) { dfree(c.d_pts_score[k]); dfree(c.d_lw_score[k]); }
   dfree(c.d_self);
@@ -157,6 +157,13 @@ ap_status build_cloud_plan(ap_items *it, const CloudPlanChoice &ch, cudaStream_t
 
 namespace {
 
+// Whether a set is boxed (kBoxedMean).
+bool boxes_pay(const CloudStore &c) {
+  double p1 = 0.0, p2 = 0.0;
+  for (int64_t v : c.h_size) { p1 += (double)v; p2 += (double)v * (double)v; }
+  return p1 > 0.0 && p2 / p1 >= kBoxedMean;
+}
+
 ap_status create_clouds(const ap_items_desc *d, ap_items *it, cudaStream_t s) {
   CloudStore &c = it->cl;
   c.dim = d->kind == AP_ITEMS_CLOUD3D ? 3 : 2;
@@ -194,6 +201,8 @@ ap_status create_clouds(const ap_items_desc *d, ap_items *it, cudaStream_t s) {
   for (int64_t sidx = 0; sidx < c.n; ++sidx) cnt32[sidx] = (int32_t)c.h_size[c.h_perm[sidx]];
   AP_TRY(dmalloc(&c.d_pts, std::max<int64_t>(c.total_pts, 4)));
   if (c.dim == 3) AP_TRY(dmalloc(&c.d_lw, std::max<int64_t>(c.total_pts, 4)));
+  c.boxed = boxes_pay(c);
+  if (c.boxed) AP_TRY(dmalloc(&c.d_boxes, (size_t)(cloud_box0(c.total_pts / 4, c.n) + 1) * 2));
   AP_TRY(dmalloc(&c.d_poff, c.n + 1));
   AP_TRY(dmalloc(&c.d_cnt, std::max<int64_t>(c.n, 1)));
   AP_TRY(dmalloc(&c.d_perm, std::max<int64_t>(c.n, 1)));
@@ -226,7 +235,8 @@ ap_status create_clouds(const ap_items_desc *d, ap_items *it, cudaStream_t s) {
     if (e == cudaSuccess) {
       auto pick = [&](int k) -> const float * { return d->data_on_host ? tmp[k] : src[k]; };
       e = launch_cloud_pack(pick(0), pick(1), pick(2), pick(3), pick(4), d_src_off, c.d_perm,
-                            c.d_poff, c.n, c.dim, c.d_pts, c.d_lw, it->d_queue + kQueueTraits, s);
+                            c.d_poff, c.n, c.dim, c.d_pts, c.d_lw, c.d_boxes, c.boxed, mx,
+                            it->d_queue + kQueueTraits, s);
     }
     for (int k = 0; k < 5; ++k)
       if (tmp[k]) cudaFreeAsync(tmp[k], s);

@@ -91,6 +91,30 @@ __device__ __forceinline__ float2 two_sum(float a, float b) {
   return make_float2(s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb)));
 }
 
+constexpr float kFar = 1e18f, kNear = 1e15f;
+
+// smallest / largest, NaN where an operand is one
+__device__ __forceinline__ float min_nan(float a, float b) {
+  float r;
+  asm("min.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ float max_nan(float a, float b) {
+  float r;
+  asm("max.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ float warp_min(float x) {
+  float r;
+  asm("redux.sync.min.NaN.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(x));
+  return r;
+}
+__device__ __forceinline__ float warp_max(float x) {
+  float r;
+  asm("redux.sync.max.NaN.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(x));
+  return r;
+}
+
 __device__ __forceinline__ uint32_t smem_u32(const void *p) {
   return (uint32_t)__cvta_generic_to_shared(p);
 }
@@ -112,6 +136,7 @@ struct TileCtx {
 struct Params {
   const float4 *pts;
   const float *lw;
+  const float4 *boxes;     // of the overlap's storage (see cloud_box0)
   const int4 *items;       // per stored item {first group, points, original id, first row}
   const int4 *bmeta;       // per block {item begin, end, first group, groups} {job0, jobs, rows, 0}
   const int2 *desc;        // [jobs][32] lane descriptors of blocks of several items
@@ -146,7 +171,7 @@ constexpr int part_size() { return MODE == GRAD ? 4 : 2; }
 template <int MODE>
 constexpr int min_ctas() { return MODE == GRAD ? 3 : 4; }
 
-template <int DIM, int MODE, int R, int SCORE>
+template <int DIM, int MODE, int R, int SCORE, bool BOX>
 __global__ void __launch_bounds__(kThreads, min_ctas<MODE>())
 overlap_kernel(Params P) {
   constexpr int NV = (MODE == GRAD) ? 4 : 1;     // partial values per (row, j)
@@ -158,7 +183,8 @@ overlap_kernel(Params P) {
   float4 *s_pts = reinterpret_cast<float4 *>(smem);
   float2 *s_lw = reinterpret_cast<float2 *>(s_pts + P.stage_cap);
   float *s_part = reinterpret_cast<float *>(s_lw) + (DIM == 3 ? P.stage_cap : 0);
-  int2 *s_j = reinterpret_cast<int2 *>(s_part + P.part_floats);  // [32] pair range of item j
+  // [32] item j's pairs in the window, first box (-1: no boxes)
+  int4 *s_j = reinterpret_cast<int4 *>(s_part + P.part_floats);
   uint64_t *s_bar = reinterpret_cast<uint64_t *>(s_j + kMaxBlockItems);
   TileCtx *s_ctx = reinterpret_cast<TileCtx *>(s_bar + 1);       // [2] this tile, the next
   int *s_next = reinterpret_cast<int *>(s_ctx + 2);              // next (job, partner) unit
@@ -239,7 +265,9 @@ overlap_kernel(Params P) {
         const int4 m = __ldg(P.items + c.j_begin + jl);
         const int b0 = 4 * (m.x - c.j_grp0), b1 = b0 + m.y;
         const int q0 = max(b0, w0), q1 = min(b1, w0 + w_pts);   // odd counts: one padding point
-        s_j[jl] = make_int2((q0 - w0) >> 1, q1 > q0 ? (q1 - w0 + 1) >> 1 : (q0 - w0) >> 1);
+        const bool boxes = BOX && !wide && m.y > kCullPoints && ((q0 - b0) & 31) == 0;
+        s_j[jl] = make_int4((q0 - w0) >> 1, q1 > q0 ? (q1 - w0 + 1) >> 1 : (q0 - w0) >> 1,
+                            boxes ? (int)cloud_box0(m.x, c.j_begin + jl) + (q0 - b0) / 32 : -1, 0);
       }
       __syncthreads();
       if (w0 == 0 && threadIdx.x == 0) fetch(s_ctx + (cur ^ 1), pop());
@@ -327,12 +355,66 @@ overlap_kernel(Params P) {
         float2 pF[RE], pC[RE], pY[RE], pT[RE];
 #pragma unroll
         for (int r = 0; r < RE; ++r) { pF[r] = z2; pC[r] = z2; pY[r] = z2; pT[r] = z2; }
-        const int2 qr = s_j[jl];
+        const int4 qr = s_j[jl];
+        // Boxes: the lane's a-points that weigh anything, then the warp's, as
+        // the sweep holds them (negated); b - a' is fl(b + (-a')), and rounding
+        // keeps order, so the gap bounds every difference the sweep forms.
+        // A warp with an a-point far out (or NaN, from its transform) sweeps
+        // everything.
+        float nx0, nx1, ny0, ny1, nz0 = 0.f, nz1 = 0.f, sa;
+        const int n_blk = (qr.y - qr.x + 15) >> 4;
+        bool boxed = qr.z >= 0;
+        if (boxed) {
+          nx0 = ny0 = nz0 = INFINITY;
+          nx1 = ny1 = nz1 = -INFINITY;
+          sa = 0.f;
+#pragma unroll
+          for (int r = 0; r < RE; ++r)
+            if (aw[r] != 0.f) {
+              nx0 = min_nan(nx0, ax[r]); nx1 = max_nan(nx1, ax[r]);
+              ny0 = min_nan(ny0, ay[r]); ny1 = max_nan(ny1, ay[r]);
+              if (DIM == 3) { nz0 = min_nan(nz0, az[r]); nz1 = max_nan(nz1, az[r]); }
+              sa = fmaxf(sa, fabsf(as[r]));
+            }
+          nx0 = warp_min(nx0); nx1 = warp_max(nx1);
+          ny0 = warp_min(ny0); ny1 = warp_max(ny1);
+          if (DIM == 3) { nz0 = warp_min(nz0); nz1 = warp_max(nz1); }
+          sa = warp_max(sa);
+          boxed = nx0 > -kNear && nx1 < kNear && ny0 > -kNear && ny1 < kNear;
+        }
+        // of 32 blocks of 16 pairs from block `base`, those with a term that
+        // may not be 0: 2^x rounds to 0 below -126 (subnormals flush), and
+        // x <= log-weight - gap^2 / (s_a + s_b)
+        auto live = [&](int base) -> uint32_t {
+          const int left = n_blk - base;
+          uint32_t mask = left >= 32 ? 0xffffffffu : (1u << left) - 1u;
+          if (boxed) {
+            bool on = false;
+            if (lane < left) {
+              const float4 u = __ldg(P.boxes + 2 * ((int64_t)qr.z + base + lane));
+              const float4 v = __ldg(P.boxes + 2 * ((int64_t)qr.z + base + lane) + 1);
+              const float gx = fmaxf(fmaxf(u.x + nx0, -(u.y + nx1)), 0.f);
+              const float gy = fmaxf(fmaxf(u.z + ny0, -(u.w + ny1)), 0.f);
+              float g2 = fmaf(gy, gy, gx * gx);
+              if (DIM == 3) {
+                const float gz = fmaxf(fmaxf(v.x + nz0, -(v.y + nz1)), 0.f);
+                g2 = fmaf(gz, gz, g2);
+              }
+              float sb = v.z, l = v.w;
+              if (SCORE == 2) {            // the score's own s2k and log-weight
+                l = 0.5f * l + 0.25f * (float)DIM * __log2f(sb / kTwoLn2) + 0.01f;
+                sb *= 2.f;
+              }
+              on = !(g2 > (127.f + l) * (sa + sb) * 1.0001f);
+            }
+            mask &= __ballot_sync(0xffffffffu, on);
+          }
+          return mask;
+        };
         auto sweep = [&](auto plain_set, auto shared) {
           constexpr bool PLAIN = decltype(plain_set)::value;   // weights 1: no log-weight
           constexpr bool ONE = decltype(shared)::value && MODE != GRAD;
-          for (int qb = qr.x; qb < qr.y; qb += 16) {
-            const int qe = min(qb + 16, qr.y);
+          auto block = [&](int qb, int qe) {
             float2 bF[RE];                  // this block's f terms (compensated below)
 #pragma unroll
             for (int r = 0; r < RE; ++r) bF[r] = z2;
@@ -392,6 +474,15 @@ overlap_kernel(Params P) {
               pC[r] = __fadd2_rn(yk, __ffma2_rn(tk, make_float2(-1.f, -1.f), pF[r]));
               pF[r] = tk;
             }
+          };
+          if (BOX) {
+            for (int base = 0; base < n_blk; base += 32)
+              for (uint32_t mask = live(base); mask; mask &= mask - 1) {
+                const int qb = qr.x + 16 * (base + __ffs(mask) - 1);
+                block(qb, min(qb + 16, qr.y));
+              }
+          } else {
+            for (int qb = qr.x; qb < qr.y; qb += 16) block(qb, min(qb + 16, qr.y));
           }
         };
         if (kRsq) {
@@ -566,31 +657,119 @@ overlap_kernel(Params P) {
 // Padding points lie far from every point of such a set, so that their terms
 // are 0 without a log-weight (squared distances stay finite).
 constexpr float kSharedMin = 8.6736174e-19f, kSharedMax = 5.7646075e17f;
-constexpr float kFar = 1e18f, kNear = 1e15f;
+
+// Place of a point in an item's storage order: strips of the item's extent
+// that hold about 128 points a square (cube), walked back and forth, so that 32
+// and 128 points in a row are near each other.  u: position in the item's
+// box, 0..1; cells: strips per axis.
+__device__ __forceinline__ uint32_t place(const float *u, int dim, int cells) {
+  auto strip = [&](float x, int n) { return min((int)(x * (float)n), n - 1); };
+  auto fine = [](float x, int steps, bool back) {
+    const int k = min((int)(x * (float)steps), steps - 1);
+    return (uint32_t)(back ? steps - 1 - k : k);
+  };
+  if (dim == 3) {
+    const int z = strip(u[2], cells), y = strip(u[1], cells);
+    const int row = (z & 1) ? cells - 1 - y : y;
+    return (uint32_t)(z * cells + row) << 12 | fine(u[0], 4096, (z * cells + row) & 1);
+  }
+  // strips in y, columns of half their width in x, y within a column
+  const int t = strip(u[1], cells), c = strip(u[0], 2 * cells);
+  const int col = (t & 1) ? 2 * cells - 1 - c : c;
+  const float in = u[1] * (float)cells - (float)t;
+  return (uint32_t)(t * 2 * cells + col) << 9 | fine(fminf(fmaxf(in, 0.f), 1.f), 512, col & 1);
+}
 
 // Pack one item per CTA into planner order, padded to a multiple of 4 points,
-// in pairs (two per thread and trip).
-__global__ void cloud_pack_kernel(const float *__restrict__ x, const float *__restrict__ y,
-                                  const float *__restrict__ z, const float *__restrict__ sigma,
-                                  const float *__restrict__ w, const int64_t *__restrict__ src_off,
-                                  const int32_t *__restrict__ perm,
-                                  const int64_t *__restrict__ poff, int64_t n, int dim,
-                                  float4 *__restrict__ pts, float *__restrict__ lw,
-                                  int32_t *__restrict__ traits) {
+// in pairs (two per thread and trip), and its boxes.  Larger items are put in
+// order first: place and index in one word, sorted in shared memory (a bitonic
+// network over the next power of two).
+constexpr int kPackThreads = 256;
+__global__ void __launch_bounds__(kPackThreads)
+cloud_pack_kernel(const float *__restrict__ x, const float *__restrict__ y,
+                  const float *__restrict__ z, const float *__restrict__ sigma,
+                  const float *__restrict__ w, const int64_t *__restrict__ src_off,
+                  const int32_t *__restrict__ perm, const int64_t *__restrict__ poff, int64_t n,
+                  int dim, float4 *__restrict__ pts, float *__restrict__ lw,
+                  float4 *__restrict__ boxes, bool boxed, int32_t *__restrict__ traits) {
+  extern __shared__ uint32_t s_order[];            // [next power of two of the largest item]
+  __shared__ float s_lo[3], s_hi[3], s_red[kPackThreads / 32][6];
   const double two_ln2 = 1.3862943611198906;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   int32_t seen = 0;
   for (int64_t s = blockIdx.x; s < n; s += gridDim.x) {
     const int64_t o = perm[s];
-    const int64_t src0 = src_off[o], cnt = src_off[o + 1] - src_off[o];
-    const int64_t q0 = poff[s] >> 1, pairs = (poff[s + 1] - poff[s]) >> 1;
-    for (int64_t k = threadIdx.x; k < pairs; k += blockDim.x) {
+    const int64_t src0 = src_off[o];
+    const int cnt = (int)(src_off[o + 1] - src0);
+    const int64_t q0 = poff[s] >> 1;
+    const int pairs = (int)((poff[s + 1] - poff[s]) >> 1);
+    const bool ordered = boxed && cnt > kCullPoints;
+    if (ordered) {
+      // the item's extent
+      float lo[3] = {INFINITY, INFINITY, INFINITY}, hi[3] = {-INFINITY, -INFINITY, -INFINITY};
+      for (int k = tid; k < cnt; k += kPackThreads) {
+        const float p[3] = {x[src0 + k], y[src0 + k], dim == 3 ? z[src0 + k] : 0.f};
+#pragma unroll
+        for (int d = 0; d < 3; ++d) { lo[d] = fminf(lo[d], p[d]); hi[d] = fmaxf(hi[d], p[d]); }
+      }
+#pragma unroll
+      for (int d = 0; d < 3; ++d) {
+        for (int m = 16; m > 0; m >>= 1) {
+          lo[d] = fminf(lo[d], __shfl_xor_sync(0xffffffffu, lo[d], m));
+          hi[d] = fmaxf(hi[d], __shfl_xor_sync(0xffffffffu, hi[d], m));
+        }
+        if (lane == 0) { s_red[warp][d] = lo[d]; s_red[warp][3 + d] = hi[d]; }
+      }
+      __syncthreads();
+      if (tid < 3) {
+        float a = INFINITY, b = -INFINITY;
+        for (int k = 0; k < kPackThreads / 32; ++k) {
+          a = fminf(a, s_red[k][tid]);
+          b = fmaxf(b, s_red[k][3 + tid]);
+        }
+        s_lo[tid] = a;
+        s_hi[tid] = b;
+      }
+      __syncthreads();
+      const float per = (float)cnt / 128.f;
+      const int cells = max(1, (int)rintf(dim == 3 ? cbrtf(per) : sqrtf(per)));   // <= 12
+      int m = 1;
+      while (m < cnt) m <<= 1;
+      for (int k = tid; k < m; k += kPackThreads) {
+        uint32_t v = 0xffffffffu;
+        if (k < cnt) {
+          float u[3];
+          const float p[3] = {x[src0 + k], y[src0 + k], dim == 3 ? z[src0 + k] : 0.f};
+#pragma unroll
+          for (int d = 0; d < 3; ++d) {
+            const float e = s_hi[d] - s_lo[d];
+            const float t = e > 0.f ? (p[d] - s_lo[d]) / e : 0.f;
+            u[d] = t >= 0.f && t <= 1.f ? t : 0.f;          // (NaN, an infinite extent)
+          }
+          v = place(u, dim, cells) << 14 | (uint32_t)k;
+        }
+        s_order[k] = v;
+      }
+      __syncthreads();
+      for (int size = 2; size <= m; size <<= 1)
+        for (int half = size >> 1; half > 0; half >>= 1) {
+          for (int k = tid; k < m / 2; k += kPackThreads) {
+            const int a = 2 * k - (k & (half - 1)), b = a + half;
+            const uint32_t va = s_order[a], vb = s_order[b];
+            if ((va > vb) == ((a & size) == 0)) { s_order[a] = vb; s_order[b] = va; }
+          }
+          __syncthreads();
+        }
+    }
+    auto source = [&](int k) { return src0 + (ordered ? (int64_t)(s_order[k] & 16383u) : k); };
+    for (int k = tid; k < pairs; k += kPackThreads) {
       // padding: far away, log-weight -inf
       float px[2] = {kFar, kFar}, py[2] = {0.f, 0.f}, pz[2] = {0.f, 0.f}, ps[2] = {-1.f, -1.f};
       float pl[2] = {-INFINITY, -INFINITY};
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
         if (2 * k + h >= cnt) continue;
-        const int64_t a = src0 + 2 * k + h;
+        const int64_t a = source(2 * k + h);
         const double sg = (double)sigma[a];
         ps[h] = (float)(-two_ln2 * sg * sg);     // stored negated
         if (!(-ps[h] >= kSharedMin && -ps[h] <= kSharedMax)) seen |= kCloudWide;
@@ -612,6 +791,41 @@ __global__ void cloud_pack_kernel(const float *__restrict__ x, const float *__re
         dst[1] = make_float4(ps[0], ps[1], pl[0], pl[1]);
       }
     }
+    if (ordered) {
+      // one warp per box, a point per lane
+      const int64_t b0 = cloud_box0(poff[s] >> 2, s);
+      for (int b = warp; b * 32 < cnt; b += kPackThreads / 32) {
+        const int k = b * 32 + lane;
+        const float wt = k < cnt ? (w ? w[source(k)] : 1.f) : 0.f;
+        const bool in = wt > 0.f;                // others have no terms
+        float lo[3], hi[3], sm = 0.f, lm = -INFINITY;
+#pragma unroll
+        for (int d = 0; d < 3; ++d) { lo[d] = INFINITY; hi[d] = -INFINITY; }
+        if (in) {
+          const int64_t a = source(k);
+          const double sg = (double)sigma[a];
+          sm = fabsf((float)(-two_ln2 * sg * sg));
+          lm = (float)log2((double)wt);
+          lo[0] = hi[0] = x[a];
+          lo[1] = hi[1] = y[a];
+          lo[2] = hi[2] = dim == 3 ? z[a] : 0.f;
+        }
+        for (int m = 16; m > 0; m >>= 1) {
+#pragma unroll
+          for (int d = 0; d < 3; ++d) {
+            lo[d] = fminf(lo[d], __shfl_xor_sync(0xffffffffu, lo[d], m));
+            hi[d] = fmaxf(hi[d], __shfl_xor_sync(0xffffffffu, hi[d], m));
+          }
+          sm = fmaxf(sm, __shfl_xor_sync(0xffffffffu, sm, m));
+          lm = fmaxf(lm, __shfl_xor_sync(0xffffffffu, lm, m));
+        }
+        if (lane == 0) {
+          boxes[2 * (b0 + b)] = make_float4(lo[0], hi[0], lo[1], hi[1]);
+          boxes[2 * (b0 + b) + 1] = make_float4(lo[2], hi[2], sm, lm);
+        }
+      }
+    }
+    __syncthreads();                             // before the order is replaced
   }
   if (seen) atomicOr(traits, seen);
 }
@@ -649,7 +863,8 @@ __global__ void cloud_rescore_kernel(const float4 *__restrict__ pts, const float
 }
 
 // S_i = C sum over a, a' in item i of w_a w_a' q^d 2^(-d^2 q^2) (SCORE 1
-// storage), one CTA per item, FP32 blocks of 64 terms folded into FP64.
+// storage), one CTA per item, FP32 blocks of 8 terms folded into FP64
+// (neighbours are stored together, so a block may hold many terms of one size).
 template <int DIM>
 __global__ void __launch_bounds__(256)
 cloud_self_kernel(const float4 *__restrict__ pts, const float *__restrict__ lw,
@@ -683,7 +898,7 @@ cloud_self_kernel(const float4 *__restrict__ pts, const float *__restrict__ lw,
         const float q = rsq_approx(qa.w + qb.w), r = q * q;
         const float e = ex2_approx(fmaf(-d2, r, la + lb));
         part = fmaf(e, DIM == 2 ? r : r * q, part);
-        if ((b & 63) == 63) { acc += (double)part; part = 0.f; }
+        if ((b & 7) == 7) { acc += widen(part); part = 0.f; }
       }
       acc += (double)part;
     }
@@ -705,9 +920,11 @@ cudaError_t launch_r(const CloudStore &cs, Params &P, cudaStream_t s) {
   P.stage_cap = MODE == COVER ? 0 : (std::min(cs.max_pts, kStagePts) + 3) & ~3;
   P.part_floats = MODE == COVER ? 0 : ((cs.max_rows * cs.max_items * kPart + 3) & ~3);
   const size_t smem = (size_t)P.stage_cap * (DIM == 3 ? 20 : 16) + (size_t)P.part_floats * 4 +
-                      kMaxBlockItems * sizeof(int2) + 8 + 2 * sizeof(TileCtx) + 16;
-  void (*kern)(Params) =
-      cs.reg_r == 2 ? overlap_kernel<DIM, MODE, 2, SCORE> : overlap_kernel<DIM, MODE, 4, SCORE>;
+                      kMaxBlockItems * sizeof(int4) + 8 + 2 * sizeof(TileCtx) + 16;
+  void (*kern)(Params) = cs.reg_r == 2 ? overlap_kernel<DIM, MODE, 2, SCORE, false>
+                         : cs.boxed && MODE != COVER
+                             ? overlap_kernel<DIM, MODE, 4, SCORE, MODE != COVER>
+                             : overlap_kernel<DIM, MODE, 4, SCORE, false>;
   // listed pairs are tiles of one item against one, a few jobs each: one
   // warp per CTA and many CTAs per SM keep the warps busy (20 ascent steps on
   // 131K listed pairs: 114 ms at 8 warps per CTA, 89 at 4, 81 at 2, 79 at 1)
@@ -744,6 +961,7 @@ Params base_params(const CloudStore &cs, int32_t *queue, int32_t *status) {
   Params P{};
   P.pts = cs.d_pts;
   P.lw = cs.d_lw;
+  P.boxes = cs.d_boxes;
   P.items = reinterpret_cast<const int4 *>(cs.d_items);
   P.bmeta = reinterpret_cast<const int4 *>(cs.d_bmeta);
   P.desc = reinterpret_cast<const int2 *>(cs.d_desc);
@@ -837,11 +1055,19 @@ cudaError_t launch_overlap_grad_q(const CloudStore &cs, int32_t *queue, const fl
 cudaError_t launch_cloud_pack(const float *x, const float *y, const float *z, const float *sigma,
                               const float *w, const int64_t *src_off, const int32_t *perm,
                               const int64_t *poff, int64_t n, int dim, float4 *pts, float *lw,
+                              float4 *boxes, bool boxed, int64_t most_points,
                               int32_t *traits, cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
-  int grid = (int)(n < 65535 ? n : 65535);
-  cloud_pack_kernel<<<grid, 128, 0, s>>>(x, y, z, sigma, w, src_off, perm, poff, n, dim, pts, lw,
-                                         traits);
+  // (up to 64 KB: 16384 points, always allowed, so that no call lowers it)
+  cudaError_t e = cudaFuncSetAttribute(cloud_pack_kernel,
+                                       cudaFuncAttributeMaxDynamicSharedMemorySize, 16384 * 4);
+  if (e != cudaSuccess) return e;
+  int64_t m = 1;
+  while (m < most_points) m <<= 1;
+  const size_t smem = boxed && most_points > kCullPoints ? (size_t)m * 4 : 0;
+  const int grid = (int)(n < 65535 ? n : 65535);
+  cloud_pack_kernel<<<grid, kPackThreads, smem, s>>>(x, y, z, sigma, w, src_off, perm, poff, n, dim,
+                                                     pts, lw, boxes, boxed, traits);
   return cudaGetLastError();
 }
 

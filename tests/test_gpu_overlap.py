@@ -172,3 +172,77 @@ def test_overlap_fragment_and_window_edges(ap, oracle_lib, dim, plan, kind):
         np.testing.assert_array_equal(one, f)
     else:
         check_overlap(one, ref, kappa, bound, f"listed {kind} {dim}d {plan}")
+
+
+def _spread_clouds(dim, weights):
+    """Items whose points reach a small part of their extent, around the sizes
+    at which blocks of 32 points are passed over, with a coarse point in some."""
+    sizes = np.array([1, 160, 161, 192, 900, 0, 1001, 2049, 2051, 4101])
+    off = np.concatenate([[0], np.cumsum(sizes)]).astype(np.int64)
+    rng = np.random.default_rng(50 + dim)
+    tot = int(off[-1])
+    pts = rng.uniform(-1, 1, (tot, 3)).astype(np.float32)
+    pts[off[4]:off[5], 0] = 0.25                 # no extent along one axis
+    sig = rng.uniform(0.01, 0.02, tot)
+    sig[off[6]::97] = 0.3
+    w = rng.uniform(0.0, 2.0, tot).astype(np.float32)
+    w[::7] = 0.0
+    return {"dim": dim, "offsets": off, "x": pts[:, 0].copy(), "y": pts[:, 1].copy(),
+            "z": pts[:, 2].copy() if dim == 3 else None, "sigma": sig.astype(np.float32),
+            "weight": w if weights else None}
+
+
+@pytest.mark.parametrize("dim", [2, 3])
+@pytest.mark.parametrize("weights", [False, True])
+def test_overlap_passes_over_far_blocks(ap, oracle_lib, dim, weights):
+    c = _spread_clouds(dim, weights)
+    n = len(c["offsets"]) - 1
+    pi, pj = oracle_lib.all_pairs(n)
+    ref, kappa, bound = oracle_lib.overlap(c, pi, pj, with_cond=True)
+    with ap.Items.from_clouds(c) as it:
+        f = it.run_pairs().cpu().numpy()
+        one = it.run_pairs_list(pi, pj).cpu().numpy()
+        it.set_plan(4, 256, 2)                   # sweeps every block
+        every = it.run_pairs().cpu().numpy()
+        assert it.last_device_error() == 0
+    check_overlap(f, ref, kappa, bound, f"blocks {dim}d")
+    # a block passed over adds exactly nothing; pieces of another length are
+    # summed in another order, in two floats, and rounded once
+    np.testing.assert_array_max_ulp(every, f, maxulp=1)
+    if dim == 2:
+        np.testing.assert_array_equal(one, f)
+    else:
+        check_overlap(one, ref, kappa, bound, f"listed blocks {dim}d")
+
+
+def test_far_blocks_under_transforms(ap, oracle_lib):
+    """Transforms that keep the clouds together, part them for good, or are no
+    numbers: the last give NaN for their own pair alone."""
+    c = _spread_clouds(2, True)
+    n = len(c["offsets"]) - 1
+    pi, pj = oracle_lib.all_pairs(n)
+    rng = np.random.default_rng(9)
+    prm = rng.uniform(-0.5, 0.5, (len(pi), 3)).astype(np.float32)
+    far = np.arange(len(pi)) % 5 == 1
+    prm[far, 1] = 1e6
+    ref, kappa, bound = oracle_lib.overlap(c, pi, pj, params=prm.astype(np.float64),
+                                           with_cond=True)
+    sizes = np.diff(c["offsets"])
+    nan = (np.arange(len(pi)) % 5 == 2) & (sizes[pi] > 0) & (sizes[pj] > 0)
+    prm[nan, 2] = np.nan
+    with ap.Items.from_clouds(c) as it:
+        p = torch.from_numpy(prm).cuda()
+        f = it.run_pairs(params=p).cpu().numpy()
+        g = it.backward(params=p)[0].cpu().numpy()
+        it.set_plan(4, 256, 2)
+        f2 = it.run_pairs(params=p).cpu().numpy()
+        g2 = it.backward(params=p)[0].cpu().numpy()
+        assert it.last_device_error() == 0
+    ok = ~nan
+    near = ok & ~far
+    check_overlap(f[near], ref[near], kappa[near], bound[near], "blocks, transforms")
+    assert np.all(f[far & ok] == 0) and np.isnan(f[nan]).all()
+    np.testing.assert_array_max_ulp(f2[ok], f[ok], maxulp=1)
+    # the sums are the same but for their order over a warp's lanes
+    scale = np.abs(g2[ok]).max()
+    np.testing.assert_allclose(g[ok], g2[ok], rtol=1e-4, atol=1e-6 * scale)

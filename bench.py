@@ -693,7 +693,7 @@ def run_sparse_workload(args):
             "probes_per_s": probes / (ms / 1e3),
             "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                          "frac": achieved / peak, "traffic": None,
-                         "kernel": "sparse_dense_kernel + sparse_join_kernel",
+                         "kernel": "sparse_gather_kernel + sparse_join_kernel",
                          "peak_kind": f"{pk_kind} HBM copy; every entry read once, every pair "
                                       "written once"},
             "gpu_launches": 3 * args.steps}

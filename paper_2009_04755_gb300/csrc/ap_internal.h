@@ -359,9 +359,10 @@ struct SparseStore {
   double *d_rs = nullptr;           // 1 / sqrt(sum of squares), NaN for none
   int32_t *d_tiles = nullptr;       // block pairs (I <= J) of 128 items
   int64_t n_tiles = 0;
-  int32_t *d_chunks = nullptr;      // [n_join + n_dense]: chunks with shared codes, by way
-  int64_t n_join = 0, n_dense = 0;
-  unsigned long long *d_heads = nullptr;   // unit queues of the two kernels
+  int32_t *d_chunks = nullptr;      // [n_join + n_gather + n_dense]: chunks with
+                                    // shared codes, by way
+  int64_t n_join = 0, n_gather = 0, n_dense = 0;
+  unsigned long long *d_heads = nullptr;   // unit queues of the three kernels
 };
 }  // namespace ap
 

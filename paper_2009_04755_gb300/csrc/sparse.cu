@@ -7,21 +7,24 @@
 // Rows are CSR (strictly increasing int32 codes, FP32 values) over an index
 // space of `dim` codes (20^k k-mers), cut into chunks of kSparseChunk codes.
 // A pair's sum needs only the codes that both rows hold, which for a code in
-// p of the n rows is p (p - 1) / 2 products.  Each chunk takes the cheaper of
-// two ways, decided at creation from its codes' counts:
+// p of the n rows is p (p - 1) / 2 products.  Each chunk takes the cheapest of
+// three ways, decided at creation from its codes' counts:
 //
 //   join    few rows per code: one CTA sorts the chunk's entries by code in
 //           shared memory (count, scan, scatter) and adds every pair of
 //           entries of a code into the FP64 output, one product each;
-//   dense   many rows per code: the FP32 Gram of the chunk's dense form, tiles
-//           of 128 x 128 rows, 32 codes at a time scattered straight from the
-//           CSR rows into shared memory (nothing dense in global memory), FP32
-//           sums over one chunk added into the FP64 output.
+//   gather  more: tiles of 128 x 128 rows, 64 codes at a time; block J is
+//           scattered dense into shared memory straight from its CSR rows, and
+//           each entry of block I multiplies the 128 values of its code;
+//   dense   a third of the rows per code and more: both blocks dense, 32 codes
+//           at a time, and an FP32 Gram of them.
 //
-// A last pass scales by the norms.  (Before, every chunk was made dense for 8
-// rows at a time in tiles of 32 x 64 rows, one product per entry of row j and
-// row i whether row i held the code or not: 256 rows of 20^6 codes, 1e5 to
-// 1.8e6 entries each, took 255 ms, 20 CTAs' work; now 10.4.)
+// Tiles keep FP32 sums over one chunk (or a part of one) and add them into the
+// FP64 output.  A last pass scales by the norms.  (Before, every chunk was made
+// dense for 8 rows at a time in tiles of 32 x 64 rows, one product per entry of
+// row j and row i whether row i held the code or not: 256 rows of 20^6 codes,
+// 1e5 to 1.8e6 entries each, took 255 ms, 20 CTAs' work; 10.5 with join and dense
+// alone, now 8.5.)
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
@@ -398,6 +401,229 @@ sparse_dense_kernel(const int64_t *__restrict__ off, const int32_t *__restrict__
   }
 }
 
+// ---------------------------------------------------------------------------
+// gather
+// ---------------------------------------------------------------------------
+// Units as the dense kernel's, but only rows B are made dense: 64 codes at a
+// time of the 128 rows of block J, a code's values side by side.  Each entry of
+// a row A takes one 512-byte read of its code's values (4 columns per lane) and
+// four FMAs per lane, so the work falls with the density of the rows A.  A warp
+// holds the 16 x 128 sums of its 16 rows A; rows that hold more of a stage's
+// codes than are staged at a time take more turns over the 16.
+// Bound by shared memory, busy 0.71 of the time: 4.5 wavefronts an entry (half a
+// read of two entries, four of values), as many again to bring the stages in.
+// 976 chunks of 256 rows of which a code is in 31: 6.2 ms, dense 8.3; with 8% of
+// the rows in a code 0.96 ms (joins 1.26), 12% 1.23 (dense 1.55), 20% 2.23
+// (2.25), 30% 3.27 (2.92).  The first form, with the further turns inside the
+// unrolled rows, fetched instructions a quarter of the time (8.2 ms).
+constexpr int kGatherStage = 64;                      // codes per stage
+constexpr int kGatherAhead = 16;                      // entries of a row staged at a time
+constexpr int kGatherBuf = (kGatherStage + 1) * kDenseLd;   // and a code of zeros
+constexpr size_t kGatherSmem =
+    (size_t)2 * kGatherBuf * 4 + 256 * 16 + (size_t)256 * kGatherAhead * 8;
+
+struct __align__(16) Row {
+  int64_t base;                          // of its entries in the CSR arrays
+  int32_t next, end;                     // relative to base
+};
+
+__global__ void __launch_bounds__(256, 2)
+sparse_gather_kernel(const int64_t *__restrict__ off, const int32_t *__restrict__ idx,
+                     const float *__restrict__ val, const int32_t *__restrict__ cptr, int64_t n,
+                     const int32_t *__restrict__ chunks, int32_t n_chunks, int32_t split,
+                     const int32_t *__restrict__ tiles, int64_t n_tiles,
+                     unsigned long long *queue, double *__restrict__ out) {
+  extern __shared__ __align__(16) float dsm[];
+  float *s_buf = dsm;                                              // [2][stage + 1][ld]
+  int2 *s_ent = reinterpret_cast<int2 *>(dsm + 2 * kGatherBuf);    // [256][kGatherAhead]
+  Row *s_row = reinterpret_cast<Row *>(s_ent + 256 * kGatherAhead);   // rows A, rows B
+  __shared__ unsigned long long s_unit;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int half = lane >> 4, sub = lane & 15;        // two rows per warp load
+  const int a0 = warp * 16, b0 = kDenseTile + warp * 16;   // this warp's rows
+
+  for (;;) {
+    if (tid == 0) s_unit = atomicAdd(queue, 1ull);
+    __syncthreads();
+    const int64_t u = (int64_t)s_unit;
+    __syncthreads();
+    if (u >= n_tiles * split * n_chunks) break;
+    const int64_t part = u / n_tiles, t = u - part * n_tiles;   // part of a chunk, tile
+    const int64_t i0 = (int64_t)tiles[2 * t] * kDenseTile;
+    const int64_t j0 = (int64_t)tiles[2 * t + 1] * kDenseTile;
+    const bool diag = i0 == j0;
+    const int64_t c = chunks[part / split];
+    const int stages = W / kGatherStage / split;
+    const int32_t code0 = (int32_t)(c * W + (part % split) * (W / split));
+    {
+      const int64_t row = tid < kDenseTile ? i0 + tid : j0 + tid - kDenseTile;
+      const bool in = row < n;
+      const int64_t base = in ? off[row] : 0;
+      int32_t lo = in ? cptr[c * n + row] : 0, hi = in ? cptr[(c + 1) * n + row] : 0;
+      const int32_t end = hi;
+      if (split > 1)                              // first entry of this part
+        while (lo < hi) {
+          const int32_t mid = lo + ((hi - lo) >> 1);
+          if (idx[base + mid] < code0) lo = mid + 1;
+          else hi = mid;
+        }
+      s_row[tid] = {base, lo, end};
+    }
+    __syncthreads();
+    float2 acc[16][2];
+#pragma unroll
+    for (int r = 0; r < 16; ++r) acc[r][0] = acc[r][1] = make_float2(0.f, 0.f);
+
+    // the next entries of a row into its staging area, one a lane
+    auto load = [&](int rr) {
+      const int4 w = *reinterpret_cast<const int4 *>(s_row + rr);
+      const int64_t base = (int64_t)(((uint64_t)(uint32_t)w.y << 32) | (uint32_t)w.x);
+      const int p = w.z + sub;
+      int2 *dst = s_ent + rr * kGatherAhead + sub;
+      if (p < w.w) {
+        cp_async4(&dst->x, idx + base + p);
+        cp_async4(&dst->y, val + base + p);
+      } else {
+        dst->x = -1;
+      }
+    };
+    auto load16 = [&](int first) {
+#pragma unroll 4
+      for (int q = 0; q < 8; ++q) load(first + 2 * q + half);
+    };
+    auto arrived = [] { asm volatile("cp.async.wait_all;" ::: "memory"); };
+    auto zero = [&](int buf) {
+      float4 *z = reinterpret_cast<float4 *>(s_buf + buf * kGatherBuf);
+      for (int k = tid; k < kGatherBuf / 4; k += 256) z[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+    };
+    // the rows B's staged entries of the stage's codes into its buffer; more
+    // while a row has them (each lane reads what it staged itself)
+    auto scatter = [&](int buf, int32_t k0) {
+      float *dst = s_buf + buf * kGatherBuf;
+      auto place = [&](int q) -> bool {
+        const int rr = b0 + 2 * q + half;
+        const int2 e = s_ent[rr * kGatherAhead + sub];
+        const bool in = (uint32_t)(e.x - k0) < (uint32_t)kGatherStage;   // codes come in order
+        if (in) dst[(e.x - k0) * kDenseLd + rr - kDenseTile] = __int_as_float(e.y);
+        const uint32_t m = __ballot_sync(0xffffffffu, in);
+        const int taken = __popc((m >> (16 * half)) & 0xffffu);
+        if (sub == 0 && taken) s_row[rr].next += taken;
+        return __any_sync(0xffffffffu, taken == kGatherAhead);
+      };
+      uint32_t more = 0;
+#pragma unroll 4
+      for (int q = 0; q < 8; ++q) more |= place(q) ? 1u << q : 0u;
+      for (; more; more &= more - 1) {
+        const int q = __ffs(more) - 1;
+        do {
+          __syncwarp();
+          load(b0 + 2 * q + half);
+          arrived();
+        } while (place(q));
+      }
+    };
+    // Staged entries of rows A, two rows at once: {code in the stage, value},
+    // {the code of zeros, 0} past the stage's; returns which lanes' are the stage's
+    auto ready = [&](int rr, int32_t k0) -> uint32_t {
+      int2 *at = s_ent + rr * kGatherAhead + sub;
+      const int2 e = *at;
+      const bool in = (uint32_t)(e.x - k0) < (uint32_t)kGatherStage;
+      *at = in ? make_int2(e.x - k0, e.y) : make_int2(kGatherStage, 0);
+      const uint32_t m = __ballot_sync(0xffffffffu, in);
+      const int taken = __popc((m >> (16 * half)) & 0xffffu);
+      if (sub == 0 && taken) s_row[rr].next += taken;
+      return m;
+    };
+    // whether some row may have more of the stage's codes
+    uint32_t have[8];
+    auto ready16 = [&](int32_t k0) -> bool {
+      bool full = false;
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {
+        have[q] = ready(a0 + 2 * q + half, k0);
+        full |= (have[q] & 0xffffu) == 0xffffu || have[q] >> 16 == 0xffffu;
+      }
+      __syncwarp();
+      return full;
+    };
+
+    load16(a0);
+    load16(b0);
+    zero(0);
+    zero(1);
+    __syncthreads();
+    arrived();
+    scatter(0, code0);
+    bool full = ready16(code0);
+    __syncthreads();
+    for (int st = 0; st < stages; ++st) {
+      const int buf = st & 1;
+      const int32_t k0 = code0 + st * kGatherStage;
+      const bool more = st + 1 < stages;
+      if (more) {
+        load16(b0);
+        if (st > 0) zero(buf ^ 1);
+      }
+      const float *Bs = s_buf + buf * kGatherBuf + 4 * lane;
+      for (;;) {
+#pragma unroll
+        for (int r = 0; r < 16; ++r) {
+          // a diagonal tile has no pair of a row with those before it
+          const bool on = !diag || 4 * lane + 3 > a0 + r;
+          const int4 *ent = reinterpret_cast<const int4 *>(s_ent + (a0 + r) * kGatherAhead);
+          const int cnt = __popc((have[r >> 1] >> (16 * (r & 1))) & 0xffffu);
+          int4 two = ent[0];
+#pragma unroll 1
+          for (int e = 0; e < cnt; e += 2) {
+            const int4 now = two;
+            two = ent[e / 2 + 1];                 // (past a row's last: not used)
+            float4 x = make_float4(0.f, 0.f, 0.f, 0.f), y = x;
+            if (on) {
+              x = *reinterpret_cast<const float4 *>(Bs + now.x * kDenseLd);
+              y = *reinterpret_cast<const float4 *>(Bs + now.z * kDenseLd);
+            }
+            const float v = __int_as_float(now.y), w = __int_as_float(now.w);
+            acc[r][0] = __ffma2_rn(make_float2(v, v), make_float2(x.x, x.y), acc[r][0]);
+            acc[r][1] = __ffma2_rn(make_float2(v, v), make_float2(x.z, x.w), acc[r][1]);
+            acc[r][0] = __ffma2_rn(make_float2(w, w), make_float2(y.x, y.y), acc[r][0]);
+            acc[r][1] = __ffma2_rn(make_float2(w, w), make_float2(y.z, y.w), acc[r][1]);
+          }
+        }
+        __syncwarp();
+        if (!full) break;
+        load16(a0);
+        arrived();
+        full = ready16(k0);
+      }
+      if (more) load16(a0);
+      __syncthreads();                            // the other buffer is clear
+      if (more) {
+        arrived();
+        scatter(buf ^ 1, k0 + kGatherStage);
+        full = ready16(k0 + kGatherStage);
+      }
+      __syncthreads();
+    }
+
+    const int ni = (int)(n - i0 < kDenseTile ? n - i0 : kDenseTile);
+    const int nj = (int)(n - j0 < kDenseTile ? n - j0 : kDenseTile);
+#pragma unroll
+    for (int r = 0; r < 16; ++r) {
+      const int il = a0 + r;
+      if (il >= ni) continue;
+      const int64_t i = i0 + il;
+      const int first = (int)(i - j0) + 1;        // pairs need j0 + jl > i
+      double *dst = out + pair_index(i, j0, n);
+#pragma unroll
+      for (int b = 0; b < 4; ++b) {
+        const int jl = 4 * lane + b;
+        if (jl >= nj || jl < first) continue;
+        atomicAdd(dst + jl, widen((b & 1) ? acc[r][b >> 1].y : acc[r][b >> 1].x));
+      }
+    }
+  }
+}
+
 // out[p] *= rs_i rs_j over the packed triangle
 __global__ void sparse_scale_kernel(double *__restrict__ out, const double *__restrict__ rs,
                                     int64_t n) {
@@ -409,9 +635,31 @@ __global__ void sparse_scale_kernel(double *__restrict__ out, const double *__re
   }
 }
 
-// measured on a GB300: see sparse_join_kernel and sparse_dense_kernel
+// Picoseconds of the whole GPU, measured on a GB300 (see the kernels); of a
+// gather, 0.7e6 a tile with hardly an entry and 23-26 an entry from sets of 2 to
+// 33% density.
 constexpr double kJoinProductPs = 5.6, kJoinEntryPs = 15.0;
 constexpr double kDenseTilePs = 2.6e6;
+constexpr double kGatherTilePs = 0.7e6, kGatherEntryPs = 23.0;
+constexpr double kJoinAlone = 0.4, kLaunchPs = 5e6;
+constexpr double kGatherUnitPs = 12e6, kGatherStagePs = 3.3e6;   // of a CTA's time
+
+// parts of a gather's chunks such that the rounds of units take least time
+struct GatherFit {
+  int32_t split;
+  double ps;
+};
+GatherFit gather_fit(int64_t chunks, int64_t n_tiles) {
+  GatherFit best{1, INFINITY};
+  const int64_t slots = 2 * (int64_t)num_sms();
+  for (int32_t split = 1; split <= 32; split *= 2) {
+    const int64_t rounds = (chunks * n_tiles * split + slots - 1) / slots;
+    const double ps = (double)rounds *
+                      (kGatherUnitPs + kGatherStagePs * (double)(W / kGatherStage / split));
+    if (ps < best.ps) best = {split, ps};
+  }
+  return best;
+}
 
 // row checks (strictly increasing codes in [0, dim)), FP64 squared norms
 constexpr int kRowThreads = 512;
@@ -531,28 +779,66 @@ ap_status create_sparse(const ap_items_desc *d, ap_items *it, cudaStream_t s) {
   std::vector<int32_t> tiles;
   dc_block_pairs((sp.n + kDenseTile - 1) / kDenseTile, tiles);
   sp.n_tiles = (int64_t)tiles.size() / 2;
-  // Each chunk by the cheaper way (picoseconds of the whole GPU): a join adds
-  // kJoinProductPs per product and kJoinEntryPs per entry, a dense chunk costs
-  // kDenseTilePs per tile whatever it holds.  A code in more rows than a join
-  // sorts at a time makes its chunk a dense one.  join chunks first in the list
-  std::vector<int32_t> join, dense;
-  for (int64_t c = 0; c < (int64_t)count.size(); ++c) {
-    const ChunkCount &k = count[c];
-    if (k.products == 0) continue;               // no code in two rows
-    const double way_join = kJoinProductPs * (double)k.products + kJoinEntryPs * (double)k.entries;
-    const bool d = k.most > kJoinCap || way_join > kDenseTilePs * (double)sp.n_tiles;
-    (d ? dense : join).push_back((int32_t)c);
+  // Each chunk by the cheapest way (picoseconds of the whole GPU): a join adds
+  // kJoinProductPs per product and kJoinEntryPs per entry; a gather kGatherTilePs
+  // per tile and kGatherEntryPs per entry and tile that has its row in block I
+  // (half the blocks, and its own); a dense chunk kDenseTilePs per tile whatever
+  // it holds.  A code in more rows than a join sorts at a time rules that out.
+  std::vector<int32_t> join, gather, dense;
+  const double blocks = (double)((sp.n + kDenseTile - 1) / kDenseTile);
+  auto way_join = [&](int32_t c) {
+    return count[c].most > kJoinCap ? INFINITY
+                                    : kJoinProductPs * (double)count[c].products +
+                                          kJoinEntryPs * (double)count[c].entries;
+  };
+  auto way_gather = [&](int32_t c) {
+    return kGatherTilePs * (double)sp.n_tiles +
+           kGatherEntryPs * (double)count[c].entries * 0.5 * (blocks + 1.0);
+  };
+  const double way_dense = kDenseTilePs * (double)sp.n_tiles;
+  for (int32_t c = 0; c < (int32_t)count.size(); ++c) {
+    if (count[c].products == 0) continue;        // no code in two rows
+    const double wj = way_join(c), wg = way_gather(c);
+    (wj <= std::min(wg, way_dense) ? join : wg <= way_dense ? gather : dense).push_back(c);
   }
   // heaviest joins first: their times differ, and the queue ends with a tail
   std::stable_sort(join.begin(), join.end(), [&](int32_t a, int32_t b) {
     return count[a].products + count[a].entries > count[b].products + count[b].entries;
   });
+  // A join is one CTA's work, which alone takes kJoinAlone of its share of the
+  // GPU's time on every CTA slot, so a few heavy ones outlast the rest: as many
+  // of them go in tiles instead, by the gather's parts, as make the two
+  // kernels' time least (600 rows of 2e6 codes: one join took 3.3 of 4.8 ms,
+  // the chunk in which the frequent codes end).
+  const double slots = 2.0 * num_sms();
+  double join_sum = 0.0, gather_sum = 0.0;
+  for (int32_t c : join) join_sum += way_join(c);
+  for (int32_t c : gather) gather_sum += way_gather(c);
+  size_t moved = 0;
+  double least = INFINITY;
+  for (size_t m = 0; m <= join.size(); ++m) {
+    const int64_t g = (int64_t)(gather.size() + m);
+    const double alone = m < join.size() ? kJoinAlone * slots * way_join(join[m]) : 0.0;
+    const double t = std::max(join_sum, alone) +
+                     (g ? std::max(gather_sum, gather_fit(g, sp.n_tiles).ps) + kLaunchPs : 0.0);
+    if (m == 0 || t < 0.9 * least) {             // (a tenth, or it is not worth the change)
+      least = t;
+      moved = m;
+    }
+    if (m == join.size() || gather_sum > least) break;
+    join_sum -= way_join(join[m]);
+    gather_sum += way_gather(join[m]);
+  }
+  gather.insert(gather.end(), join.begin(), join.begin() + moved);
+  join.erase(join.begin(), join.begin() + moved);
   sp.n_join = (int64_t)join.size();
+  sp.n_gather = (int64_t)gather.size();
   sp.n_dense = (int64_t)dense.size();
+  join.insert(join.end(), gather.begin(), gather.end());
   join.insert(join.end(), dense.begin(), dense.end());
   AP_TRY(dmalloc(&sp.d_chunks, std::max<size_t>(join.size(), 1)));
   AP_TRY(dmalloc(&sp.d_tiles, std::max<size_t>(tiles.size(), 2)));
-  AP_TRY(dmalloc(&sp.d_heads, 2));
+  AP_TRY(dmalloc(&sp.d_heads, 3));
   if (!join.empty())
     AP_TRY(cudaMemcpyAsync(sp.d_chunks, join.data(), join.size() * 4, cudaMemcpyHostToDevice, s));
   if (!tiles.empty())
@@ -564,7 +850,7 @@ ap_status create_sparse(const ap_items_desc *d, ap_items *it, cudaStream_t s) {
 
 cudaError_t launch_sparse_cosine(const SparseStore &sp, void *out, int coverage, cudaStream_t s) {
   if (sp.n_tiles <= 0) return cudaSuccess;
-  cudaError_t e = cudaMemsetAsync(sp.d_heads, 0, 2 * sizeof(*sp.d_heads), s);
+  cudaError_t e = cudaMemsetAsync(sp.d_heads, 0, 3 * sizeof(*sp.d_heads), s);
   if (e != cudaSuccess) return e;
   const int64_t slots = 2 * (int64_t)num_sms();      // two CTAs per SM, both kernels
   if (coverage) {
@@ -576,6 +862,17 @@ cudaError_t launch_sparse_cosine(const SparseStore &sp, void *out, int coverage,
   double *o = reinterpret_cast<double *>(out);
   e = cudaMemsetAsync(o, 0, (size_t)(sp.n * (sp.n - 1) / 2) * sizeof(double), s);
   if (e != cudaSuccess) return e;
+  if (sp.n_gather > 0) {
+    e = cudaFuncSetAttribute(sparse_gather_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)kGatherSmem);
+    if (e != cudaSuccess) return e;
+    const int32_t split = gather_fit(sp.n_gather, sp.n_tiles).split;
+    const int64_t units = sp.n_gather * sp.n_tiles * split;
+    sparse_gather_kernel<<<(int)std::min(slots, units), 256, kGatherSmem, s>>>(
+        sp.d_off, sp.d_idx, sp.d_val, sp.d_cptr, sp.n, sp.d_chunks + sp.n_join,
+        (int32_t)sp.n_gather, split, sp.d_tiles, sp.n_tiles, sp.d_heads + 2, o);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  }
   if (sp.n_dense > 0) {
     e = cudaFuncSetAttribute(sparse_dense_kernel<0>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)kDenseSmem);
@@ -585,7 +882,7 @@ cudaError_t launch_sparse_cosine(const SparseStore &sp, void *out, int coverage,
     while (split < 32 && sp.n_dense * sp.n_tiles * split < slots) split *= 2;
     const int64_t units = sp.n_dense * sp.n_tiles * split;
     sparse_dense_kernel<0><<<(int)std::min(slots, units), 256, kDenseSmem, s>>>(
-        sp.d_off, sp.d_idx, sp.d_val, sp.d_cptr, sp.n, sp.d_chunks + sp.n_join,
+        sp.d_off, sp.d_idx, sp.d_val, sp.d_cptr, sp.n, sp.d_chunks + sp.n_join + sp.n_gather,
         (int32_t)sp.n_dense, split, sp.d_tiles, sp.n_tiles, sp.d_heads, out);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }

@@ -88,7 +88,10 @@ def test_cosine_rejects_bad_rows(ap):
     (130, 4097, 1500, 4097),      # dense chunks, two row blocks, a chunk of one code
     (129, 20000, 5, 60),          # join chunks, a ragged row block
     (40, 12288, 8, 4000),         # rows a hundred times as heavy as others
-    (700, 8192, 20, 300)])        # join chunks sorted in several rounds
+    (700, 8192, 20, 300),         # join chunks sorted in several rounds
+    (200, 8192, 700, 1200),       # gather chunks
+    (129, 10000, 600, 9000),      # rows with more entries in 64 codes than are staged at a time
+    (150, 8300, 3500, 4500)])     # dense chunks, one of 108 codes
 def test_cosine_join_and_dense_chunks(ap, oracle_lib, n, dim, lo, hi):
     rng = np.random.default_rng(n)
     sizes = np.exp(rng.uniform(np.log(lo), np.log(hi), n)).astype(np.int64).clip(lo, hi)

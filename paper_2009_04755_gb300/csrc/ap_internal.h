@@ -10,6 +10,7 @@
 
 #include <functional>
 #include <memory>
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -146,7 +147,6 @@ struct CloudPlanHost {
 struct CloudStore {
   int dim = 2;
   int64_t n = 0;
-  bool unit_weights = true;
   std::vector<int64_t> h_size;      // points per item (original order)
   std::vector<int32_t> h_perm;      // storage position -> original item id
   std::vector<int64_t> h_poff;      // padded offsets in storage order [n+1]
@@ -372,6 +372,7 @@ struct ap_items {
   ap::CloudStore cl;
   ap::VecStore vec;
   ap::SparseStore sp;
+  std::mutex list_mutex;            // over vec.d_list, until a list run has finished
   int32_t *d_status = nullptr;      // [0] device error code, [1..] scratch
   int32_t *d_queue = nullptr;       // tile-queue heads (one per launch slot)
   float *d_scratch = nullptr;       // generic scratch

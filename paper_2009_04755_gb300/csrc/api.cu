@@ -182,7 +182,6 @@ ap_status create_clouds(const ap_items_desc *d, ap_items *it, cudaStream_t s) {
   int64_t mx = 0;
   for (int64_t v : c.h_size) mx = std::max(mx, v);
   if (mx > (int64_t)4 * 32 * kOverlapMaxRows) return AP_ERR_UNSUPPORTED;   // > 16384 points
-  c.unit_weights = (d->weight == nullptr);
 
   for (int64_t v : c.h_size) c.total_pts += round_up(v, 4);
   CloudPlanChoice ch = choose_cloud_plan(c);

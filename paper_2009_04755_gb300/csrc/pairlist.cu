@@ -341,7 +341,8 @@ cudaError_t launch_pearson_list(VecStore &v, bool split, const int32_t *pi,
   const int64_t least = (v.Dp + most - 1) / most;
   L.slice_cols = (std::max(std::max<int64_t>(std::min(share, spread), 1024), least) + 255) / 256 * 256;
   L.n_slices = (v.Dp + L.slice_cols - 1) / L.slice_cols;
-  // the handle's list buffer (the call before has synchronised its stream):
+  // the handle's list buffer (its lock held, and the call before has
+  // synchronised its stream):
   // partial sums, then the index arrays
   const size_t head = (size_t)(L.n_slices * n_pairs) * sizeof(double);
   const size_t ints_at = (head + 15) / 16 * 16, bytes = ints_at + h.ints.size() * 4;
@@ -422,6 +423,8 @@ extern "C" ap_status ap_run_pairs_list(ap_items *it, int32_t fn, int32_t precisi
       if (e == cudaSuccess) e = cudaStreamSynchronize(s);   // before the index buffer goes
       dfree(d_idx);
     } else {
+      // runs of several threads take the list buffer in turn
+      std::lock_guard<std::mutex> lock(it->list_mutex);
       e = launch_pearson_list(it->vec, split, pi, pj, n_pairs, reinterpret_cast<double *>(out), s);
       if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     }

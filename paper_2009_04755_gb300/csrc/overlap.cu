@@ -774,7 +774,7 @@ cloud_pack_kernel(const float *__restrict__ x, const float *__restrict__ y,
         ps[h] = (float)(-two_ln2 * sg * sg);     // stored negated
         if (!(-ps[h] >= kSharedMin && -ps[h] <= kSharedMax)) seen |= kCloudWide;
         const float wt = w ? w[a] : 1.f;
-        pl[h] = (wt > 0.f) ? (float)log2((double)wt) : -INFINITY;
+        pl[h] = wt == 1.f ? 0.f : (wt > 0.f) ? (float)log2((double)wt) : -INFINITY;
         px[h] = x[a];
         py[h] = y[a];
         if (dim == 3) pz[h] = z[a];
@@ -792,23 +792,26 @@ cloud_pack_kernel(const float *__restrict__ x, const float *__restrict__ y,
       }
     }
     if (ordered) {
-      // one warp per box, a point per lane
+      // one warp per box, a point per lane, as just stored (FP64, and log2 in
+      // it, is slow here)
+      __syncthreads();
       const int64_t b0 = cloud_box0(poff[s] >> 2, s);
       for (int b = warp; b * 32 < cnt; b += kPackThreads / 32) {
-        const int k = b * 32 + lane;
-        const float wt = k < cnt ? (w ? w[source(k)] : 1.f) : 0.f;
-        const bool in = wt > 0.f;                // others have no terms
+        const int k = b * 32 + lane, h = k & 1;
         float lo[3], hi[3], sm = 0.f, lm = -INFINITY;
 #pragma unroll
         for (int d = 0; d < 3; ++d) { lo[d] = INFINITY; hi[d] = -INFINITY; }
-        if (in) {
-          const int64_t a = source(k);
-          const double sg = (double)sigma[a];
-          sm = fabsf((float)(-two_ln2 * sg * sg));
-          lm = (float)log2((double)wt);
-          lo[0] = hi[0] = x[a];
-          lo[1] = hi[1] = y[a];
-          lo[2] = hi[2] = dim == 3 ? z[a] : 0.f;
+        if (k < cnt) {
+          const int64_t q = q0 + (k >> 1);
+          const float4 u = pts[2 * q], v = pts[2 * q + 1];
+          const float l = dim == 3 ? lw[2 * q + h] : h ? v.w : v.z;
+          if (!(l == -INFINITY)) {                // others have no terms
+            sm = fabsf(dim == 3 ? (h ? v.w : v.z) : (h ? v.y : v.x));
+            lm = l;
+            lo[0] = hi[0] = h ? u.y : u.x;
+            lo[1] = hi[1] = h ? u.w : u.z;
+            lo[2] = hi[2] = dim == 3 ? (h ? v.y : v.x) : 0.f;
+          }
         }
         for (int m = 16; m > 0; m >>= 1) {
 #pragma unroll

@@ -166,8 +166,8 @@ typedef struct ap_run_stats {
 } ap_run_stats;
 
 /* Tile plan of a point-cloud set: blocks of at most block_items items and
- * block_pts padded points (one block is staged in shared memory per tile),
- * reg_r a-points held per lane (chunks of 32*reg_r points).  sorted = items
+ * block_pts padded points (a tile stages one block in shared memory, 2048
+ * points at a time), reg_r a-points held per lane.  sorted = items
  * stored largest first (decided at creation).  rate = point pairs per second
  * the tuner measured for the chosen plan. */
 typedef struct ap_plan {
@@ -244,7 +244,7 @@ ap_status ap_update_items(ap_items *items, const float *data, int32_t data_on_ho
  *   fn = AP_FN_COSINE: sparse vectors; out double[P].
  *   fn = AP_FN_GMM_L2, AP_FN_BHATTACHARYYA: clouds; out float[P]; params as
  *        for the overlap.  The first call of each builds a re-scaled copy of
- *        the storage (16 bytes a point, + 4 for 3-D weights) and, for the L2
+ *        the storage (16 bytes a point, 20 in 3-D) and, for the L2
  *        distance, the self terms S_i; later calls reuse them.
  * Errors: AP_ERR_INVALID_ARG (fn/kind mismatch, NULL out with P > 0, params
  * with 3-D clouds), AP_ERR_STATE (representation not built), AP_ERR_CUDA,

@@ -16,7 +16,7 @@
 //   gather  more: tiles of 128 x 128 rows, 64 codes at a time; block J is
 //           scattered dense into shared memory straight from its CSR rows, and
 //           each entry of block I multiplies the 128 values of its code;
-//   dense   a third of the rows per code and more: both blocks dense, 32 codes
+//   dense   about a fifth of the rows per code and more: both blocks dense, 32 codes
 //           at a time, and an FP32 Gram of them.
 //
 // Tiles keep FP32 sums over one chunk (or a part of one) and add them into the

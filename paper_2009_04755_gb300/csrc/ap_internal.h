@@ -75,9 +75,10 @@ __device__ __forceinline__ double widen(float x) {
 // kBoxedMean points on (over points, so that large items count): clouds over
 // [-1, 1]^2 with sigma 0.01-0.03 / 0.02-0.05 ran 0.98x / 0.97x as fast with
 // boxes at 200-300 points, 1.08x / 0.98x at 400-600, 1.17x / 0.98x at 600-760
-// under transforms, 1.38x / 1.09x at 800-1200; over [-1, 1]^3 1.15x / 1.00x at
-// 800-1200 and 1.77x / 1.08x at 2000-3000; GMM L2 of 256 particles of 1000-2000
-// points 22.1 -> 13.7 ms.  Terms of one size then follow one another in the
+// under transforms, 1.38x / 1.09x at 800-1200 (2-D with strips of the extent;
+// strips by rank came after); over [-1, 1]^3 1.15x / 1.00x at 800-1200 and 1.77x
+// / 1.08x at 2000-3000; GMM L2 of 256 particles of 1000-2000
+// points 22.1 -> 12.1 ms.  Terms of one size then follow one another in the
 // block sums: errors against 64 bits 4.8e-8 -> 5.1e-8 (2-D overlap; 5.9e-8 with
 // plain sums over blocks), 5.5e-8 -> 5.6e-8 (3-D), 2.7e-8 -> 2.5e-8 (GMM L2).
 // An item of up to kCullPoints fills a warp or little more: no part of it is far

@@ -91,7 +91,11 @@ __device__ __forceinline__ float2 two_sum(float a, float b) {
   return make_float2(s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb)));
 }
 
-constexpr float kFar = 1e18f, kNear = 1e15f;
+// Padding points lie at x = kFar.  The points of a set that is swept without
+// log-weights lie within kNear of 0 and have |s2k| <= kSharedMax: a point that
+// its transform takes past 2 kNear has no term with them, but it might have one
+// with the padding, so such points stop at kPark, from where they have neither.
+constexpr float kFar = 1e18f, kNear = 1e15f, kPark = 5e17f;
 
 // smallest / largest, NaN where an operand is one
 __device__ __forceinline__ float min_nan(float a, float b) {
@@ -346,6 +350,7 @@ overlap_kernel(Params P) {
               const float ux = __fadd_rn(ax[r], ttx), uy = __fadd_rn(ay[r], tty);
               ax[r] = __fmaf_rn(cth, ux, __fmul_rn(sth, uy));
               ay[r] = __fmaf_rn(cth, uy, __fmul_rn(-sth, ux));
+              if (plain && ax[r] < -kPark && ax[r] > -INFINITY) ax[r] = -kPark;
             }
           }
         }

@@ -246,3 +246,36 @@ def test_far_blocks_under_transforms(ap, oracle_lib):
     # the sums are the same but for their order over a warp's lanes
     scale = np.abs(g2[ok]).max()
     np.testing.assert_allclose(g[ok], g2[ok], rtol=1e-4, atol=1e-6 * scale)
+
+
+@pytest.mark.parametrize("plan", [None, (4, 256, 2)])     # with boxes and without
+def test_clouds_moved_onto_the_padding(ap, plan):
+    """Unit weights, odd sizes: a pair parked far away by its transform has no
+    term with the points that fill its partner's storage up (x = 1e18, with
+    whose x these translations coincide), whichever call asks."""
+    sizes = np.array([1, 3, 5, 33, 129, 161, 1001, 2049])
+    off = np.concatenate([[0], np.cumsum(sizes)]).astype(np.int64)
+    rng = np.random.default_rng(3)
+    pts = rng.uniform(-0.3, 0.3, (2, int(off[-1]))).astype(np.float32)
+    c = {"dim": 2, "offsets": off, "x": pts[0], "y": pts[1], "z": None, "weight": None,
+         "sigma": rng.uniform(0.2, 0.4, int(off[-1])).astype(np.float32)}
+    n = len(sizes)
+    pi, pj = np.triu_indices(n, 1)
+    away = torch.zeros(len(pi), 3, device="cuda")
+    away[:, 1] = 1e18                            # moved points at x = -1e18: nothing there
+    onto = torch.zeros(len(pi), 3, device="cuda")
+    onto[:, 1] = -torch.linspace(0.4e18, 1.6e18, len(pi), device="cuda")
+    onto[::2, 1] = -1e18
+    with ap.Items.from_clouds(c) as it:
+        if plan:
+            it.set_plan(*plan)
+        assert torch.all(it.run_pairs(params=onto) == 0)
+        assert torch.all(it.run_pairs_list(pi, pj, params=onto) == 0)
+        assert torch.equal(it.run_pairs(ap.AP_FN_GMM_L2, params=onto),
+                           it.run_pairs(ap.AP_FN_GMM_L2, params=away))
+        assert torch.all(it.run_pairs(ap.AP_FN_BHATTACHARYYA, params=onto) == 0)
+        for g, f in (it.backward(params=onto), it.backward_list(pi, pj, params=onto)):
+            assert torch.all(f == 0) and torch.all(g == 0)
+        p, f, flags = it.ascent(onto.clone(), 3, 1e-2)
+        assert torch.all(f == 0) and torch.all(flags == 1) and torch.equal(p, onto)
+        assert it.last_device_error() == 0

@@ -442,10 +442,12 @@ cudaError_t launch_vec_prep(const float *X, int64_t row0, int64_t out_row0, int6
 // mean correction of pairs the Gram kernel already scaled by rs_i rs_j
 cudaError_t launch_pair_correct(double *out, const double *rs, const double *delta, int64_t n,
                                 int64_t D, cudaStream_t s);
-// out[p] = (out[p] - D delta_i delta_j) rs_i rs_j over the packed triangle
-// out[p] = (sum over r of planes[r][p] - D delta_i delta_j) rs_i rs_j
+// out[p] = (sum over r of planes[r][p] - D delta_i delta_j) rs_i rs_j; NaN for
+// every pair where the status word is set
 cudaError_t launch_pair_planes(double *out, const float *planes, int64_t k, const double *rs,
-                               const double *delta, int64_t n, int64_t D, cudaStream_t s);
+                               const double *delta, const int32_t *status, int64_t n, int64_t D,
+                               cudaStream_t s);
+// out[p] = (out[p] - D delta_i delta_j) rs_i rs_j over the packed triangle
 cudaError_t launch_pair_finalize(double *out, const double *rs, const double *delta, int64_t n,
                                  int64_t D, cudaStream_t s);
 // columns [col0, col0 + width) of rows row0.. (cols of them real, staged

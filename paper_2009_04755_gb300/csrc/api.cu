@@ -524,7 +524,8 @@ ap_status ap_run_pairs(ap_items *it, int32_t fn, int32_t precision, const float 
         AP_TRY(launch_gram_tc2_store(v.tmap_hi, v.tmap_lo, v.n, v.d_pair_units, v.n_pair_units,
                                      v.n_planes, it->d_queue, it->d_status, v.d_planes,
                                      it->wait_budget_ns, it->debug, s));
-        AP_TRY(launch_pair_planes(o, v.d_planes, v.n_planes, v.d_rs, v.d_delta_all, v.n, v.D, s));
+        AP_TRY(launch_pair_planes(o, v.d_planes, v.n_planes, v.d_rs, v.d_delta_all, it->d_status,
+                                  v.n, v.D, s));
       } else {
         AP_TRY(cudaMemsetAsync(out, 0, (size_t)(n * (n - 1) / 2) * sizeof(double), s));
         if (pairs)

@@ -482,11 +482,15 @@ __global__ void slice_finalize_kernel(double *__restrict__ out, const double *__
 }
 
 // the same over the planes of a split Gram: FP32 partial sums in order, FP64.
-// Bound by the FP64 additions (two per clock and SM), k of them a pair.
+// Bound by the FP64 additions (two per clock and SM), k of them a pair.  Where
+// a Gram left early (the status word is set), planes hold what an earlier call
+// or nothing wrote: every pair is then NaN.
 __global__ void pair_planes_kernel(double *__restrict__ out, const float *__restrict__ planes,
                                    int64_t k, const double *__restrict__ rs,
-                                   const double *__restrict__ delta, int64_t n, int64_t D) {
+                                   const double *__restrict__ delta,
+                                   const int32_t *__restrict__ status, int64_t n, int64_t D) {
   const int64_t P = n * (n - 1) / 2;
+  const bool left = *status != 0;
   for (int64_t i = blockIdx.x; i < n - 1; i += gridDim.x) {
     const double ri = rs[i], di = (double)D * delta[i];
     const int64_t p0 = pair_index(i, i + 1, n);
@@ -495,7 +499,8 @@ __global__ void pair_planes_kernel(double *__restrict__ out, const float *__rest
       double g = 0.0;
 #pragma unroll 8
       for (int64_t r = 0; r < k; ++r) g += widen(__ldcs(src + r * P));
-      out[p0 + (j - i - 1)] = (g - di * delta[j]) * (ri * rs[j]);
+      out[p0 + (j - i - 1)] = left ? __longlong_as_double(0x7ff8000000000000ll)
+                                   : (g - di * delta[j]) * (ri * rs[j]);
     }
   }
 }
@@ -760,10 +765,11 @@ cudaError_t launch_pair_correct(double *out, const double *rs, const double *del
 }
 
 cudaError_t launch_pair_planes(double *out, const float *planes, int64_t k, const double *rs,
-                               const double *delta, int64_t n, int64_t D, cudaStream_t s) {
+                               const double *delta, const int32_t *status, int64_t n, int64_t D,
+                               cudaStream_t s) {
   if (n < 2) return cudaSuccess;
   const int grid = (int)(n - 1 < 65535 ? n - 1 : 65535);
-  pair_planes_kernel<<<grid, 256, 0, s>>>(out, planes, k, rs, delta, n, D);
+  pair_planes_kernel<<<grid, 256, 0, s>>>(out, planes, k, rs, delta, status, n, D);
   return cudaGetLastError();
 }
 

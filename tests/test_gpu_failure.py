@@ -62,6 +62,28 @@ def test_wait_runs_out_with_mmas_in_flight(ap, oracle_lib, k_split):
             assert np.abs(got - ref).max() < 1e-4
 
 
+@pytest.mark.parametrize("flag", [1, 2])
+def test_early_leave_shows_no_earlier_result(ap, flag):
+    """Ranges whose partial sums stay with the handle: a run that leaves early
+    gives NaN, not the vectors of the run before, and so does every run until
+    the code has been read."""
+    n, D = 300, 2048
+    old, new = synth.vectors_grouped(n, D, seed=1).cuda(), synth.vectors_grouped(n, D, seed=2).cuda()
+    with ap.Items.from_vectors(old) as it:
+        it.set_plan(128, 256, 0, 4)
+        before = it.run_pairs()
+        assert torch.isfinite(before).all()
+        it.update(new)
+        it.set_debug(flag, wait_budget_ns=50_000_000)
+        assert torch.isnan(it.run_pairs()).all()
+        it.set_debug(0, 0)
+        assert torch.isnan(it.run_pairs()).all()
+        assert it.last_device_error() in (1, 2, 3)
+        after = it.run_pairs()
+        assert torch.isfinite(after).all() and not torch.equal(after, before)
+        assert it.last_device_error() == 0
+
+
 def test_set_debug_rejects_unknown_flag(ap):
     X = torch.randn(10, 64, device="cuda")
     with ap.Items.from_vectors(X) as it:

@@ -21,6 +21,7 @@
 #include <stdint.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "ap_internal.h"
 
@@ -532,10 +533,15 @@ __global__ void pair_correct_kernel(double *__restrict__ out, const double *__re
 constexpr int kF32Tile = 128;
 constexpr int kF32K = 16;
 constexpr int kF32Pad = 4;
+constexpr int64_t kF32Wide = (1ll << 31) / 512;
 
 // PARTIAL = 1: the unit's partial Gram is added into FP64 `out` (zeroed by
 // the caller, scaled by the pass that follows); 0: whole tiles, scaled here.
-template <int COVER, int PARTIAL>
+// WIDE = 1: rows of kF32Wide 16-column blocks and more, whose offsets in a row
+// block pass int32 (2^31 vectors of 16 bytes, at 2^26 columns).  The others keep
+// to int32: with 64-bit offsets or pointers that advance, at 128 registers a
+// thread, 1024 x 65,536 ran 1.46 to 1.61 ms, 1.41 so.
+template <int COVER, int PARTIAL, int WIDE>
 __global__ void __launch_bounds__(256, 2)
 gram_f32_kernel(const float *__restrict__ C, int64_t n, int64_t Dp,
                 const double *__restrict__ rs, const int32_t *__restrict__ tiles,
@@ -546,7 +552,7 @@ gram_f32_kernel(const float *__restrict__ C, int64_t n, int64_t Dp,
   __shared__ int s_tile;
   const int tid = threadIdx.x;
   const int tx = tid & 15, ty = tid >> 4;
-  const int nk = (int)(Dp / kF32K);          // < 2^27 k-blocks (int32 keeps registers free)
+  const int nk = (int)(Dp / kF32K);          // < 2^27: a row block of 2^31 columns is 1 TiB
 
   for (;;) {
     if (tid == 0) s_tile = atomicAdd(queue, 1);
@@ -573,11 +579,12 @@ gram_f32_kernel(const float *__restrict__ C, int64_t n, int64_t Dp,
       for (int b = 0; b < 4; ++b) acc[a][b] = make_float2(0.f, 0.f);
 
     float4 ra[2], rb[2];
+    using Offset = std::conditional_t<WIDE, int64_t, int>;
     auto gload = [&](int kb) {
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
-        ra[h] = __ldg(ablk + kb * 512 + tid + 256 * h);
-        rb[h] = __ldg(bblk + kb * 512 + tid + 256 * h);
+        ra[h] = __ldg(ablk + (Offset)kb * 512 + tid + 256 * h);
+        rb[h] = __ldg(bblk + (Offset)kb * 512 + tid + 256 * h);
       }
     };
     auto sstore = [&](int buf) {
@@ -655,8 +662,9 @@ gram_f32_kernel(const float *__restrict__ C, int64_t n, int64_t Dp,
 // quarters full, 40.6 ms, 35.1 ms in ranges.)
 int32_t f32_k_split(int64_t n_tiles, int64_t nk, int64_t slots) {
   constexpr int64_t kF32UnitBlocks = 12, kMost = 64;
-  int64_t best = 1, cost = INT64_MAX;
-  for (int64_t k = 1; k <= std::min(nk, kMost); ++k) {
+  const int64_t least = nk >= kF32Wide ? 2 : 1;      // wide rows always go in ranges
+  int64_t best = least, cost = INT64_MAX;
+  for (int64_t k = least; k <= std::min(nk, kMost); ++k) {
     const int64_t c = ((n_tiles * k + slots - 1) / slots) *
                       ((nk + k - 1) / k + (k > 1 ? 2 : 1) * kF32UnitBlocks);
     if (c < cost) { cost = c; best = k; }
@@ -805,7 +813,7 @@ cudaError_t launch_gram_f32(const float *C, int64_t n, int64_t Dp, const double 
   // issuing where 8 left it idle a third of the time)
   int per_sm = 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-          &per_sm, coverage ? gram_f32_kernel<1, 0> : gram_f32_kernel<0, 1>, 256, 0) !=
+          &per_sm, coverage ? gram_f32_kernel<1, 0, 0> : gram_f32_kernel<0, 1, 0>, 256, 0) !=
           cudaSuccess ||
       per_sm < 1) {
     cudaGetLastError();
@@ -821,14 +829,14 @@ cudaError_t launch_gram_f32(const float *C, int64_t n, int64_t Dp, const double 
   const int grid = (int)std::min<int64_t>(slots, n_tiles * k_split);
   const int32_t nt = (int32_t)n_tiles;
   if (coverage)
-    gram_f32_kernel<1, 0><<<grid, 256, 0, s>>>(C, n, Dp, rs, tiles, nt, 1, queue, out, delta,
-                                               (double)D);
+    gram_f32_kernel<1, 0, 0><<<grid, 256, 0, s>>>(C, n, Dp, rs, tiles, nt, 1, queue, out, delta,
+                                                  (double)D);
   else if (k_split == 1)
-    gram_f32_kernel<0, 0><<<grid, 256, 0, s>>>(C, n, Dp, rs, tiles, nt, 1, queue, out, delta,
-                                               (double)D);
+    gram_f32_kernel<0, 0, 0><<<grid, 256, 0, s>>>(C, n, Dp, rs, tiles, nt, 1, queue, out, delta,
+                                                  (double)D);
   else
-    gram_f32_kernel<0, 1><<<grid, 256, 0, s>>>(C, n, Dp, rs, tiles, nt, k_split, queue, out, delta,
-                                               (double)D);
+    (Dp / kF32K < kF32Wide ? gram_f32_kernel<0, 1, 0> : gram_f32_kernel<0, 1, 1>)
+        <<<grid, 256, 0, s>>>(C, n, Dp, rs, tiles, nt, k_split, queue, out, delta, (double)D);
   e = cudaGetLastError();
   if (e != cudaSuccess || k_split == 1) return e;
   return launch_pair_finalize(reinterpret_cast<double *>(out), rs, delta, n, D, s);

@@ -117,3 +117,17 @@ def test_pearson_out_of_core_8192x3m_sampled(ap, oracle_lib):
     assert abs(st["reuse_R"] - 1.625) < 1e-9
     assert st["h2d_bytes"] == int(1.625 * n) * D * 4
     del Xh
+
+
+def test_pearson_fp32_beyond_2_26_columns(ap, oracle_lib):
+    """A row block of the FP32 copy passes 2^31 vectors of 16 bytes at 2^26
+    columns: two correlated rows whose last columns outweigh the others."""
+    D = (1 << 26) + 100
+    X = synth.vectors_grouped(2, D, seed=4, device="cuda")
+    X[:, -90:] *= 2000.0
+    ref = oracle_lib.pearson(X.cpu().numpy(), np.array([0]), np.array([1]))
+    with ap.Items.from_vectors(X, precisions=(ap.AP_PREC_FP32,)) as it:
+        got = it.run_pairs(ap.AP_FN_PEARSON, ap.AP_PREC_FP32).cpu().numpy()
+        assert it.last_device_error() == 0
+    # 64 ranges of a million columns in FP32: 2^-24 sqrt(2^20) of a range's sum
+    assert abs(ref[0]) > 1e-2 and abs(got[0] - ref[0]) <= 2.0 ** -14

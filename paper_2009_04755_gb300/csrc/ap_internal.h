@@ -622,9 +622,18 @@ void dfree(T *&p) {
   p = nullptr;
 }
 
+// A copy from pageable memory, and what the null stream was given before it, done
+// for every stream on return.  cudaMemcpy by itself returns when the source has been
+// staged, and a stream that does not wait for the null stream (a non-blocking
+// one) may then read what was there before.
+inline cudaError_t upload_now(void *dst, const void *src, size_t bytes) {
+  const cudaError_t e = cudaMemcpy(dst, src, bytes, cudaMemcpyHostToDevice);
+  return e == cudaSuccess ? cudaStreamSynchronize(nullptr) : e;
+}
+
 struct CloudPlanChoice { int32_t block_items, block_pts, reg_r; bool sorted; };
 CloudPlanChoice choose_cloud_plan(const CloudStore &c);
-ap_status build_cloud_plan(ap_items *it, const CloudPlanChoice &ch, cudaStream_t s = nullptr);
+ap_status build_cloud_plan(ap_items *it, const CloudPlanChoice &ch, cudaStream_t s);
 // copy a plan to the device into c (its plan buffers hold nothing before)
 ap_status upload_cloud_plan(CloudStore &c, const CloudPlanHost &h, cudaStream_t s);
 void free_cloud_plan(CloudStore &c);

@@ -342,7 +342,7 @@ ap_status create_vectors(const ap_items_desc *d, ap_items *it, cudaStream_t s) {
     AP_TRY(dmalloc(&v.d_g64, tc_scratch_doubles(num_sms())));
     AP_TRY(dmalloc(&v.d_tiles_tc, std::max<size_t>(tiles.size(), 2)));
     if (!tiles.empty())
-      AP_TRY(cudaMemcpy(v.d_tiles_tc, tiles.data(), tiles.size() * 4, cudaMemcpyHostToDevice));
+      AP_TRY(upload_now(v.d_tiles_tc, tiles.data(), tiles.size() * 4));
     ap_status st = set_vector_plan(it, -1);
     if (st != AP_OK) return st;
   }
@@ -354,7 +354,7 @@ ap_status create_vectors(const ap_items_desc *d, ap_items *it, cudaStream_t s) {
     v.n_tiles_f32 = (int64_t)tiles.size() / 2;
     AP_TRY(dmalloc(&v.d_tiles_f32, std::max<size_t>(tiles.size(), 2)));
     if (!tiles.empty())
-      AP_TRY(cudaMemcpy(v.d_tiles_f32, tiles.data(), tiles.size() * 4, cudaMemcpyHostToDevice));
+      AP_TRY(upload_now(v.d_tiles_f32, tiles.data(), tiles.size() * 4));
   }
   if (d->data_on_host && v.n > 0) {
     // ~256 MB per staging half
@@ -658,6 +658,7 @@ int32_t ap_last_device_error(ap_items *it) {
     // an aborted launch leaves its queue part-way
     cudaMemset(it->d_queue + kQueueClouds, 0, sizeof v);
     cudaMemset(it->d_queue + kQueuePairs, 0, sizeof v);
+    cudaStreamSynchronize(nullptr);              // a run on any stream may follow
   }
   return v;
 }

@@ -239,8 +239,7 @@ ap_status cloud_list_plan(ap_items *it, const int32_t *pi, const int32_t *pj, in
     std::vector<int32_t> single;
     single_item_blocks(c, c.reg_r, single);
     AP_TRY(dmalloc(&c.d_bmeta_single, std::max<size_t>(single.size(), 8)));
-    AP_TRY(cudaMemcpy(c.d_bmeta_single, single.data(), single.size() * 4,
-                      cudaMemcpyHostToDevice));
+    AP_TRY(upload_now(c.d_bmeta_single, single.data(), single.size() * 4));
   }
   if (c.list_cap < n_pairs) {
     AP_TRY(cudaStreamSynchronize(s));              // the old list may still be read
@@ -256,7 +255,8 @@ ap_status cloud_list_plan(ap_items *it, const int32_t *pi, const int32_t *pj, in
     tiles[2 * k] = c.h_iperm[pi[k]];
     tiles[2 * k + 1] = c.h_iperm[pj[k]];
   }
-  AP_TRY(cudaMemcpy(c.d_list_tiles, tiles.data(), tiles.size() * 4, cudaMemcpyHostToDevice));
+  // (a pageable source: staged before the call returns)
+  AP_TRY(cudaMemcpyAsync(c.d_list_tiles, tiles.data(), tiles.size() * 4, cudaMemcpyHostToDevice, s));
   lc = c;
   lc.list_mode = true;
   lc.d_bmeta = c.d_bmeta_single;

@@ -261,9 +261,9 @@ static ap_status install_schedule(VecStore &v) {
   AP_TRY(dmalloc(&v.d_units, std::max<size_t>(units.size(), kOocTileInts)));
   AP_TRY(dmalloc(&v.d_cover_units, std::max<size_t>(cover.size(), kOocTileInts)));
   if (!units.empty())
-    AP_TRY(cudaMemcpy(v.d_units, units.data(), units.size() * 4, cudaMemcpyHostToDevice));
+    AP_TRY(upload_now(v.d_units, units.data(), units.size() * 4));
   if (!cover.empty())
-    AP_TRY(cudaMemcpy(v.d_cover_units, cover.data(), cover.size() * 4, cudaMemcpyHostToDevice));
+    AP_TRY(upload_now(v.d_cover_units, cover.data(), cover.size() * 4));
   v.ooc_loads = 0;
   v.ooc_uses = 0;
   for (const OocStep &st : v.steps) {
@@ -282,6 +282,7 @@ static ap_status alloc_pool(VecStore &v) {
   AP_TRY(dmalloc(&v.d_pool_lo, (size_t)pool_rows * v.Dp));
   AP_TRY(cudaMemset(v.d_pool_hi, 0, (size_t)pool_rows * v.Dp * 2));
   AP_TRY(cudaMemset(v.d_pool_lo, 0, (size_t)pool_rows * v.Dp * 2));
+  AP_TRY(cudaStreamSynchronize(nullptr));          // before a run on any stream
   AP_TRY_ST(alloc_raw_ring(v, std::max<int64_t>(2, v.group), (size_t)kMacro * v.ld));
   AP_TRY(make_tc_tensor_maps(v.d_pool_hi, v.d_pool_lo, pool_rows, v.Dp, &v.tmap_pool_hi,
                              &v.tmap_pool_lo));
@@ -336,6 +337,7 @@ static ap_status alloc_slices(VecStore &v) {
     AP_TRY(dmalloc(&v.d_slice_lo[b], elems));
     AP_TRY(cudaMemset(v.d_slice_hi[b], 0, elems * 2));
     AP_TRY(cudaMemset(v.d_slice_lo[b], 0, elems * 2));
+    AP_TRY(cudaStreamSynchronize(nullptr));        // before a run on any stream
     AP_TRY(make_tc_tensor_maps(v.d_slice_hi[b], v.d_slice_lo[b], v.n, v.slice_cols,
                                &v.tmap_slice_hi[b], &v.tmap_slice_lo[b]));
     AP_TRY(cudaEventCreateWithFlags(&v.ev_slice_ready[b], cudaEventDisableTiming));
@@ -355,13 +357,13 @@ static ap_status alloc_slices(VecStore &v) {
   v.n_slice_units = (int64_t)units.size() / kOocTileInts;
   AP_TRY(dmalloc(&v.d_slice_units, std::max<size_t>(units.size(), kOocTileInts)));
   if (!units.empty())
-    AP_TRY(cudaMemcpy(v.d_slice_units, units.data(), units.size() * 4, cudaMemcpyHostToDevice));
+    AP_TRY(upload_now(v.d_slice_units, units.data(), units.size() * 4));
   std::vector<int32_t> cover;
   pair_units(v.n, nch, tc2_pairs(), 1, cover);
   v.n_slice_cover = (int64_t)cover.size() / kOocTileInts;
   AP_TRY(dmalloc(&v.d_slice_cover, std::max<size_t>(cover.size(), kOocTileInts)));
   if (!cover.empty())
-    AP_TRY(cudaMemcpy(v.d_slice_cover, cover.data(), cover.size() * 4, cudaMemcpyHostToDevice));
+    AP_TRY(upload_now(v.d_slice_cover, cover.data(), cover.size() * 4));
   return AP_OK;
 }
 
@@ -693,7 +695,7 @@ static ap_status build_stream_units(VecStore &v, int64_t C) {
   dfree(v.d_stream_units);
   AP_TRY(dmalloc(&v.d_stream_units, std::max<size_t>(units.size(), kOocTileInts)));
   if (!units.empty())
-    AP_TRY(cudaMemcpy(v.d_stream_units, units.data(), units.size() * 4, cudaMemcpyHostToDevice));
+    AP_TRY(upload_now(v.d_stream_units, units.data(), units.size() * 4));
   return AP_OK;
 }
 

@@ -185,7 +185,7 @@ ap_status upload_units(const std::vector<int32_t> &units, int32_t **d, int64_t *
   *n = 0;
   AP_TRY(dmalloc(d, std::max<size_t>(units.size(), kOocTileInts)));
   if (!units.empty())
-    AP_TRY(cudaMemcpy(*d, units.data(), units.size() * 4, cudaMemcpyHostToDevice));
+    AP_TRY(upload_now(*d, units.data(), units.size() * 4));
   *n = (int64_t)units.size() / kOocTileInts;
   return AP_OK;
 }
@@ -255,7 +255,9 @@ extern "C" ap_status ap_set_plan(ap_items *it, const ap_plan *plan) {
   CloudPlanChoice ch{plan->block_items, plan->block_pts, plan->reg_r, it->cl.sorted};
   cudaError_t e = cudaDeviceSynchronize();      // the old plan may still be in use
   if (e != cudaSuccess) return from_cuda(e);
-  return build_cloud_plan(it, ch);
+  AP_TRY_ST(build_cloud_plan(it, ch, nullptr));
+  AP_TRY(cudaStreamSynchronize(nullptr));       // a run on any stream may follow
+  return AP_OK;
 }
 
 extern "C" ap_status ap_tune(ap_items *it, int32_t mode, void *stream, ap_plan *out) {
@@ -357,8 +359,9 @@ extern "C" ap_status ap_tune(ap_items *it, int32_t mode, void *stream, ap_plan *
   if (e1) cudaEventDestroy(e1);
   if (st != AP_OK) return st;
   if (best_rate > 0) {
-    st = build_cloud_plan(it, best);
+    st = build_cloud_plan(it, best, s);
     if (st != AP_OK) return st;
+    AP_TRY(cudaStreamSynchronize(s));            // a run on any stream may follow
   }
   if (out) {
     ap_get_plan(it, out);

@@ -95,3 +95,36 @@ def test_handles_of_one_kernel_keep_their_launch_shapes(ap):
         for _ in range(2):
             assert torch.equal(a.run_pairs(), fa) and torch.equal(b.run_pairs(), fb)
             assert a.run_pairs_list([0, 3], [1, 5]).shape == (2,)
+
+
+def test_new_plans_are_there_for_every_stream(ap):
+    """A run on a side stream straight after set_plan, tune or a list's first
+    call, with nothing that waits in between: plans of megabytes, whose copies
+    take longer than the launch."""
+    rng = np.random.default_rng(4)
+    sizes = rng.integers(3, 12, 2500)
+    off = np.concatenate([[0], np.cumsum(sizes)]).astype(np.int64)
+    pts = rng.uniform(-1, 1, (2, int(off[-1]))).astype(np.float32)
+    c = {"dim": 2, "offsets": off, "x": pts[0], "y": pts[1], "z": None, "weight": None,
+         "sigma": rng.uniform(0.1, 0.2, int(off[-1])).astype(np.float32)}
+    side = torch.cuda.Stream()
+    pi, pj = np.triu_indices(400, 1)
+    with ap.Items.from_clouds(c) as it:
+        ref = it.run_pairs()
+        one = it.run_pairs_list(pi, pj)
+        out, few = torch.zeros_like(ref), torch.zeros_like(one)
+        torch.cuda.synchronize()
+        for plan in [(8, 384, 4), (2, 64, 4), (32, 2048, 4), (3, 8192, 4)] * 3:
+            it.set_plan(*plan)
+            it.run_pairs(out=out, stream=side)
+            side.synchronize()
+            assert torch.equal(out, ref), plan
+            it.set_plan(plan[0], plan[1], 2)      # other one-item blocks
+            it.run_pairs_list(pi[::2], pj[::2], out=few[:len(pi[::2])], stream=side)
+            it.run_pairs_list(pi, pj, out=few, stream=side)
+            side.synchronize()
+            torch.testing.assert_close(few, one, rtol=1e-6, atol=0)
+        it.tune(0, stream=side)
+        it.run_pairs(out=out)
+        torch.testing.assert_close(out, ref, rtol=1e-6, atol=0)
+        assert it.last_device_error() == 0

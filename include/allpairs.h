@@ -18,7 +18,11 @@
  *         p(i, j) = i*n - i*(i+1)/2 + (j - i - 1),     P = n(n-1)/2 entries,
  *     the row-major enumeration of the strict upper triangle.  n < 2 gives
  *     P = 0 and every call returns AP_OK without touching memory.
- *   - One handle is not thread-safe; different handles are independent.
+ *   - One handle is not thread-safe, and its runs share queues, plans and partial
+ *     sums: order them on one stream, or by events.  Runs that overlap on the GPU
+ *     all the same may give wrong results, but spoil no later run.  (Pearson lists
+ *     alone, ap_run_pairs_list, may come from several threads: they take turns.)
+ *     Different handles are independent.
  *   - Device waits inside the kernels are bounded; when one runs out the
  *     kernel records a code readable with ap_last_device_error() and the call
  *     that synchronises next reports AP_ERR_TIMEOUT.

@@ -8,6 +8,7 @@
 #include <cuda_bf16.h>
 #include <stdint.h>
 
+#include <atomic>
 #include <functional>
 #include <memory>
 #include <mutex>
@@ -375,7 +376,8 @@ struct ap_items {
   ap::SparseStore sp;
   std::mutex list_mutex;            // over vec.d_list, until a list run has finished
   int32_t *d_status = nullptr;      // [0] device error code, [1..] scratch
-  int32_t *d_queue = nullptr;       // tile-queue heads (one per launch slot)
+  int32_t *d_queue = nullptr;       // device words, see kQueueTraits
+  std::atomic<uint32_t> launches{0};     // launches given a queue head (take_queue)
   float *d_scratch = nullptr;       // generic scratch
   int64_t scratch_bytes = 0;
   ap_run_stats stats{};
@@ -392,6 +394,31 @@ struct ap_items {
 };
 
 namespace ap {
+
+// ---------------------------------------------------------------------------
+// words of a handle's d_queue block, and unit queues
+// ---------------------------------------------------------------------------
+// [0] unit-queue head of the launches that clear it themselves, [1] status word,
+// [2] scratch, traits of a cloud set (some s2k or coordinate is outside the range
+// in which two terms may share a reciprocal; some weight is not 1), two heads for
+// captured launches, and a ring of heads.
+constexpr int kQueueTraits = 3, kQueueCaptured = 4, kQueueRing = 64;
+constexpr uint32_t kQueueHeads = 64;
+constexpr int kQueueWords = kQueueRing + (int)kQueueHeads;
+// The queue of one launch: `head` is 0 when the launch starts, and the launch
+// clears `ahead`.  Launches take the heads of the ring in turn and clear the one
+// half the ring on, so that a run costs no clearing of its own (a memset before
+// a small set's one kernel takes 2 of 10 us), and whatever a head is left at (by a
+// device wait that ran out, by runs that overlapped) is gone when it comes round.
+struct UnitQueue {
+  int32_t *words, *head, *ahead;
+};
+// the next head of the ring; where the stream is being captured, a head that a
+// memset in front of the launch clears, since a replay finds it as it was left
+cudaError_t take_queue(ap_items *it, cudaStream_t s, UnitQueue *q);
+// a queue taken for a launch that does not take place: clears `ahead` in its
+// stead and returns e
+cudaError_t leave_queue(const UnitQueue &q, cudaStream_t s, cudaError_t e);
 
 // ---------------------------------------------------------------------------
 // host planners (plan.cpp)
@@ -495,7 +522,7 @@ cudaError_t launch_gram_tc(const void *tmap_hi, const void *tmap_lo, int64_t n, 
 // chunk}; atomic = 1 adds partial Grams into FP64 out, 0 writes G rs_i rs_j
 // of whole block pairs, coverage = 1 counts pairs into int32 out.
 cudaError_t launch_gram_tc2(const void *tmap_hi, const void *tmap_lo, int64_t n, const double *rs,
-                            const int32_t *units, int64_t n_units, int32_t *queue,
+                            const int32_t *units, int64_t n_units, const UnitQueue &queue,
                             int32_t *status, double *g64, void *out, int coverage, int atomic,
                             uint64_t budget, int32_t debug, cudaStream_t s);
 // split-K units of the resident set, listed by pair_units with k_split ranges
@@ -503,8 +530,8 @@ cudaError_t launch_gram_tc2(const void *tmap_hi, const void *tmap_lo, int64_t n,
 // planes[r][n (n - 1) / 2]
 cudaError_t launch_gram_tc2_store(const void *tmap_hi, const void *tmap_lo, int64_t n,
                                   const int32_t *units, int64_t n_units, int64_t k_split,
-                                  int32_t *queue, int32_t *status, float *planes, uint64_t budget,
-                                  int32_t debug, cudaStream_t s);
+                                  const UnitQueue &queue, int32_t *status, float *planes,
+                                  uint64_t budget, int32_t debug, cudaStream_t s);
 // CTA pairs of one launch (clusters of two that fit on the device at once)
 int64_t tc2_pairs();
 // units of the CTA-pair Gram over the resident set: macro pairs (I <= J, 256
@@ -553,18 +580,18 @@ cudaError_t launch_pearson_list(VecStore &v, bool split, const int32_t *pi,
 
 // clouds (overlap.cu)
 cudaError_t launch_overlap(const CloudStore &cs, const float *params, float *out,
-                           int coverage, int32_t *queue, cudaStream_t s);
+                           int coverage, const UnitQueue &queue, cudaStream_t s);
 // adjoint (params_io == NULL: grad_params = grad_out * grad f) or one fused
 // ascent step (params_io != NULL: params_io += eta grad f / f where f >= fmin)
-cudaError_t launch_overlap_grad_q(const CloudStore &cs, int32_t *queue, const float *params,
-                                  const float *grad_out, float *grad_params, float *f_out,
-                                  float eta, float fmin, float *params_io, int32_t *flags,
-                                  cudaStream_t s);
+cudaError_t launch_overlap_grad_q(const CloudStore &cs, const UnitQueue &queue,
+                                  const float *params, const float *grad_out,
+                                  float *grad_params, float *f_out, float eta, float fmin,
+                                  float *params_io, int32_t *flags, cudaStream_t s);
 // particle scores (score 1 GMM L2 distance, 2 Bhattacharyya cost) on the
 // re-scaled storage pts / lw; self = the L2 self terms (score 1)
 cudaError_t launch_score(const CloudStore &cs, int score, const float4 *pts, const float *lw,
-                         const double *self, const float *params, float *out, int32_t *queue,
-                         cudaStream_t s);
+                         const double *self, const float *params, float *out,
+                         const UnitQueue &queue, cudaStream_t s);
 cudaError_t launch_cloud_rescore(const CloudStore &cs, int score, float4 *pts_out, float *lw_out,
                                  cudaStream_t s);
 cudaError_t launch_cloud_self(const CloudStore &cs, const float4 *pts, const float *lw,
@@ -573,14 +600,7 @@ cudaError_t launch_cloud_self(const CloudStore &cs, const float4 *pts, const flo
 ap_status create_sparse(const ap_items_desc *d, ap_items *it, cudaStream_t s);
 void free_sparse(SparseStore &sp);
 cudaError_t launch_sparse_cosine(const SparseStore &sp, void *out, int coverage, cudaStream_t s);
-// words of a handle's d_queue block: [0] tile-queue head, [1] status word,
-// [2] scratch, and for clouds their own queue head (zero between launches:
-// the CTA that takes the last pop resets it) and traits of the set: some s2k
-// or coordinate is outside the range in which two terms may share a
-// reciprocal; some weight is not 1
-constexpr int kQueueClouds = 3, kQueueTraits = 4;
-constexpr int kQueuePairs = 5;          // head of the CTA-pair Gram's queue, reset the same way
-constexpr int32_t kCloudWide = 1, kCloudWeighted = 2;
+constexpr int32_t kCloudWide = 1, kCloudWeighted = 2;   // traits of a set, see below
 // tiles at the end of a cloud plan's list that are split: one per CTA slot
 // (four CTAs of four warps per SM)
 constexpr int64_t kSplitTailPerSm = 4;

@@ -47,6 +47,27 @@ ap_status from_cuda(cudaError_t e) {
   return e == cudaErrorMemoryAllocation ? AP_ERR_OOM : AP_ERR_CUDA;
 }
 
+cudaError_t take_queue(ap_items *it, cudaStream_t s, UnitQueue *q) {
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (s) {                              // (the legacy stream cannot be captured)
+    const cudaError_t e = cudaStreamIsCapturing(s, &cap);
+    if (e != cudaSuccess) return e;
+  }
+  if (cap != cudaStreamCaptureStatusNone) {
+    *q = {it->d_queue, it->d_queue + kQueueCaptured, nullptr};
+    return cudaMemsetAsync(q->head, 0, sizeof(int32_t), s);
+  }
+  const uint32_t k = it->launches.fetch_add(1, std::memory_order_relaxed);
+  int32_t *ring = it->d_queue + kQueueRing;
+  *q = {it->d_queue, ring + k % kQueueHeads, ring + (k + kQueueHeads / 2) % kQueueHeads};
+  return cudaSuccess;
+}
+
+cudaError_t leave_queue(const UnitQueue &q, cudaStream_t s, cudaError_t e) {
+  if (q.ahead) cudaMemsetAsync(q.ahead, 0, sizeof(int32_t), s);
+  return e;
+}
+
 namespace {
 
 int64_t round_up(int64_t v, int64_t m) { return (v + m - 1) / m * m; }
@@ -439,8 +460,8 @@ ap_status ap_create_items(const ap_items_desc *desc, void *stream, ap_items **ou
   it->kind = desc->kind;
   cudaGetDevice(&it->device);
   ap_status st = AP_OK;
-  cudaError_t e = dmalloc(&it->d_queue, 64);
-  if (e == cudaSuccess) e = cudaMemsetAsync(it->d_queue, 0, 64 * sizeof(int32_t), s);
+  cudaError_t e = dmalloc(&it->d_queue, kQueueWords);
+  if (e == cudaSuccess) e = cudaMemsetAsync(it->d_queue, 0, kQueueWords * sizeof(int32_t), s);
   if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&it->copy_stream, cudaStreamNonBlocking);
   if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&it->graph_stream, cudaStreamNonBlocking);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&it->ev_a, cudaEventDisableTiming);
@@ -516,26 +537,30 @@ ap_status ap_run_pairs(ap_items *it, int32_t fn, int32_t precision, const float 
     if (use_split && !have_split) return AP_ERR_STATE;
     if (!use_split && !have_f32) return AP_ERR_STATE;
     const bool pairs = v.mma_ctas == 2;
+    UnitQueue q;
     if (use_split && !cover && v.k_split > 0) {
       // split-K units in waves: partial Grams in planes that the scaling pass
       // sums, or added in FP64 into `out`
       double *o = reinterpret_cast<double *>(out);
       if (pairs && v.d_planes) {
+        AP_TRY(take_queue(it, s, &q));
         AP_TRY(launch_gram_tc2_store(v.tmap_hi, v.tmap_lo, v.n, v.d_pair_units, v.n_pair_units,
-                                     v.n_planes, it->d_queue, it->d_status, v.d_planes,
+                                     v.n_planes, q, it->d_status, v.d_planes,
                                      it->wait_budget_ns, it->debug, s));
         AP_TRY(launch_pair_planes(o, v.d_planes, v.n_planes, v.d_rs, v.d_delta_all, it->d_status,
                                   v.n, v.D, s));
       } else {
         AP_TRY(cudaMemsetAsync(out, 0, (size_t)(n * (n - 1) / 2) * sizeof(double), s));
-        if (pairs)
+        if (pairs) {
+          AP_TRY(take_queue(it, s, &q));
           AP_TRY(launch_gram_tc2(v.tmap_hi, v.tmap_lo, v.n, v.d_rs, v.d_pair_units,
-                                 v.n_pair_units, it->d_queue, it->d_status, v.d_g64, out, 0, 1,
+                                 v.n_pair_units, q, it->d_status, v.d_g64, out, 0, 1,
                                  it->wait_budget_ns, it->debug, s));
-        else
+        } else {
           AP_TRY(launch_gram_tc(v.tmap_hi, v.tmap_lo, v.n, v.Dp, v.d_rs, v.d_panel_units,
                                 v.n_panel_units, it->d_queue, it->d_status, v.d_g64, out, 0, 1,
                                 it->wait_budget_ns, it->debug, s));
+        }
         AP_TRY(launch_pair_finalize(o, v.d_rs, v.d_delta_all, v.n, v.D, s));
       }
       it->stats.tiles = pairs ? v.n_pair_units : v.n_panel_units;
@@ -543,8 +568,9 @@ ap_status ap_run_pairs(ap_items *it, int32_t fn, int32_t precision, const float 
       it->stats.tile_n = kTcTileN;
     } else if (use_split && pairs) {
       // whole block pairs (or coverage) on CTA pairs
+      AP_TRY(take_queue(it, s, &q));
       AP_TRY(launch_gram_tc2(v.tmap_hi, v.tmap_lo, v.n, v.d_rs, v.d_pair_whole, v.n_pair_whole,
-                             it->d_queue, it->d_status, v.d_g64, out, cover, 0,
+                             q, it->d_status, v.d_g64, out, cover, 0,
                              it->wait_budget_ns, it->debug, s));
       if (!cover)
         AP_TRY(launch_pair_correct(reinterpret_cast<double *>(out), v.d_rs, v.d_delta_all, v.n,
@@ -578,15 +604,19 @@ ap_status ap_run_pairs(ap_items *it, int32_t fn, int32_t precision, const float 
     const int score = fn == AP_FN_GMM_L2 ? 1 : 2;
     AP_TRY_ST(ensure_score_storage(it, score, s));
     const CloudStore &c = it->cl;
+    UnitQueue q;
+    AP_TRY(take_queue(it, s, &q));
     AP_TRY(launch_score(c, score, c.d_pts_score[score - 1], c.d_lw_score[score - 1], c.d_self,
-                        params, reinterpret_cast<float *>(out), it->d_queue, s));
+                        params, reinterpret_cast<float *>(out), q, s));
     it->stats.tiles = it->cl.n_tiles;
     it->stats.item_loads = it->cl.n;
     it->stats.reuse_R = 1.0;
     it->stats.slot_hit_rate = 1.0;
     return AP_OK;
   }
-  AP_TRY(launch_overlap(it->cl, params, reinterpret_cast<float *>(out), cover, it->d_queue, s));
+  UnitQueue q;
+  AP_TRY(take_queue(it, s, &q));
+  AP_TRY(launch_overlap(it->cl, params, reinterpret_cast<float *>(out), cover, q, s));
   it->stats.tiles = it->cl.n_tiles;
   it->stats.item_loads = it->cl.n;
   it->stats.reuse_R = 1.0;
@@ -601,8 +631,11 @@ ap_status ap_backward(ap_items *it, const float *params, const float *grad_out,
   if (it->kind != AP_ITEMS_CLOUD2D) return AP_ERR_INVALID_ARG;
   if (it->cl.n < 2) return AP_OK;
   if (!grad_params) return AP_ERR_INVALID_ARG;
-  AP_TRY(launch_overlap_grad_q(it->cl, it->d_queue, params, grad_out, grad_params, f_out, 0.f, 0.f,
-                               nullptr, nullptr, reinterpret_cast<cudaStream_t>(stream)));
+  cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
+  UnitQueue q;
+  AP_TRY(take_queue(it, s, &q));
+  AP_TRY(launch_overlap_grad_q(it->cl, q, params, grad_out, grad_params, f_out, 0.f, 0.f, nullptr,
+                               nullptr, s));
   return AP_OK;
 }
 
@@ -617,12 +650,13 @@ ap_status ap_ascent(ap_items *it, float *params, int32_t n_steps, float eta, flo
   GraphKey key{params, f_out, flags, nullptr, eta, fmin, n_steps};
   ap_items *h = it;
   return run_graphed(it, key, s, [h, params, n_steps, eta, fmin, f_out, flags](cudaStream_t cs) {
-    for (int32_t k = 0; k < n_steps; ++k) {
-      cudaError_t e = launch_overlap_grad_q(h->cl, h->d_queue, nullptr, nullptr, nullptr, f_out,
-                                            eta, fmin, params, flags, cs);
-      if (e != cudaSuccess) return e;
-    }
-    return cudaSuccess;
+    // captured: the first head cleared here, each other by the step before
+    int32_t *heads = h->d_queue + kQueueCaptured;
+    cudaError_t e = cudaMemsetAsync(heads, 0, sizeof(int32_t), cs);
+    for (int32_t k = 0; k < n_steps && e == cudaSuccess; ++k)
+      e = launch_overlap_grad_q(h->cl, {h->d_queue, heads + (k & 1), heads + (~k & 1)}, nullptr,
+                                nullptr, nullptr, f_out, eta, fmin, params, flags, cs);
+    return e;
   });
 }
 
@@ -655,9 +689,6 @@ int32_t ap_last_device_error(ap_items *it) {
   if (cudaMemcpy(&v, it->d_status, sizeof v, cudaMemcpyDeviceToHost) != cudaSuccess) return -1;
   if (v != 0) {
     cudaMemset(it->d_status, 0, sizeof v);
-    // an aborted launch leaves its queue part-way
-    cudaMemset(it->d_queue + kQueueClouds, 0, sizeof v);
-    cudaMemset(it->d_queue + kQueuePairs, 0, sizeof v);
     cudaStreamSynchronize(nullptr);              // a run on any stream may follow
   }
   return v;

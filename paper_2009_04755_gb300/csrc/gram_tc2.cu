@@ -151,8 +151,9 @@ template <int OUT>
 __global__ void __maxnreg__(168)
 gram_tc2_kernel(const __grid_constant__ CUtensorMap tm_hi, const __grid_constant__ CUtensorMap tm_lo,
                 int64_t n, const double *__restrict__ rs, const int32_t *__restrict__ units,
-                int32_t n_units, int32_t *queue, int32_t *status, double *__restrict__ g64,
-                void *out, SplitOrder order, uint64_t budget, int32_t debug) {
+                int32_t n_units, int32_t *queue, int32_t *ahead, int32_t *status,
+                double *__restrict__ g64, void *out, SplitOrder order, uint64_t budget,
+                int32_t debug) {
   constexpr bool COVER = OUT == kCover;
   extern __shared__ uint8_t smem_raw[];
   uint8_t *smem = reinterpret_cast<uint8_t *>(
@@ -246,6 +247,7 @@ gram_tc2_kernel(const __grid_constant__ CUtensorMap tm_hi, const __grid_constant
     uint32_t us = 0, uph = 0, ps = 0, pph = 0;
     int32_t round = 0;                     // phase of every stage in this pass of the ring
     bool stop = false;
+    if (ahead && blockIdx.x == 0) *ahead = 0;
     while (!stop) {
       int32_t t;
       if (leader) {
@@ -253,12 +255,7 @@ gram_tc2_kernel(const __grid_constant__ CUtensorMap tm_hi, const __grid_constant
           abort_pair(DEV_TIMEOUT_UNIT);
           break;
         }
-        // each pair of CTAs pops once past the last unit; the last of these
-        // pops leaves the queue as it was found (an aborted run does not, and
-        // nothing runs until the host has cleared the status and the queue)
         t = atomicAdd(queue, 1);
-        if (t == n_units + (int32_t)(gridDim.x >> 1) - 1)
-          *reinterpret_cast<volatile int32_t *>(queue) = 0;
         if (*s_abort || *reinterpret_cast<volatile int32_t *>(status) != 0) t = n_units;
         if (t > n_units) t = n_units;
         ring[us] = t;
@@ -540,7 +537,8 @@ gram_tc2_kernel(const __grid_constant__ CUtensorMap tm_hi, const __grid_constant
 }
 
 using Kern2 = void (*)(CUtensorMap, CUtensorMap, int64_t, const double *, const int32_t *, int32_t,
-                       int32_t *, int32_t *, double *, void *, SplitOrder, uint64_t, int32_t);
+                       int32_t *, int32_t *, int32_t *, double *, void *, SplitOrder, uint64_t,
+                       int32_t);
 
 Kern2 pick(int out) {
   switch (out) {
@@ -603,26 +601,26 @@ int64_t tc2_pairs() {
 
 namespace {
 cudaError_t launch(const void *tmap_hi, const void *tmap_lo, int64_t n, const double *rs,
-                   const int32_t *units, int64_t n_units, int32_t *queue, int32_t *status,
+                   const int32_t *units, int64_t n_units, const UnitQueue &queue, int32_t *status,
                    double *g64, void *out, int what, SplitOrder order, uint64_t budget,
                    int32_t debug, cudaStream_t s) {
-  if (n_units <= 0) return cudaSuccess;
-  if (n_units > INT32_MAX / 2) return cudaErrorInvalidValue;
-  cudaError_t e = ensure_attr(what);
-  if (e != cudaSuccess) return e;
+  if (n_units <= 0) return leave_queue(queue, s, cudaSuccess);
+  cudaError_t e = n_units > INT32_MAX / 2 ? cudaErrorInvalidValue : ensure_attr(what);
+  if (e != cudaSuccess) return leave_queue(queue, s, e);
   int64_t pairs = tc2_pairs();
   if (pairs > n_units) pairs = n_units;
   cudaLaunchAttribute attr[1];
   cudaLaunchConfig_t cfg = launch_cfg((int)pairs, s, attr);
-  return cudaLaunchKernelEx(&cfg, pick(what), *reinterpret_cast<const CUtensorMap *>(tmap_hi),
-                            *reinterpret_cast<const CUtensorMap *>(tmap_lo), n, rs, units,
-                            (int32_t)n_units, queue + kQueuePairs, status, g64, out, order,
-                            (uint64_t)(budget ? budget : kWaitBudgetNs), debug);
+  e = cudaLaunchKernelEx(&cfg, pick(what), *reinterpret_cast<const CUtensorMap *>(tmap_hi),
+                         *reinterpret_cast<const CUtensorMap *>(tmap_lo), n, rs, units,
+                         (int32_t)n_units, queue.head, queue.ahead, status, g64, out, order,
+                         (uint64_t)(budget ? budget : kWaitBudgetNs), debug);
+  return e == cudaSuccess ? e : leave_queue(queue, s, e);
 }
 }  // namespace
 
 cudaError_t launch_gram_tc2(const void *tmap_hi, const void *tmap_lo, int64_t n, const double *rs,
-                            const int32_t *units, int64_t n_units, int32_t *queue,
+                            const int32_t *units, int64_t n_units, const UnitQueue &queue,
                             int32_t *status, double *g64, void *out, int coverage, int atomic,
                             uint64_t budget, int32_t debug, cudaStream_t s) {
   return launch(tmap_hi, tmap_lo, n, rs, units, n_units, queue, status, g64, out,
@@ -631,8 +629,8 @@ cudaError_t launch_gram_tc2(const void *tmap_hi, const void *tmap_lo, int64_t n,
 
 cudaError_t launch_gram_tc2_store(const void *tmap_hi, const void *tmap_lo, int64_t n,
                                   const int32_t *units, int64_t n_units, int64_t k_split,
-                                  int32_t *queue, int32_t *status, float *planes, uint64_t budget,
-                                  int32_t debug, cudaStream_t s) {
+                                  const UnitQueue &queue, int32_t *status, float *planes,
+                                  uint64_t budget, int32_t debug, cudaStream_t s) {
   const SplitOrder order{(int32_t)(n_units / k_split), (int32_t)tc2_pairs(), (int32_t)k_split};
   return launch(tmap_hi, tmap_lo, n, nullptr, units, n_units, queue, status, nullptr, planes,
                 kStore, order, budget, debug, s);

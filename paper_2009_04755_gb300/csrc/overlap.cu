@@ -147,7 +147,7 @@ struct Params {
   const int32_t *tiles;
   int64_t n_tiles;
   int64_t n_items;
-  int32_t *queue;
+  int32_t *queue, *ahead;  // this launch's head, one it clears for another (or NULL)
   int32_t *status;
   const int32_t *traits;   // kCloudWide, kCloudWeighted
   int32_t stage_cap;       // points that fit the shared staging buffer (a multiple of 4)
@@ -215,16 +215,10 @@ overlap_kernel(Params P) {
       dst->diag = !P.list_mode && b.x < a.y;
     }
   };
-  // the first tile of a CTA is its index; each later pop takes the next, and
-  // each CTA's last one fails, so that a run makes n_tiles pops: the last
-  // leaves the queue as it was found (with the status word set it does not,
-  // and nothing runs until the host has cleared both)
-  auto pop = [&]() {
-    const int r = atomicAdd(P.queue, 1);
-    if (r == (int)P.n_tiles - 1) *reinterpret_cast<volatile int32_t *>(P.queue) = 0;
-    return r + (int)gridDim.x;
-  };
+  // the first tile of a CTA is its index; each later pop takes the next
+  auto pop = [&]() { return atomicAdd(P.queue, 1) + (int)gridDim.x; };
   if (threadIdx.x == 0) {
+    if (blockIdx.x == 0 && P.ahead) *P.ahead = 0;
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar) : "memory");
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     fetch(s_ctx, blockIdx.x);
@@ -925,7 +919,7 @@ cloud_self_kernel(const float4 *__restrict__ pts, const float *__restrict__ lw,
 }
 
 template <int DIM, int MODE, int SCORE = 0>
-cudaError_t launch_r(const CloudStore &cs, Params &P, cudaStream_t s) {
+cudaError_t launch_r(const CloudStore &cs, const UnitQueue &queue, Params &P, cudaStream_t s) {
   constexpr int kPart = part_size<MODE>();
   P.stage_cap = MODE == COVER ? 0 : (std::min(cs.max_pts, kStagePts) + 3) & ~3;
   P.part_floats = MODE == COVER ? 0 : ((cs.max_rows * cs.max_items * kPart + 3) & ~3);
@@ -955,19 +949,20 @@ cudaError_t launch_r(const CloudStore &cs, Params &P, cudaStream_t s) {
       e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     if (e == cudaSuccess)
       e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, optin);
-    if (e != cudaSuccess) return e;
     int per_sm = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem);
-    if (e != cudaSuccess) return e;
+    if (e == cudaSuccess)
+      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem);
+    if (e != cudaSuccess) return leave_queue(queue, s, e);
     slots = (int64_t)num_sms() * std::max(per_sm, 1);
     cs.fits->push_back({reinterpret_cast<const void *>(kern), smem, threads, slots});
   }
   const int64_t grid = std::min(slots, P.n_tiles);
   kern<<<(int)grid, threads, smem, s>>>(P);
-  return cudaGetLastError();
+  e = cudaGetLastError();
+  return e == cudaSuccess ? e : leave_queue(queue, s, e);
 }
 
-Params base_params(const CloudStore &cs, int32_t *queue, int32_t *status) {
+Params base_params(const CloudStore &cs, const UnitQueue &queue) {
   Params P{};
   P.pts = cs.d_pts;
   P.lw = cs.d_lw;
@@ -978,35 +973,33 @@ Params base_params(const CloudStore &cs, int32_t *queue, int32_t *status) {
   P.tiles = cs.d_tiles;
   P.n_tiles = cs.n_tiles;
   P.n_items = cs.n;
-  P.queue = queue + kQueueClouds;
-  P.status = status;
-  P.traits = queue + kQueueTraits;
+  P.queue = queue.head;
+  P.ahead = queue.ahead;
+  P.status = queue.words + 1;
+  P.traits = queue.words + kQueueTraits;
   P.list_mode = cs.list_mode ? 1 : 0;
   return P;
 }
 
 }  // namespace
 
-// status word lives right after the queue counter (see api.cu)
-static inline int32_t *status_of(int32_t *queue) { return queue + 1; }
-
 cudaError_t launch_overlap(const CloudStore &cs, const float *params, float *out, int coverage,
-                           int32_t *queue, cudaStream_t s) {
-  if (cs.n_tiles <= 0) return cudaSuccess;
-  Params P = base_params(cs, queue, status_of(queue));
+                           const UnitQueue &queue, cudaStream_t s) {
+  if (cs.n_tiles <= 0) return leave_queue(queue, s, cudaSuccess);
+  Params P = base_params(cs, queue);
   P.out = out;
   P.params = params;
   if (coverage)
-    return cs.dim == 3 ? launch_r<3, COVER>(cs, P, s) : launch_r<2, COVER>(cs, P, s);
-  if (params) return launch_r<2, FWD_T>(cs, P, s);
-  return cs.dim == 3 ? launch_r<3, FWD>(cs, P, s) : launch_r<2, FWD>(cs, P, s);
+    return cs.dim == 3 ? launch_r<3, COVER>(cs, queue, P, s) : launch_r<2, COVER>(cs, queue, P, s);
+  if (params) return launch_r<2, FWD_T>(cs, queue, P, s);
+  return cs.dim == 3 ? launch_r<3, FWD>(cs, queue, P, s) : launch_r<2, FWD>(cs, queue, P, s);
 }
 
 cudaError_t launch_score(const CloudStore &cs, int score, const float4 *pts, const float *lw,
-                         const double *self, const float *params, float *out, int32_t *queue,
-                         cudaStream_t s) {
-  if (cs.n_tiles <= 0) return cudaSuccess;
-  Params P = base_params(cs, queue, status_of(queue));
+                         const double *self, const float *params, float *out,
+                         const UnitQueue &queue, cudaStream_t s) {
+  if (cs.n_tiles <= 0) return leave_queue(queue, s, cudaSuccess);
+  Params P = base_params(cs, queue);
   P.pts = pts;
   P.lw = lw;
   P.out = out;
@@ -1015,11 +1008,11 @@ cudaError_t launch_score(const CloudStore &cs, int score, const float4 *pts, con
   P.score_c = score == 1 ? pow(0.6931471805599453 / 3.141592653589793, 0.5 * cs.dim)
                          : pow(8.0 * 0.6931471805599453, 0.5 * cs.dim);
   if (score == 1) {
-    if (params) return launch_r<2, FWD_T, 1>(cs, P, s);
-    return cs.dim == 3 ? launch_r<3, FWD, 1>(cs, P, s) : launch_r<2, FWD, 1>(cs, P, s);
+    if (params) return launch_r<2, FWD_T, 1>(cs, queue, P, s);
+    return cs.dim == 3 ? launch_r<3, FWD, 1>(cs, queue, P, s) : launch_r<2, FWD, 1>(cs, queue, P, s);
   }
-  if (params) return launch_r<2, FWD_T, 2>(cs, P, s);
-  return cs.dim == 3 ? launch_r<3, FWD, 2>(cs, P, s) : launch_r<2, FWD, 2>(cs, P, s);
+  if (params) return launch_r<2, FWD_T, 2>(cs, queue, P, s);
+  return cs.dim == 3 ? launch_r<3, FWD, 2>(cs, queue, P, s) : launch_r<2, FWD, 2>(cs, queue, P, s);
 }
 
 cudaError_t launch_cloud_rescore(const CloudStore &cs, int score, float4 *pts_out, float *lw_out,
@@ -1045,12 +1038,12 @@ cudaError_t launch_cloud_self(const CloudStore &cs, const float4 *pts, const flo
   return cudaGetLastError();
 }
 
-cudaError_t launch_overlap_grad_q(const CloudStore &cs, int32_t *queue, const float *params,
-                                  const float *grad_out, float *grad_params, float *f_out,
-                                  float eta, float fmin, float *params_io, int32_t *flags,
-                                  cudaStream_t s) {
-  if (cs.n_tiles <= 0) return cudaSuccess;
-  Params P = base_params(cs, queue, status_of(queue));
+cudaError_t launch_overlap_grad_q(const CloudStore &cs, const UnitQueue &queue,
+                                  const float *params, const float *grad_out,
+                                  float *grad_params, float *f_out, float eta, float fmin,
+                                  float *params_io, int32_t *flags, cudaStream_t s) {
+  if (cs.n_tiles <= 0) return leave_queue(queue, s, cudaSuccess);
+  Params P = base_params(cs, queue);
   P.params = params;
   P.grad_out = grad_out;
   P.grad_params = grad_params;
@@ -1059,7 +1052,7 @@ cudaError_t launch_overlap_grad_q(const CloudStore &cs, int32_t *queue, const fl
   P.flags = flags;
   P.eta = eta;
   P.fmin = fmin;
-  return launch_r<2, GRAD>(cs, P, s);
+  return launch_r<2, GRAD>(cs, queue, P, s);
 }
 
 cudaError_t launch_cloud_pack(const float *x, const float *y, const float *z, const float *sigma,

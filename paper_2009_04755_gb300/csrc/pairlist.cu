@@ -433,14 +433,16 @@ extern "C" ap_status ap_run_pairs_list(ap_items *it, int32_t fn, int32_t precisi
   }
   CloudStore lc;
   AP_TRY_ST(cloud_list_plan(it, pi, pj, n_pairs, s, lc));
-  if (fn == AP_FN_OVERLAP)
-    AP_TRY(launch_overlap(lc, params, reinterpret_cast<float *>(out), 0, it->d_queue, s));
-  else {
-    const int score = fn == AP_FN_GMM_L2 ? 1 : 2;
-    AP_TRY_ST(ensure_score_storage(it, score, s));
+  const int score = fn == AP_FN_GMM_L2 ? 1 : 2;
+  if (fn != AP_FN_OVERLAP) AP_TRY_ST(ensure_score_storage(it, score, s));
+  UnitQueue q;
+  AP_TRY(take_queue(it, s, &q));
+  if (fn == AP_FN_OVERLAP) {
+    AP_TRY(launch_overlap(lc, params, reinterpret_cast<float *>(out), 0, q, s));
+  } else {
     const CloudStore &c = it->cl;
     AP_TRY(launch_score(lc, score, c.d_pts_score[score - 1], c.d_lw_score[score - 1], c.d_self,
-                        params, reinterpret_cast<float *>(out), it->d_queue, s));
+                        params, reinterpret_cast<float *>(out), q, s));
   }
   return AP_OK;
 }
@@ -457,8 +459,10 @@ extern "C" ap_status ap_backward_list(ap_items *it, const int32_t *pi, const int
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   CloudStore lc;
   AP_TRY_ST(cloud_list_plan(it, pi, pj, n_pairs, s, lc));
-  AP_TRY(launch_overlap_grad_q(lc, it->d_queue, params, grad_out, grad_params, f_out, 0.f, 0.f,
-                               nullptr, nullptr, s));
+  UnitQueue q;
+  AP_TRY(take_queue(it, s, &q));
+  AP_TRY(launch_overlap_grad_q(lc, q, params, grad_out, grad_params, f_out, 0.f, 0.f, nullptr,
+                               nullptr, s));
   return AP_OK;
 }
 
@@ -473,8 +477,11 @@ extern "C" ap_status ap_ascent_list(ap_items *it, const int32_t *pi, const int32
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   CloudStore lc;
   AP_TRY_ST(cloud_list_plan(it, pi, pj, n_pairs, s, lc));
-  for (int32_t k = 0; k < n_steps; ++k)
-    AP_TRY(launch_overlap_grad_q(lc, it->d_queue, nullptr, nullptr, nullptr, f_out, eta, fmin,
-                                 params, flags, s));
+  for (int32_t k = 0; k < n_steps; ++k) {
+    UnitQueue q;
+    AP_TRY(take_queue(it, s, &q));
+    AP_TRY(launch_overlap_grad_q(lc, q, nullptr, nullptr, nullptr, f_out, eta, fmin, params, flags,
+                                 s));
+  }
   return AP_OK;
 }

@@ -378,9 +378,11 @@ static ap_status alloc_slices(VecStore &v) {
 static ap_status run_slices(ap_items *it, void *out, int coverage, cudaStream_t s) {
   VecStore &v = it->vec;
   const int64_t P = v.n * (v.n - 1) / 2;
+  UnitQueue q;
   if (coverage) {
+    AP_TRY(take_queue(it, s, &q));
     AP_TRY(launch_gram_tc2(v.tmap_slice_hi[0], v.tmap_slice_lo[0], v.n, v.d_rs, v.d_slice_cover,
-                           v.n_slice_cover, it->d_queue, it->d_status, v.d_g64, out, 1, 0,
+                           v.n_slice_cover, q, it->d_status, v.d_g64, out, 1, 0,
                            it->wait_budget_ns, it->debug, s));
     it->stats.tiles = v.n_slice_cover;
     it->stats.item_loads = 0;
@@ -444,8 +446,9 @@ static ap_status run_slices(ap_items *it, void *out, int coverage, cudaStream_t 
     AP_TRY(cudaEventRecord(v.ev_slice_ready[b], it->prep_stream));
     AP_TRY(cudaStreamWaitEvent(s, v.ev_slice_ready[b], 0));
     const int t_gram = tr.begin(0, AP_STAGE_GRAM, c, 0, s);
+    AP_TRY(take_queue(it, s, &q));
     AP_TRY(launch_gram_tc2(v.tmap_slice_hi[b], v.tmap_slice_lo[b], v.n, v.d_rs, v.d_slice_units,
-                           v.n_slice_units, it->d_queue, it->d_status, v.d_g64, out, 0, 1,
+                           v.n_slice_units, q, it->d_status, v.d_g64, out, 0, 1,
                            it->wait_budget_ns, it->debug, s));
     tr.end(t_gram, s);
     AP_TRY(cudaEventRecord(v.ev_slice_done[b], s));
@@ -790,9 +793,11 @@ ap_status stream_load_and_run(ap_items *it, const float *h, double *out, cudaStr
         AP_TRY(cudaStreamWaitEvent(s, v.ev_prepped[b], 0));
         const auto &uc = v.stream_cols[(size_t)(c * M + m)];
         const int t_gram = tr.begin(0, AP_STAGE_GRAM, seq, 0, s);
+        UnitQueue q;
+        AP_TRY(take_queue(it, s, &q));
         AP_TRY(launch_gram_tc2(v.tmap_hi, v.tmap_lo, v.n, v.d_rs,
                                v.d_stream_units + uc.first * kOocTileInts, uc.second,
-                               it->d_queue, it->d_status, v.d_g64, out, 0, 1, it->wait_budget_ns,
+                               q, it->d_status, v.d_g64, out, 0, 1, it->wait_budget_ns,
                                it->debug, s));
         tr.end(t_gram, s);
       }
@@ -832,10 +837,12 @@ ap_status stream_load_and_run(ap_items *it, const float *h, double *out, cudaStr
     v.ring_used[b] = 1;
     AP_TRY(cudaStreamWaitEvent(s, v.ev_prepped[b], 0));
     const int t_gram = tr.begin(0, AP_STAGE_GRAM, (int64_t)m, 0, s);
+    UnitQueue q;
+    AP_TRY(take_queue(it, s, &q));
     AP_TRY(launch_gram_tc2(v.tmap_hi, v.tmap_lo, v.n, v.d_rs,
                            v.d_stream_units + v.stream_cols[m].first * kOocTileInts,
-                           v.stream_cols[m].second, it->d_queue, it->d_status, v.d_g64, out, 0,
-                           1, it->wait_budget_ns, it->debug, s));
+                           v.stream_cols[m].second, q, it->d_status, v.d_g64, out, 0, 1,
+                           it->wait_budget_ns, it->debug, s));
     tr.end(t_gram, s);
   }
   const int t_fin = tr.begin(0, AP_STAGE_FINALIZE, 0, 0, s);

@@ -326,9 +326,12 @@ extern "C" ap_status ap_tune(ap_items *it, int32_t mode, void *stream, ap_plan *
         st = upload_cloud_plan(cand, plan, s);
         if (st != AP_OK) break;
         auto launch = [&]() {
-          return mode == 0 ? launch_overlap(cand, nullptr, d_out, 0, it->d_queue, s)
-                           : launch_overlap_grad_q(cand, it->d_queue, nullptr, nullptr, d_g, d_out,
-                                                   0.f, 0.f, nullptr, nullptr, s);
+          UnitQueue q;
+          const cudaError_t taken = take_queue(it, s, &q);
+          if (taken != cudaSuccess) return taken;
+          return mode == 0 ? launch_overlap(cand, nullptr, d_out, 0, q, s)
+                           : launch_overlap_grad_q(cand, q, nullptr, nullptr, d_g, d_out, 0.f, 0.f,
+                                                   nullptr, nullptr, s);
         };
         float ms_best = 1e30f;
         e = launch();

@@ -128,3 +128,41 @@ def test_new_plans_are_there_for_every_stream(ap):
         it.run_pairs(out=out)
         torch.testing.assert_close(out, ref, rtol=1e-6, atol=0)
         assert it.last_device_error() == 0
+
+
+def test_runs_that_overlap_spoil_no_later_run(ap):
+    """Runs of one handle on two streams at once, of unequal numbers of tiles
+    (which programs should not do: the header says so): later runs are whole,
+    more of them than there are queue heads, and so is a replayed capture."""
+    c = synth.clouds_uniform(n=150, dim=2, size=(5, 60), seed=6)
+    pi, pj = np.triu_indices(150, 1)
+    a, b = torch.cuda.Stream(), torch.cuda.Stream()
+    with ap.Items.from_clouds(c) as it:
+        ref = it.run_pairs()
+        one, x, y = torch.empty_like(ref), torch.empty_like(ref), torch.zeros_like(ref)
+        torch.cuda.synchronize()
+        for _ in range(40):
+            it.run_pairs(out=x, stream=a)
+            it.run_pairs(out=y, stream=b)
+            it.run_pairs_list(pi[:777], pj[:777], out=one, stream=b)
+            it.run_pairs(out=x, stream=a)
+        torch.cuda.synchronize()
+        for _ in range(150):
+            x.zero_()
+            it.run_pairs(out=x)
+            assert torch.equal(x, ref)
+        p0 = torch.zeros(len(pi), 3, device="cuda")
+        p1, f1, _ = it.ascent(p0.clone(), 5, 1e-3)
+        p2, f2 = p0.clone(), None
+        for _ in range(5):                       # odd numbers of steps: the heads alternate
+            p2, f2, _ = it.ascent(p2, 1, 1e-3)
+        assert torch.equal(p1, p2) and torch.equal(f1, f2)
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g):
+            it.run_pairs(out=x)
+            it.run_pairs(out=y)
+        for _ in range(3):
+            x.zero_(), y.zero_()
+            g.replay()
+            assert torch.equal(x, ref) and torch.equal(y, ref)
+        assert it.last_device_error() == 0

@@ -460,11 +460,11 @@ cudaError_t launch_vec_mean(const float *X, int64_t n, int64_t D, int64_t ld, do
 // evenly spread samples), then the centred split / FP32 copies and the FP64
 // sums of c and c^2 in one pass, then delta = mean - shift, ss and rs; rows
 // whose shift missed the mean by D delta^2 > ss / 64 are redone from the
-// exact mean.
-cudaError_t launch_vec_prep(const float *X, int64_t row0, int64_t out_row0, int64_t n, int64_t D,
-                            int64_t ld, int64_t Dp, __nv_bfloat16 *hi, __nv_bfloat16 *lo,
-                            float *c32, double *shift, double *delta, double *ss, double *rs,
-                            cudaStream_t s);
+// exact mean.  set_rows: the rows of the whole set (see prep_cluster).
+cudaError_t launch_vec_prep(const float *X, int64_t row0, int64_t out_row0, int64_t n,
+                            int64_t set_rows, int64_t D, int64_t ld, int64_t Dp,
+                            __nv_bfloat16 *hi, __nv_bfloat16 *lo, float *c32, double *shift,
+                            double *delta, double *ss, double *rs, cudaStream_t s);
 // out[p] -= (D delta_i rs_i)(delta_j rs_j) over the packed triangle: the
 // mean correction of pairs the Gram kernel already scaled by rs_i rs_j
 cudaError_t launch_pair_correct(double *out, const double *rs, const double *delta, int64_t n,

@@ -275,7 +275,7 @@ ap_status vec_load(ap_items *it, const float *data, int on_host, cudaStream_t s)
   const bool split = (v.precisions & (1u << AP_PREC_SPLIT_BF16)) != 0;
   const bool f32 = (v.precisions & (1u << AP_PREC_FP32)) != 0;
   if (!on_host) {
-    AP_TRY(launch_vec_prep(data, 0, 0, v.n, v.D, v.ld, v.Dp, split ? v.d_hi : nullptr,
+    AP_TRY(launch_vec_prep(data, 0, 0, v.n, v.n, v.D, v.ld, v.Dp, split ? v.d_hi : nullptr,
                            split ? v.d_lo : nullptr, f32 ? v.d_c32 : nullptr, v.d_mu,
                            v.d_delta_all, v.d_ss, v.d_rs, s));
     return AP_OK;
@@ -304,9 +304,9 @@ ap_status vec_load(ap_items *it, const float *data, int on_host, cudaStream_t s)
     if (e == cudaSuccess) e = cudaEventRecord(copied[b], it->copy_stream);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(s, copied[b], 0);
     if (e == cudaSuccess)
-      e = launch_vec_prep(stage, r0, r0, nr, v.D, v.ld, v.Dp, split ? v.d_hi : nullptr,
+      e = launch_vec_prep(stage, r0, r0, nr, v.n, v.D, v.ld, v.Dp, split ? v.d_hi : nullptr,
                           split ? v.d_lo : nullptr, f32 ? v.d_c32 : nullptr, v.d_mu,
-                           v.d_delta_all, v.d_ss, v.d_rs, s);
+                          v.d_delta_all, v.d_ss, v.d_rs, s);
     if (e == cudaSuccess) e = cudaEventRecord(done[b], s);
   }
   if (e != cudaSuccess) st = from_cuda(e);

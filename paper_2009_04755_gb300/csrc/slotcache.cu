@@ -538,7 +538,7 @@ ap_status run_out_of_core(ap_items *it, void *out, int coverage, cudaStream_t s)
         AP_TRY(cudaEventRecord(v.ev_raw_ready[b], it->copy_stream));
         AP_TRY(cudaStreamWaitEvent(s, v.ev_raw_ready[b], 0));
         const size_t slot_off = (size_t)slot * kMacro * v.Dp;
-        AP_TRY(launch_vec_prep(raw, r0, 0, rows, v.D, v.ld, v.Dp, v.d_pool_hi + slot_off,
+        AP_TRY(launch_vec_prep(raw, r0, 0, rows, v.n, v.D, v.ld, v.Dp, v.d_pool_hi + slot_off,
                                v.d_pool_lo + slot_off, nullptr, v.d_mu, v.d_delta_all, v.d_ss,
                                v.d_rs, s));
         AP_TRY(cudaEventRecord(v.ev_raw_free[b], s));
@@ -828,7 +828,7 @@ ap_status stream_load_and_run(ap_items *it, const float *h, double *out, cudaStr
     AP_TRY(cudaEventRecord(v.ev_raw_ready[b], it->copy_stream));
     AP_TRY(cudaStreamWaitEvent(it->prep_stream, v.ev_raw_ready[b], 0));
     const int t_prep = tr.begin(2, AP_STAGE_PREPROCESS, (int64_t)m, 0, it->prep_stream);
-    AP_TRY(launch_vec_prep(raw, r0, r0, rows, v.D, v.ld, v.Dp, split ? v.d_hi : nullptr,
+    AP_TRY(launch_vec_prep(raw, r0, r0, rows, v.n, v.D, v.ld, v.Dp, split ? v.d_hi : nullptr,
                            split ? v.d_lo : nullptr, f32 ? v.d_c32 : nullptr, v.d_mu,
                            v.d_delta_all, v.d_ss, v.d_rs, it->prep_stream));
     tr.end(t_prep, it->prep_stream);

@@ -732,7 +732,9 @@ cudaError_t launch_vec_split_cols(const float *X, int64_t row0, int64_t n, int64
 // CTAs per row, a power of two, at most eight: as many as give every SM its
 // four, while each keeps 2048 columns; and eight of a row so long that each
 // still has 65,536 (4096 x 2^20: 5.47 ms with eight, 6.31 with one, whose writes
-// meet 608 rows at once; 1000 x 50,000: 88 us with one, 97 with two)
+// meet 608 rows at once; 1000 x 50,000: 88 us with one, 97 with two).  n are the
+// rows of the set, not of a launch: a row's sums come in the same order, and so
+// have the same bits, from the device at once and from the host in pieces.
 int prep_cluster(int64_t n, int64_t Dp) {
   int c = 1;
   while (c < 8 && ((n * c < 4 * (int64_t)num_sms() && Dp / (2 * c) >= 2048) ||
@@ -741,12 +743,12 @@ int prep_cluster(int64_t n, int64_t Dp) {
   return c;
 }
 
-cudaError_t launch_vec_prep(const float *X, int64_t row0, int64_t out_row0, int64_t n, int64_t D,
-                            int64_t ld, int64_t Dp, __nv_bfloat16 *hi, __nv_bfloat16 *lo,
-                            float *c32, double *shift, double *delta, double *ss, double *rs,
-                            cudaStream_t s) {
+cudaError_t launch_vec_prep(const float *X, int64_t row0, int64_t out_row0, int64_t n,
+                            int64_t set_rows, int64_t D, int64_t ld, int64_t Dp,
+                            __nv_bfloat16 *hi, __nv_bfloat16 *lo, float *c32, double *shift,
+                            double *delta, double *ss, double *rs, cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
-  const int c = prep_cluster(n, Dp);
+  const int c = prep_cluster(set_rows, Dp);
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(std::min<int64_t>(n, 1 << 24) * c), 1, 1);
   cfg.blockDim = dim3(kSplitThreads, 1, 1);

@@ -82,6 +82,19 @@ def test_pearson_host_source_equals_device_source(ap):
     assert np.array_equal(a, b)
 
 
+def test_pearson_host_source_in_pieces_equals_device_source(ap):
+    """671 rows of 100,000 fill a staging buffer: the 29 of the second piece
+    are summed as the set's others are."""
+    n, D = 700, 100_000
+    X = synth.vectors_grouped(n, D, seed=5, device="cuda")
+    Xh = X.cpu().pin_memory()
+    with ap.Items.from_vectors(X) as a, ap.Items.from_vectors(Xh) as b:
+        ra, rb = a.run_pairs(), b.run_pairs()
+        assert torch.equal(ra, rb)
+        a.update(Xh)
+        assert torch.equal(a.run_pairs(), rb)
+
+
 def test_pearson_update_items_reuses_storage(ap, oracle_lib):
     n, D = 150, 512
     X1 = synth.vectors_grouped(n, D, seed=1)

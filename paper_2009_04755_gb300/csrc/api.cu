@@ -114,16 +114,25 @@ CloudPlanChoice choose_cloud_plan(const CloudStore &c) {
   // original order to know which item of a pair is moved)
   ch.sorted = (c.dim == 3) && mx > 4 * std::max<int64_t>(mn, 1);
   ch.reg_r = 4;
-  // blocks of about 1/60 of the points: 1800 tiles, 12 per SM before the last
-  // ones are split (256 clouds of 64-128 points: 420 points a block 126 us, 256
-  // 140, 768 134); at least 384, below which a small set's launch is all tiles
-  // (48 clouds of 20-60 points: 8.2 us with 384, 10.2 with 64); at most
-  // kCloudBlockPts, which one staging window holds.  Eight items at most: more would take shared memory for their
-  // partial sums from the CTAs.
+  // Blocks of about 1/60 of the points: 1800 tiles, 12 per SM before the last ones
+  // are split (256 clouds of 64-128 points: 420 points a block 126 us, 256 140,
+  // 768 134); at least 384, below which a small set's launch is all tiles (48
+  // clouds of 20-60 points: 8.2 us with 384, 10.2 with 64); at most kCloudBlockPts,
+  // which one staging window holds.
   constexpr int64_t kCloudBlockPts = 2048;
   const int64_t want = (c.total_pts / 60 + 3) / 4 * 4;
   ch.block_pts = (int32_t)std::min(std::max<int64_t>(want, 384), kCloudBlockPts);
-  ch.block_items = 8;
+  // Items of a block: 8, and twice as many while whole blocks of them make more
+  // than kMostTiles tiles.  Sets of few small clouds run best in eights (700 of 20
+  // points 88 us, in sixteens 93; 32 of them 6.2 us, 8.0); those of many spend their
+  // time on tiles (1000 of 20 points 160 us, in sixteens 156; 2400 832 us in
+  // eights, 745 in thirty-twos; 20,000 56.5 ms and a list of 3.1 million tiles, 47.2
+  // ms and 0.2 million).
+  constexpr int64_t kMostTiles = 6000;
+  for (ch.block_items = 8; ch.block_items < kOverlapMaxBlockItems; ch.block_items *= 2) {
+    const int64_t nb = (c.n + ch.block_items - 1) / ch.block_items;
+    if (nb * (nb + 1) / 2 <= kMostTiles) break;
+  }
   return ch;
 }
 

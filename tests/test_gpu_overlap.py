@@ -279,3 +279,16 @@ def test_clouds_moved_onto_the_padding(ap, plan):
         p, f, flags = it.ascent(onto.clone(), 3, 1e-2)
         assert torch.all(f == 0) and torch.all(flags == 1) and torch.equal(p, onto)
         assert it.last_device_error() == 0
+
+
+@pytest.mark.parametrize("n,items,tiles", [(700, 8, 8000), (1200, 16, 12_000), (5000, 32, 32_000)])
+def test_tiles_of_many_small_clouds(ap, n, items, tiles):
+    """Blocks take more items as sets of small clouds grow, so that the list
+    of tiles grows with the pairs' work and not with the square of the eighths."""
+    c = synth.clouds_uniform(n=n, dim=2, size=(2, 6), seed=n)
+    with ap.Items.from_clouds(c) as it:
+        assert it.plan()["block_items"] == items and it.stats()["tiles"] < tiles
+        assert torch.all(it.run_pairs(ap.AP_FN_COVERAGE) == 1)
+        f = it.run_pairs()
+        it.set_plan(8, 384, 4)
+        assert torch.equal(it.run_pairs(), f)

@@ -858,8 +858,14 @@ __global__ void cloud_rescore_kernel(const float4 *__restrict__ pts, const float
     float2 s2k = dim == 3 ? make_float2(q.z, q.w) : make_float2(q.x, q.y);   // padding: -1
     float2 l = dim == 3 ? l2[k] : make_float2(q.z, q.w);
     if (score == 2) {
-      l.x = 0.5f * l.x + 0.25f * (float)dim * __log2f(-s2k.x / ln2x2);
-      l.y = 0.5f * l.y + 0.25f * (float)dim * __log2f(-s2k.y / ln2x2);
+      // log2 of the mantissa and the exponent apart: one rounding of the size of l
+      auto half = [&](float lw, float s) {
+        int e;
+        const float m = frexpf(-s / ln2x2, &e), d4 = 0.25f * (float)dim;
+        return fmaf(d4, (float)e, fmaf(d4, log2f(m), 0.5f * lw));
+      };
+      l.x = half(l.x, s2k.x);
+      l.y = half(l.y, s2k.y);
     }
     const float f = (score == 2 ? 2.f : 1.f) * (dim == 3 ? -1.f : 1.f);
     s2k.x *= f;

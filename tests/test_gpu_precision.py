@@ -47,3 +47,49 @@ def test_few_points_take_a_reciprocal_each(ap, dim, weights):
     few = torch.from_numpy((sizes[pi] <= 8) & (sizes[pj] <= 8)).cuda()
     many = torch.from_numpy((sizes[pi] > 8) & (sizes[pj] > 8)).cuda()
     assert torch.equal(f[few], g[few]) and not torch.equal(f[many], g[many])
+
+
+def _pairs64(c, fn):
+    """The cost of every pair (no transforms) in 64 bits, plain torch."""
+    off, dim = c["offsets"], c["dim"]
+    n = len(off) - 1
+    x = torch.stack([torch.from_numpy(c[k]).cuda().double() for k in "xyz"[:dim]], 1)
+    s = torch.from_numpy(c["sigma"]).cuda().double()
+    w = torch.ones_like(s) if c["weight"] is None else torch.from_numpy(c["weight"]).cuda().double()
+    item = torch.repeat_interleave(torch.arange(n, device="cuda"),
+                                   torch.from_numpy(np.diff(off)).cuda())
+    out = torch.zeros(n, n, dtype=torch.float64, device="cuda")
+    for i in range(n - 1):
+        a = slice(int(off[i]), int(off[i + 1]))
+        for b0 in range(int(off[i + 1]), len(s), 1 << 16):
+            b = slice(b0, min(len(s), b0 + (1 << 16)))
+            s2 = s[a, None] ** 2 + s[b][None] ** 2
+            d2 = sum((x[a, k][:, None] - x[b, k][None]) ** 2 for k in range(dim))
+            if fn == "overlap":
+                t = torch.exp(-d2 / (2 * s2)) * w[a, None] * w[b][None]
+            else:
+                t = ((2 * s[a, None] * s[b][None] / s2) ** (dim / 2) * torch.exp(-d2 / (4 * s2))
+                     * (w[a, None] * w[b][None]).sqrt())
+            out[i].index_add_(0, item[b], t.sum(0))
+    pi, pj = torch.triu_indices(n, n, 1, device="cuda")
+    return out[pi, pj]
+
+
+def _off(f, ref):
+    f = f.double()
+    return (float((f - ref).norm() / ref.norm()),                 # in the 2-norm
+            float(((f - ref) / ref).pow(2).mean().sqrt()))        # relative, rms
+
+
+@pytest.mark.parametrize("dim", [2, 3])
+@pytest.mark.parametrize("weights", [False, True])
+def test_bhattacharyya_log_weights_are_rounded_once(ap, dim, weights):
+    """A term's two log-weights carry one rounding each of an ulp of theirs
+    (uniform: 12^-0.5 of it rms), times ln 2, beside the terms' own 1e-7."""
+    c = _clouds(np.full(60, 100), dim, 2, 0.1, (0.02, 0.05), weights)
+    with ap.Items.from_clouds(c) as it:
+        f = it.run_pairs(ap.AP_FN_BHATTACHARYYA)
+    l = 0.25 * dim * np.log2(c["sigma"].astype(np.float64) ** 2)
+    ulp = 2.0 ** (np.floor(np.log2(np.abs(l).max())) - 23)
+    bound = np.log(2) * np.sqrt(2.0) * ulp / np.sqrt(12.0) + 1e-7
+    assert _off(f, _pairs64(c, "bhattacharyya"))[1] < bound

@@ -167,9 +167,10 @@ struct Params {
   double score_c;          // SCORE 1, 2: the constant C
 };
 
-// floats of one partial sum: the adjoint's f and three components, or f in two
+// floats of one partial sum: f in two, the first and the last, and the adjoint's
+// three components
 template <int MODE>
-constexpr int part_size() { return MODE == GRAD ? 4 : 2; }
+constexpr int part_size() { return MODE == GRAD ? 5 : 2; }
 
 // CTAs of four warps per SM that the registers must allow
 template <int MODE>
@@ -187,7 +188,9 @@ template <int DIM, int MODE, int R, int SCORE, bool BOX>
 __global__ void __launch_bounds__(kThreads, min_ctas<MODE>())
 overlap_kernel(Params P) {
   constexpr int NV = (MODE == GRAD) ? 4 : 1;     // partial values per (row, j)
-  constexpr bool kTwo = MODE != GRAD;            // f as a sum of two floats
+  // a-points that a sum of f spans before it is held in two floats (as points, so
+  // that a piece of up to 32 has the same bits whatever lanes it sits on)
+  constexpr int kTwoFrom = MODE == GRAD ? 32 : 0;
   constexpr int kPart = part_size<MODE>();       // floats per (row, j)
   constexpr int kUnroll = DIM == 3 ? 2 : 4;
   constexpr bool kRsq = SCORE != 0 && DIM == 3;  // terms need q^3: rsqrt, not a reciprocal
@@ -511,11 +514,13 @@ overlap_kernel(Params P) {
         // carried as an unevaluated sum of two floats, which more than makes
         // up for them (256 clouds: 4.9e-8 off in the 2-norm, 5.9e-8 with plain
         // sums and a reciprocal each); 3% of a pass of 64-128 points, less of
-        // larger items.
+        // larger items.  The adjoint's f is so from 32 points on, which makes up
+        // for a fragment of 128 where 64 used to meet in FP64 (150 points: 5.9e-8,
+        // 6.8e-8 with plain sums, 6.2e-8 with those of 64); 1.5% of an ascent step.
         float s[NV][RE], lo[RE];
 #pragma unroll
         for (int r = 0; r < RE; ++r) {
-          if (kTwo) {
+          if (kTwoFrom == 0) {
             const float2 h = two_sum(pF[r].x, pF[r].y);
             s[0][r] = __fmul_rn(aw[r], h.x);
             lo[r] = __fmaf_rn(aw[r], __fadd_rn(h.y, __fadd_rn(pC[r].x, pC[r].y)),
@@ -533,10 +538,6 @@ overlap_kernel(Params P) {
           }
         }
         auto add2 = [](float &h, float &l, float h2, float l2) {
-          if (!kTwo) {
-            h = __fadd_rn(h, h2);
-            return;
-          }
           const float2 t = two_sum(h, h2);
           h = t.x;
           l = __fadd_rn(t.y, __fadd_rn(l, l2));
@@ -545,7 +546,8 @@ overlap_kernel(Params P) {
         for (int o = 1; o < RE; o <<= 1) {
 #pragma unroll
           for (int r = 0; r < RE; r += 2 * o) {
-            add2(s[0][r], lo[r], s[0][r + o], lo[r + o]);
+            if (kTwoFrom == 0) add2(s[0][r], lo[r], s[0][r + o], lo[r + o]);
+            else s[0][r] = __fadd_rn(s[0][r], s[0][r + o]);
 #pragma unroll
             for (int q = 1; q < NV; ++q) s[q][r] = __fadd_rn(s[q][r], s[q][r + o]);
           }
@@ -557,8 +559,13 @@ overlap_kernel(Params P) {
         for (int o = 1; o < 32; o <<= 1) {
           const bool in = t + o < len;
           const float fh = __shfl_down_sync(0xffffffffu, v[0], o);
-          const float fl = kTwo ? __shfl_down_sync(0xffffffffu, vl, o) : 0.f;
-          if (in) add2(v[0], vl, fh, fl);
+          if (o * RE >= kTwoFrom) {
+            const float fl =
+                o * RE > kTwoFrom || kTwoFrom == 0 ? __shfl_down_sync(0xffffffffu, vl, o) : 0.f;
+            if (in) add2(v[0], vl, fh, fl);
+          } else if (in) {
+            v[0] = __fadd_rn(v[0], fh);
+          }
 #pragma unroll
           for (int q = 1; q < NV; ++q) {
             const float x = __shfl_down_sync(0xffffffffu, v[q], o);
@@ -568,13 +575,13 @@ overlap_kernel(Params P) {
         if (active && t == 0) {
           float *dst = s_part + ((size_t)row * nJ + jl) * kPart;
           if (w0) {
-            add2(v[0], vl, dst[0], kTwo ? dst[kPart - 1] : 0.f);
+            add2(v[0], vl, dst[0], dst[kPart - 1]);
 #pragma unroll
             for (int q = 1; q < NV; ++q) v[q] = __fadd_rn(v[q], dst[q]);
           }
 #pragma unroll
           for (int q = 0; q < NV; ++q) dst[q] = v[q];
-          if (kTwo) dst[kPart - 1] = vl;
+          dst[kPart - 1] = vl;
         }
       };
 
@@ -618,7 +625,7 @@ overlap_kernel(Params P) {
       const int r0 = c.job0 >= 0 ? mi.w : 0, r1 = r0 + cloud_rows(mi.y, R);
       for (int row = r0; row < r1; ++row) {
         const float *src = s_part + ((size_t)row * nJ + jl) * kPart;
-        sF += kTwo ? (double)src[0] + (double)src[kPart - 1] : (double)src[0];
+        sF += (double)src[0] + (double)src[kPart - 1];
         if (MODE == GRAD) { sX += (double)src[1]; sY += (double)src[2]; sT += (double)src[3]; }
       }
       if (MODE == FWD || MODE == FWD_T) {

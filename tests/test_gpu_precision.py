@@ -93,3 +93,36 @@ def test_bhattacharyya_log_weights_are_rounded_once(ap, dim, weights):
     ulp = 2.0 ** (np.floor(np.log2(np.abs(l).max())) - 23)
     bound = np.log(2) * np.sqrt(2.0) * ulp / np.sqrt(12.0) + 1e-7
     assert _off(f, _pairs64(c, "bhattacharyya"))[1] < bound
+
+
+def _pose64(c, params):
+    """f and df/d(theta, tx, ty) of every pair under its transform, 64 bits."""
+    off, P = c["offsets"], params.double()
+    n = len(off) - 1
+    x, y, s = (torch.from_numpy(c[k]).cuda().double() for k in ("x", "y", "sigma"))
+    f, g = [], []
+    for p, (i, j) in enumerate(zip(*np.triu_indices(n, 1))):
+        a, b = slice(int(off[i]), int(off[i + 1])), slice(int(off[j]), int(off[j + 1]))
+        co, si = torch.cos(P[p, 0]), torch.sin(P[p, 0])
+        rx, ry = co * x[b] - si * y[b], si * x[b] + co * y[b]
+        dx, dy = x[a, None] - (rx + P[p, 1])[None], y[a, None] - (ry + P[p, 2])[None]
+        s2 = s[a, None] ** 2 + s[b][None] ** 2
+        e = torch.exp(-(dx * dx + dy * dy) / (2 * s2))
+        gx, gy = (e / s2 * dx).sum(0), (e / s2 * dy).sum(0)
+        f.append(e.sum())
+        g.append(torch.stack([(gy * rx - gx * ry).sum(), gx.sum(), gy.sum()]))
+    return torch.stack(f), torch.stack(g)
+
+
+def test_adjoint_cost_is_as_close_as_the_cost(ap):
+    """The adjoint's f sums 32 points in FP32 (five roundings, each of its
+    level's share: 0.6 of a last one's 2^-24 / 3^0.5, beside the 5.6e-8 of the
+    terms and of the result) and what follows in two floats."""
+    c = _clouds(np.full(48, 150), 2, 3, 0.5, (0.02, 0.05))
+    params = torch.randn(48 * 47 // 2, 3, generator=torch.Generator("cuda").manual_seed(3),
+                         device="cuda") * 0.1
+    with ap.Items.from_clouds(c) as it:
+        f = it.run_pairs(params=params)
+        _, fb = it.backward(params=params)
+    ref, _ = _pose64(c, params)
+    assert _off(fb, ref)[1] < np.hypot(_off(f, ref)[1], 0.6 * 2.0 ** -24 / np.sqrt(3.0))

@@ -191,6 +191,11 @@ overlap_kernel(Params P) {
   // a-points that a sum of f spans before it is held in two floats (as points, so
   // that a piece of up to 32 has the same bits whatever lanes it sits on)
   constexpr int kTwoFrom = MODE == GRAD ? 32 : 0;
+  // Where neighbours are stored together, the adjoint's terms of one sign follow
+  // one another and cancel late, so they are summed by blocks first (2-norm of the
+  // gradient's error at 1500 points: 1.4e-7, 2.4e-7 in one sum, 1.75e-7 in one sum
+  // over points as given).
+  constexpr bool kBlockwise = MODE == GRAD && BOX;
   constexpr int kPart = part_size<MODE>();       // floats per (row, j)
   constexpr int kUnroll = DIM == 3 ? 2 : 4;
   constexpr bool kRsq = SCORE != 0 && DIM == 3;  // terms need q^3: rsqrt, not a reciprocal
@@ -362,10 +367,14 @@ overlap_kernel(Params P) {
         }
         // the sweep over item j: each packed operation takes two b-points
         // against one a-point held in both halves
+        float uY[RE], uT[RE];                    // kBlockwise: pY, pT of the blocks before
         const float2 z2 = make_float2(0.f, 0.f);
         float2 pF[RE], pC[RE], pY[RE], pT[RE];
 #pragma unroll
-        for (int r = 0; r < RE; ++r) { pF[r] = z2; pC[r] = z2; pY[r] = z2; pT[r] = z2; }
+        for (int r = 0; r < RE; ++r) {
+          pF[r] = z2; pC[r] = z2; pY[r] = z2; pT[r] = z2;
+          uY[r] = uT[r] = 0.f;
+        }
         const int4 qr = s_j[jl];
         // Boxes: the lane's a-points that weigh anything, then the warp's, as
         // the sweep holds them (negated); b - a' is fl(b + (-a')), and rounding
@@ -484,6 +493,12 @@ overlap_kernel(Params P) {
               const float2 tk = __fadd2_rn(pF[r], yk);
               pC[r] = __fadd2_rn(yk, __ffma2_rn(tk, make_float2(-1.f, -1.f), pF[r]));
               pF[r] = tk;
+              if (kBlockwise) {
+                uY[r] = __fadd_rn(uY[r], __fadd_rn(pY[r].x, pY[r].y));
+                uT[r] = __fadd_rn(uT[r], __fadd_rn(pT[r].x, pT[r].y));
+                pY[r] = z2;
+                pT[r] = z2;
+              }
             }
           };
           if (BOX) {
@@ -530,7 +545,8 @@ overlap_kernel(Params P) {
             lo[r] = 0.f;
           }
           if (MODE == GRAD) {
-            const float gx = __fadd_rn(pY[r].x, pY[r].y), gy = __fadd_rn(pT[r].x, pT[r].y);
+            const float gx = kBlockwise ? uY[r] : __fadd_rn(pY[r].x, pY[r].y);
+            const float gy = kBlockwise ? uT[r] : __fadd_rn(pT[r].x, pT[r].y);
             s[NV > 1 ? 1 : 0][r] = __fmul_rn(aw[r], gx);
             s[NV > 2 ? 2 : 0][r] = __fmul_rn(aw[r], gy);
             s[NV > 3 ? 3 : 0][r] =

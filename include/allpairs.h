@@ -170,8 +170,10 @@ typedef struct ap_run_stats {
 } ap_run_stats;
 
 /* Tile plan of a point-cloud set: blocks of at most block_items items and
- * block_pts padded points (a tile stages one block in shared memory, 2048
- * points at a time), reg_r a-points held per lane.  sorted = items
+ * min(block_pts, 2048) padded points, which a tile stages in shared memory (a
+ * larger item is a block by itself, staged 2048 points at a time), reg_r
+ * a-points held per lane.  A pair has the same bits in every plan of the same
+ * reg_r.  sorted = items
  * stored largest first (decided at creation).  rate = point pairs per second
  * the tuner measured for the chosen plan. */
 typedef struct ap_plan {

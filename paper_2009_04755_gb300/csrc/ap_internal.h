@@ -436,7 +436,8 @@ void make_blocks(const std::vector<int64_t> &poff, const std::vector<int64_t> &c
 // jobs, and the tiles in the order they are popped, the last split_tail of
 // them split into one tile per item of J
 void make_cloud_plan(const std::vector<int64_t> &poff, const std::vector<int64_t> &cnt,
-                     const std::vector<int32_t> &perm, int64_t split_tail, int32_t block_items, int32_t block_pts, int32_t reg_r, CloudPlanHost &out);
+                     const std::vector<int32_t> &perm, int64_t split_tail, int32_t block_items,
+                     int32_t block_pts, int32_t reg_r, CloudPlanHost &out);
 
 // ---------------------------------------------------------------------------
 // kernel launchers
@@ -606,6 +607,7 @@ constexpr int32_t kCloudWide = 1, kCloudWeighted = 2;   // traits of a set, see 
 constexpr int64_t kSplitTailPerSm = 4;
 constexpr int kOverlapMaxRows = 128;      // partial rows of a block of several items
 constexpr int kOverlapMaxBlockItems = 32;
+constexpr int kCloudStagePts = 2048;      // points of the staging buffer of a J block
 cudaError_t launch_cloud_pack(const float *x, const float *y, const float *z,
                               const float *sigma, const float *w, const int64_t *src_off,
                               const int32_t *perm, const int64_t *poff, int64_t n, int dim,

@@ -117,11 +117,10 @@ CloudPlanChoice choose_cloud_plan(const CloudStore &c) {
   // Blocks of about 1/60 of the points: 1800 tiles, 12 per SM before the last ones
   // are split (256 clouds of 64-128 points: 420 points a block 126 us, 256 140,
   // 768 134); at least 384, below which a small set's launch is all tiles (48
-  // clouds of 20-60 points: 8.2 us with 384, 10.2 with 64); at most kCloudBlockPts,
-  // which one staging window holds.
-  constexpr int64_t kCloudBlockPts = 2048;
+  // clouds of 20-60 points: 8.2 us with 384, 10.2 with 64); at most kCloudStagePts,
+  // which the staging buffer holds.
   const int64_t want = (c.total_pts / 60 + 3) / 4 * 4;
-  ch.block_pts = (int32_t)std::min(std::max<int64_t>(want, 384), kCloudBlockPts);
+  ch.block_pts = (int32_t)std::min<int64_t>(std::max<int64_t>(want, 384), kCloudStagePts);
   // Items of a block: 8, and twice as many while whole blocks of them make more
   // than kMostTiles tiles.  Sets of few small clouds run best in eights (700 of 20
   // points 88 us, in sixteens 93; 32 of them 6.2 us, 8.0); those of many spend their

@@ -63,7 +63,6 @@ namespace ap {
 namespace {
 
 constexpr int kThreads = 128;
-constexpr int kStagePts = 2048;      // points of the staging buffer, at most
 constexpr int kMaxBlockItems = kOverlapMaxBlockItems;
 constexpr float kTwoLn2 = 1.3862943611198906f;
 
@@ -256,8 +255,9 @@ overlap_kernel(Params P) {
     const int j_pts = 4 * c.j_grps;
     if (MODE == COVER && threadIdx.x == 0) fetch(s_ctx + (cur ^ 1), pop());
 
-    // the J block goes through the staging buffer in windows of stage_cap
-    // points (one, unless an item is larger)
+    // the J block goes through the staging buffer at once, or an item larger than
+    // that (a block by itself, so that every plan cuts it alike) in windows of
+    // stage_cap points
     for (int w0 = 0; MODE != COVER && (w0 == 0 || w0 < j_pts); w0 += P.stage_cap) {
       const int w_pts = min(P.stage_cap, j_pts - w0);
       if (threadIdx.x == 0) {
@@ -997,7 +997,7 @@ cloud_self_kernel(const float4 *__restrict__ pts, const float *__restrict__ lw,
 template <int DIM, int MODE, int SCORE = 0>
 cudaError_t launch_r(const CloudStore &cs, const UnitQueue &queue, Params &P, cudaStream_t s) {
   constexpr int kPart = part_size<MODE>();
-  P.stage_cap = MODE == COVER ? 0 : (std::min(cs.max_pts, kStagePts) + 3) & ~3;
+  P.stage_cap = MODE == COVER ? 0 : (std::min(cs.max_pts, kCloudStagePts) + 3) & ~3;
   P.part_floats = MODE == COVER ? 0 : ((cs.max_rows * cs.max_items * kPart + 3) & ~3);
   const size_t smem = (size_t)P.stage_cap * (DIM == 3 ? 20 : 16) + (size_t)P.part_floats * 4 +
                       kMaxBlockItems * sizeof(int4) + 8 + 2 * sizeof(TileCtx) + 16;

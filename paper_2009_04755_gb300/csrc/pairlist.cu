@@ -7,7 +7,7 @@
 // list mode puts tile t's transform and outputs at index t; the transform
 // acts on b, as it acts on the second item of a packed pair.  A pair listed
 // in packed order (a < b) therefore gets exactly the operations, and the
-// bits, of the all-pairs run.
+// bits, of the all-pairs run (of a plan of the same points per lane).
 //
 // Vectors run over the resident centred rows (split BF16 or FP32 copy), the
 // same three products per column as the tensor-core Gram, summed in FP32 over
@@ -254,6 +254,9 @@ ap_status cloud_list_plan(ap_items *it, const int32_t *pi, const int32_t *pj, in
   for (int64_t k = 0; k < n_pairs; ++k) {
     tiles[2 * k] = c.h_iperm[pi[k]];
     tiles[2 * k + 1] = c.h_iperm[pj[k]];
+    // sets stored by size (3-D, without transforms): as the all-pairs run takes
+    // them, the earlier in the storage first
+    if (c.sorted && tiles[2 * k] > tiles[2 * k + 1]) std::swap(tiles[2 * k], tiles[2 * k + 1]);
   }
   // (a pageable source: staged before the call returns)
   AP_TRY(cudaMemcpyAsync(c.d_list_tiles, tiles.data(), tiles.size() * 4, cudaMemcpyHostToDevice, s));

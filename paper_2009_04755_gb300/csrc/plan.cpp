@@ -141,7 +141,10 @@ void make_cloud_plan(const std::vector<int64_t> &poff, const std::vector<int64_t
                      const std::vector<int32_t> &perm, int64_t split_tail, int32_t block_items,
                      int32_t block_pts, int32_t reg_r, CloudPlanHost &out) {
   out = CloudPlanHost();
-  make_blocks(poff, cnt, block_items, block_pts, reg_r, kOverlapMaxRows, out.bstart);
+  // several items fit the staging buffer: a window that cut one of them would
+  // sum it in another order than other plans do, and lose its boxes
+  make_blocks(poff, cnt, block_items, std::min(block_pts, kCloudStagePts), reg_r,
+              kOverlapMaxRows, out.bstart);
   const int64_t nb = (int64_t)out.bstart.size() - 1, n = (int64_t)cnt.size();
   out.items.resize((size_t)n * 4);
   out.bmeta.reserve((size_t)(nb + n) * 8);

@@ -290,66 +290,65 @@ extern "C" ap_status ap_tune(ap_items *it, int32_t mode, void *stream, ap_plan *
   const int32_t rmin = min_reg_r(c);
   for (int32_t rr : {2, 4}) {
     if (rr < rmin) continue;
-    for (int32_t bp : {2048, 4096, 8192}) {
-      for (int32_t bi : {2, 4, 8, 16, 32}) {
-        if (e != cudaSuccess || st != AP_OK) break;
-        CloudPlanHost plan;
-        make_cloud_plan(c.h_poff, cnt, c.h_perm, 0, bi, bp, rr, plan);
-        const std::vector<int32_t> &bstart = plan.bstart, &tiles = plan.tiles;
-        const int64_t nt = (int64_t)tiles.size() / 2;
-        std::vector<double> cost(nt);
-        double total = 0;
-        for (int64_t t = 0; t < nt; ++t) {
-          cost[t] = tile_cost(bstart, cnt, tiles[2 * t], tiles[2 * t + 1]);
-          total += cost[t];
-        }
-        // evenly spread sample of about `budget` point pairs, at least a few
-        // tiles per SM
-        int64_t stride = 1;
-        if (total > budget) stride = (int64_t)std::ceil(total / budget);
-        stride = std::min<int64_t>(stride, std::max<int64_t>(1, nt / (8LL * num_sms())));
-        std::vector<int32_t> sample;
-        double scost = 0;
-        for (int64_t t = 0; t < nt; t += stride) {
-          sample.push_back(tiles[2 * t]);
-          sample.push_back(tiles[2 * t + 1]);
-          scost += cost[t];
-        }
-        plan.tiles.swap(sample);
-        // a shallow copy of the set with the sample's plan
-        free_cloud_plan(cand);
-        cand = c;
-        cand.d_bmeta = cand.d_desc = cand.d_items = cand.d_tiles = nullptr;
-        cand.block_items = bi;
-        cand.block_pts = bp;
-        cand.reg_r = rr;
-        st = upload_cloud_plan(cand, plan, s);
-        if (st != AP_OK) break;
-        auto launch = [&]() {
-          UnitQueue q;
-          const cudaError_t taken = take_queue(it, s, &q);
-          if (taken != cudaSuccess) return taken;
-          return mode == 0 ? launch_overlap(cand, nullptr, d_out, 0, q, s)
-                           : launch_overlap_grad_q(cand, q, nullptr, nullptr, d_g, d_out, 0.f, 0.f,
-                                                   nullptr, nullptr, s);
-        };
-        float ms_best = 1e30f;
-        e = launch();
-        for (int rep = 0; rep < 2 && e == cudaSuccess; ++rep) {
-          e = cudaEventRecord(e0, s);
-          if (e == cudaSuccess) e = launch();
-          if (e == cudaSuccess) e = cudaEventRecord(e1, s);
-          if (e == cudaSuccess) e = cudaEventSynchronize(e1);
-          float ms = 0;
-          if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, e0, e1);
-          ms_best = std::min(ms_best, ms);
-        }
-        if (e != cudaSuccess) break;
-        const double rate = scost / (ms_best * 1e-3);
-        if (rate > best_rate) {
-          best_rate = rate;
-          best = {bi, bp, rr, c.sorted};
-        }
+    const int32_t bp = kCloudStagePts;           // more makes no other blocks
+    for (int32_t bi : {2, 4, 8, 16, 32}) {
+      if (e != cudaSuccess || st != AP_OK) break;
+      CloudPlanHost plan;
+      make_cloud_plan(c.h_poff, cnt, c.h_perm, 0, bi, bp, rr, plan);
+      const std::vector<int32_t> &bstart = plan.bstart, &tiles = plan.tiles;
+      const int64_t nt = (int64_t)tiles.size() / 2;
+      std::vector<double> cost(nt);
+      double total = 0;
+      for (int64_t t = 0; t < nt; ++t) {
+        cost[t] = tile_cost(bstart, cnt, tiles[2 * t], tiles[2 * t + 1]);
+        total += cost[t];
+      }
+      // evenly spread sample of about `budget` point pairs, at least a few
+      // tiles per SM
+      int64_t stride = 1;
+      if (total > budget) stride = (int64_t)std::ceil(total / budget);
+      stride = std::min<int64_t>(stride, std::max<int64_t>(1, nt / (8LL * num_sms())));
+      std::vector<int32_t> sample;
+      double scost = 0;
+      for (int64_t t = 0; t < nt; t += stride) {
+        sample.push_back(tiles[2 * t]);
+        sample.push_back(tiles[2 * t + 1]);
+        scost += cost[t];
+      }
+      plan.tiles.swap(sample);
+      // a shallow copy of the set with the sample's plan
+      free_cloud_plan(cand);
+      cand = c;
+      cand.d_bmeta = cand.d_desc = cand.d_items = cand.d_tiles = nullptr;
+      cand.block_items = bi;
+      cand.block_pts = bp;
+      cand.reg_r = rr;
+      st = upload_cloud_plan(cand, plan, s);
+      if (st != AP_OK) break;
+      auto launch = [&]() {
+        UnitQueue q;
+        const cudaError_t taken = take_queue(it, s, &q);
+        if (taken != cudaSuccess) return taken;
+        return mode == 0 ? launch_overlap(cand, nullptr, d_out, 0, q, s)
+                         : launch_overlap_grad_q(cand, q, nullptr, nullptr, d_g, d_out, 0.f, 0.f,
+                                                 nullptr, nullptr, s);
+      };
+      float ms_best = 1e30f;
+      e = launch();
+      for (int rep = 0; rep < 2 && e == cudaSuccess; ++rep) {
+        e = cudaEventRecord(e0, s);
+        if (e == cudaSuccess) e = launch();
+        if (e == cudaSuccess) e = cudaEventRecord(e1, s);
+        if (e == cudaSuccess) e = cudaEventSynchronize(e1);
+        float ms = 0;
+        if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, e0, e1);
+        ms_best = std::min(ms_best, ms);
+      }
+      if (e != cudaSuccess) break;
+      const double rate = scost / (ms_best * 1e-3);
+      if (rate > best_rate) {
+        best_rate = rate;
+        best = {bi, bp, rr, c.sorted};
       }
     }
   }

@@ -226,3 +226,41 @@ def test_pearson_list_groups_and_slices(ap, oracle_lib, prec, D):
         got = it.run_pairs_list(pi, pj, ap.AP_FN_PEARSON, prec).cpu().numpy()
         assert np.all(np.abs(got - ref) <= tol), float((np.abs(got - ref) / tol).max())
     it.close()
+
+
+@pytest.mark.parametrize("dim,sizes", [(3, (2, 150)), (3, (30, 2600)), (2, (2, 150)), (2, (700, 2600))])
+@pytest.mark.parametrize("weights", [False, True])
+def test_bits_of_a_pair_in_every_plan_and_list(ap, dim, sizes, weights):
+    """Blocks of one item and of thirty-two, plans that ask for more points than
+    are staged at a time, sets stored by size, pieces that share warps, with
+    boxes and without: cost, scores, gradient and the adjoint's cost."""
+    rng = np.random.default_rng(dim + sizes[1])
+    n = 40 if sizes[1] < 1000 else 14
+    sz = rng.integers(sizes[0], sizes[1] + 1, n)
+    sz[:3] = [sizes[0], sizes[1], (sizes[0] + sizes[1]) // 2]
+    off = np.concatenate([[0], np.cumsum(sz)]).astype(np.int64)
+    f = lambda lo, hi: rng.uniform(lo, hi, int(off[-1])).astype(np.float32)
+    c = {"dim": dim, "offsets": off, "x": f(-1, 1), "y": f(-1, 1),
+         "z": f(-1, 1) if dim == 3 else None, "sigma": f(0.05, 0.1),
+         "weight": f(0.5, 1.5) if weights else None}
+    pi, pj = np.triu_indices(n, 1)
+    fns = (ap.AP_FN_OVERLAP, ap.AP_FN_GMM_L2, ap.AP_FN_BHATTACHARYYA)
+    prm = torch.randn(len(pi), 3, generator=torch.Generator("cuda").manual_seed(1),
+                      device="cuda") * 0.1 if dim == 2 else None
+
+    def results(it, listed):
+        out = [it.run_pairs_list(pi, pj, fn) if listed else it.run_pairs(fn) for fn in fns]
+        if dim == 2:
+            out += it.backward_list(pi, pj, prm) if listed else it.backward(prm)
+        return out
+
+    with ap.Items.from_clouds(c) as it:
+        ref = results(it, False)
+        got = {"list": results(it, True)}
+        for plan in [(1, 64, 4), (5, 300, 4), (32, 8192, 4), (32, 2048, 4)]:
+            it.set_plan(*plan)
+            got[plan] = results(it, False)
+        assert it.last_device_error() == 0
+    for key, out in got.items():
+        for k, (a, b) in enumerate(zip(ref, out)):
+            assert torch.equal(a, b), (key, k)

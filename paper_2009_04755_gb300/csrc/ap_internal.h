@@ -330,12 +330,11 @@ struct NvtxRange {
 namespace ap {
 // a captured launch sequence, replayed with cudaGraphLaunch
 struct GraphKey {
-  const void *a, *b, *c, *d;       // buffers the sequence reads / writes
+  const void *a, *b, *c;           // buffers the sequence reads / writes
   float eta, fmin;
   int32_t n;
   bool operator==(const GraphKey &o) const {
-    return a == o.a && b == o.b && c == o.c && d == o.d && eta == o.eta &&
-           fmin == o.fmin && n == o.n;
+    return a == o.a && b == o.b && c == o.c && eta == o.eta && fmin == o.fmin && n == o.n;
   }
 };
 struct GraphEntry {
@@ -503,10 +502,8 @@ cudaError_t launch_slice_finalize(const double *part, const double *part_c, int6
                                   int64_t D, double *delta, double *ss, double *rs, double *out,
                                   cudaStream_t s);
 cudaError_t launch_gram_f32(const float *C, int64_t n, int64_t Dp, const double *rs,
-                            const int32_t *tiles, int64_t n_tiles, int32_t *queue,
-                            void *out, int coverage, int64_t row0, int64_t n_total,
-                            cudaStream_t s, const double *delta = nullptr,
-                            int64_t D = 0);
+                            const int32_t *tiles, int64_t n_tiles, int32_t *queue, void *out,
+                            int coverage, const double *delta, int64_t D, cudaStream_t s);
 // tensor-core split-BF16 Gram (gram_tc.cu)
 constexpr int kTcTileM = 128;    // rows of the I block per tile
 constexpr int kTcTileN = 256;    // rows of the J block per tile

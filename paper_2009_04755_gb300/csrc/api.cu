@@ -598,7 +598,7 @@ ap_status ap_run_pairs(ap_items *it, int32_t fn, int32_t precision, const float 
       it->stats.tile_n = kTcTileN;
     } else {
       AP_TRY(launch_gram_f32(v.d_c32, v.n, v.Dp, v.d_rs, v.d_tiles_f32, v.n_tiles_f32,
-                             it->d_queue, out, cover, 0, v.n, s, v.d_delta_all, v.D));
+                             it->d_queue, out, cover, v.d_delta_all, v.D, s));
       it->stats.tiles = v.n_tiles_f32;
       it->stats.tile_m = 128;
       it->stats.tile_n = 128;
@@ -655,7 +655,7 @@ ap_status ap_ascent(ap_items *it, float *params, int32_t n_steps, float eta, flo
   if (!params) return AP_ERR_INVALID_ARG;
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   // the n_steps fused steps are replayed as one CUDA graph
-  GraphKey key{params, f_out, flags, nullptr, eta, fmin, n_steps};
+  GraphKey key{params, f_out, flags, eta, fmin, n_steps};
   ap_items *h = it;
   return run_graphed(it, key, s, [h, params, n_steps, eta, fmin, f_out, flags](cudaStream_t cs) {
     // captured: the first head cleared here, each other by the step before

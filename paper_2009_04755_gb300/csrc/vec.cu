@@ -806,8 +806,7 @@ cudaError_t launch_slice_finalize(const double *part, const double *part_c, int6
 
 cudaError_t launch_gram_f32(const float *C, int64_t n, int64_t Dp, const double *rs,
                             const int32_t *tiles, int64_t n_tiles, int32_t *queue, void *out,
-                            int coverage, int64_t, int64_t, cudaStream_t s, const double *delta,
-                            int64_t D) {
+                            int coverage, const double *delta, int64_t D, cudaStream_t s) {
   if (n_tiles <= 0) return cudaSuccess;
   cudaError_t e = cudaMemsetAsync(queue, 0, sizeof(int32_t), s);
   if (e != cudaSuccess) return e;

@@ -185,8 +185,13 @@ typedef struct ap_plan {
   /* vector sets only: 0 runs each 128 x 256 tile over all columns in one
    * unit; k >= 1 splits every tile's columns into k ranges and runs them
    * range by range inside waves of one tile per SM, so the tiles in flight
-   * read the same columns and share them in L2; the partial Grams meet in
-   * FP64 in the output, which a last pass scales by rs_i rs_j.  The default
+   * read the same columns and share them in L2.  A last pass scales the sums of
+   * a pair's ranges by rs_i rs_j.  With CTA pairs (mma_ctas 2), ranges of at
+   * most 16384 columns and k n (n - 1) / 2 floats within 256 MB, the partial
+   * Grams are stored in FP32 planes, which the handle allocates at creation and
+   * in ap_set_plan and keeps, and the pass adds them in order: runs repeat their
+   * bits, and a run that leaves early gives NaN.  Else, and where that
+   * allocation fails, they meet in FP64 in the output.  The default
    * (set at creation, and by ap_set_plan with k_split = -1): ranges of at most
    * 16384 and at least 64 columns, as many as fill whole rounds of the units
    * that run at once; 0 where that gives one range */
@@ -246,8 +251,12 @@ ap_status ap_update_items(ap_items *items, const float *data, int32_t data_on_ho
  *        transform applied to the second item j.
  *   fn = AP_FN_PEARSON: vectors; out double[P]; precision selects the Gram
  *        path (the representation must have been built at creation).
+ *        AP_PREC_FP32 adds the FP32 sums of column ranges in FP64 in no fixed
+ *        order (exact, so without effect, unless they differ in size by 2^28).
  *   fn = AP_FN_COVERAGE: any kind; out int32[P] is incremented.
- *   fn = AP_FN_COSINE: sparse vectors; out double[P].
+ *   fn = AP_FN_COSINE: sparse vectors; out double[P].  FP32 products and tile
+ *        sums meet in FP64 in no fixed order: runs may differ by a few units of
+ *        FP64's last place (20 of 32,640 pairs by 3.4e-16 of their value).
  *   fn = AP_FN_GMM_L2, AP_FN_BHATTACHARYYA: clouds; out float[P]; params as
  *        for the overlap.  The first call of each builds a re-scaled copy of
  *        the storage (16 bytes a point, 20 in 3-D) and, for the L2
@@ -551,8 +560,10 @@ ap_status ap_pipe_rate(int32_t pipe, double *per_clk_per_sm, double *per_s, doub
  *   data: device float[n_items][ld] (row-major, dim <= ld values per row,
  *         ld = 0 means ld = dim), caller-owned, read only;
  *   out:  device double[n_items(n_items-1)/2], packed as above, written.
- * Same arithmetic as ap_run_pairs(AP_FN_PEARSON, AP_PREC_FP32): FP64 mean and
- * norm per item, FP32 centring and Gram, FP64 scaling.  It calls no
+ * As ap_run_pairs(AP_FN_PEARSON, AP_PREC_FP32): FP64 mean and norm per item,
+ * FP32 centring and Gram, FP64 scaling; but a pair's products are summed over
+ * the whole row in FP32, where that call sums column ranges and adds them in
+ * FP64 (a third of the error at 65,536 columns).  It calls no
  * cudaMalloc, cudaFree or other allocating routine: its working memory (item
  * means, inverse norms, the tile-queue counter) is one file-scope
  * `static __device__` array of AP_NOALLOC_SCRATCH_BYTES bytes that every GPU

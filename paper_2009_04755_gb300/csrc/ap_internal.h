@@ -73,15 +73,20 @@ __device__ __forceinline__ double widen(float x) {
 //
 // What boxes save hangs on how far the Gaussians reach against the extent of
 // the items; looking at them costs 2-6%.  A set is boxed from a mean of
-// kBoxedMean points on (over points, so that large items count): clouds over
-// [-1, 1]^2 with sigma 0.01-0.03 / 0.02-0.05 ran 0.98x / 0.97x as fast with
-// boxes at 200-300 points, 1.08x / 0.98x at 400-600, 1.17x / 0.98x at 600-760
-// under transforms, 1.38x / 1.09x at 800-1200 (2-D with strips of the extent;
-// strips by rank came after); over [-1, 1]^3 1.15x / 1.00x at 800-1200 and 1.77x
-// / 1.08x at 2000-3000; GMM L2 of 256 particles of 1000-2000
-// points 22.1 -> 12.1 ms.  Terms of one size then follow one another in the
-// block sums: errors against 64 bits 4.8e-8 -> 5.1e-8 (2-D overlap; 5.9e-8 with
-// plain sums over blocks), 5.5e-8 -> 5.6e-8 (3-D), 2.7e-8 -> 2.5e-8 (GMM L2).
+// kBoxedMean points on (over points, so that large items count).  Times without
+// boxes over those with them, clouds over [-1, 1]^dim with sigma 0.01-0.03 /
+// 0.02-0.05:
+//   points      2-D overlap    its adjoint    2-D GMM L2     3-D overlap
+//   200-300     0.98 / 0.96    1.02 / 0.97    1.01 / 0.95    1.15 / 0.99
+//   400-600     1.18 / 0.96    1.19 / 0.98    1.23 / 1.00    0.98 / 0.96
+//   600-760     1.32 / 1.04    1.30 / 1.03    1.34 / 1.06    1.04 / 0.97
+//   800-1200    1.52 / 1.16    1.50 / 1.14    1.54 / 1.18    1.15 / 1.00
+//   2000-3000   2.06 / 1.33    2.06 / 1.32    2.13 / 1.37    1.80 / 1.10
+// and 50-5000 lognormal (1240 over points) 1.31 / 1.08 in 2-D, 1.16 / 1.02 in
+// 3-D; GMM L2 of 256 particles of 1000-2000 points 22.1 -> 12.1 ms.  Putting the
+// points in order takes part of a set's creation (1000 lognormal 3-D clouds 2.0
+// -> 2.3 ms).  Terms of one size then follow one another, which the sums allow for
+// (kBlockwise, kTree).
 // An item of up to kCullPoints fills a warp or little more: no part of it is far
 // from the rest.
 constexpr int64_t kCullPoints = 160;

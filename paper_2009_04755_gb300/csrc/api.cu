@@ -166,8 +166,8 @@ ap_status build_cloud_plan(ap_items *it, const CloudPlanChoice &ch, cudaStream_t
   std::vector<int64_t> cnt(c.n);
   for (int64_t s = 0; s < c.n; ++s) cnt[s] = c.h_size[c.h_perm[s]];
   CloudPlanHost h;
-  make_cloud_plan(c.h_poff, cnt, c.h_perm, kSplitTailPerSm * num_sms(), ch.block_items, ch.block_pts,
-                  ch.reg_r, h);
+  make_cloud_plan(c.h_poff, cnt, c.h_perm, kSplitTailPerSm * num_sms(), ch.block_items,
+                  ch.block_pts, ch.reg_r, h);
   free_cloud_plan(c);
   c.fits->clear();
   AP_TRY_ST(upload_cloud_plan(c, h, s));

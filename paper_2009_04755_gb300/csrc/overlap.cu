@@ -47,8 +47,9 @@
 // plain FMAs for its three-operand sums.  Measured before / after with the
 // fragments that share warps and the split tail of the tile list: 256 2-D
 // clouds of 64-128 points 197 / 119 us, 1000 lognormal 3-D clouds 50.8 / 41.2
-// ms, the L2 score of 256 clouds of 1000-2000 points 27.2 / 22.1 ms, one
-// adjoint step of 400 clouds of 100-400 points 2.12 / 1.92 ms.
+// ms, the L2 score of 256 clouds of 1000-2000 points 27.2 / 22.1 ms (12.1 with
+// the boxes of large sets, kBoxedMean), one adjoint step of 400 clouds of 100-400
+// points 2.12 / 1.92 ms.
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
@@ -731,9 +732,10 @@ constexpr float kSharedMin = 8.6736174e-19f, kSharedMax = 5.7646075e17f;
 // in pairs (two per thread and trip), and its boxes.  Larger items are put in
 // order first, so that 128 and 32 points in a row are near each other.  In 2-D
 // sorted by y and cut into strips of whole warps' 128 points, each strip sorted
-// by x, each 64 points by y: strips of the extent, which leave a warp's points
-// over two or three cells, kept more blocks (GMM L2 of 256 particles of 1000-2000
-// points 13.7 ms, now 12.1).  In 3-D rows of the extent, by x: blocks thin in x are
+// by x (the sort-tile-recursive packing of R-trees: Leutenegger, Lopez and
+// Edgington, 1997), each 64 points by y: strips of the extent, which leave a
+// warp's points over two or three cells, kept more blocks (GMM L2 of 256 particles
+// of 1000-2000 points 13.7 ms, now 12.1).  In 3-D rows of the extent, by x: blocks thin in x are
 // passed over more often than cubes where items are cut once or twice an axis
 // (strips by rank ran the lognormal set 1% slower).  Key and index are one
 // word, sorted in shared memory (a bitonic network over the next power of two).

@@ -664,8 +664,9 @@ namespace ap {
 
 // Units of the streamed run: column m holds the pairs (a <= m, m) of macros,
 // addressed directly in the resident arrays (row block = item block), as
-// CTA-pair units in waves like the resident schedule (column ranges of
-// ~16384 columns, two units per SM at least).  With C column chunks, each
+// CTA-pair units in waves like the resident schedule (column ranges of at most
+// 16384 columns, as many as fill whole rounds of units: default_k_split).  With
+// C column chunks, each
 // (chunk, column) entry holds those pairs over the chunk's columns only.
 static ap_status build_stream_units(VecStore &v, int64_t C) {
   const int64_t M = (v.n + kMacro - 1) / kMacro;

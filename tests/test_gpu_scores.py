@@ -22,7 +22,7 @@ def _gpu(ap, c, fn, params=None, twice=False):
     with ap.Items.from_clouds(c) as it:
         prm = None if params is None else torch.as_tensor(params, dtype=torch.float32).cuda()
         out = it.run_pairs(fn, params=prm).cpu().numpy()
-        if twice:                                  # the cached storage and graph
+        if twice:                                  # the cached storage
             again = it.run_pairs(fn, params=prm).cpu().numpy()
             np.testing.assert_array_equal(again, out)
         assert it.last_device_error() == 0

@@ -1,6 +1,6 @@
-"""GPU checks of the tile-plan autotuner and of CUDA-graph replay: any plan
-the tuner can pick gives results within tolerance of the oracle, replays are
-bit-identical to direct launches, and explicit plans round-trip."""
+"""GPU checks of the tile-plan autotuner and of the ascent's CUDA graph: any
+plan the tuner can pick gives results within tolerance of the oracle, replays
+and repeated launches are bit-identical, and explicit plans round-trip."""
 import numpy as np
 import pytest
 
@@ -31,7 +31,7 @@ def test_tune_then_parity_2d(ap, oracle_lib):
         assert plan["reg_r"] in (2, 4)
         assert it.plan()["block_items"] == plan["block_items"]
         f1 = it.run_pairs().cpu().numpy()
-        f2 = it.run_pairs().cpu().numpy()          # replayed from the cached graph
+        f2 = it.run_pairs().cpu().numpy()
     check_overlap(f1, ref, kappa, bound, "tuned 2d")
     assert np.array_equal(f1, f2)
 
@@ -78,11 +78,19 @@ def test_graph_replay_respects_new_buffers(ap):
     with ap.Items.from_clouds(c) as it:
         a = it.run_pairs().clone()
         out = torch.zeros_like(a)
-        it.run_pairs(out=out)                     # a new output buffer: a new graph
+        it.run_pairs(out=out)                     # a new output buffer
         assert torch.equal(a, out)
-        it.set_plan(4, 2048, 4)                   # a new plan invalidates the graphs
+        first, second = (torch.zeros(len(a), 3, device="cuda") for _ in range(2))
+        p1, f1, _ = it.ascent(first, 3, 1e-3)     # captured for these buffers
+        p2, f2, _ = it.ascent(second, 3, 1e-3)    # other parameters: another graph
+        assert torch.equal(p1, p2) and torch.equal(f1, f2) and p1 is first and p2 is second
+        assert bool((first != 0).any())
+        it.set_plan(4, 2048, 2)                   # a new plan invalidates the graphs
         b = it.run_pairs()
         assert torch.allclose(a, b, rtol=1e-5, atol=0)
+        p3, f3, _ = it.ascent(first.zero_(), 3, 1e-3)
+        torch.testing.assert_close(p3, p2, rtol=1e-4, atol=1e-6)
+        torch.testing.assert_close(f3, f2, rtol=1e-5, atol=0)
 
 
 def test_handles_of_one_kernel_keep_their_launch_shapes(ap):

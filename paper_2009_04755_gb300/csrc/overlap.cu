@@ -680,7 +680,8 @@ overlap_kernel(Params P) {
       const int r0 = c.job0 >= 0 ? mi.w : 0, r1 = r0 + cloud_rows(mi.y, R);
       for (int row = r0; row < r1; ++row) {
         const float *src = s_part + ((size_t)row * nJ + jl) * kPart;
-        sF += (double)src[0] + (double)src[kPart - 1];
+        // (a sum that left the FP32 range has no rounding error to add)
+        sF += (double)src[0] + (isinf(src[0]) ? 0.0 : (double)src[kPart - 1]);
         if (MODE == GRAD) { sX += (double)src[1]; sY += (double)src[2]; sT += (double)src[3]; }
       }
       if (MODE == FWD || MODE == FWD_T) {

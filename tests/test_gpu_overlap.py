@@ -292,3 +292,29 @@ def test_tiles_of_many_small_clouds(ap, n, items, tiles):
         f = it.run_pairs()
         it.set_plan(8, 384, 4)
         assert torch.equal(it.run_pairs(), f)
+
+
+@pytest.mark.parametrize("dim", [2, 3])
+def test_sums_beyond_the_fp32_range_are_infinite(ap, dim):
+    """Weights whose products leave the range: infinity for the pairs that hold
+    two of them, whatever way the sums go, and numbers for the others."""
+    sizes = np.array([1, 2, 30, 200, 1500, 3, 40, 160])
+    off = np.concatenate([[0], np.cumsum(sizes)]).astype(np.int64)
+    rng = np.random.default_rng(8)
+    pts = rng.uniform(-0.01, 0.01, (3, int(off[-1]))).astype(np.float32)
+    w = np.ones(int(off[-1]), np.float32)
+    heavy = [0, 2, 3, 4]
+    w[off[heavy]] = 1e30
+    c = {"dim": dim, "offsets": off, "x": pts[0], "y": pts[1], "z": pts[2] if dim == 3 else None,
+         "sigma": np.full(int(off[-1]), 0.5, np.float32), "weight": w}
+    pi, pj = np.triu_indices(len(sizes), 1)
+    both = torch.from_numpy(np.isin(pi, heavy) & np.isin(pj, heavy)).cuda()
+    with ap.Items.from_clouds(c) as it:
+        fs = [it.run_pairs(), it.run_pairs_list(pi, pj)]
+        if dim == 2:
+            zero = torch.zeros(len(pi), 3, device="cuda")
+            fs += [it.run_pairs(params=zero), it.backward(zero)[1]]
+        it.set_plan(4, 256, 2)
+        fs.append(it.run_pairs())
+        for f in fs:
+            assert torch.all(torch.isposinf(f[both])) and torch.all(torch.isfinite(f[~both]))
